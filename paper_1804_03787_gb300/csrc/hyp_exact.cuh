@@ -2,12 +2,12 @@
 //
 // GB300 runs FP64 at a small fraction of its FP32 rate, and a 4-point
 // homography in FP64 was the bottleneck of the per-window fit.  Here the
-// projective-basis solution H ~ B adj(A) (see minimal_h in
-// kernels_planes.cu) is formed exactly in 128-bit integers -- window-local
-// coordinates keep every entry below 2^89 -- and the FP32 evaluation form is
-// derived from exact integer numerators with one rounding each; the
-// translation, which needs ~1e-7 px absolute accuracy on flows of hundreds of
-// pixels, is split into hi + lo with an exact integer remainder.
+// projective-basis solution H ~ B adj(A) is formed exactly in 128-bit
+// integers -- frames up to 32767 px a side keep every entry below 2^89 -- and
+// the FP32 evaluation form is derived from exact integer numerators with one
+// rounding each; the translation, which needs ~1e-7 px absolute accuracy on
+// flows of hundreds of pixels, is split into hi + lo with an exact integer
+// remainder.
 #pragma once
 
 #include <stdint.h>
@@ -55,52 +55,59 @@ __host__ __device__ __forceinline__ float i128_to_float(i128 x) {
 }
 
 // 4-point homography, exact: H = B adj(A) with the projective bases of the
-// source points (A) and target points (B); window-local integer coordinates
-// (|source| <= 48, |target| < 2^15).
+// source points (A) and target points (B); window-local integer coordinates.
+// With every point taken relative to the fourth pair (p3, q3), the lambdas
+// are the cross products l_k of the other two source points, the target
+// weights the cross products mu_k, sum_k mu_k (q_k - q3) = 0, and
+//   H = T(q3) H' T(-p3),   H' = sum_k w_k (q_k - q3, 1) adj(P')_k,   w_k = mu_k l_i l_j,
+// the same integers as the products with the untranslated points, in 18 wide
+// products instead of 45, most of them on short factors.  Bounds for windows
+// up to 96 px (|l| < 2^14.2) and target differences below 2^23 (frames below
+// 2^15 a side; imported offsets may leave the frame): |mu| < 2^47,
+// |w| < 2^75.4, |H| < 2^110.
 __host__ __device__ inline void minimal_h_exact(const int* px, const int* py, const int* qx, const int* qy,
                                                 i128* H) {
-    int A[9];
-    {
-        const int x1 = px[0], x2 = px[1], x3 = px[2], y1 = py[0], y2 = py[1], y3 = py[2];
-        const int l0 = (y2 - y3) * px[3] + (x3 - x2) * py[3] + (x2 * y3 - x3 * y2);
-        const int l1 = (y3 - y1) * px[3] + (x1 - x3) * py[3] + (x3 * y1 - x1 * y3);
-        const int l2 = (y1 - y2) * px[3] + (x2 - x1) * py[3] + (x1 * y2 - x2 * y1);
-        A[0] = l0 * x1; A[1] = l1 * x2; A[2] = l2 * x3;
-        A[3] = l0 * y1; A[4] = l1 * y2; A[5] = l2 * y3;
-        A[6] = l0;      A[7] = l1;      A[8] = l2;
+    int dx[3], dy[3];
+    int64_t X[3], Y[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        dx[k] = px[k] - px[3];
+        dy[k] = py[k] - py[3];
+        X[k] = qx[k] - qx[3];
+        Y[k] = qy[k] - qy[3];
     }
+    int l[3];
     int64_t mu[3];
-    {
-        const int64_t x1 = qx[0], x2 = qx[1], x3 = qx[2], y1 = qy[0], y2 = qy[1], y3 = qy[2];
-        mu[0] = (y2 - y3) * qx[3] + (x3 - x2) * qy[3] + (x2 * y3 - x3 * y2);
-        mu[1] = (y3 - y1) * qx[3] + (x1 - x3) * qy[3] + (x3 * y1 - x1 * y3);
-        mu[2] = (y1 - y2) * qx[3] + (x2 - x1) * qy[3] + (x1 * y2 - x2 * y1);
+    i128 w[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int i = (k + 1) % 3, j = (k + 2) % 3;
+        l[k] = dx[i] * dy[j] - dx[j] * dy[i];
+        mu[k] = X[i] * Y[j] - X[j] * Y[i];
     }
-    int64_t adj[9];
-    adj[0] = (int64_t)A[4] * A[8] - (int64_t)A[5] * A[7];
-    adj[1] = (int64_t)A[2] * A[7] - (int64_t)A[1] * A[8];
-    adj[2] = (int64_t)A[1] * A[5] - (int64_t)A[2] * A[4];
-    adj[3] = (int64_t)A[5] * A[6] - (int64_t)A[3] * A[8];
-    adj[4] = (int64_t)A[0] * A[8] - (int64_t)A[2] * A[6];
-    adj[5] = (int64_t)A[2] * A[3] - (int64_t)A[0] * A[5];
-    adj[6] = (int64_t)A[3] * A[7] - (int64_t)A[4] * A[6];
-    adj[7] = (int64_t)A[1] * A[6] - (int64_t)A[0] * A[7];
-    adj[8] = (int64_t)A[0] * A[4] - (int64_t)A[1] * A[3];
-    // H = Q diag(mu) adj(A) = Q C with C = diag(mu) adj(A).  Bounds for windows
-    // up to 96 px (|source| <= 48) and frames up to 32767 px (|target| < 2^15):
-    // |A| < 2^19.4, |adj| < 2^39.8, |mu| < 2^32.6, so C needs 128 bits
-    // (< 2^72.4) and |H| < 2^89 (Q holds 16-bit coordinates, last row 1).
-    i128 Cm[9];
+    // H' (its third column is (0, 0, h22))
+    i128 h[3][2] = {}, h22 = (i128)((int64_t)l[0] * l[1] * l[2]) * (mu[0] + mu[1] + mu[2]);
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) Cm[k * 3 + c] = (i128)mu[k] * adj[k * 3 + c];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        H[0 * 3 + c] = Cm[c] * qx[0] + Cm[3 + c] * qx[1] + Cm[6 + c] * qx[2];
-        H[1 * 3 + c] = Cm[c] * qy[0] + Cm[3 + c] * qy[1] + Cm[6 + c] * qy[2];
-        H[2 * 3 + c] = Cm[c] + Cm[3 + c] + Cm[6 + c];
+    for (int k = 0; k < 3; ++k) {
+        const int i = (k + 1) % 3, j = (k + 2) % 3;
+        w[k] = (i128)mu[k] * ((int64_t)l[i] * l[j]);
+        const i128 a = w[k] * (dy[i] - dy[j]), b = w[k] * (dx[j] - dx[i]);
+        h[0][0] += a * X[k];
+        h[0][1] += b * X[k];
+        h[1][0] += a * Y[k];
+        h[1][1] += b * Y[k];
+        h[2][0] += a;
+        h[2][1] += b;
     }
+    H[6] = h[2][0];
+    H[7] = h[2][1];
+    H[8] = h22 - h[2][0] * px[3] - h[2][1] * py[3];
+    H[0] = h[0][0] + h[2][0] * qx[3];
+    H[1] = h[0][1] + h[2][1] * qx[3];
+    H[2] = H[8] * qx[3] - h[0][0] * px[3] - h[0][1] * py[3];
+    H[3] = h[1][0] + h[2][0] * qy[3];
+    H[4] = h[1][1] + h[2][1] * qy[3];
+    H[5] = H[8] * qy[3] - h[1][0] * px[3] - h[1][1] * py[3];
 }
 
 // num / den (den > 0) as hi + lo floats: hi the rounded quotient, lo the

@@ -516,45 +516,6 @@ __device__ __forceinline__ void min_eigvec9(const double (&M)[45], double (&x)[9
     }
 }
 
-// Draws hypothesis k of a window: Philox indices into the N matches; false if
-// the sample is degenerate (three source or three target points collinear).
-// The homography is exact (128-bit integers, see hyp_exact.cuh).
-__device__ __forceinline__ bool draw_hypothesis(const float4* match, int N, int cell, int k, uint32_t tag,
-                                                uint32_t pair_id, uint32_t k0, uint32_t k1, i128* Hk) {
-    const uint4 w = philox((uint32_t)cell, (uint32_t)k, tag, pair_id, k0, k1);
-    const uint32_t idx[4] = {bounded_u32(w.x, (uint32_t)N), bounded_u32(w.y, (uint32_t)N),
-                             bounded_u32(w.z, (uint32_t)N), bounded_u32(w.w, (uint32_t)N)};
-    int px[4], py[4], qx[4], qy[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        // the match coordinates are small exact integers held as floats: adding
-        // 1.5 * 2^23 puts the integer in the low mantissa bits (no conversion op)
-        const float4 m = match[idx[j]];
-        px[j] = __float_as_int(m.x + 12582912.f) - 0x4B400000;
-        py[j] = __float_as_int(m.y + 12582912.f) - 0x4B400000;
-        qx[j] = __float_as_int((m.x + m.z) + 12582912.f) - 0x4B400000;
-        qy[j] = __float_as_int((m.y + m.w) + 12582912.f) - 0x4B400000;
-    }
-    bool degen = false;
-    const int T3[4][3] = {{0, 1, 2}, {0, 1, 3}, {0, 2, 3}, {1, 2, 3}};
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        const int a = T3[t][0], b = T3[t][1], c = T3[t][2];
-        degen |= collinear3(px[a], py[a], px[b], py[b], px[c], py[c]);
-        degen |= collinear3(qx[a], qy[a], qx[b], qy[b], qx[c], qy[c]);
-    }
-    if (degen) return false;
-    minimal_h_exact(px, py, qx, qy, Hk);
-    return true;
-}
-
-// The same out of line (the winner's redraw, once per window: the scoring
-// loop keeps the only inline copy).
-__device__ __noinline__ void draw_hypothesis_ool(const float4* match, int N, int cell, int k, uint32_t tag,
-                                                 uint32_t pair_id, uint32_t k0, uint32_t k1, i128* Hk) {
-    draw_hypothesis(match, N, cell, k, tag, pair_id, k0, k1, Hk);
-}
-
 // The exact hypothesis as doubles in window-local coordinates, oriented like
 // its evaluation form (positive denominator at the window centre) and scaled
 // by a power of two (largest entry in [1, 2)): the FP64 stand-in of the
@@ -576,9 +537,6 @@ __device__ __forceinline__ void exact_local_fp64(const i128* Hk, double* Hl) {
 //   (C) ransac_finish, a group per window: rescoring of the refit (kept unless
 //       it has fewer inliers), the colour-overlap count and the model record.
 
-// Windows with at most this many matches score each hypothesis on one thread.
-constexpr int kLaneScoreMax = 64;
-
 // mef_inlier_pt out of line (loose hypotheses are rare: the callers' loops stay small).
 __device__ __noinline__ bool mef_inlier_pt_ool(const Mef& m, float4 mt, float t2, bool& unc) {
     return mef_inlier_pt(m, mt.x, mt.y, mt.z, mt.w, t2, unc);
@@ -586,105 +544,6 @@ __device__ __noinline__ bool mef_inlier_pt_ool(const Mef& m, float4 mt, float t2
 // The certified test of a match: the FP32 decision, and unc when it is within its rounding bound.
 __device__ __forceinline__ bool cert_inlier(const Mef& m, const float4& mt, float t2, bool& unc) {
     return mef_loose(m) ? mef_inlier_pt_ool(m, mt, t2, unc) : mef_inlier_c(m, mt.x, mt.y, mt.z, mt.w, t2, unc);
-}
-
-// Support of a loose hypothesis (per-match bounds), the warp's lanes over the
-// matches: the FP32 count and the number of uncertain tests, on every lane.
-// Abandoned (x = -1) once even its optimistic count plus the matches left
-// cannot exceed bound.  Out of line: rare, and the scoring loops stay small in
-// the instruction cache.  tests: residual tests done (counter).
-__device__ __noinline__ int2 loose_score_warp(const float4* match, int N, const Mef& m, float t2, int bound,
-                                              int& tests) {
-    const int lane = threadIdx.x & 31;
-    int s2 = 0, u2 = 0;
-    for (int c = 0; c < N; c += 128) {
-        int sl = 0, ul = 0;
-        for (int j = c + lane; j < min(N, c + 128); j += 32) {
-            const float4 mt = match[j];
-            bool unc;
-            sl += mef_inlier_pt(m, mt.x, mt.y, mt.z, mt.w, t2, unc);
-            ul += unc;
-        }
-        s2 += (int)__reduce_add_sync(FULL, (unsigned)sl);
-        u2 += (int)__reduce_add_sync(FULL, (unsigned)ul);
-        tests += min(128, N - c);
-        if (s2 + u2 + max(N - c - 128, 0) <= bound) return make_int2(-1, 0);
-    }
-    return make_int2(s2, u2);
-}
-
-// Support of a loose hypothesis on at most 64 matches (per-match bounds), the
-// warp's lanes over the matches: the FP32 count on every lane, the uncertain
-// tests (bit j of unc: match j) and the FP32 decisions among them (bit j of
-// uin).  Out of line (rare).  tests: residual tests done (counter).
-__device__ __noinline__ int loose_score64(const float4* match, int N, const Mef& m, float t2,
-                                          unsigned long long& unc, unsigned long long& uin) {
-    const int lane = threadIdx.x & 31;
-    int score = 0;
-    unc = 0;
-    uin = 0;
-    for (int c = 0; c < N; c += 32) {
-        const int j = c + lane;
-        bool in = false, u = false;
-        if (j < N) {
-            const float4 mt = match[j];
-            in = mef_inlier_pt(m, mt.x, mt.y, mt.z, mt.w, t2, u);
-        }
-        const unsigned bi = __ballot_sync(FULL, in), bu = __ballot_sync(FULL, u);
-        score += __popc(bi);
-        unc |= (unsigned long long)bu << c;
-        uin |= (unsigned long long)(bu & bi) << c;
-    }
-    return score;
-}
-
-// The exact count of a hypothesis from its FP32 count on at most 64 matches:
-// each uncertain test (bit j of unc) decided again in FP64 with Hl, the
-// hypothesis's exact form, replacing its FP32 decision (bit j of uin).  One
-// thread; nfp64 counts the FP64 decisions.
-__device__ __noinline__ int resolve_uncertain(const float4* match, const double* Hl, float t2, unsigned long long unc,
-                                              unsigned long long uin, int score, int& nfp64) {
-    for (; unc; unc &= unc - 1) {
-        const int j = __ffsll((long long)unc) - 1;
-        const float4 mt = match[j];
-        score += (int)hyp_inlier_fp64(Hl, mt.x, mt.y, mt.z, mt.w, (double)t2) - (int)((uin >> j) & 1ull);
-        ++nfp64;
-    }
-    return score;
-}
-// The same from the 128-bit hypothesis itself (kept in shared memory since it was drawn).
-__device__ __noinline__ int resolve_uncertain_hk(const float4* match, const i128* hk, float t2,
-                                                 unsigned long long unc, unsigned long long uin, int score,
-                                                 int& nfp64) {
-    double Hl[9];
-    {
-        i128 H[9];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) H[q] = hk[q];
-        exact_local_fp64(H, Hl);
-    }
-    return resolve_uncertain(match, Hl, t2, unc, uin, score, nfp64);
-}
-
-// The same with the warp's lanes over the matches (every lane gets the score).
-__device__ __noinline__ int exact_score_warp(const float4* match, int N, const Mef& m, const double* Hl, float t2,
-                                             int& nfp64) {
-    const int lane = threadIdx.x & 31;
-    int score = 0;
-    for (int c = 0; c < N; c += 32) {
-        const int j = c + lane;
-        bool in = false, unc = false;
-        if (j < N) {
-            const float4 mt = match[j];
-            in = cert_inlier(m, mt, t2, unc);
-            if (unc) {
-                in = hyp_inlier_fp64(Hl, mt.x, mt.y, mt.z, mt.w, (double)t2);
-                ++nfp64;
-            }
-        }
-        score += __popc(__ballot_sync(FULL, in));
-    }
-    return score;
 }
 
 // Exact integer of a small integer-valued float: adding 1.5 * 2^23 puts it in
@@ -698,6 +557,350 @@ __device__ __forceinline__ void window_origin(const LevelGeom& g, int cell, int&
     y0 = win_pos(g.gy, g.h, cyw);
     ox = x0 + g.s / 2;
     oy = y0 + g.s / 2;
+}
+
+// The window's matches in raster order, in shared memory, as planes of floats holding exact integers (so a lane
+// loads four consecutive matches with one 16-byte load per plane): the pixel u in window coordinates, and its
+// target u + v relative to the window's reference offset v0.  Entries past N, up to the next multiple of `pad`,
+// are no match's inlier.
+struct Window {
+    float *x, *y, *qx, *qy;
+    int N;
+    float v0x, v0y;
+    float U;     // half the window side: bounds |u|
+    float vq;    // largest component of |u + v - v0|
+    float vmax;  // largest component of |v|
+    __device__ __forceinline__ float4 match(int j) const {
+        const float a = x[j], b = y[j];
+        return make_float4(a, b, (qx[j] + v0x) - a, (qy[j] + v0y) - b);
+    }
+};
+// A target no hypothesis reaches within the inlier radius (its square stays finite for any accepted hypothesis).
+constexpr float kFarTarget = 1e15f;
+// Up to this |u + v - v0|, differences of targets stay below 2^15 and their cross products fit 32 bits.
+constexpr float kFastReach = 16383.f;
+
+// Gathers the window's matches (stage 1: every pixel; stage 2: the residual ones) into planes of `cap` floats.
+template <class G>
+__device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, const LevelGeom& g, int stage, int dir,
+                                              int cell, float* planes, int cap, int pad, Window& w) {
+    const int tid = grp.rank(), s = g.s, W = pv.W;
+    int x0, y0, ox, oy;
+    window_origin<G>(g, cell, x0, y0, ox, oy);
+    const int2* nnf = pv.nnf[dir];
+    const uint8_t* resid = pv.resid[dir];
+    w.x = planes;
+    w.y = planes + cap;
+    w.qx = planes + 2 * cap;
+    w.qy = planes + 3 * cap;
+    int N = 0;
+    for (int base = 0; base < s * s; base += G::size) {
+        const int j = base + tid;
+        bool take = j < s * s;
+        const int yl = j / s, xl = j - yl * s, i = (y0 + yl) * W + x0 + xl;
+        int at = j, total = min(G::size, s * s - base);
+        if (stage != 1) {
+            take = take && resid[i];
+            at = N + grp.scan(take, total);
+        }
+        if (take) {
+            const int2 v = nnf[i];
+            const int ux = x0 + xl - ox, uy = y0 + yl - oy;
+            w.x[at] = (float)ux;
+            w.y[at] = (float)uy;
+            w.qx[at] = (float)(ux + v.x);
+            w.qy[at] = (float)(uy + v.y);
+        }
+        N += total;
+    }
+    w.N = N;
+    w.U = 0.5f * (float)s;
+    grp.sync();
+    // reference offset: the component-wise median of eight matches spread over the list (any value is correct;
+    // one near the window's main motion keeps the rounding bounds of its hypotheses small)
+    float mx = 0.f, my = 0.f;
+    if (N > 0) {
+        const int lane = tid & 31, j = ((2 * (lane & 7) + 1) * N) >> 4;
+        mx = w.qx[j] - w.x[j];
+        my = w.qy[j] - w.y[j];
+    }
+    int rx = 0, ry = 0;
+#pragma unroll
+    for (int l = 0; l < 8; ++l) {
+        const float a = __shfl_sync(FULL, mx, l), b = __shfl_sync(FULL, my, l);
+        const bool before = l < (int)(threadIdx.x & 7);
+        rx += a < mx || (a == mx && before);
+        ry += b < my || (b == my && before);
+    }
+    w.v0x = __shfl_sync(FULL, mx, __ffs(__ballot_sync(FULL, rx == 3)) - 1);
+    w.v0y = __shfl_sync(FULL, my, __ffs(__ballot_sync(FULL, ry == 3)) - 1);
+    grp.sync();
+    float vm = 0.f, vq = 0.f;
+    for (int j = tid; j < N; j += G::size) {
+        const float ax = w.qx[j], ay = w.qy[j], bx = ax - w.v0x, by = ay - w.v0y;
+        vm = fmaxf(vm, fmaxf(fabsf(ax - w.x[j]), fabsf(ay - w.y[j])));
+        vq = fmaxf(vq, fmaxf(fabsf(bx), fabsf(by)));
+        w.qx[j] = bx;
+        w.qy[j] = by;
+    }
+    for (int j = N + tid; j < (N + pad - 1) / pad * pad; j += G::size) {
+        w.x[j] = w.y[j] = 0.f;
+        w.qx[j] = w.qy[j] = kFarTarget;
+    }
+    // integers: exact as keys; the larger of the two decides which bound holds, so one reduction each
+    w.vmax = (float)grp.max((unsigned long long)vm);
+    w.vq = (float)grp.max((unsigned long long)vq);
+    grp.sync();
+}
+
+// ---- hypotheses
+// Four Philox indices into the N matches of a window.
+__device__ __forceinline__ void draw_indices(int N, int cell, int k, uint32_t tag, uint32_t pair_id, uint32_t k0,
+                                             uint32_t k1, int idx[4]) {
+    const uint4 r = philox((uint32_t)cell, (uint32_t)k, tag, pair_id, k0, k1);
+    idx[0] = (int)bounded_u32(r.x, (uint32_t)N);
+    idx[1] = (int)bounded_u32(r.y, (uint32_t)N);
+    idx[2] = (int)bounded_u32(r.z, (uint32_t)N);
+    idx[3] = (int)bounded_u32(r.w, (uint32_t)N);
+}
+
+// Hypothesis k of a window, exact (128-bit integers, hyp_exact.cuh), in window coordinates; false if the sample is
+// degenerate (three source or three target points collinear).
+__device__ __forceinline__ bool draw_exact(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id,
+                                           uint32_t k0, uint32_t k1, i128* Hk) {
+    int idx[4], px[4], py[4], qx[4], qy[4];
+    draw_indices(w.N, cell, k, tag, pair_id, k0, k1, idx);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        px[j] = exact_int(w.x[idx[j]]);
+        py[j] = exact_int(w.y[idx[j]]);
+        qx[j] = exact_int(w.qx[idx[j]] + w.v0x);
+        qy[j] = exact_int(w.qy[idx[j]] + w.v0y);
+    }
+    bool degen = false;
+    const int T3[4][3] = {{0, 1, 2}, {0, 1, 3}, {0, 2, 3}, {1, 2, 3}};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const int a = T3[t][0], b = T3[t][1], c = T3[t][2];
+        degen |= collinear3(px[a], py[a], px[b], py[b], px[c], py[c]);
+        degen |= collinear3(qx[a], qy[a], qx[b], qy[b], qx[c], qy[c]);
+    }
+    if (degen) return false;
+    minimal_h_exact(px, py, qx, qy, Hk);
+    return true;
+}
+
+// A hypothesis in FP32, for scoring: den(u) = c0 + g0 ux + g1 uy (positive at the window centre), the target
+// relative to v0 times den, X(u) = xc + x0 ux + x1 uy and Y(u) likewise, and kap, a bound of everything rounding
+// can do to the inlier test: with n = (X - qx den, Y - qy den), an inlier has |n| < t den, so it passes
+// |n| <= t den + kap as computed, and a match that passes |n| < t den - kap as computed is an inlier.
+struct FastHyp {
+    float g0, g1, c0, kap, x0, x1, xc, pad0, y0, y1, yc, pad1;
+};
+enum { HYP_DEAD = 0, HYP_OK = 1, HYP_LOOSE = 2 };  // degenerate; scored in FP32; the FP32 form says too little
+// t widened by 2^-20: covers the relative roundings of both sides of the comparison (at most 6 units of 2^-24).
+__device__ __forceinline__ float t_above(float t2) { return sqrtf(t2) * (1.f + 9.5367431640625e-07f); }
+__device__ __forceinline__ float t_below(float t2) { return sqrtf(t2) * (1.f - 9.5367431640625e-07f); }
+
+// Draws hypothesis k and solves it in FP32.  Relative to the fourth pair, with the cross products l_k, mu_k of
+// hyp_exact.cuh (exact: floats below 2^24 and 32-bit integers) and rho_k = mu_k / (M l_k), M = sum mu, the form's
+// coefficients are sums over k of rho_k (dy_i - dy_j), rho_k (dx_j - dx_i) and their products with the target
+// differences, normalised to 1 at p3.  The degeneracy test is exact: the eight triangle areas are the l_k, the mu_k
+// and their sums.
+// Rounding, in units of u = 2^-24, first order: mu, M, M l one each, the division 4 (2 ulp): rho 7; a product with
+// an exact integer 8, the sums 11 (g) and 12 (h00..h11).  With e_k = |rho_k| (|dy_i - dy_j| + |dx_j - dx_i|),
+// S = U sum e_k and SQ = U sum e_k (|X_k| + |Y_k|): den carries at most 28 (1 + S), X and Y together at most
+// 32 (SQ + |q3|_1 (1 + S)), n in addition |q|_1 28 (1 + S).  A match that can pass has
+// |q|_1 <= (|X| + |Y|) / den + 2 t, which the window's extremes of the form bound where den stays positive; else
+// the window's largest |q| does.  (34 and 30 below leave the second order room.)
+__device__ __forceinline__ int fast_hypothesis(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id,
+                                               uint32_t k0, uint32_t k1, float t, FastHyp& h) {
+    if (!(w.vq <= kFastReach)) return HYP_LOOSE;  // uniform over the window
+    int idx[4];
+    draw_indices(w.N, cell, k, tag, pair_id, k0, k1, idx);
+    const float p3x = w.x[idx[3]], p3y = w.y[idx[3]], q3x = w.qx[idx[3]], q3y = w.qy[idx[3]];
+    float dx[3], dy[3], X[3], Y[3], l[3];
+    int Xi[3], Yi[3], mu[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        dx[j] = w.x[idx[j]] - p3x;
+        dy[j] = w.y[idx[j]] - p3y;
+        X[j] = w.qx[idx[j]] - q3x;
+        Y[j] = w.qy[idx[j]] - q3y;
+        Xi[j] = exact_int(X[j]);
+        Yi[j] = exact_int(Y[j]);
+    }
+    bool degen = false;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int a = (j + 1) % 3, b = (j + 2) % 3;
+        l[j] = dx[a] * dy[b] - dx[b] * dy[a];
+        mu[j] = Xi[a] * Yi[b] - Xi[b] * Yi[a];
+        degen |= l[j] == 0.f || mu[j] == 0;
+    }
+    const int M = (int)((unsigned)mu[0] + (unsigned)mu[1] + (unsigned)mu[2]);
+    if (degen || l[0] + l[1] + l[2] == 0.f || M == 0) return HYP_DEAD;
+    const float Mf = (float)M;
+    float S = 0.f, SQ = 0.f, h00 = 0.f, h01 = 0.f, h10 = 0.f, h11 = 0.f;
+    h.g0 = h.g1 = 0.f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int a = (j + 1) % 3, b = (j + 2) % 3;
+        const float rho = __fdividef((float)mu[j], Mf * l[j]);
+        const float al = rho * (dy[a] - dy[b]), be = rho * (dx[b] - dx[a]);
+        const float e = fabsf(al) + fabsf(be);
+        S += e;
+        SQ = fmaf(e, fabsf(X[j]) + fabsf(Y[j]), SQ);
+        h.g0 += al;
+        h.g1 += be;
+        h00 = fmaf(al, X[j], h00);
+        h01 = fmaf(be, X[j], h01);
+        h10 = fmaf(al, Y[j], h10);
+        h11 = fmaf(be, Y[j], h11);
+    }
+    h.c0 = fmaf(-h.g1, p3y, fmaf(-h.g0, p3x, 1.f));
+    h.x0 = fmaf(q3x, h.g0, h00);
+    h.x1 = fmaf(q3x, h.g1, h01);
+    h.xc = fmaf(-h01, p3y, fmaf(-h00, p3x, q3x * h.c0));
+    h.y0 = fmaf(q3y, h.g0, h10);
+    h.y1 = fmaf(q3y, h.g1, h11);
+    h.yc = fmaf(-h11, p3y, fmaf(-h10, p3x, q3y * h.c0));
+    const float u = 5.9604644775390625e-08f, U = w.U;
+    const float one = fmaf(U, S, 1.f), ed = 30.f * u * one;
+    const float dc = h.c0 - 0.5f * (h.g0 + h.g1);
+    if (!(fabsf(dc) > 2.f * ed)) return HYP_LOOSE;  // its orientation needs the exact form
+    if (dc < 0.f) {
+        h.g0 = -h.g0, h.g1 = -h.g1, h.c0 = -h.c0;
+        h.x0 = -h.x0, h.x1 = -h.x1, h.xc = -h.xc;
+        h.y0 = -h.y0, h.y1 = -h.y1, h.yc = -h.yc;
+    }
+    const float dmin = h.c0 - (fabsf(h.g0) + fabsf(h.g1)) * U - 2.f * ed;
+    float Q = 2.f * w.vq;
+    if (dmin > 0.f) {
+        const float XY = fabsf(h.xc) + fabsf(h.yc) + (fabsf(h.x0) + fabsf(h.x1) + fabsf(h.y0) + fabsf(h.y1)) * U;
+        Q = fminf(Q, __fdividef(1.05f * XY + t, dmin) + 2.2f * t);
+    }
+    h.kap = 1.0001f * fmaf(34.f * u, fmaf(fabsf(q3x) + fabsf(q3y) + Q, one, SQ * U), t * ed);
+    return h.kap < 1e6f ? HYP_OK : HYP_LOOSE;  // a wide bound still excludes most; NaN: loose
+}
+
+// The form of a hypothesis with every coefficient in both halves of a pair, for tests of two matches per
+// instruction on the packed FP32x2 pipe; the denominator negated, so that no product needs a sign change.
+struct PairHyp {
+    float2 g0, g1, c0, kap, x0, x1, xc, y0, y1, yc;
+};
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ PairHyp pair_hyp(const FastHyp& h) {
+    PairHyp p;
+    p.g0 = both(-h.g0), p.g1 = both(-h.g1), p.c0 = both(-h.c0), p.kap = both(-h.kap);
+    p.x0 = both(h.x0), p.x1 = both(h.x1), p.xc = both(h.xc);
+    p.y0 = both(h.y0), p.y1 = both(h.y1), p.yc = both(h.yc);
+    return p;
+}
+// How many of two matches can be inliers: 12 FP32 operations a match (three linear forms, two residuals, the
+// comparison squared with a negative radius cut to zero), the count from the sign bit of |n|^2 - radius^2.
+__device__ __forceinline__ void count_pair(const PairHyp& h, float2 t, float2 ux, float2 uy, float2 qx, float2 qy,
+                                           int& cnt) {
+    const float2 nd = __ffma2_rn(h.g1, uy, __ffma2_rn(h.g0, ux, h.c0));  // -den
+    const float2 nx = __ffma2_rn(qx, nd, __ffma2_rn(h.x1, uy, __ffma2_rn(h.x0, ux, h.xc)));
+    const float2 ny = __ffma2_rn(qy, nd, __ffma2_rn(h.y1, uy, __ffma2_rn(h.y0, ux, h.yc)));
+    const float2 m = __ffma2_rn(t, nd, h.kap);  // -(t den + kap)
+    const float2 n2 = __ffma2_rn(nx, nx, __fmul2_rn(ny, ny));
+    const float ma = fminf(m.x, 0.f), mb = fminf(m.y, 0.f);
+    cnt += (int)(__float_as_uint(fmaf(-ma, ma, n2.x)) >> 31) + (int)(__float_as_uint(fmaf(-mb, mb, n2.y)) >> 31);
+}
+// The same for the four matches from index j (a multiple of 4).
+__device__ __forceinline__ void count_quad(const Window& w, const PairHyp& h, float2 t, int j, int& cnt) {
+    const float4 x = *reinterpret_cast<const float4*>(w.x + j), y = *reinterpret_cast<const float4*>(w.y + j);
+    const float4 a = *reinterpret_cast<const float4*>(w.qx + j), b = *reinterpret_cast<const float4*>(w.qy + j);
+    count_pair(h, t, make_float2(x.x, x.y), make_float2(y.x, y.y), make_float2(a.x, a.y), make_float2(b.x, b.y), cnt);
+    count_pair(h, t, make_float2(x.z, x.w), make_float2(y.z, y.w), make_float2(a.z, a.w), make_float2(b.z, b.w), cnt);
+}
+
+// One match against a scored hypothesis: sure (an inlier whatever the rounding) and maybe (possibly one).
+__device__ __forceinline__ void test_match(const Window& w, const FastHyp& h, float tl, float th, int j, bool& sure,
+                                           bool& maybe) {
+    const float ux = w.x[j], uy = w.y[j];
+    const float den = fmaf(h.g1, uy, fmaf(h.g0, ux, h.c0));
+    const float nx = fmaf(-w.qx[j], den, fmaf(h.x1, uy, fmaf(h.x0, ux, h.xc)));
+    const float ny = fmaf(-w.qy[j], den, fmaf(h.y1, uy, fmaf(h.y0, ux, h.yc)));
+    const float n2 = fmaf(nx, nx, ny * ny);
+    const float a = fmaf(th, den, h.kap), b = fmaf(tl, den, -h.kap);
+    maybe = a > 0.f && n2 < a * a;
+    sure = b > 0.f && n2 < b * b;
+}
+
+// The order of two hypotheses: more inliers, then the lower index.  Zero is below every hypothesis.
+__device__ __forceinline__ unsigned long long hyp_key(int score, int k) {
+    return ((unsigned long long)(unsigned)(score + 1) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)k);
+}
+__device__ __forceinline__ int key_score(unsigned long long key) { return (int)(key >> 32) - 1; }
+__device__ __forceinline__ int key_index(unsigned long long key) {
+    return (int)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
+}
+
+// The certified test of a match by the exact hypothesis: its FP32 evaluation form, and FP64 (Hl) where that is
+// within its rounding bound.
+__device__ __forceinline__ bool exact_inlier(const Mef& m, const double* Hl, const float4& mt, float t2, int& nfp64) {
+    bool unc;
+    const bool in = cert_inlier(m, mt, t2, unc);
+    if (!unc) return in;
+    ++nfp64;
+    return hyp_inlier_fp64(Hl, mt.x, mt.y, mt.z, mt.w, (double)t2);
+}
+
+// What a warp counts of its work (profiling counters).
+struct RansacStats {
+    int tests = 0, fp64 = 0, loose = 0;
+};
+
+// The exact support of hypothesis k, by one warp: -1 if its sample is degenerate, or as soon as it cannot reach
+// `floor` (a key).  Out of line: for the few hypotheses that contend with uncertain tests, and the loose ones.
+__device__ __noinline__ int exact_support(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id,
+                                          uint32_t k0, uint32_t k1, float t2, unsigned long long floor,
+                                          RansacStats& st) {
+    const int lane = threadIdx.x & 31;
+    double Hl[9];
+    Mef m;
+    {
+        i128 Hk[9];
+        if (!draw_exact(w, cell, k, tag, pair_id, k0, k1, Hk) || !make_mef_exact(Hk, m)) return -1;
+        exact_local_fp64(Hk, Hl);
+    }
+    mef_set_bounds(m, w.U, w.vmax, t2);
+    int score = 0, f = 0;
+    for (int c = 0; c < w.N; c += 128) {
+#pragma unroll 1
+        for (int j = c + lane; j < c + 128 + lane; j += 32) {
+            const bool in = j < w.N && exact_inlier(m, Hl, w.match(j), t2, f);
+            score += __popc(__ballot_sync(FULL, in));
+        }
+        st.tests += min(128, w.N - c);
+        if (hyp_key(score + max(w.N - c - 128, 0), k) < floor) return -1;
+    }
+    st.fp64 += (int)__reduce_add_sync(FULL, (unsigned)f);
+    return score;
+}
+
+// The support of scored hypothesis k (its form in `form`, shared memory), by one warp: the FP32 count if no test is
+// uncertain, else exact; -1 if it cannot reach `floor`.  Out of line (contenders only).
+__device__ __noinline__ int contender_support(const Window& w, const FastHyp* form, int cell, int k, uint32_t tag,
+                                              uint32_t pair_id, uint32_t k0, uint32_t k1, float t2,
+                                              unsigned long long floor, RansacStats& st) {
+    const FastHyp h = *form;
+    const float tl = t_below(t2), th = t_above(t2);
+    int lo = 0, hi = 0;
+    for (int j = threadIdx.x & 31; j < w.N; j += 32) {
+        bool sure, maybe;
+        test_match(w, h, tl, th, j, sure, maybe);
+        lo += sure;
+        hi += maybe;
+    }
+    lo = (int)__reduce_add_sync(FULL, (unsigned)lo);
+    hi = (int)__reduce_add_sync(FULL, (unsigned)hi);
+    st.tests += w.N;
+    if (hyp_key(hi, k) < floor) return -1;
+    return hi == lo ? lo : exact_support(w, cell, k, tag, pair_id, k0, k1, t2, floor, st);
 }
 
 // The window's matches in raster order into `match`; returns their number.
@@ -758,9 +961,9 @@ struct DistSum {
 // Refit inputs on the winner's inliers, for ransac_fit (out of line: once per window, and its 24 integer
 // moments would otherwise crowd the registers of the hypothesis loop).
 template <class G>
-__device__ __noinline__ void winner_moments(const G& grp, const float4* match, int N, const Mef* wmef,
-                                            const double* whl, float t2, int wscore, RefitWork* rw) {
-    const int tid = grp.rank();
+__device__ __noinline__ void winner_moments(const G& grp, const Window& w, const Mef* wmef, const double* whl, float t2,
+                                            int wscore, RefitWork* rw) {
+    const int tid = grp.rank(), N = w.N;
     // Hartley centroids (exact integer sums), mean distances, and the DLT moments as exact integers about the
     // rounded centroids
     const Mef wm = *wmef;
@@ -776,7 +979,7 @@ __device__ __noinline__ void winner_moments(const G& grp, const float4* match, i
     unsigned long long inm = 0;
     int sx = 0, sy = 0, tx = 0, ty = 0;
     for (int j = tid, c = 0; j < N; j += G::size, ++c) {
-        const float4 mt = match[j];
+        const float4 mt = w.match(j);
         if (winner_inlier(mt)) {
             inm |= 1ull << c;
             sx += exact_int(mt.x);
@@ -802,7 +1005,7 @@ __device__ __noinline__ void winner_moments(const G& grp, const float4* match, i
 #pragma unroll
     for (int q = 0; q < 24; ++q) R[q] = 0;
     for (; inm; inm &= inm - 1) {
-        const float4 mt = match[tid + (__ffsll((long long)inm) - 1) * G::size];
+        const float4 mt = w.match(tid + (__ffsll((long long)inm) - 1) * G::size);
         dsum.add(nw * exact_int(mt.x) - sx, nw * exact_int(mt.y) - sy);
         dtsum.add(nw * exact_int(mt.x + mt.z) - tx, nw * exact_int(mt.y + mt.w) - ty);
         const int X = exact_int(mt.x) - cx, Y = exact_int(mt.y) - cy;
@@ -836,310 +1039,261 @@ __device__ __noinline__ void winner_moments(const G& grp, const float4* match, i
     }
 }
 
-template <class G, int ST, bool LANE>
-__device__ void ransac_fit(const G& grp, const PairView& pv, const LevelGeom& g, int level, int stage,
-                           const PlaneParams& pp, int dir, int cell, float4* match, Mef* hyp, int* gbest, int* kfull,
-                           Mef* wmef, void* hx) {
-    const int tid = grp.rank();
-    const int id = (g.base + cell) * 2 + (stage - 1);
+// The window's model record, cleared before its fit.
+__device__ __forceinline__ void clear_model(const PairView& pv, int dir, int id, int N, RefitWork* rw) {
     int* mi = pv.mi[dir] + (size_t)id * kMI;
-    RefitWork* rw = pv.rw[dir] + cell;
-    if (G::size > 32 && tid == 0) {
-        *gbest = -1;
-        *kfull = 0x7fffffff;
-    }
-    const int N = gather_matches<G>(grp, pv, g, stage, dir, cell, match);
-    if (tid == 0) {
-        for (int k = 0; k < kMI; ++k) mi[k] = 0;
-        mi[MI_NIN] = N;
-        mi[MI_BESTK] = -1;
-        for (int k = 0; k < 9; ++k) pv.mh[dir][(size_t)id * 9 + k] = 0.0;
-        Mef z = {};
-        pv.mef[dir][id] = z;
-        rw->status = 0;
-    }
-    if (N < pp.min_inliers || N < 4) return;
-    // the largest |offset| component among the matches, and the window's half side: the bounds of the FP32 tests
-    float vloc = 0.f;
-    for (int j = tid; j < N; j += G::size) {
-        const float4 mt = match[j];
-        vloc = fmaxf(vloc, fmaxf(fabsf(mt.z), fabsf(mt.w)));
-    }
-    const float V = (float)grp.max((unsigned long long)vloc);  // integers: exact as a key
-    const float U = 0.5f * (float)g.s;
-    if (tid == 0) rw->vmax = V;
+    for (int k = 0; k < kMI; ++k) mi[k] = 0;
+    mi[MI_NIN] = N;
+    mi[MI_BESTK] = -1;
+    for (int k = 0; k < 9; ++k) pv.mh[dir][(size_t)id * 9 + k] = 0.0;
+    pv.mef[dir][id] = Mef{};
+    rw->status = 0;
+}
 
-    // Hypotheses.  Few matches: each thread draws and scores its own
-    // hypotheses k = rank, rank + size, ... in full.  Otherwise each warp of
-    // the group draws 32 at a time (one per lane), then scores them in index
-    // order with its lanes over the matches, 128 at a time, and abandons one
-    // as soon as it cannot win: its inliers so far plus the matches left fall
-    // below the best score of the group (any index), or do not exceed the
-    // best of this warp's earlier, lower-index hypotheses.  The winner (most
-    // inliers, lowest index) is never abandoned, so the outcome is that of
-    // scoring every hypothesis in full.  Once a hypothesis has all N matches
-    // as inliers, hypotheses of higher index can at most tie and are not
-    // drawn at all.
-    // Counts are certified: a count with uncertain FP32 tests bounds the exact
-    // count by count +- uncertain; a hypothesis whose optimistic count could
-    // still win gets its exact count at once (its uncertain tests decided in
-    // FP64 with its exact form).  hx keeps each lane's hypothesis since it was
-    // drawn: in the one-hypothesis-per-lane kernel (LANE) as its 128-bit
-    // entries (converted only when needed), else as its exact form in FP64.
-    const float t2 = pp.t2;
-    const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
-    constexpr int NW = G::size / 32;
-    const int lane = tid & 31;
-    Mef* hb = hyp + (tid >> 5) * 32;
-    i128* hkw = reinterpret_cast<i128*>(hx) + (tid >> 5) * (32 * 9);    // LANE: this warp's 32 hypotheses
-    double* hlw = reinterpret_cast<double*>(hx) + (tid >> 5) * (32 * 9);  // else: their exact forms
-    int best_score = -1, best_k = 0x7fffffff, tests = 0;
-    int nfp64 = 0, nloose = 0;  // tests decided in FP64, hypotheses tested with per-match bounds (counters)
-    // LANE: the warp's best hypothesis so far (its key, its 128-bit entries after the 32 lanes' in hx, its
-    // evaluation form in *wmef), so that the winner needs no second draw
-    unsigned long long wbest_key = 0ull;
-    i128* wslot = reinterpret_cast<i128*>(hx) + 32 * 9;
-    if (LANE || N <= kLaneScoreMax) {
-        int group_best = -1;  // the group's best exact count after the previous rounds
-        for (int r = 0; r * G::size < pp.num_hyp; ++r) {
-            const int k = r * G::size + tid;
-            Mef m;
-            bool ok = false;
-            if (k < pp.num_hyp) {
-                i128 Hk[9];
-                ok = draw_hypothesis(match, N, cell, k, tag, pv.pair_id, pp.k0, pp.k1, Hk) && make_mef_exact(Hk, m);
-                if (LANE) {
+// The winner drawn again, exact, by one warp (out of line, once per window).
+__device__ __noinline__ void emit_winner(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id, uint32_t k0,
+                                         uint32_t k1, float t2, Mef* wmef, double* whl, RefitWork* rw) {
+    const int lane = threadIdx.x & 31;
+    i128 Hk[9];
+    draw_exact(w, cell, k, tag, pair_id, k0, k1, Hk);
+    double Hl[9];
+    exact_local_fp64(Hk, Hl);
 #pragma unroll
-                    for (int q = 0; q < 9; ++q) hkw[lane * 9 + q] = Hk[q];
-                } else if (ok) {
-                    exact_local_fp64(Hk, hlw + lane * 9);
-                }
-            }
-            // FP32 count; the uncertain tests (bit j: match j) and the FP32 decisions among them: the exact
-            // count is within score +- popc(um)
-            int score = 0;
-            unsigned long long um = 0, im = 0;
-            bool loose = false;
-            if (ok) {
-                mef_set_bounds(m, U, V, t2);
-                loose = mef_loose(m);
-                nloose += loose;
-                if (!loose) {  // two matches per instruction on the packed FP32x2 pipe
-                    const Mef2 m2 = mef2_of(m);
-                    const float ef = m.ef, eden = __int_as_float(m.eden);
-                    int j = 0;
-                    for (; j + 1 < N; j += 2) {
-                        bool ia, ib, ua, ub;
-                        mef_inlier2_c(m2, ef, eden, match[j], match[j + 1], t2, ia, ib, ua, ub);
-                        score += (int)ia + (int)ib;
-                        if (ua || ub) {
-                            const unsigned long long ba = (unsigned long long)ua << j, bb = (unsigned long long)ub
-                                                                                                  << (j + 1);
-                            um |= ba | bb;
-                            im |= (ia ? ba : 0ull) | (ib ? bb : 0ull);
-                        }
-                    }
-                    if (j < N) {
-                        const float4 mt = match[j];
-                        bool unc;
-                        const bool in = mef_inlier_c(m, mt.x, mt.y, mt.z, mt.w, t2, unc);
-                        score += in;
-                        if (unc) {
-                            um |= 1ull << j;
-                            if (in) im |= 1ull << j;
-                        }
-                    }
-                }
-                tests += N;
-            }
-            hb[lane] = m;
-            __syncwarp();
-            // loose hypotheses (per-match bounds): the warp scores them together, lanes over the matches
-            for (unsigned lm = __ballot_sync(FULL, loose); lm; lm &= lm - 1) {
-                const int l = __ffs(lm) - 1;
-                unsigned long long ul, il;
-                const int sl = loose_score64(match, N, hb[l], t2, ul, il);
-                if (lane == l) {
-                    score = sl;
-                    um = ul;
-                    im = il;
-                }
-            }
-            const int unc_n = __popcll(um);
-            // A hypothesis with uncertain tests that could beat the best so far (this thread's, the group's of
-            // earlier rounds: lower indices) and that no hypothesis of this round surely beats gets its exact
-            // count.  Without uncertain tests its count is exact.
-            const int rlo = (int)__reduce_max_sync(FULL, (unsigned)(ok ? score - unc_n + 1 : 0)) - 1;
-            const int hi = score + unc_n;
-            bool exact = unc_n == 0;
-            if (ok && !exact && hi > max(best_score, group_best) && hi >= rlo) {
-                score = LANE ? resolve_uncertain_hk(match, hkw + lane * 9, t2, um, im, score, nfp64)
-                             : resolve_uncertain(match, hlw + lane * 9, t2, um, im, score, nfp64);
-                exact = true;
-            }
-            __syncwarp();
-            if (ok && exact && score > best_score) {
-                best_score = score;
-                best_k = k;
-            }
-            if (LANE) {  // the warp's best so far (most inliers, lowest index) into its slot when it changes
-                const unsigned long long key =
-                    best_score < 0 ? 0ull
-                                   : (((unsigned long long)(best_score + 1)) << 32) |
-                                         (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_k);
-                const unsigned long long wk = grp.max(key);
-                if (wk != wbest_key) {  // a hypothesis of this round: its lane still holds it in hkw and hb
-                    const int wl = __ffs(__ballot_sync(FULL, key == wk)) - 1;
-                    if (lane < 9) wslot[lane] = hkw[wl * 9 + lane];
-                    if (lane == 9) *wmef = hb[wl];
-                    wbest_key = wk;
-                }
-                __syncwarp();
-                group_best = (int)(wk >> 32) - 1;
-                // all N matches inliers: every later round has higher indices and can at most tie
-                if (group_best >= N) break;
-            } else {
-                // all N matches inliers: every later round has higher indices and can at most tie
-                if (grp.any(best_score >= N)) break;
-                group_best = (int)grp.max((unsigned long long)(best_score + 1)) - 1;
-            }
+    for (int q = 0; q < 9; ++q)
+        if (lane == q) {
+            whl[q] = Hl[q];
+            rw->hx[q] = Hk[q];
         }
+    if (lane == 0) {
+        Mef m0;
+        make_mef_exact(Hk, m0);
+        mef_set_bounds(m0, w.U, w.vmax, t2);
+        *wmef = m0;
+        rw->mef0 = m0;
+        rw->vmax = w.vmax;
     }
-    for (int b = tid >> 5; !LANE && N > kLaneScoreMax && b * 32 < pp.num_hyp; b += NW) {
-        // a hypothesis with all N matches inliers at a lower index than this batch: nothing here can win
-        if ((NW > 1 ? *(volatile int*)kfull : (best_score >= N ? best_k : 0x7fffffff)) < b * 32) break;
-        const int k = b * 32 + lane;
-        bool ok = false;
-        if (k < pp.num_hyp) {
-            i128 Hk[9];
-            Mef m;
-            ok = draw_hypothesis(match, N, cell, k, tag, pv.pair_id, pp.k0, pp.k1, Hk) && make_mef_exact(Hk, m);
-            if (ok) {
-                mef_set_bounds(m, U, V, t2);
-                nloose += mef_loose(m);
-                hb[lane] = m;
-                exact_local_fp64(Hk, hlw + lane * 9);
-            }
-        }
-        unsigned todo = __ballot_sync(FULL, ok);
-        __syncwarp();
-        while (todo) {
-            const int l = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const Mef2 m2 = mef2_of(hb[l]);
-            const float ef = hb[l].ef, eden = __int_as_float(hb[l].eden);
-            const bool loose = mef_loose(hb[l]);  // warp-uniform
-            // abandon when reach < group best or reach <= this warp's best
-            const int bound = max(NW > 1 ? *(volatile int*)gbest - 1 : -1, best_score);
-            int score = 0, unc_n = 0;  // FP32 count, uncertain tests: the exact count is within score +- unc_n
-            bool alive = true;
-            if (loose) {  // per-match bounds, out of line
-                const int2 su = loose_score_warp(match, N, hb[l], t2, bound, tests);
-                score = su.x;
-                unc_n = su.y;
-                alive = su.x >= 0 && score + unc_n > bound;
-            }
-            for (int c = 0; !loose && c < N; c += 128) {
-                int uc = 0;  // this lane's uncertain tests in the chunk
-#pragma unroll
-                for (int u = 0; u < 4; u += 2) {  // matches j and j + 32 of this lane, tested as a pair
-                    const int j = c + 32 * u + lane;
-                    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float4 ma = j < N ? match[j] : z, mb = j + 32 < N ? match[j + 32] : z;
-                    bool ia, ib, ua, ub;
-                    mef_inlier2_c(m2, ef, eden, ma, mb, t2, ia, ib, ua, ub);
-                    uc += (ua && j < N) + (ub && j + 32 < N);
-                    score += __popc(__ballot_sync(FULL, ia && j < N)) + __popc(__ballot_sync(FULL, ib && j + 32 < N));
-                }
-                if (__any_sync(FULL, uc != 0)) unc_n += (int)__reduce_add_sync(FULL, (unsigned)uc);
-                tests += min(128, N - c);
-                // abandoned only if even every uncertain test turning in its favour could not win
-                if (score + unc_n + max(N - c - 128, 0) <= bound) {
-                    alive = false;
-                    break;
-                }
-            }
-            if (alive && unc_n > 0) {  // a contender with uncertain tests: its exact count
-                int f = 0;
-                score = exact_score_warp(match, N, hb[l], hlw + l * 9, t2, f);
-                const unsigned tf = __reduce_add_sync(FULL, (unsigned)f);
-                if (lane == 0) nfp64 += (int)tf;
-                alive = score > bound;
-            }
-            if (alive) {  // more inliers than every earlier hypothesis of this warp
-                best_score = score;
-                best_k = b * 32 + l;
-                if (NW > 1 && lane == 0) {
-                    atomicMax(gbest, score);
-                    if (score >= N) atomicMin(kfull, best_k);
-                }
-            }
-        }
-        __syncwarp();
-    }
+}
+
+// What follows the search: the winner drawn again, exact, with its evaluation form and its FP64 form for uncertain
+// tests (whl, shared memory), and the refit's inputs on its inliers.  best: the winner's key, 0 if there is none.
+template <class G>
+__device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, const Window& w, const PlaneParams& pp,
+                                           int dir, int cell, int id, uint32_t tag, unsigned long long best,
+                                           const RansacStats& st, Mef* wmef, double* whl, RefitWork* rw) {
+    const int tid = grp.rank();
+    int* mi = pv.mi[dir] + (size_t)id * kMI;
     if (pv.evals) {  // residual tests performed, those decided in FP64, loose hypotheses (profiling)
-        const bool per_lane = LANE || N <= kLaneScoreMax;
-        const int t = grp.sum(per_lane || lane == 0 ? tests : 0);
-        const int f = grp.sum(nfp64);
-        const int lo = grp.sum(per_lane || lane == 0 ? nloose : 0);
+        const bool one = (tid & 31) == 0;
+        const int t = grp.sum(one ? st.tests : 0), f = grp.sum(one ? st.fp64 : 0), lo = grp.sum(one ? st.loose : 0);
         if (tid == 0) {
             atomicAdd(&pv.evals[GPM_COUNT_RANSAC], (unsigned long long)t);
             atomicAdd(&pv.evals[GPM_COUNT_RANSAC_FP64], (unsigned long long)f);
             atomicAdd(&pv.evals[GPM_COUNT_RANSAC_LOOSE], (unsigned long long)lo);
         }
     }
-    // most inliers, then lowest hypothesis index
-    const unsigned long long key =
-        best_score < 0 ? 0ull
-                       : (((unsigned long long)(best_score + 1)) << 32) |
-                             (unsigned long long)(0xFFFFFFFFu - (uint32_t)best_k);
-    const unsigned long long wkey = grp.max(key);
-    if (wkey == 0ull) {  // every sample degenerate: no winner, best score -1
+    if (best == 0ull) {  // every sample degenerate: no winner, best score -1
         if (tid == 0) mi[MI_BESTSCORE] = -1;
         return;
     }
-    const int wscore = (int)(wkey >> 32) - 1;
-    const int wk = (int)(0xFFFFFFFFu - (uint32_t)(wkey & 0xFFFFFFFFull));
-    // the winner's exact form for its FP64 tests, in the first 72 bytes of hx (the scan is over: every warp
-    // of the group has passed the reduction above)
-    double* whl = reinterpret_cast<double*>(hx);
-    if (tid < 32) {  // first warp: the winner again, exact (LANE: from the warp's slot), and its evaluation form
-        i128 Hk[9];
-        if (LANE) {
-#pragma unroll
-            for (int q = 0; q < 9; ++q) Hk[q] = wslot[q];
-        } else {
-            draw_hypothesis_ool(match, N, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, Hk);
-        }
-        {
-            double Hl[9];
-            exact_local_fp64(Hk, Hl);
-            __syncwarp();
-#pragma unroll
-            for (int q = 0; q < 9; ++q)
-                if (tid == q) whl[q] = Hl[q];
-        }
+    const int wscore = key_score(best), wk = key_index(best);
+    if (tid < 32) {  // first warp
+        emit_winner(w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, pp.t2, wmef, whl, rw);
         if (tid == 0) {
-            Mef m0;
-            if (LANE) {
-                m0 = *wmef;
-            } else {
-                make_mef_exact(Hk, m0);
-                mef_set_bounds(m0, U, V, t2);
-            }
-            *wmef = m0;
-            rw->mef0 = m0;
             mi[MI_BESTK] = wk;
             mi[MI_BESTSCORE] = wscore;
         }
-#pragma unroll
-        for (int q = 0; q < 9; ++q)
-            if (tid == q) rw->hx[q] = Hk[q];
     }
     grp.sync();
     if (wscore < 4) return;
+    winner_moments<G>(grp, w, wmef, whl, pp.t2, wscore, rw);
+}
 
-    winner_moments<G>(grp, match, N, wmef, whl, t2, wscore, rw);
+// The search keeps the hypothesis with the most inliers (lowest index on ties).  Every hypothesis is bounded, not
+// counted: `maybe` tests give the most inliers it can have, whatever the rounding of its FP32 form, and it is
+// dropped as soon as those and the matches not yet tested leave it below the best support known.  Only contenders
+// are counted exactly, their uncertain tests decided in FP64 with the exact hypothesis; hypotheses whose FP32 form
+// says too little (ill-conditioned samples, windows with far-flung imported offsets) are counted exactly at once.
+// The outcome is that of counting every hypothesis exactly.  Once one has every match as an inlier, later ones can
+// at most tie and are not drawn.
+
+// Windows up to 16 x 16, one warp each: 32 hypotheses at a time, one per lane, each lane testing its own against
+// the matches four at a time (every lane reads the same ones: broadcasts).  The quads go in four interleaved
+// passes spread over the window; after each, lanes that cannot win drop out, and once few are left the warp counts
+// those one by one with its lanes over the matches.
+// What bounds it: instruction fetch, then the FP32 pipe in the tests (12 operations a match).  1024x436, stage 1:
+// the 16 px windows 1.44 -> 0.64 ms, the 8 px windows 1.73 -> 1.12 ms, against scoring exact 128-bit hypotheses.
+__device__ __forceinline__ unsigned long long search_warp(const Window& w, const PlaneParams& pp, int cell,
+                                                          uint32_t tag, uint32_t pair_id, FastHyp* slot,
+                                                          RansacStats& st) {
+    const int lane = threadIdx.x & 31, N = w.N, nq = (N + 3) >> 2;
+    const float t = t_above(pp.t2);
+    const float2 tt = both(t);
+    unsigned long long best = 0ull;
+    for (int b = 0; b < pp.num_hyp; b += 32) {
+        if (key_score(best) >= N) break;
+        const int k = b + lane;
+        FastHyp h;
+        const int status =
+            k < pp.num_hyp ? fast_hypothesis(w, cell, k, tag, pair_id, pp.k0, pp.k1, t, h) : (int)HYP_DEAD;
+        st.loose += __popc(__ballot_sync(FULL, status == HYP_LOOSE));
+        unsigned alive = __ballot_sync(FULL, status == HYP_OK);
+        int cnt = 0, left = 4 * nq;  // maybe tests passed; matches not yet tested
+        if (alive) {
+            const PairHyp ph = pair_hyp(h);
+            for (int pass = 0; pass < 4; ++pass) {
+                int done = 0;
+#pragma unroll 2
+                for (int q = pass; q < nq; q = (q | 3) + 1 + ((q + 1) & 3)) {  // 4 i + ((i + pass) & 3)
+                    count_quad(w, ph, tt, 4 * q, cnt);
+                    done += 4;
+                }
+                left -= done;
+                st.tests += done * __popc(alive);
+                alive = __ballot_sync(FULL, status == HYP_OK && hyp_key(cnt + min(left, N), k) >= best);
+                if (__popc(alive) <= 2 * (3 - pass)) break;
+            }
+        }
+        // contenders, the most promising first
+        const int reach = status == HYP_OK ? cnt + max(min(left, N), 0) : (status == HYP_LOOSE ? N : -1);
+        alive |= __ballot_sync(FULL, status == HYP_LOOSE);
+        while (alive) {
+            const bool in = (alive >> lane) & 1u;
+            const int top = (int)__reduce_max_sync(FULL, (unsigned)(in ? reach + 1 : 0)) - 1;
+            const unsigned ok = __ballot_sync(FULL, in && reach == top && status == HYP_OK);
+            const int l = __ffs(ok ? ok : __ballot_sync(FULL, in && reach == top)) - 1;
+            if (lane == l) *slot = h;
+            __syncwarp();
+            const int score =
+                ok ? contender_support(w, slot, cell, b + l, tag, pair_id, pp.k0, pp.k1, pp.t2, best, st)
+                   : exact_support(w, cell, b + l, tag, pair_id, pp.k0, pp.k1, pp.t2, best, st);
+            __syncwarp();
+            if (score >= 0) best = max(best, hyp_key(score, b + l));
+            alive &= ~(1u << l);
+            alive &= __ballot_sync(FULL, hyp_key(reach, k) >= best);
+        }
+    }
+    return best;
+}
+
+// Larger windows, one block of 256 threads each: 256 hypotheses a round, solved one per thread into shared memory.
+// The warps first test every hypothesis on an eighth of the matches (chunks of 128, spread over the window); the
+// one with the most is counted from below on all of them, by the whole block, which gives the bound the others have
+// to reach from the start; then the warps take the hypotheses that still can, one at a time, chunk by chunk.
+// What bounds it: the FP32 pipe and the shared loads of the tests.  1024x436, stage 1: the 64 px windows 1.99 ->
+// 0.85 ms, the 32 px windows 1.03 -> 0.59 ms, against scoring in index order from exact 128-bit hypotheses.
+constexpr int kHypRound = 256;
+struct BlockSearch {
+    FastHyp form[kHypRound];
+    short cnt[kHypRound];           // maybe tests passed in the first chunks; -1: not scored
+    short todo[kHypRound];          // the hypotheses to finish, loose ones from the back
+    unsigned long long best;        // a lower bound of the best key; the winner's at the end
+    int next, n_ok, n_loose;
+};
+__device__ __forceinline__ unsigned long long search_block(const BlockGroup<256>& grp, const Window& w,
+                                                           const PlaneParams& pp, int cell, uint32_t tag,
+                                                           uint32_t pair_id, BlockSearch& bs, RansacStats& st) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, N = w.N;
+    const float t = t_above(pp.t2), tl = t_below(pp.t2);
+    const float2 tt = both(t);
+    const int nch = (N + 127) >> 7, nfirst = max(1, nch >> 3);
+    // visiting order of the chunks: i -> i * step mod nch, step coprime to nch
+    int step = max(1, (3 * nch) >> 3);
+    for (;; ++step) {
+        int a = step, b = nch;
+        while (b) {
+            const int r = a % b;
+            a = b;
+            b = r;
+        }
+        if (a == 1) break;
+    }
+    volatile unsigned long long* vbest = &bs.best;
+    if (tid == 0) bs.best = 0ull;
+    __syncthreads();
+    for (int b = 0; b < pp.num_hyp; b += kHypRound) {
+        if (key_score(*vbest) >= N) break;  // block-uniform: the barrier below has passed since it was written
+        const int k = b + tid;
+        int status = HYP_DEAD;
+        {
+            FastHyp h;
+            if (k < pp.num_hyp) status = fast_hypothesis(w, cell, k, tag, pair_id, pp.k0, pp.k1, t, h);
+            if (status == HYP_OK) bs.form[tid] = h;
+        }
+        bs.cnt[tid] = status == HYP_OK ? 0 : -1;
+        if (tid == 0) bs.next = bs.n_ok = bs.n_loose = 0;
+        __syncthreads();
+        for (int e = warp; e < kHypRound; e += 8) {
+            if (bs.cnt[e] < 0) continue;  // warp-uniform
+            const PairHyp ph = pair_hyp(bs.form[e]);
+            int c = 0, ch = 0;
+            for (int i = 0; i < nfirst; ++i) {
+                count_quad(w, ph, tt, 128 * ch + 4 * lane, c);
+                ch += step;
+                if (ch >= nch) ch -= nch;
+            }
+            c = (int)__reduce_add_sync(FULL, (unsigned)c);
+            if (lane == 0) bs.cnt[e] = (short)c;
+            st.tests += 128 * nfirst;
+        }
+        __syncthreads();
+        const int rest = 128 * (nch - nfirst);
+        {
+            const int mine = bs.cnt[tid];
+            const unsigned long long lead = grp.max(mine >= 0 ? hyp_key(mine, k) : 0ull);
+            if (lead && hyp_key(min(key_score(lead) + rest, N), key_index(lead)) >= *vbest) {  // block-uniform
+                const FastHyp h = bs.form[key_index(lead) - b];
+                int lo = 0;
+                for (int j = tid; j < N; j += 256) {
+                    bool sure, maybe;
+                    test_match(w, h, tl, t, j, sure, maybe);
+                    lo += sure;
+                }
+                lo = grp.sum(lo);
+                if (tid == 0) bs.best = max(bs.best, hyp_key(lo, key_index(lead)));
+                st.tests += lane == 0 ? N / 8 : 0;
+                __syncthreads();
+            }
+            const bool go = mine >= 0 && hyp_key(min(mine + rest, N), k) >= *vbest;
+            if (go) bs.todo[atomicAdd(&bs.n_ok, 1)] = (short)tid;
+            if (status == HYP_LOOSE) bs.todo[kHypRound - 1 - atomicAdd(&bs.n_loose, 1)] = (short)tid;
+        }
+        __syncthreads();
+        const int n_ok = bs.n_ok, n_all = n_ok + bs.n_loose;
+        for (;;) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&bs.next, 1);
+            at = __shfl_sync(FULL, at, 0);
+            if (at >= n_all) break;
+            const bool loose = at >= n_ok;
+            const int e = bs.todo[loose ? kHypRound - 1 - (at - n_ok) : at];
+            int score = -1;
+            if (loose) {
+                ++st.loose;
+                if (hyp_key(N, b + e) >= *vbest)
+                    score = exact_support(w, cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, *vbest, st);
+            } else {
+                const PairHyp ph = pair_hyp(bs.form[e]);
+                int have = bs.cnt[e], left = rest, ch = (int)((long long)nfirst * step % nch);
+                bool alive = hyp_key(min(have + left, N), b + e) >= *vbest;
+                while (alive && left > 0) {
+                    int c = 0;
+                    count_quad(w, ph, tt, 128 * ch + 4 * lane, c);
+                    ch += step;
+                    if (ch >= nch) ch -= nch;
+                    left -= 128;
+                    have += (int)__reduce_add_sync(FULL, (unsigned)c);
+                    st.tests += 128;
+                    alive = hyp_key(min(have + left, N), b + e) >= *vbest;
+                }
+                if (alive)
+                    score = contender_support(w, &bs.form[e], cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, *vbest, st);
+            }
+            if (score >= 0 && lane == 0) atomicMax(&bs.best, hyp_key(score, b + e));
+            __syncwarp();
+        }
+        __syncthreads();
+    }
+    return *vbest;
 }
 
 // (B) Normalised DLT refit of each window whose fit is pending, one thread
@@ -1355,38 +1509,32 @@ __device__ void ransac_finish(const G& grp, const PairView& pv, const LevelGeom&
     }
 }
 
-// Windows up to 16 x 16: one warp per window, eight windows per block.
-// Dynamic shared memory: 8 x MS matches, 8 x 32 hypotheses (evaluation
-// forms), then per warp the exact hypotheses (LANE: 32 x 9 128-bit entries
-// and the warp's best so far, 9 more; else 32 x 9 doubles).  LANE: windows
-// of at most kLaneScoreMax pixels, whose hypotheses are all scored one per
-// lane (the other scoring path is not compiled in).
-constexpr int ransac_warp_match_stride(bool lane) { return lane ? kLaneScoreMax : 256; }
-constexpr size_t ransac_warp_hx_bytes(bool lane) { return lane ? (32 * 9 + 9) * sizeof(i128) : 32 * 9 * sizeof(double); }
-// Windows (warps) per block of the warp-per-window fit.
+// (A) Windows up to 16 x 16: one warp per window, kRansacWarps windows per block.  CAP: the most matches a window
+// has (64 for sides up to 8, else 256).
 constexpr int kRansacWarps = 4;
-constexpr size_t ransac_warp_smem(bool lane) {
-    return kRansacWarps * (ransac_warp_match_stride(lane) * sizeof(float4) + 32 * sizeof(Mef) +
-                           ransac_warp_hx_bytes(lane));
-}
-template <int ST, bool LANE>
+template <int CAP>
 __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     k_ransac_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
-    constexpr int MS = ransac_warp_match_stride(LANE);
-    extern __shared__ float4 warp_dyn[];
+    __shared__ __align__(16) float planes[kRansacWarps][4 * CAP];
+    __shared__ FastHyp slot[kRansacWarps];
     __shared__ Mef wmef[kRansacWarps];
-    const int warp = threadIdx.x >> 5;
+    __shared__ double whl[kRansacWarps][9];
+    const int warp = threadIdx.x >> 5, dir = blockIdx.y;
     const int cell = blockIdx.x * kRansacWarps + warp;
     if (cell >= g.ncells()) return;
-    float4* match = warp_dyn + warp * MS;
-    Mef* hyp = reinterpret_cast<Mef*>(warp_dyn + kRansacWarps * MS) + warp * 32;
-    char* hx = reinterpret_cast<char*>(warp_dyn + kRansacWarps * MS + kRansacWarps * 32 * 4) +
-               (size_t)warp * ransac_warp_hx_bytes(LANE);
-    WarpGroup grp;
-    ransac_fit<WarpGroup, ST, LANE>(grp, pv, g, level, stage, pp, blockIdx.y, cell, match, hyp, nullptr, nullptr,
-                                    &wmef[warp], hx);
+    const WarpGroup grp;
+    const int id = (g.base + cell) * 2 + (stage - 1);
+    RefitWork* rw = pv.rw[dir] + cell;
+    Window w;
+    gather_window(grp, pv, g, stage, dir, cell, planes[warp], CAP, 4, w);
+    if (grp.rank() == 0) clear_model(pv, dir, id, w.N, rw);
+    if (w.N < pp.min_inliers || w.N < 4) return;
+    const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
+    RansacStats st;
+    const unsigned long long best = search_warp(w, pp, cell, tag, pv.pair_id, &slot[warp], st);
+    finish_fit(grp, pv, w, pp, dir, cell, id, tag, best, st, &wmef[warp], whl[warp], rw);
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
@@ -1400,23 +1548,32 @@ __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constan
     ransac_finish<WarpGroup, ST>(grp, pv, g, stage, pp, blockIdx.y, cell, match[warp]);
 }
 
-// Larger windows: one 256-thread block per window (matches in dynamic shared memory).
-template <int ST>
-__global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
+// Larger windows: one 256-thread block per window (matches in dynamic shared memory: four planes of block_cap(s)).
+__host__ __device__ constexpr int block_cap(int s) { return (s * s + 127) / 128 * 128; }
+__global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__ Batch bt, int level, int stage,
+                                                         PlaneParams pp) {
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
-    if ((int)blockIdx.x >= g.ncells()) return;  // past this pair's windows (block-uniform)
-    extern __shared__ float4 match_dyn[];
+    const int cell = blockIdx.x, dir = blockIdx.y;
+    if (cell >= g.ncells()) return;  // past this pair's windows (block-uniform)
+    extern __shared__ __align__(16) float planes_dyn[];
     __shared__ double red_d[8];
     __shared__ int red_i[8];
     __shared__ unsigned long long red_u[8];
-    __shared__ Mef hyp[8 * 32];
+    __shared__ __align__(16) BlockSearch bs;
     __shared__ Mef wmef;
-    __shared__ int gbest, kfull;
-    BlockGroup<256> grp{red_d, red_i, red_u};
-    __shared__ double hl[8 * 32 * 9];  // the exact forms of the block's 8 x 32 hypotheses in flight
-    ransac_fit<BlockGroup<256>, ST, false>(grp, pv, g, level, stage, pp, blockIdx.y, blockIdx.x, match_dyn, hyp,
-                                           &gbest, &kfull, &wmef, hl);
+    __shared__ double whl[9];
+    const BlockGroup<256> grp{red_d, red_i, red_u};
+    const int id = (g.base + cell) * 2 + (stage - 1);
+    RefitWork* rw = pv.rw[dir] + cell;
+    Window w;
+    gather_window(grp, pv, g, stage, dir, cell, planes_dyn, block_cap(g.s), 128, w);
+    if (threadIdx.x == 0) clear_model(pv, dir, id, w.N, rw);
+    if (w.N < pp.min_inliers || w.N < 4) return;
+    const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
+    RansacStats st;
+    const unsigned long long best = search_block(grp, w, pp, cell, tag, pv.pair_id, bs, st);
+    finish_fit(grp, pv, w, pp, dir, cell, id, tag, best, st, &wmef, whl, rw);
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
@@ -1902,32 +2059,24 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
                              const PlaneParams& pp, cudaStream_t st) {
     const int nc = max_cells;
     if (s <= 16) {
-        static bool wattr_set = false;
-        if (!wattr_set) {
-            cudaFuncSetAttribute(k_ransac_warp<ST, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)ransac_warp_smem(false));
-            cudaFuncSetAttribute(k_ransac_warp<ST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)ransac_warp_smem(true));
-            wattr_set = true;
-        }
         const dim3 fgrid((nc + kRansacWarps - 1) / kRansacWarps, 2, np), grid((nc + 7) / 8, 2, np);
-        if (s * s <= kLaneScoreMax)
-            k_ransac_warp<ST, true><<<fgrid, 32 * kRansacWarps, ransac_warp_smem(true), st>>>(bt, level, stage, pp);
+        if (s <= 8)
+            k_ransac_warp<64><<<fgrid, 32 * kRansacWarps, 0, st>>>(bt, level, stage, pp);
         else
-            k_ransac_warp<ST, false><<<fgrid, 32 * kRansacWarps, ransac_warp_smem(false), st>>>(bt, level, stage, pp);
+            k_ransac_warp<256><<<fgrid, 32 * kRansacWarps, 0, st>>>(bt, level, stage, pp);
         k_refit_solve<<<dim3((2 * nc + 63) / 64, 1, np), 64, 0, st>>>(bt, level, pp);
         k_ransac_finish_warp<ST><<<grid, 256, 0, st>>>(bt, level, stage, pp);
         return;
     }
-    const size_t smem = (size_t)s * s * sizeof(float4);
+    const size_t smem = (size_t)s * s * sizeof(float4), fit_smem = (size_t)block_cap(s) * sizeof(float4);
     static bool attr_set = false;
     if (!attr_set) {
         const int mx = kMaxCell * kMaxCell * (int)sizeof(float4);  // the largest window's matches
-        cudaFuncSetAttribute(k_ransac_block<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        cudaFuncSetAttribute(k_ransac_block, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
         cudaFuncSetAttribute(k_ransac_finish_block<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
         attr_set = true;
     }
-    k_ransac_block<ST><<<dim3(nc, 2, np), 256, smem, st>>>(bt, level, stage, pp);
+    k_ransac_block<<<dim3(nc, 2, np), 256, fit_smem, st>>>(bt, level, stage, pp);
     k_refit_solve<<<dim3((2 * nc + 63) / 64, 1, np), 64, 0, st>>>(bt, level, pp);
     k_ransac_finish_block<ST><<<dim3(nc, 2, np), 256, smem, st>>>(bt, level, stage, pp);
 }
