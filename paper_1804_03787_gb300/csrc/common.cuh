@@ -476,10 +476,11 @@ struct Labels {
 // solve, finish) and reused by every level and stage.
 struct __align__(16) RefitWork {
     long long mom[24];      // exact DLT moments of the winner's inliers about (cx, cy, cu, cv)
-    __int128 hx[9];         // the winning hypothesis, exact
+    int sample[16];         // the winner's sample, window-local: source x[4], y[4], target x[4], y[4]
     Mef mef0, mef1;         // evaluation forms (origin 0) of the winner and of the refit, with test bounds
-    double hl_r[9];         // the refit in window-local coordinates, denominator 1 at the window centre (FP64 tests)
-    double ds, dt;          // sums of the inliers' distances to the source / target centroids
+    double hl_w[9], hl_r[9];  // the winner and the refit in window-local coordinates, denominator positive at the
+                              // window centre (FP64 tests)
+    double ds, dt;          // sums of nin times the inliers' distances to the source / target centroids
     double ha_w[9], ha_r[9];  // absolute homographies of the winner and of the refit
     int cx, cy, cu, cv;     // integer centres of the moments
     int status;             // 2: refit pending (set by the fit), else the window is final

@@ -78,20 +78,19 @@ __host__ __device__ inline void minimal_h_exact(const int* px, const int* py, co
     }
     int l[3];
     int64_t mu[3];
-    i128 w[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const int i = (k + 1) % 3, j = (k + 2) % 3;
         l[k] = dx[i] * dy[j] - dx[j] * dy[i];
         mu[k] = X[i] * Y[j] - X[j] * Y[i];
     }
-    // H' (its third column is (0, 0, h22))
+    // H' (its third column is (0, 0, h22)); rolled: the few threads that run this wait for its instructions
     i128 h[3][2] = {}, h22 = (i128)((int64_t)l[0] * l[1] * l[2]) * (mu[0] + mu[1] + mu[2]);
-#pragma unroll
+#pragma unroll 1
     for (int k = 0; k < 3; ++k) {
         const int i = (k + 1) % 3, j = (k + 2) % 3;
-        w[k] = (i128)mu[k] * ((int64_t)l[i] * l[j]);
-        const i128 a = w[k] * (dy[i] - dy[j]), b = w[k] * (dx[j] - dx[i]);
+        const i128 w = (i128)mu[k] * ((int64_t)l[i] * l[j]);
+        const i128 a = w * (dy[i] - dy[j]), b = w * (dx[j] - dx[i]);
         h[0][0] += a * X[k];
         h[0][1] += b * X[k];
         h[1][0] += a * Y[k];
@@ -140,18 +139,27 @@ __host__ __device__ inline bool make_mef_exact(const i128* Hin, Mef& m) {
     i128 dc2 = 2 * Hin[8] - (Hin[6] + Hin[7]);  // twice the denominator at the centre (-0.5, -0.5)
     if (dc2 == 0) return false;
     const bool flip = dc2 < 0;
+#pragma unroll 1
     for (int k = 0; k < 9; ++k) H[k] = flip ? -Hin[k] : Hin[k];
     if (flip) dc2 = -dc2;
     const float rd = 1.f / i128_to_float(dc2);  // one reciprocal, then products (about 1 ulp each)
-    m.b0 = i128_to_float(2 * H[0] - dc2) * rd;
-    m.h1 = i128_to_float(2 * H[1]) * rd;
-    split_ratio(2 * H[2], dc2, rd, m.h2h, m.h2l);
-    m.h3 = i128_to_float(2 * H[3]) * rd;
-    m.b4 = i128_to_float(2 * H[4] - dc2) * rd;
-    split_ratio(2 * H[5], dc2, rd, m.h5h, m.h5l);
-    m.g0 = i128_to_float(2 * H[6]) * rd;
-    m.g1 = i128_to_float(2 * H[7]) * rd;
-    m.e0 = i128_to_float(2 * H[8] - dc2) * rd;
+    float c[9];
+#pragma unroll 1
+    for (int k = 0; k < 9; ++k) c[k] = i128_to_float(2 * H[k] - ((k & 3) == 0 ? dc2 : 0)) * rd;  // k = 0, 4, 8: less 1
+    m.b0 = c[0];
+    m.h1 = c[1];
+    m.h3 = c[3];
+    m.b4 = c[4];
+    m.g0 = c[6];
+    m.g1 = c[7];
+    m.e0 = c[8];
+    float t[2][2];
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) split_ratio(2 * H[2 + 3 * k], dc2, rd, t[k][0], t[k][1]);
+    m.h2h = t[0][0];
+    m.h2l = t[0][1];
+    m.h5h = t[1][0];
+    m.h5l = t[1][1];
     m.ef = 0.f;
     m.ox = 0;
     m.oy = 0;
@@ -177,13 +185,13 @@ __host__ __device__ __forceinline__ int u128_bits(u128 u) {
 // 64-bit integer conversion or an FP64 divide issues on the slow FP64 pipe).
 __host__ __device__ inline void exact_to_double_pow2(const i128* H, double* D, bool flip) {
     int bl[9], E = 0;
-#pragma unroll
+#pragma unroll 1
     for (int k = 0; k < 9; ++k) {
         const u128 u = H[k] < 0 ? (u128)0 - (u128)H[k] : (u128)H[k];
         bl[k] = u128_bits(u);
         E = bl[k] > E ? bl[k] : E;
     }
-#pragma unroll
+#pragma unroll 1
     for (int k = 0; k < 9; ++k) {
         const bool neg = H[k] < 0;
         const u128 u = neg ? (u128)0 - (u128)H[k] : (u128)H[k];
@@ -205,6 +213,7 @@ __host__ __device__ inline void exact_to_double_pow2(const i128* H, double* D, b
 
 // The first n entries of an exact homography as doubles (unnormalised).
 __host__ __device__ inline void exact_to_double(const i128* H, double* D, int n = 9) {
+#pragma unroll 1
     for (int k = 0; k < n; ++k) {
         const bool neg = H[k] < 0;
         const u128 u = neg ? (u128)0 - (u128)H[k] : (u128)H[k];

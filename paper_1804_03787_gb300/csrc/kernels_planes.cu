@@ -107,24 +107,8 @@ struct WarpGroup {
         for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
         return v;
     }
-    __device__ int sum(int v) const {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-        return v;
-    }
-    __device__ unsigned long long max(unsigned long long v) const {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const unsigned long long o = __shfl_xor_sync(FULL, v, off);
-            v = o > v ? o : v;
-        }
-        return v;
-    }
-    __device__ long long sum(long long v) const {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-        return v;
-    }
+    __device__ int sum(int v) const { return (int)__reduce_add_sync(FULL, (unsigned)v); }
+    __device__ unsigned max(unsigned v) const { return __reduce_max_sync(FULL, v); }
     __device__ bool any(bool p) const { return __any_sync(FULL, p); }
     // exclusive prefix of `take` over the group and the total
     __device__ int scan(bool take, int& total) const {
@@ -153,8 +137,7 @@ struct BlockGroup {
         return t;
     }
     __device__ int sum(int v) const {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+        v = (int)__reduce_add_sync(FULL, (unsigned)v);
         __syncthreads();
         if ((threadIdx.x & 31) == 0) red_i[threadIdx.x >> 5] = v;
         __syncthreads();
@@ -162,17 +145,16 @@ struct BlockGroup {
         for (int w = 0; w < NT / 32; ++w) t += red_i[w];
         return t;
     }
-    __device__ bool any(bool p) const { return __syncthreads_or(p) != 0; }
-    __device__ long long sum(long long v) const {  // exact: integer addition in any order
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+    __device__ unsigned max(unsigned v) const {
+        v = __reduce_max_sync(FULL, v);
         __syncthreads();
-        if ((threadIdx.x & 31) == 0) red_u[threadIdx.x >> 5] = (unsigned long long)v;
+        if ((threadIdx.x & 31) == 0) red_i[threadIdx.x >> 5] = (int)v;
         __syncthreads();
-        unsigned long long t = 0;
-        for (int w = 0; w < NT / 32; ++w) t += red_u[w];
-        return (long long)t;
+        unsigned t = 0;
+        for (int w = 0; w < NT / 32; ++w) t = (unsigned)red_i[w] > t ? (unsigned)red_i[w] : t;
+        return t;
     }
+    __device__ bool any(bool p) const { return __syncthreads_or(p) != 0; }
     __device__ unsigned long long max(unsigned long long v) const {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
@@ -647,9 +629,8 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
         w.x[j] = w.y[j] = 0.f;
         w.qx[j] = w.qy[j] = kFarTarget;
     }
-    // integers: exact as keys; the larger of the two decides which bound holds, so one reduction each
-    w.vmax = (float)grp.max((unsigned long long)vm);
-    w.vq = (float)grp.max((unsigned long long)vq);
+    w.vmax = (float)grp.max((unsigned)vm);  // non-negative integers
+    w.vq = (float)grp.max((unsigned)vq);
     grp.sync();
 }
 
@@ -935,6 +916,19 @@ __device__ int gather_matches(const G& grp, const PairView& pv, const LevelGeom&
     return N;
 }
 
+// A positive normal float, and an integer in [1, 2^62], as doubles: assembled from their bits (a conversion issues on
+// the FP64 pipe, 64 cycles a warp instruction on GB300); above 2^53 the integer is converted, rounded once.
+__device__ __forceinline__ double double_of(float f) {
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+__device__ __forceinline__ double double_of(long long K) {
+    const int lz = __clzll(K);
+    const unsigned long long m = (unsigned long long)K << lz;
+    if (m & 0x7FFull) return (double)K;
+    return __longlong_as_double(((long long)(1085 - lz) << 52) + (long long)(m >> 11));
+}
+
 // Sum of |(a, b)| over a lane's points, for exact integers a, b: each root of
 // the sum of squares K (exact in 64-bit integers, rounded once to FP64 above
 // 2^53) to about 1e-14 relative, added in FP64.  The least-squares refit of a thin, ill-conditioned support
@@ -942,100 +936,82 @@ __device__ int gather_matches(const G& grp, const PairView& pv, const LevelGeom&
 // FP32 rounding (with FP32 roots, refits moved by ~1e-6).  The root: the FP32
 // root s0 and reciprocal 1 / (2 s0), then one Newton step in FP64,
 // s0 + (K - s0^2) / (2 s0): its error is about s0 times the square of s0's
-// relative error (2^-23), against some ten FP64 operations of a full FP64
-// root on GB300's slow FP64 pipe.
-struct DistSum {
-    double s = 0.0;
-    __device__ __forceinline__ void add(int a, int b) {
-        const long long K = (long long)a * a + (long long)b * b;  // exact: |a|, |b| < 2^31
-        const float fa = (float)a, fb = (float)b;
-        const float s0 = sqrtf(fmaf(fa, fa, fb * fb));
-        if (!(s0 > 0.f)) return;  // K = 0
-        const double sd = (double)s0;
-        const double e = fma(-sd, sd, (double)K);
-        s += fma(e, (double)(0.5f / s0), sd);
-    }
-    __device__ __forceinline__ double total() const { return s; }
-};
+// relative error (2^-23), for three FP64 operations.
+__device__ __forceinline__ void add_dist(double& s, int a, int b) {
+    const long long K = (long long)a * a + (long long)b * b;  // exact: |a|, |b| < 2^31
+    const float fa = (float)a, fb = (float)b;
+    const float s0 = sqrtf(fmaf(fa, fa, fb * fb));
+    if (!(s0 > 0.f)) return;  // K = 0
+    const double sd = double_of(s0);
+    const double e = fma(-sd, sd, double_of(K));
+    s += fma(e, double_of(0.5f / s0), sd);
+}
 
-// Refit inputs on the winner's inliers, for ransac_fit (out of line: once per window, and its 24 integer
-// moments would otherwise crowd the registers of the hypothesis loop).
-template <class G>
-__device__ __noinline__ void winner_moments(const G& grp, const Window& w, const Mef* wmef, const double* whl, float t2,
-                                            int wscore, RefitWork* rw) {
-    const int tid = grp.rank(), N = w.N;
-    // Hartley centroids (exact integer sums), mean distances, and the DLT moments as exact integers about the
-    // rounded centroids
-    const Mef wm = *wmef;
-    // the winner's inlier test, certified: an uncertain one is decided in FP64 with the exact winner
-    auto winner_inlier = [&](const float4& mt) -> bool {
-        bool unc;
-        const bool in = cert_inlier(wm, mt, t2, unc);
-        return unc ? hyp_inlier_fp64(whl, mt.x, mt.y, mt.z, mt.w, (double)t2) : in;
+// The warp's totals of the lanes' 24 moments, one on each lane whose low two index bits are below 3 (`slot`: its
+// index): five exchange steps halve what a lane keeps, 24 exchanges in all instead of 120.
+__device__ __forceinline__ long long warp_moments(const long long (&R)[24], int& slot) {
+    const int lane = threadIdx.x & 31;
+    long long a[12], b[6], c[4], d[2];
+    auto step = [&](bool hi, long long lo_v, long long hi_v, int off) {
+        const long long send = hi ? lo_v : hi_v;
+        return (hi ? hi_v : lo_v) + __shfl_xor_sync(FULL, send, off);
     };
-    // the winner's inliers among this thread's matches (bit c: match tid + c G::size; N <= 64 G::size for
-    // every group: 256 matches per warp window, 96 x 96 per block window)
-    static_assert(kMaxCell * kMaxCell <= 64 * 256 && 16 * 16 <= 64 * 32, "inlier mask too small");
-    unsigned long long inm = 0;
-    int sx = 0, sy = 0, tx = 0, ty = 0;
-    for (int j = tid, c = 0; j < N; j += G::size, ++c) {
-        const float4 mt = w.match(j);
-        if (winner_inlier(mt)) {
-            inm |= 1ull << c;
-            sx += exact_int(mt.x);
-            sy += exact_int(mt.y);
-            tx += exact_int(mt.x + mt.z);
-            ty += exact_int(mt.y + mt.w);
-        }
-    }
-    sx = grp.sum(sx);
-    sy = grp.sum(sy);
-    tx = grp.sum(tx);
-    ty = grp.sum(ty);
-    const float fn = (float)wscore;
-    const float fmx = __fdiv_rn((float)sx, fn), fmy = __fdiv_rn((float)sy, fn);
-    const float fmqx = __fdiv_rn((float)tx, fn), fmqy = __fdiv_rn((float)ty, fn);
-    const int cx = __float2int_rn(fmx), cy = __float2int_rn(fmy), cu = __float2int_rn(fmqx), cv = __float2int_rn(fmqy);
-    // Hartley scales: distances to the exact centroids, as n |p - mean| = |n p - sum| from exact integers
-    // (the least-squares refit of a noisy support moves with its normalisation, so the scale must carry no
-    // more than float rounding)
-    const int nw = wscore;  // n |coordinate| < 2^31 for frames up to 32767 px and windows up to 96 px
-    DistSum dsum, dtsum;
-    long long R[24];
 #pragma unroll
-    for (int q = 0; q < 24; ++q) R[q] = 0;
-    for (; inm; inm &= inm - 1) {
-        const float4 mt = w.match(tid + (__ffsll((long long)inm) - 1) * G::size);
-        dsum.add(nw * exact_int(mt.x) - sx, nw * exact_int(mt.y) - sy);
-        dtsum.add(nw * exact_int(mt.x + mt.z) - tx, nw * exact_int(mt.y + mt.w) - ty);
-        const int X = exact_int(mt.x) - cx, Y = exact_int(mt.y) - cy;
-        const int U = exact_int(mt.x + mt.z) - cu, V = exact_int(mt.y + mt.w) - cv;
-        const int zz[6] = {X * X, X * Y, X, Y * Y, Y, 1};
-        const int w3 = U * U + V * V;
+    for (int q = 0; q < 12; ++q) a[q] = step(lane & 16, R[q], R[q + 12], 16);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            R[q] += zz[q];
-            R[6 + q] += (long long)U * zz[q];
-            R[12 + q] += (long long)V * zz[q];
-            R[18 + q] += (long long)w3 * zz[q];
-        }
-    }
-    const double ds = grp.sum(dsum.total()) / (double)nw;  // sums of |p - mean|
-    const double dt = grp.sum(dtsum.total()) / (double)nw;
+    for (int q = 0; q < 6; ++q) b[q] = step(lane & 8, a[q], a[q + 6], 8);
 #pragma unroll
-    for (int q = 0; q < 24; ++q) {
-        const long long t = grp.sum(R[q]);
-        if (tid == q) rw->mom[q] = t;
+    for (int q = 0; q < 3; ++q) c[q] = step(lane & 4, b[q], b[q + 3], 4);
+    c[3] = 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) d[q] = step(lane & 2, c[q], c[q + 2], 2);
+    const int low = lane & 3;
+    slot = low < 3 ? ((lane & 16) ? 12 : 0) + ((lane & 8) ? 6 : 0) + ((lane & 4) ? 3 : 0) + low : -1;
+    return step(lane & 1, d[0], d[1], 1);
+}
+// Totals of the 24 moments over the group, into out; scratch: 24 values per warp (blocks).
+__device__ __forceinline__ void group_moments(const WarpGroup&, const long long (&R)[24], long long*, long long* out) {
+    int q;
+    const long long t = warp_moments(R, q);
+    if (q >= 0) out[q] = t;
+}
+template <int NT>
+__device__ __forceinline__ void group_moments(const BlockGroup<NT>&, const long long (&R)[24], long long* scratch,
+                                              long long* out) {
+    int q;
+    const long long t = warp_moments(R, q);
+    if (q >= 0) scratch[(threadIdx.x >> 5) * 24 + q] = t;
+    __syncthreads();
+    if (threadIdx.x < 24) {
+        long long v = 0;
+        for (int w = 0; w < NT / 32; ++w) v += scratch[w * 24 + threadIdx.x];
+        out[threadIdx.x] = v;
     }
-    if (tid == 0) {
-        rw->ds = ds;
-        rw->dt = dt;
-        rw->cx = cx;
-        rw->cy = cy;
-        rw->cu = cu;
-        rw->cv = cv;
-        rw->nin = wscore;
-        rw->status = 2;
+}
+// The warp's sums of two doubles, each added in the order of an exchange over lane distances 16, 8, 4, 2, 1, in one
+// chain of five additions: lanes 0-15 keep the first, lanes 16-31 the second.
+__device__ __forceinline__ double warp_sum_pair(double first, double second) {
+    const bool hi = threadIdx.x & 16;
+    double v = (hi ? second : first) + __shfl_xor_sync(FULL, hi ? first : second, 16);
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+    return v;
+}
+__device__ __forceinline__ void group_dists(const WarpGroup&, double s, double t, double*, RefitWork* rw) {
+    const double v = warp_sum_pair(s, t);
+    if ((threadIdx.x & 31) == 0) rw->ds = v;
+    if ((threadIdx.x & 31) == 16) rw->dt = v;
+}
+template <int NT>
+__device__ __forceinline__ void group_dists(const BlockGroup<NT>&, double s, double t, double* scratch, RefitWork* rw) {
+    const double v = warp_sum_pair(s, t);
+    const int lane = threadIdx.x & 31;
+    if ((lane & 15) == 0) scratch[(threadIdx.x >> 5) * 2 + (lane >> 4)] = v;
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double a = 0;
+        for (int w = 0; w < NT / 32; ++w) a += scratch[w * 2 + threadIdx.x];  // in warp order
+        (threadIdx.x ? rw->dt : rw->ds) = a;
     }
 }
 
@@ -1050,37 +1026,26 @@ __device__ __forceinline__ void clear_model(const PairView& pv, int dir, int id,
     rw->status = 0;
 }
 
-// The winner drawn again, exact, by one warp (out of line, once per window).
-__device__ __noinline__ void emit_winner(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id, uint32_t k0,
-                                         uint32_t k1, float t2, Mef* wmef, double* whl, RefitWork* rw) {
-    const int lane = threadIdx.x & 31;
+// The exact hypothesis k in FP64 (shared memory), by one warp: for the winner's uncertain tests.  Out of line (rare).
+__device__ __noinline__ void winner_fp64(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id, uint32_t k0,
+                                         uint32_t k1, double* whl) {
     i128 Hk[9];
     draw_exact(w, cell, k, tag, pair_id, k0, k1, Hk);
     double Hl[9];
     exact_local_fp64(Hk, Hl);
-#pragma unroll
-    for (int q = 0; q < 9; ++q)
-        if (lane == q) {
-            whl[q] = Hl[q];
-            rw->hx[q] = Hk[q];
-        }
-    if (lane == 0) {
-        Mef m0;
-        make_mef_exact(Hk, m0);
-        mef_set_bounds(m0, w.U, w.vmax, t2);
-        *wmef = m0;
-        rw->mef0 = m0;
-        rw->vmax = w.vmax;
-    }
+    if ((threadIdx.x & 31) == 0)
+        for (int q = 0; q < 9; ++q) whl[q] = Hl[q];
 }
 
-// What follows the search: the winner drawn again, exact, with its evaluation form and its FP64 form for uncertain
-// tests (whl, shared memory), and the refit's inputs on its inliers.  best: the winner's key, 0 if there is none.
+// What follows the search: the refit's inputs on the winner's inliers (Hartley centroids as exact integer sums,
+// distances, and the DLT moments as exact integers about the rounded centroids) and the winner's sample, from which
+// the solve (a thread per window) forms the exact homography.  best: the winner's key, 0 if there is none; whl: 9
+// doubles of shared memory; scratch: 24 values per warp of a block.
 template <class G>
 __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, const Window& w, const PlaneParams& pp,
                                            int dir, int cell, int id, uint32_t tag, unsigned long long best,
-                                           const RansacStats& st, Mef* wmef, double* whl, RefitWork* rw) {
-    const int tid = grp.rank();
+                                           const RansacStats& st, double* whl, long long* scratch, RefitWork* rw) {
+    const int tid = grp.rank(), N = w.N;
     int* mi = pv.mi[dir] + (size_t)id * kMI;
     if (pv.evals) {  // residual tests performed, those decided in FP64, loose hypotheses (profiling)
         const bool one = (tid & 31) == 0;
@@ -1095,17 +1060,98 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
         if (tid == 0) mi[MI_BESTSCORE] = -1;
         return;
     }
-    const int wscore = key_score(best), wk = key_index(best);
-    if (tid < 32) {  // first warp
-        emit_winner(w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, pp.t2, wmef, whl, rw);
-        if (tid == 0) {
-            mi[MI_BESTK] = wk;
-            mi[MI_BESTSCORE] = wscore;
+    const int nw = key_score(best), wk = key_index(best);
+    if (tid == 0) {
+        mi[MI_BESTK] = wk;
+        mi[MI_BESTSCORE] = nw;
+    }
+    if (nw < 4) return;
+    // the winner's inliers among this thread's matches (bit c: match tid + c G::size; N <= 64 G::size for every
+    // group: 256 matches per warp window, 96 x 96 per block window), uncertain ones decided in FP64
+    static_assert(kMaxCell * kMaxCell <= 64 * 256 && 16 * 16 <= 64 * 32, "inlier mask too small");
+    unsigned long long inm = 0, um = 0;
+    {
+        FastHyp h;
+        const float tl = t_below(pp.t2), th = t_above(pp.t2);
+        const bool scored = fast_hypothesis(w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, th, h) == HYP_OK;
+        for (int j = tid, c = 0; j < N; j += G::size, ++c) {
+            bool sure = false, maybe = true;
+            if (scored) test_match(w, h, tl, th, j, sure, maybe);
+            if (sure)
+                inm |= 1ull << c;
+            else if (maybe)
+                um |= 1ull << c;
         }
     }
-    grp.sync();
-    if (wscore < 4) return;
-    winner_moments<G>(grp, w, wmef, whl, pp.t2, wscore, rw);
+    if (grp.any(um != 0)) {
+        if (tid < 32) winner_fp64(w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, whl);
+        grp.sync();
+        for (; um; um &= um - 1) {
+            const int c = __ffsll((long long)um) - 1;
+            const float4 mt = w.match(tid + c * G::size);
+            if (hyp_inlier_fp64(whl, mt.x, mt.y, mt.z, mt.w, (double)pp.t2)) inm |= 1ull << c;
+        }
+    }
+    int sx = 0, sy = 0, tx = 0, ty = 0;  // target sums about v0
+    for (unsigned long long m = inm; m; m &= m - 1) {
+        const int j = tid + (__ffsll((long long)m) - 1) * G::size;
+        sx += exact_int(w.x[j]);
+        sy += exact_int(w.y[j]);
+        tx += exact_int(w.qx[j]);
+        ty += exact_int(w.qy[j]);
+    }
+    const int v0x = exact_int(w.v0x), v0y = exact_int(w.v0y);
+    sx = grp.sum(sx);
+    sy = grp.sum(sy);
+    tx = grp.sum(tx) + nw * v0x;
+    ty = grp.sum(ty) + nw * v0y;
+    const float fn = (float)nw;
+    const int cx = __float2int_rn(__fdiv_rn((float)sx, fn)), cy = __float2int_rn(__fdiv_rn((float)sy, fn));
+    const int cu = __float2int_rn(__fdiv_rn((float)tx, fn)), cv = __float2int_rn(__fdiv_rn((float)ty, fn));
+    // Hartley scales: distances to the exact centroids, as n |p - mean| = |n p - sum| from exact integers
+    // (the least-squares refit of a noisy support moves with its normalisation, so the scale must carry no
+    // more than float rounding); n |coordinate| < 2^31 for frames up to 32767 px and windows up to 96 px
+    double ds = 0.0, dt = 0.0;
+    long long R[24];
+#pragma unroll
+    for (int q = 0; q < 24; ++q) R[q] = 0;
+    for (; inm; inm &= inm - 1) {
+        const int j = tid + (__ffsll((long long)inm) - 1) * G::size;
+        const int ax = exact_int(w.x[j]), ay = exact_int(w.y[j]);
+        const int bx = exact_int(w.qx[j]) + v0x, by = exact_int(w.qy[j]) + v0y;
+        add_dist(ds, nw * ax - sx, nw * ay - sy);
+        add_dist(dt, nw * bx - tx, nw * by - ty);
+        const int X = ax - cx, Y = ay - cy, U = bx - cu, V = by - cv;
+        const int zz[6] = {X * X, X * Y, X, Y * Y, Y, 1};
+        const int w3 = U * U + V * V;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            R[q] += zz[q];
+            R[6 + q] += (long long)U * zz[q];
+            R[12 + q] += (long long)V * zz[q];
+            R[18 + q] += (long long)w3 * zz[q];
+        }
+    }
+    group_dists(grp, ds, dt, reinterpret_cast<double*>(whl), rw);
+    group_moments(grp, R, scratch, rw->mom);
+    if (tid < 4) {
+        int idx[4];
+        draw_indices(N, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, idx);
+        const int j = tid == 0 ? idx[0] : (tid == 1 ? idx[1] : (tid == 2 ? idx[2] : idx[3]));
+        rw->sample[tid] = exact_int(w.x[j]);
+        rw->sample[4 + tid] = exact_int(w.y[j]);
+        rw->sample[8 + tid] = exact_int(w.qx[j]) + v0x;
+        rw->sample[12 + tid] = exact_int(w.qy[j]) + v0y;
+    }
+    if (tid == 0) {
+        rw->cx = cx;
+        rw->cy = cy;
+        rw->cu = cu;
+        rw->cv = cv;
+        rw->nin = nw;
+        rw->vmax = w.vmax;
+        rw->status = 2;
+    }
 }
 
 // The search keeps the hypothesis with the most inliers (lowest index on ties).  Every hypothesis is bounded, not
@@ -1121,7 +1167,8 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
 // passes spread over the window; after each, lanes that cannot win drop out, and once few are left the warp counts
 // those one by one with its lanes over the matches.
 // What bounds it: instruction fetch, then the FP32 pipe in the tests (12 operations a match).  1024x436, stage 1:
-// the 16 px windows 1.44 -> 0.64 ms, the 8 px windows 1.73 -> 1.12 ms, against scoring exact 128-bit hypotheses.
+// the 16 px windows 1.44 -> 0.41 ms, the 8 px windows 1.73 -> 0.53 ms, against scoring exact 128-bit hypotheses
+// (0.64 and 1.12 ms of these gains while the winner was still solved here, in 180 KB of code, not 97).
 __device__ __forceinline__ unsigned long long search_warp(const Window& w, const PlaneParams& pp, int cell,
                                                           uint32_t tag, uint32_t pair_id, FastHyp* slot,
                                                           RansacStats& st) {
@@ -1180,7 +1227,7 @@ __device__ __forceinline__ unsigned long long search_warp(const Window& w, const
 // one with the most is counted from below on all of them, by the whole block, which gives the bound the others have
 // to reach from the start; then the warps take the hypotheses that still can, one at a time, chunk by chunk.
 // What bounds it: the FP32 pipe and the shared loads of the tests.  1024x436, stage 1: the 64 px windows 1.99 ->
-// 0.85 ms, the 32 px windows 1.03 -> 0.59 ms, against scoring in index order from exact 128-bit hypotheses.
+// 0.77 ms, the 32 px windows 1.03 -> 0.47 ms, against scoring in index order from exact 128-bit hypotheses.
 constexpr int kHypRound = 256;
 struct BlockSearch {
     FastHyp form[kHypRound];
@@ -1311,12 +1358,20 @@ __global__ void __launch_bounds__(64) k_refit_solve(const __grid_constant__ Batc
     if (rw->status != 2) return;
     int x0, y0, ox, oy;
     window_origin<WarpGroup>(g, cell, x0, y0, ox, oy);
-    // the winner, normalised by its largest entry
+    // the winner, exact, from its sample: its evaluation form with test bounds, its FP64 form for uncertain tests,
+    // and itself normalised by its largest entry (a thread per window: the 128-bit solve serves 32 windows an
+    // instruction here; by the fit's warp per window it took a third of the 8 px level's instructions)
     double Hw[9];
-    i128 hx[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) hx[q] = rw->hx[q];
-    exact_to_double(hx, Hw, 9);
+    {
+        i128 hx[9];
+        minimal_h_exact(rw->sample, rw->sample + 4, rw->sample + 8, rw->sample + 12, hx);
+        Mef m0;
+        make_mef_exact(hx, m0);
+        mef_set_bounds(m0, 0.5f * (float)g.s, rw->vmax, pp.t2);
+        rw->mef0 = m0;
+        exact_local_fp64(hx, rw->hl_w);
+        exact_to_double(hx, Hw, 9);
+    }
     double f = 0;
 #pragma unroll
     for (int q = 0; q < 9; ++q) f = fmax(f, fabs(Hw[q]));
@@ -1335,7 +1390,7 @@ __global__ void __launch_bounds__(64) k_refit_solve(const __grid_constant__ Batc
     const double inv_n = 1.0 / (double)rw->nin;
     const double dx = R[2] * inv_n, dy = R[4] * inv_n, du = R[11] * inv_n, dv = R[17] * inv_n;
     const double mx = rw->cx + dx, my = rw->cy + dy, mqx = rw->cu + du, mqy = rw->cv + dv;
-    const double ds = rw->ds * inv_n, dt = rw->dt * inv_n;
+    const double n_in = (double)rw->nin, ds = rw->ds / n_in * inv_n, dt = rw->dt / n_in * inv_n;  // mean distances
     if (!(ds > 1e-12 && dt > 1e-12)) return;
     const double ss = sqrt(2.0) / ds, sq = sqrt(2.0) / dt;
     const double iss = ds * 0.70710678118654752440, isq = dt * 0.70710678118654752440;  // 1 / ss, 1 / sq
@@ -1445,16 +1500,7 @@ __device__ void ransac_finish(const G& grp, const PairView& pv, const LevelGeom&
     const bool use_refit = have_refit && rcount >= wscore;
     Mef fm = use_refit ? rw->mef1 : rw->mef0;
     // the chosen model in FP64 (local coordinates), for decisions the FP32 form cannot certify
-    double Hl[9];
-    if (use_refit) {
-#pragma unroll
-        for (int q = 0; q < 9; ++q) Hl[q] = rw->hl_r[q];
-    } else {
-        i128 hx[9];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) hx[q] = rw->hx[q];
-        exact_local_fp64(hx, Hl);
-    }
+    const double* Hl = use_refit ? rw->hl_r : rw->hl_w;
     const int count = use_refit ? rcount : wscore;
     const void* src = pv.img[dir];
     const void* tgt = pv.img[1 - dir];
@@ -1519,7 +1565,6 @@ __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     const LevelGeom g = bt.geom(blockIdx.z, level);
     __shared__ __align__(16) float planes[kRansacWarps][4 * CAP];
     __shared__ FastHyp slot[kRansacWarps];
-    __shared__ Mef wmef[kRansacWarps];
     __shared__ double whl[kRansacWarps][9];
     const int warp = threadIdx.x >> 5, dir = blockIdx.y;
     const int cell = blockIdx.x * kRansacWarps + warp;
@@ -1534,7 +1579,7 @@ __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
     RansacStats st;
     const unsigned long long best = search_warp(w, pp, cell, tag, pv.pair_id, &slot[warp], st);
-    finish_fit(grp, pv, w, pp, dir, cell, id, tag, best, st, &wmef[warp], whl[warp], rw);
+    finish_fit(grp, pv, w, pp, dir, cell, id, tag, best, st, whl[warp], nullptr, rw);
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
@@ -1561,8 +1606,7 @@ __global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__
     __shared__ int red_i[8];
     __shared__ unsigned long long red_u[8];
     __shared__ __align__(16) BlockSearch bs;
-    __shared__ Mef wmef;
-    __shared__ double whl[9];
+    __shared__ double whl[16];  // also two sums per warp
     const BlockGroup<256> grp{red_d, red_i, red_u};
     const int id = (g.base + cell) * 2 + (stage - 1);
     RefitWork* rw = pv.rw[dir] + cell;
@@ -1573,7 +1617,7 @@ __global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__
     const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
     RansacStats st;
     const unsigned long long best = search_block(grp, w, pp, cell, tag, pv.pair_id, bs, st);
-    finish_fit(grp, pv, w, pp, dir, cell, id, tag, best, st, &wmef, whl, rw);
+    finish_fit(grp, pv, w, pp, dir, cell, id, tag, best, st, whl, reinterpret_cast<long long*>(bs.form), rw);
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
