@@ -225,15 +225,33 @@ __device__ __forceinline__ bool plane_geometry_ok(const double* Hl, int s, int r
     return ok && det > 0 && det >= scale_min * scale_min && det <= scale_max * scale_max;
 }
 
+// A positive normal float as a double, assembled from its bits (a conversion issues on the FP64 pipe, 64 cycles a
+// warp instruction on GB300).
+__device__ __forceinline__ double double_of(float f) {
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+// a < b for non-negative doubles that are not NaN, by their bits (a comparison issues on the FP64 pipe too).
+__device__ __forceinline__ bool less_bits(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+// d < 0, by its bits.
+__device__ __forceinline__ bool negative(double d) {
+    return (unsigned long long)__double_as_longlong(d) - 0x8000000000000001ull < 0x7FF0000000000000ull;
+}
+// Half of a normal double well above the smallest, by its exponent.
+__device__ __forceinline__ double half_of(double r) {
+    return __hiloint2double(__double2hiint(r) - 0x00100000, __double2loint(r));
+}
+
 // 1 / sqrt(n) for a positive normal double: an FP32 estimate refined by two
 // Newton steps (relative error ~1e-16), far fewer FP64 operations than a
 // correctly rounded square root and division.  Inverse iteration only needs a
 // scale close to the unit norm.
+__device__ __noinline__ double rsqrt_wide(double n) { return 1.0 / sqrt(n); }
 __device__ __forceinline__ double rsqrt_nr(double n) {
-    if (!(n > 1e-30 && n < 1e30)) return 1.0 / sqrt(n);  // outside the FP32 estimate's range
-    double r = (double)rsqrtf((float)n);
+    if (!(less_bits(1e-30, n) && less_bits(n, 1e30))) return rsqrt_wide(n);  // outside the FP32 estimate's range
+    double r = double_of(rsqrtf((float)n));
 #pragma unroll
-    for (int k = 0; k < 2; ++k) r = fma(0.5 * r, fma(-n * r, r, 1.0), r);
+    for (int k = 0; k < 2; ++k) r = fma(half_of(r), fma(-n * r, r, 1.0), r);
     return r;
 }
 
@@ -263,6 +281,124 @@ __device__ __forceinline__ bool cholesky9(double (&A)[45], double (&rd)[9]) {
     return ok;
 }
 
+// State of an inverse iteration after e.it steps.
+struct EigState {
+    double sigma, tr, prev, before;  // shift, trace, the last step's change (1e300 after a shift) and the one before
+    int reshifts, slow, it;
+    bool above;  // the last ratio of changes was above 0.5
+};
+// The warp's matrices (packed, one column per lane), and the one window whose iteration the whole warp carries on:
+// the factor of M - sigma I and the vector so far.
+struct EigShared {
+    double M[45][32];
+    EigState e;
+    double A[45], rd[9], x[9];
+};
+constexpr int kEigSteps = 200;
+
+// |d| as bits, which order non-negative doubles (0 for NaN, which fmax would pass over).
+__device__ __forceinline__ unsigned long long abs_bits(double d) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(d) & 0x7FFFFFFFFFFFFFFFull;
+    return b > 0x7FF0000000000000ull ? 0ull : b;
+}
+// diff / prev > 0.9 for 0 < prev / 2 < diff, both normal: from the leading 24 bits, or divided where those are too
+// close to say.
+__device__ __forceinline__ bool ratio_above_0p9(double diff, double prev) {
+    const int hd = __double2hiint(diff), hp = __double2hiint(prev), de = (hd >> 20) - (hp >> 20);
+    if (de > 1) return true;
+    const float md = __int_as_float(0x3F800000 | ((hd & 0xFFFFF) << 3) | ((unsigned)__double2loint(diff) >> 29));
+    const float mp = __int_as_float(0x3F800000 | ((hp & 0xFFFFF) << 3) | ((unsigned)__double2loint(prev) >> 29));
+    const float r = __fdividef(md, mp) * (de > 0 ? 2.f : (de < 0 ? 0.5f : 1.f));
+    return fabsf(r - 0.9f) > 1e-5f ? r > 0.9f : diff / prev > 0.9;
+}
+
+// After a step that changed the unit vector by diff.
+// Stopping: the step's change is below 1e-12 and, when the iteration converges slowly (a small eigen-gap
+// against the shift's distance), so is the remaining error extrapolated from the ratio of successive changes
+// (a small change per step alone would stop a slow iteration far from the vector).  A slow iteration is
+// re-shifted at the current vector's Rayleigh quotient minus twice its residual (still below the smallest
+// eigenvalue), a few times at most.  An iteration that stays slow after them measures the eigen-gap: with
+// the ratio q of successive changes, (lambda_1 - sigma) / (lambda_2 - sigma) = q gives lambda_2 - lambda_1 =
+// (rho - sigma)(1 - q) / q (rho, the Rayleigh quotient, for lambda_1); below 1e-11 of the trace (at most 9
+// times the largest eigenvalue), the gap is far below the 1e-8 of the largest eigenvalue at which the
+// smallest eigenvector is no longer determined to the 1e-6 a refit is compared at, and the iteration stops.
+// The comparisons of q = diff / prev, rounded, with 0.5 are those of diff with prev / 2 (exact), and the one with
+// 0.9 rarely needs the quotient: it is divided only where its value counts.
+//
+// Whether the iteration has converged; notes in e how fast it does.
+__device__ __forceinline__ bool eig_converged(double diff, EigState& e) {
+    const double prev = e.prev;
+    e.before = prev;
+    e.prev = diff;
+    bool below, slow;  // q < 0.5, q > 0.9
+    if (less_bits(1e-280, prev) && !less_bits(1e300, prev) && !less_bits(1e300, diff) && less_bits(1e-280, diff)) {
+        const double h = half_of(prev);
+        below = less_bits(diff, h);
+        e.above = less_bits(h, diff);
+        slow = e.above && ratio_above_0p9(diff, prev);
+    } else {
+        const double q = diff / prev;
+        below = q < 0.5;
+        e.above = q > 0.5;
+        slow = q > 0.9;
+    }
+    e.slow = slow ? e.slow + 1 : 0;  // q >= 1: no convergence at all (a gap below what rounding resolves)
+    // 1e-12 is far below what the rescore (1e-5 near-tie band) and the
+    // model comparison (1e-6) can see
+    if (!less_bits(diff, 1e-12)) return false;
+    if (below) return true;
+    const double q = diff / prev;
+    return diff * q / (1.0 - fmin(q, 0.999999)) < 1e-13;
+}
+// The gap test or the re-shift that is due after a step (column `col` of M is the matrix): 0 stop, 1 go on, 2 go on
+// with the factor B (and 1 / its diagonal, rdB) of the matrix less the new shift.  Out of line: rare, and inlined the
+// compiler fuses parts of it into the caller's arithmetic, which changes the last bits.
+__device__ __noinline__ int eig_gap_or_shift(const double (*M)[32], int col, const double* x, EigState* e, double* B_out,
+                                             double* rd_out) {
+    auto sym = [](int i, int j) { return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i; };
+    double Mx[9], xx = 0, rho = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        double t = 0;
+#pragma unroll
+        for (int j = 0; j < 9; ++j) t = fma(M[sym(i, j)][col], x[j], t);
+        Mx[i] = t;
+        xx = fma(x[i], x[i], xx);
+        rho = fma(x[i], t, rho);
+    }
+    rho /= xx;
+    if (e->reshifts >= 4) {
+        const double q = e->prev / e->before;
+        const double gap = q < 1.0 ? (rho - e->sigma) * (1.0 - q) / q : 0.0;
+        return gap < 1e-11 * e->tr ? 0 : 1;
+    }
+    ++e->reshifts;
+    double rr = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const double r = fma(-rho, x[i], Mx[i]);
+        rr = fma(r, r, rr);
+    }
+    const double sig2 = rho - 2.0 * sqrt(rr / xx);
+    if (!(sig2 > e->sigma)) return 1;
+    double B[45], rd2[9];
+#pragma unroll
+    for (int q = 0; q < 45; ++q) B[q] = M[q][col];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) B[i * (i + 1) / 2 + i] -= sig2;
+    if (!cholesky9(B, rd2)) return 1;
+    e->sigma = sig2;
+    e->prev = 1e300;
+#pragma unroll
+    for (int q = 0; q < 45; ++q) B_out[q] = B[q];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) rd_out[i] = rd2[i];
+    return 2;
+}
+__device__ __forceinline__ bool eig_check_due(const EigState& e) {
+    return e.reshifts < 4 ? e.it >= 2 && e.above : e.slow >= 4 && (e.slow & 3) == 0;
+}
+
 // Unit eigenvector of the smallest eigenvalue of the 9 x 9 symmetric positive
 // semi-definite matrix M (lower triangle packed, row i at i(i+1)/2), from the
 // start x.  The FP64 pipe of this GPU issues a warp instruction in about 64
@@ -278,7 +414,9 @@ __device__ __forceinline__ bool cholesky9(double (&A)[45], double (&rd)[9]) {
 //     is not positive definite (the bound did not hold), the shift falls back
 //     to -1e-13 tr, plain inverse iteration.
 // One thread per window: each FP64 warp instruction serves 32 windows.
-__device__ __forceinline__ void min_eigvec9(const double (&M)[45], double (&x)[9]) {
+// eig_start does 1 and 2 and the first factor, eig_thread and eig_warp the steps.
+__device__ __forceinline__ void eig_start(const double (&M)[45], double (&x)[9], double (&A)[45], double (&rd)[9],
+                                          EigState& e) {
     auto sym = [](int i, int j) { return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i; };
     double tr = 0;
 #pragma unroll
@@ -380,7 +518,6 @@ __device__ __forceinline__ void min_eigvec9(const double (&M)[45], double (&x)[9
     double sigma = rho - 2.0 * sqrt(rr * ixx);
     if (!(sigma > floor_shift)) sigma = floor_shift;
     // 3. shifted inverse iteration in FP64
-    double A[45], rd[9];
 #pragma unroll
     for (int q = 0; q < 45; ++q) A[q] = M[q];
 #pragma unroll
@@ -398,104 +535,148 @@ __device__ __forceinline__ void min_eigvec9(const double (&M)[45], double (&x)[9
 #pragma unroll
         for (int i = 0; i < 9; ++i) x[i] *= s0;
     }
-    // Stopping: the step's change is below 1e-12 and, when the iteration converges slowly (a small eigen-gap
-    // against the shift's distance), so is the remaining error extrapolated from the ratio of successive changes
-    // (a small change per step alone would stop a slow iteration far from the vector).  A slow iteration is
-    // re-shifted at the current vector's Rayleigh quotient minus twice its residual (still below the smallest
-    // eigenvalue), a few times at most.  An iteration that stays slow after them measures the eigen-gap: with
-    // the ratio q of successive changes, (lambda_1 - sigma) / (lambda_2 - sigma) = q gives lambda_2 - lambda_1 =
-    // (rho - sigma)(1 - q) / q (rho, the Rayleigh quotient, for lambda_1); below 1e-11 of the trace (at most 9
-    // times the largest eigenvalue), the gap is far below the 1e-8 of the largest eigenvalue at which the
-    // smallest eigenvector is no longer determined to the 1e-6 a refit is compared at, and the iteration stops.
-    double prev = 1e300;
-    int reshifts = 0, slow = 0;
-    for (int it = 0; it < 200; ++it) {
-        double y[9];
+    e.sigma = sigma;
+    e.tr = tr;
+    e.prev = 1e300;
+    e.reshifts = e.slow = e.it = 0;
+}
+
+// One step on this thread; false: the iteration is over.
+__device__ __forceinline__ bool eig_thread(const double (*M)[32], double (&x)[9], double (&A)[45], double (&rd)[9],
+                                           EigState& e) {
+    double y[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {  // L z = x
-            double t = x[i];
+    for (int i = 0; i < 9; ++i) {  // L z = x
+        double t = x[i];
 #pragma unroll
-            for (int k = 0; k < i; ++k) t = fma(-A[i * (i + 1) / 2 + k], y[k], t);
-            y[i] = t * rd[i];
-        }
+        for (int k = 0; k < i; ++k) t = fma(-A[i * (i + 1) / 2 + k], y[k], t);
+        y[i] = t * rd[i];
+    }
 #pragma unroll
-        for (int i = 8; i >= 0; --i) {  // L^T y = z
-            double t = y[i];
+    for (int i = 8; i >= 0; --i) {  // L^T y = z
+        double t = y[i];
 #pragma unroll
-            for (int k = i + 1; k < 9; ++k) t = fma(-A[k * (k + 1) / 2 + i], y[k], t);
-            y[i] = t * rd[i];
-        }
-        double n = 0, dot = 0;
+        for (int k = i + 1; k < 9; ++k) t = fma(-A[k * (k + 1) / 2 + i], y[k], t);
+        y[i] = t * rd[i];
+    }
+    double n = 0, dot = 0;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            n = fma(y[i], y[i], n);
-            dot = fma(y[i], x[i], dot);
-        }
-        double sc = rsqrt_nr(n);
-        if (dot < 0) sc = -sc;
-        double diff = 0;
+    for (int i = 0; i < 9; ++i) {
+        n = fma(y[i], y[i], n);
+        dot = fma(y[i], x[i], dot);
+    }
+    double sc = rsqrt_nr(n);
+    if (negative(dot)) sc = -sc;
+    unsigned long long diff = 0;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            y[i] *= sc;
-            diff = fmax(diff, fabs(y[i] - x[i]));
-            x[i] = y[i];
-        }
-        // 1e-12 is far below what the rescore (1e-5 near-tie band) and the
-        // model comparison (1e-6) can see
-        const double q = diff / prev;  // convergence ratio of the last step
-        prev = diff;
-        if (diff < 1e-12 && (q < 0.5 || diff * q / (1.0 - fmin(q, 0.999999)) < 1e-13)) break;
-        slow = q > 0.9 ? slow + 1 : 0;  // q >= 1: no convergence at all (a gap below what rounding resolves)
-        if (reshifts >= 4 && slow >= 4 && (slow & 3) == 0) {  // the gap, from the convergence ratio
-            double xx3 = 0, rho3 = 0;
+    for (int i = 0; i < 9; ++i) {
+        y[i] *= sc;
+        diff = max(diff, abs_bits(y[i] - x[i]));
+        x[i] = y[i];
+    }
+    if (eig_converged(__longlong_as_double((long long)diff), e)) return false;
+    if (eig_check_due(e)) {
+        double xc[9], B[45], rdB[9];  // copies: the call must not force x, A and rd out of registers
+        EigState ec = e;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                double t = 0;
+        for (int i = 0; i < 9; ++i) xc[i] = x[i];
+        const int what = eig_gap_or_shift(M, threadIdx.x, xc, &ec, B, rdB);
+        e = ec;
+        if (what == 0) return false;
+        if (what == 2) {
 #pragma unroll
-                for (int j = 0; j < 9; ++j) t = fma(M[sym(i, j)], x[j], t);
-                xx3 = fma(x[i], x[i], xx3);
-                rho3 = fma(x[i], t, rho3);
-            }
-            const double gap = q < 1.0 ? (rho3 / xx3 - sigma) * (1.0 - q) / q : 0.0;
-            if (gap < 1e-11 * tr) break;
-        }
-        if (it >= 2 && q > 0.5 && reshifts < 4) {
-            double Mx2[9], xx2 = 0, rho2 = 0;
+            for (int q = 0; q < 45; ++q) A[q] = B[q];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                double t = 0;
-#pragma unroll
-                for (int j = 0; j < 9; ++j) t = fma(M[sym(i, j)], x[j], t);
-                Mx2[i] = t;
-                xx2 = fma(x[i], x[i], xx2);
-                rho2 = fma(x[i], t, rho2);
-            }
-            rho2 /= xx2;
-            double rr2 = 0;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const double r = fma(-rho2, x[i], Mx2[i]);
-                rr2 = fma(r, r, rr2);
-            }
-            const double sig2 = rho2 - 2.0 * sqrt(rr2 / xx2);
-            if (sig2 > sigma) {
-                double B[45], rd2[9];
-#pragma unroll
-                for (int q2 = 0; q2 < 45; ++q2) B[q2] = M[q2];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) B[i * (i + 1) / 2 + i] -= sig2;
-                if (cholesky9(B, rd2)) {
-#pragma unroll
-                    for (int q2 = 0; q2 < 45; ++q2) A[q2] = B[q2];
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) rd[i] = rd2[i];
-                    sigma = sig2;
-                    prev = 1e300;
-                }
-            }
-            ++reshifts;
+            for (int i = 0; i < 9; ++i) rd[i] = rdB[i];
         }
     }
+    return ++e.it < kEigSteps;
+}
+
+// The iteration of one window (its state in sh, its matrix in column `col`), carried on by the whole warp: the few
+// windows that need many steps (supports of 4 or 5 matches with a nearly two-dimensional null space: up to 200) set
+// the launch's duration, and a step on one thread is some 140 FP64 instructions of 64 cycles each.  Every operation
+// and its order per result are those of eig_thread, so the bits are the same: the forward substitution by columns,
+// lane i holding row i; the backward one (whose order leaves no parallelism) on every lane; the two dot products on
+// even and odd lanes; scaling and difference with lane i on entry i.  About 80 FP64 instructions a step; the eight
+// solves of a 1024x436 pair 3.15 -> 2.36 ms.  The solve kernel hands a window over once it is the warp's last and 4
+// steps are done (98.5 % of the windows need no more): two or more are cheaper side by side on their threads.
+__device__ __noinline__ void eig_warp(EigShared& sh, int col) {
+    const int lane = threadIdx.x & 31, row = min(lane, 8);
+    double A[45], rd[9], x[9], Lr[8], rdr = 0;
+    EigState e = sh.e;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) x[i] = sh.x[i];
+    int loaded = -1;
+    for (;;) {
+        if (loaded != e.reshifts) {  // the factor may be new
+            loaded = e.reshifts;
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < 45; ++q) A[q] = sh.A[q];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) rd[i] = sh.rd[i];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) Lr[k] = sh.A[row * (row + 1) / 2 + min(k, row)];
+            rdr = sh.rd[row];
+        }
+        double z[9], own = x[0];
+#pragma unroll
+        for (int i = 1; i < 9; ++i) own = row == i ? x[i] : own;
+        double t = own;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {  // L z = x
+            z[k] = __shfl_sync(FULL, t * rdr, k);
+            if (k < 8) t = row > k ? fma(-Lr[k < 8 ? k : 0], z[k], t) : t;
+        }
+        double y[9];
+#pragma unroll
+        for (int i = 8; i >= 0; --i) {  // L^T y = z
+            double u = z[i];
+#pragma unroll
+            for (int k = i + 1; k < 9; ++k) u = fma(-A[k * (k + 1) / 2 + i], y[k], u);
+            y[i] = u * rd[i];
+        }
+        double acc = 0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) acc = fma(y[i], (lane & 1) ? x[i] : y[i], acc);
+        const double n = __shfl_sync(FULL, acc, 0), dot = __shfl_sync(FULL, acc, 1);
+        double sc = rsqrt_nr(n);
+        if (negative(dot)) sc = -sc;
+        double yr = y[0];
+#pragma unroll
+        for (int i = 1; i < 9; ++i) yr = row == i ? y[i] : yr;
+        yr *= sc;
+        const unsigned long long d = abs_bits(yr - own);
+        const unsigned hi = __reduce_max_sync(FULL, (unsigned)(d >> 32));
+        const unsigned lo = __reduce_max_sync(FULL, (unsigned)(d >> 32) == hi ? (unsigned)d : 0u);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) x[i] = __shfl_sync(FULL, yr, i);
+        if (eig_converged(__longlong_as_double((long long)(((unsigned long long)hi << 32) | lo)), e)) break;
+        if (eig_check_due(e)) {  // the same on every lane
+            double xc[9], B[45], rdB[9];
+            EigState ec = e;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) xc[i] = x[i];
+            const int what = eig_gap_or_shift(sh.M, col, xc, &ec, B, rdB);
+            e = ec;
+            if (what == 0) break;
+            if (what == 2) {
+                __syncwarp();
+                if (lane == 0) {
+                    for (int q = 0; q < 45; ++q) sh.A[q] = B[q];
+                    for (int i = 0; i < 9; ++i) sh.rd[i] = rdB[i];
+                }
+            }
+        }
+        if (++e.it >= kEigSteps) break;
+    }
+    __syncwarp();
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) sh.x[i] = x[i];
+    }
+    __syncwarp();
 }
 
 // The exact hypothesis as doubles in window-local coordinates, oriented like
@@ -916,12 +1097,7 @@ __device__ int gather_matches(const G& grp, const PairView& pv, const LevelGeom&
     return N;
 }
 
-// A positive normal float, and an integer in [1, 2^62], as doubles: assembled from their bits (a conversion issues on
-// the FP64 pipe, 64 cycles a warp instruction on GB300); above 2^53 the integer is converted, rounded once.
-__device__ __forceinline__ double double_of(float f) {
-    const unsigned b = __float_as_uint(f);
-    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
-}
+// An integer in [1, 2^62] as a double, from its bits; above 2^53 it is converted, rounded once.
 __device__ __forceinline__ double double_of(long long K) {
     const int lz = __clzll(K);
     const unsigned long long m = (unsigned long long)K << lz;
@@ -1343,19 +1519,13 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<256>
     return *vbest;
 }
 
-// (B) Normalised DLT refit of each window whose fit is pending, one thread
-// per window and direction: centred, Hartley-scaled moments from the exact
-// integer ones, the smallest eigenvector of A^T A started from the winner,
-// denormalisation, and the geometry checks of the winner and of the refit.
-__global__ void __launch_bounds__(64) k_refit_solve(const __grid_constant__ Batch bt, int level, PlaneParams pp) {
-    const PairView& pv = bt.view(blockIdx.z);
-    const LevelGeom g = bt.geom(blockIdx.z, level);
-    const int nc = g.ncells();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 2 * nc) return;
-    const int dir = t / nc, cell = t - dir * nc;
-    RefitWork* rw = pv.rw[dir] + cell;
-    if (rw->status != 2) return;
+// The frames a refit is normalised in, for its way back.
+struct RefitFrame {
+    double ss, isq, mx, my, mqx, mqy;
+};
+// One window's normalised DLT matrix M and start x; false if the support has no extent.
+__device__ __forceinline__ bool refit_system(RefitWork* rw, const LevelGeom& g, const PlaneParams& pp, int cell,
+                                             double (&A)[45], double (&x)[9], RefitFrame& f) {
     int x0, y0, ox, oy;
     window_origin<WarpGroup>(g, cell, x0, y0, ox, oy);
     // the winner, exact, from its sample: its evaluation form with test bounds, its FP64 form for uncertain tests,
@@ -1372,10 +1542,10 @@ __global__ void __launch_bounds__(64) k_refit_solve(const __grid_constant__ Batc
         exact_local_fp64(hx, rw->hl_w);
         exact_to_double(hx, Hw, 9);
     }
-    double f = 0;
+    double big = 0;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) f = fmax(f, fabs(Hw[q]));
-    const double rf = 1.0 / f;
+    for (int q = 0; q < 9; ++q) big = fmax(big, fabs(Hw[q]));
+    const double rf = 1.0 / big;
 #pragma unroll
     for (int q = 0; q < 9; ++q) Hw[q] *= rf;
     rw->geo_w = plane_geometry_ok(Hw, g.s, pp.radius, pp.scale_min, pp.scale_max) ? 1 : 0;
@@ -1391,7 +1561,7 @@ __global__ void __launch_bounds__(64) k_refit_solve(const __grid_constant__ Batc
     const double dx = R[2] * inv_n, dy = R[4] * inv_n, du = R[11] * inv_n, dv = R[17] * inv_n;
     const double mx = rw->cx + dx, my = rw->cy + dy, mqx = rw->cu + du, mqy = rw->cv + dv;
     const double n_in = (double)rw->nin, ds = rw->ds / n_in * inv_n, dt = rw->dt / n_in * inv_n;  // mean distances
-    if (!(ds > 1e-12 && dt > 1e-12)) return;
+    if (!(ds > 1e-12 && dt > 1e-12)) return false;
     const double ss = sqrt(2.0) / ds, sq = sqrt(2.0) / dt;
     const double iss = ds * 0.70710678118654752440, isq = dt * 0.70710678118654752440;  // 1 / ss, 1 / sq
     // centre the source terms (per raw weight 1, U, V, U^2 + V^2), then the weights
@@ -1419,13 +1589,11 @@ __global__ void __launch_bounds__(64) k_refit_solve(const __grid_constant__ Batc
         mom[12 + q] = sq * sz[q] * c2;
         mom[18 + q] = sq * sq * sz[q] * c3;
     }
-    double A[45];
 #pragma unroll
     for (int i = 0; i < 9; ++i)
 #pragma unroll
         for (int j = 0; j <= i; ++j) A[i * (i + 1) / 2 + j] = dlt_entry(mom, i, j);
     // start: the winner in the normalised frames, h0 = Tq Hw Tp^-1
-    double x[9];
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -1437,7 +1605,16 @@ __global__ void __launch_bounds__(64) k_refit_solve(const __grid_constant__ Batc
                               : (c == 1 ? Hw[k * 3 + 1] * iss : Hw[k * 3] * mx + Hw[k * 3 + 1] * my + Hw[k * 3 + 2]);
             x[r * 3 + c] = r == 0 ? sq * (b[0] - mqx * b[2]) : (r == 1 ? sq * (b[1] - mqy * b[2]) : b[2]);
         }
-    min_eigvec9(A, x);
+    f = RefitFrame{ss, isq, mx, my, mqx, mqy};
+    return true;
+}
+
+// The refit from the eigenvector x: denormalised, its evaluation and FP64 forms, the geometry checks.
+__device__ __forceinline__ void refit_record(RefitWork* rw, const LevelGeom& g, const PlaneParams& pp, int cell,
+                                             const double (&x)[9], const RefitFrame& f) {
+    int x0, y0, ox, oy;
+    window_origin<WarpGroup>(g, cell, x0, y0, ox, oy);
+    const double ss = f.ss, isq = f.isq, mx = f.mx, my = f.my, mqx = f.mqx, mqy = f.mqy;
     // Hr = Tq^-1 h Tp
     double Hr[9];
 #pragma unroll
@@ -1464,6 +1641,58 @@ __global__ void __launch_bounds__(64) k_refit_solve(const __grid_constant__ Batc
     rw->geo_r = plane_geometry_ok(Hr, g.s, pp.radius, pp.scale_min, pp.scale_max) ? 1 : 0;
     local_to_abs(Hr, ox, oy, rw->ha_r);
     rw->refit_ok = 1;
+}
+
+// (B) Normalised DLT refit of each window whose fit is pending, one thread
+// per window and direction: centred, Hartley-scaled moments from the exact
+// integer ones, the smallest eigenvector of A^T A started from the winner,
+// denormalisation, and the geometry checks of the winner and of the refit.
+__global__ void __launch_bounds__(32) k_refit_solve(const __grid_constant__ Batch bt, int level, PlaneParams pp) {
+    const PairView& pv = bt.view(blockIdx.z);
+    const LevelGeom g = bt.geom(blockIdx.z, level);
+    __shared__ EigShared sh;
+    const int nc = g.ncells(), lane = threadIdx.x;
+    const int t = blockIdx.x * 32 + lane;
+    const int dir = min(t / max(nc, 1), 1), cell = t - dir * nc;
+    RefitWork* rw = pv.rw[dir] + cell;
+    RefitFrame f;
+    double x[9], A[45], rd[9];
+    EigState e;
+    const bool todo = t < 2 * nc && rw->status == 2;
+    bool act = todo;
+    if (act) {
+        double M[45];
+        act = refit_system(rw, g, pp, cell, M, x, f);
+        if (act) {
+#pragma unroll
+            for (int q = 0; q < 45; ++q) sh.M[q][lane] = M[q];
+            eig_start(M, x, A, rd, e);
+        }
+    }
+    const bool refit = act;
+    unsigned left;
+    for (int step = 0;; ++step) {
+        left = __ballot_sync(FULL, act);
+        if (!left || (step >= 4 && __popc(left) == 1)) break;
+        if (act) act = eig_thread(sh.M, x, A, rd, e);
+    }
+    if (left) {  // one window's iteration goes on
+        if (act) {
+            sh.e = e;
+#pragma unroll
+            for (int q = 0; q < 45; ++q) sh.A[q] = A[q];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) sh.rd[i] = rd[i], sh.x[i] = x[i];
+        }
+        __syncwarp();
+        eig_warp(sh, __ffs(left) - 1);
+        if (act) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) x[i] = sh.x[i];
+        }
+    }
+    if (!refit) return;
+    refit_record(rw, g, pp, cell, x, f);
 }
 
 // (C) Rescore the refit on the window's matches, choose, count colour
@@ -2108,7 +2337,7 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
             k_ransac_warp<64><<<fgrid, 32 * kRansacWarps, 0, st>>>(bt, level, stage, pp);
         else
             k_ransac_warp<256><<<fgrid, 32 * kRansacWarps, 0, st>>>(bt, level, stage, pp);
-        k_refit_solve<<<dim3((2 * nc + 63) / 64, 1, np), 64, 0, st>>>(bt, level, pp);
+        k_refit_solve<<<dim3((2 * nc + 31) / 32, 1, np), 32, 0, st>>>(bt, level, pp);
         k_ransac_finish_warp<ST><<<grid, 256, 0, st>>>(bt, level, stage, pp);
         return;
     }
@@ -2121,7 +2350,7 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
         attr_set = true;
     }
     k_ransac_block<<<dim3(nc, 2, np), 256, fit_smem, st>>>(bt, level, stage, pp);
-    k_refit_solve<<<dim3((2 * nc + 63) / 64, 1, np), 64, 0, st>>>(bt, level, pp);
+    k_refit_solve<<<dim3((2 * nc + 31) / 32, 1, np), 32, 0, st>>>(bt, level, pp);
     k_ransac_finish_block<ST><<<dim3(nc, 2, np), 256, smem, st>>>(bt, level, stage, pp);
 }
 void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int stage, const PlaneParams& pp,
