@@ -502,7 +502,7 @@ struct PairView {
     float* cost[2];
     uint8_t* frozen[2];
     uint8_t* cue[2];
-    uint8_t* resid[2];
+    uint8_t* resid[2];    // fit: pixels without a first-stage plane; sweeps: pixels that moved in their last half-iteration
     Labels acc[2], tent[2], st1[2], lvl[2];
     double* mh[2];        // [m][9] absolute homographies
     Mef* mef[2];          // [m]

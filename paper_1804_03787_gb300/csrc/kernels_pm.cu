@@ -750,27 +750,6 @@ __device__ __forceinline__ float box_threshold(float bc) {
     return fmaf(bc, 1.52587890625e-05f, bc) + 3.814697265625e-06f;
 }
 
-// load_patch for a square colour patch whose source texels are staged in shared memory (tile origin (x0, y0) in
-// image coordinates, row length TW): the same taps, target indices into the padded copy (row length Wp).
-template <int R, int ST, int TW>
-__device__ __forceinline__ void load_patch_tile(LanePatch<R>& lp, const void* tile, int x0, int y0, int W, int H,
-                                                int px, int py, int lane, int Wp) {
-#pragma unroll
-    for (int j = 0; j < Patch<R>::NT; ++j) {
-        const int t = lane + 32 * j;
-        const int tt = t < Patch<R>::T ? t : 0;
-        const int dy = tt / Patch<R>::D - R, dx = tt % Patch<R>::D - R;
-        lp.tx[j] = min(max(px + dx, 0), W - 1);
-        lp.ty[j] = min(max(py + dy, 0), H - 1);
-        lp.tidx[j] = (lp.ty[j] + kPad) * Wp + lp.tx[j] + kPad;
-        lp.a[j] = ldpix_shared<ST>(tile, (lp.ty[j] - y0 + R) * TW + lp.tx[j] - x0 + R);
-        lp.fx[j] = 0.f;
-        lp.fy[j] = 0.f;
-    }
-    set_interior_box(lp, max(px - R, 0), min(px + R, W - 1), max(py - R, 0), min(py + R, H - 1), W, H);
-    lp.warped = false;
-}
-
 // ---------------------------------------------------------------- sweep
 // PLANES: levels >= 1 (restricted pixel list, plane-distorted patches, plane
 // candidates); otherwise level 0 with the census data term (level 0 with
@@ -783,6 +762,12 @@ __device__ __forceinline__ void load_patch_tile(LanePatch<R>& lp, const void* ti
 // around the best offset after A, radius R0 >> k on lane k.  The warp walks
 // each list in lane order through one evaluation site (a small kernel body
 // keeps the instruction cache warm) and accepts with the strict-less rule.
+// After the first iteration only the offsets of neighbours that moved in
+// their last half-iteration are candidates of list A, and no window's model:
+// the others were candidates at this pixel's visit one iteration ago, so
+// their cost is at least the best of then, and the best never rises (an
+// offset that became the best is repeated by it).  pv.resid is free during
+// the sweeps and holds which pixels moved.
 // CENSUS (level 0 only): the census data term on the frames' code images.
 template <int R, int ST, bool PLANES, bool CENSUS>
 __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Batch bt, int level, int it, int phase, uint32_t k0,
@@ -798,6 +783,7 @@ __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Bat
     const void* src = CENSUS ? (const void*)pv.code[dir] : pv.img[dir];
     const void* tgt = CENSUS ? (const void*)pv.code[1 - dir] : pv.img[1 - dir];
     int2* __restrict__ nnf = pv.nnf[dir];
+    uint8_t* __restrict__ moved = pv.resid[dir];
     const int nw = gridDim.x * (blockDim.x >> 5);
     const int hw = (W + 1) >> 1;
     const int total = !PLANES ? H * hw : pv.list_count[dir * 2 + phase];
@@ -836,7 +822,8 @@ __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Bat
             const Mef* G = home_plane(g, pv.mef[dir], x, y);
             if (G) warp_taps<R>(lp, *G, x, y, W, H, lane);
         }
-        int2 best = nnf[i];
+        const int2 before = nnf[i];
+        int2 best = before;
         float bc = pv.cost[dir][i];  // raw sum of the incumbent
         int ithr = CENSUS ? 0 : abandon_threshold(bc);
         int nev = 0, ntap = 0;
@@ -846,12 +833,12 @@ __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Bat
         if (lane < 4) {
             const int nx = x + (lane == 0 ? -1 : (lane == 1 ? 1 : 0));
             const int ny = y + (lane == 2 ? -1 : (lane == 3 ? 1 : 0));
-            if (nx >= 0 && nx < W && ny >= 0 && ny < H) {
+            if (nx >= 0 && nx < W && ny >= 0 && ny < H && (it == 0 || moved[ny * W + nx])) {
                 cand = nnf[ny * W + nx];
                 const int tx = x + cand.x, ty = y + cand.y;
                 ok = tx >= 0 && tx < W && ty >= 0 && ty < H;
             }
-        } else if (PLANES && lane < 4 + 18) {
+        } else if (PLANES && it == 0 && lane < 4 + 18) {
             int fx0, nrx, fy0, nry;
             const int nxw = covering_range(g.gx, g.s, g.h, x, fx0, nrx);
             const int nyw = covering_range(g.gy, g.s, g.h, y, fy0, nry);
@@ -922,8 +909,12 @@ __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Bat
             }
         }
         if (lane == 0) {
-            nnf[i] = best;
-            pv.cost[dir][i] = bc;
+            const bool m = best.x != before.x || best.y != before.y;
+            moved[i] = m;
+            if (m) {
+                nnf[i] = best;
+                pv.cost[dir][i] = bc;
+            }
             if (pv.evals) {
                 atomicAdd(&pv.evals[PLANES ? GPM_COUNT_SWEEP_PLANE : GPM_COUNT_SWEEP0], (unsigned long long)nev);
                 atomicAdd(&pv.evals[PLANES ? GPM_COUNT_SWEEP_PLANE_TAPS : GPM_COUNT_SWEEP0_TAPS],
@@ -934,23 +925,32 @@ __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Bat
 }
 
 // ---------------------------------------------------------------- level-0 sweep, two layouts
-// Tiles of the level-0 sweep: 16 pixels of one colour by 8 rows (32 x 8 image pixels), each of the block's four
-// warps owning two rows, one pixel per lane.  The staged source region is the tile grown by r, in rows of TW
-// texels (TW congruent to 2r + 1 modulo 8, so that eight consecutive taps of a patch row fall on eight distinct
-// 16-byte bank groups).
+// Tiles of the level-0 sweep: 16 pixels of one colour by `rows` rows (32 x rows image pixels), the block's four
+// warps owning 4 rows pixels each, one pixel per lane: rows = 8 fills the lanes and shares the staging best; small
+// frames take 4, 2 or 1, so that the launch still covers the chip (sweep0_rows).  The staged source region is the
+// tile grown by r, in rows of TW texels (TW congruent to 2r + 1 modulo 8, so that eight consecutive taps of a patch
+// row fall on eight distinct 16-byte bank groups).
 template <int R>
 struct Tile0L {
-    static constexpr int TXC = 16, TY = 8, TX = 2 * TXC, WARPS = 4;
+    static constexpr int TXC = 16, TYMAX = 8, TX = 2 * TXC, WARPS = 4;
     static constexpr int TW0 = TX + 2 * R;
     static constexpr int TW = TW0 + ((2 * R + 1 - TW0) % 8 + 8) % 8;
-    static constexpr int TH = TY + 2 * R;
+    static constexpr int TH = TYMAX + 2 * R;
 };
 // Search radii R0 >> k >= 1 for frames below 2^15 pixels a side: at most 15.
 constexpr int kMaxRadii = 16;
 
-int sweep0_tiles(int W, int H) {
+int sweep0_tiles(int W, int H, int rows) {
     const int hw = (W + 1) >> 1;
-    return ((hw + Tile0L<1>::TXC - 1) / Tile0L<1>::TXC) * ((H + Tile0L<1>::TY - 1) / Tile0L<1>::TY);
+    return ((hw + Tile0L<1>::TXC - 1) / Tile0L<1>::TXC) * ((H + rows - 1) / rows);
+}
+// The most rows a tile may have with at least four blocks per SM in the launch (a block's warps walk their pixels
+// one after another, so a launch of fewer blocks lasts as long as one of that many): 128x96 takes 1 row, 253x187
+// four, from 512x384 on 8.
+int sweep0_rows(int W, int H, int pairs, int nsm) {
+    int rows = Tile0L<1>::TYMAX;
+    while (rows > 1 && (int64_t)sweep0_tiles(W, H, rows) * 2 * pairs < 4 * nsm) rows >>= 1;
+    return rows;
 }
 
 // A candidate offset in one word (|c.x|, |c.y| < 2^15 for frames below 2^15 pixels a side).
@@ -965,72 +965,101 @@ __device__ __forceinline__ void list_push(uint32_t (*list)[32], int& n, int2 c, 
     if (!dup) list[n++][lane] = key;
 }
 
-// Raw tap sums of N candidate offsets of one square patch (off[q] = c.y * Wp + c.x into the padded target copy),
-// all in full: each lane accumulates its taps in the order of tap_sum_in and the totals are warp_sum_q23's, so
-// each sum is bitwise tap_sum_in's; the N candidates' gathers of a chunk are in flight together.
-template <int R, int ST, int N>
-__device__ __forceinline__ void tap_sums_sq(const LanePatch<R>& lp, const void* tgtp, const int* off, float* sum,
-                                            int lane) {
-    float s[N];
+// One pixel's patch, one tap per lane and chunk: the source texels, and the taps' byte offsets into the padded target
+// copy at offset 0 (frames hold at most 2^26 texels of 16 bytes, so 32 bits address the copy).
+template <int R>
+struct SquarePatch {
+    float4 a[Patch<R>::NT];
+    unsigned at[Patch<R>::NT];
+};
+// What a lane's taps add to a pixel whose patch stays inside the frame: its texels in the staged tile and in the
+// padded copy (constants of the lane, so that such a pixel's patch takes two additions a tap; clamping every tap's
+// coordinates took eleven instructions).
+template <int R>
+struct TapOffsets {
+    int tile[Patch<R>::NT];
+    unsigned at[Patch<R>::NT];
+};
+template <int R, int ST, int TW>
+__device__ __forceinline__ void load_square(SquarePatch<R>& sp, const TapOffsets<R>& to, const void* tile, int x0, int y0,
+                                            int W, int H, int px, int py, bool inside, int lane, int Wp) {
+    constexpr unsigned B = sizeof(typename TexelOf<ST>::type);
+    if (inside) {  // warp-uniform
+        const int tp = (py - y0) * TW + (px - x0);
+        const unsigned ap = (unsigned)((py + kPad) * Wp + px + kPad) * B;
 #pragma unroll
-    for (int q = 0; q < N; ++q) s[q] = 0.f;
-#pragma unroll
-    for (int j = 0; j < Patch<R>::NT; ++j) {
-        if (lane + 32 * j < Patch<R>::T) {
-            float4 v[N];
-#pragma unroll
-            for (int q = 0; q < N; ++q) v[q] = ldpix<ST>(tgtp, lp.tidx[j] + off[q]);
-#pragma unroll
-            for (int q = 0; q < N; ++q) s[q] += absdiff3(lp.a[j], make_float3(v[q].x, v[q].y, v[q].z));
+        for (int j = 0; j < Patch<R>::NT; ++j) {
+            sp.a[j] = ldpix_shared<ST>(tile, tp + to.tile[j]);
+            sp.at[j] = ap + to.at[j];
         }
+        return;
     }
 #pragma unroll
-    for (int q = 0; q < N; ++q) sum[q] = warp_sum_q23(s[q]);
+    for (int j = 0; j < Patch<R>::NT; ++j) {
+        const int t = lane + 32 * j;
+        const int tt = t < Patch<R>::T ? t : 0;
+        const int dy = tt / Patch<R>::D - R, dx = tt % Patch<R>::D - R;
+        const int tx = min(max(px + dx, 0), W - 1), ty = min(max(py + dy, 0), H - 1);
+        sp.at[j] = (unsigned)((ty + kPad) * Wp + tx + kPad) * B;
+        sp.a[j] = ldpix_shared<ST>(tile, (ty - y0 + R) * TW + tx - x0 + R);
+    }
 }
 
 // Maximum number of one pixel's candidates whose costs are summed together.
 constexpr int kSweep0Group = 3;
 
+// N listed candidates of one square patch, from the k-th: their raw tap sums, all in full, each lane accumulating its
+// taps in the order of tap_sum_in and the totals warp_sum_q23's times 2^23 (an exact scaling, so they compare
+// alike; best costs are held scaled too); the N candidates' gathers of a chunk are in flight together.  Then the
+// strict-less updates in list order.
 template <int R, int ST, int N>
-__device__ __forceinline__ void eval_group(const LanePatch<R>& lp, const void* tgtp, int Wp,
-                                           const uint32_t (*list)[32], int p, int k, int2& best, float& bc) {
+__device__ __forceinline__ void eval_group(const SquarePatch<R>& sp, const void* tgtp, int Wp,
+                                           const uint32_t (*list)[32], int p, int k, int lane, int2& best, float& bc) {
+    constexpr unsigned B = sizeof(typename TexelOf<ST>::type);
     int2 c[N];
-    int off[N];
-    float sum[N];
+    unsigned off[N];
+    float s[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) {
         c[q] = unpack_off(list[k + q][p]);
-        off[q] = c[q].y * Wp + c[q].x;
+        off[q] = (unsigned)(c[q].y * Wp + c[q].x) * B;
+        s[q] = 0.f;
     }
-    tap_sums_sq<R, ST, N>(lp, tgtp, off, sum, (int)(threadIdx.x & 31));
 #pragma unroll
-    for (int q = 0; q < N; ++q)
-        if (sum[q] < bc) {
-            bc = sum[q];
+    for (int j = 0; j < Patch<R>::NT; ++j) {
+        if (lane + 32 * j < Patch<R>::T) {
+            float4 v[N];
+#pragma unroll
+            for (int q = 0; q < N; ++q) v[q] = ldpix<ST>(static_cast<const char*>(tgtp) + (sp.at[j] + off[q]), 0);
+#pragma unroll
+            for (int q = 0; q < N; ++q) s[q] += absdiff3(sp.a[j], make_float3(v[q].x, v[q].y, v[q].z));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        const float sum = (float)__reduce_add_sync(FULL, __float2uint_rn(s[q] * 8388608.f));
+        if (sum < bc) {
+            bc = sum;
             best = c[q];
         }
+    }
 }
 
 // The warp (one tap per lane) evaluates the n listed candidates of one pixel in list order, up to kSweep0Group
 // at a time, with the strict-less rule (every cost summed in full, then the updates in list order): best / bc
 // are warp-uniform on entry and on return.
 template <int R, int ST>
-__device__ __forceinline__ void eval_listed(const LanePatch<R>& lp, const void* tgtp, int Wp,
-                                            const uint32_t (*list)[32], int p, int n, int2& best, float& bc,
-                                            unsigned& nev, unsigned& ntap) {
+__device__ __forceinline__ void eval_listed(const SquarePatch<R>& sp, const void* tgtp, int Wp,
+                                            const uint32_t (*list)[32], int p, int n, int lane, int2& best, float& bc) {
     for (int k = 0; k < n;) {
         const int g = min(n - k, kSweep0Group);
-        if (g >= 4)
-            eval_group<R, ST, 4>(lp, tgtp, Wp, list, p, k, best, bc);
-        else if (g == 3)
-            eval_group<R, ST, 3>(lp, tgtp, Wp, list, p, k, best, bc);
+        if (g == 3)
+            eval_group<R, ST, 3>(sp, tgtp, Wp, list, p, k, lane, best, bc);
         else if (g == 2)
-            eval_group<R, ST, 2>(lp, tgtp, Wp, list, p, k, best, bc);
+            eval_group<R, ST, 2>(sp, tgtp, Wp, list, p, k, lane, best, bc);
         else
-            eval_group<R, ST, 1>(lp, tgtp, Wp, list, p, k, best, bc);
+            eval_group<R, ST, 1>(sp, tgtp, Wp, list, p, k, lane, best, bc);
         k += g;
-        nev += g;
-        ntap += g * Patch<R>::T;
     }
 }
 
@@ -1039,12 +1068,13 @@ __device__ __forceinline__ void eval_listed(const LanePatch<R>& lp, const void* 
 // neighbours; (B) random search around the best offset after A, radius R0 >> k for k = 0, 1, ... (Philox words,
 // two radii per call).  A candidate replaces the best only if its raw tap sum is strictly lower, in list order;
 // candidates that repeat the best or an earlier entry, or that the patch-sum bound rules out, cannot win and are
-// not listed.  The per-pixel scalar work runs with one pixel per lane: the neighbours' offsets, the Philox words
+// not listed, nor are, after the first iteration, the offsets of neighbours that did not move (see k_pm_sweep).
+// The per-pixel scalar work runs with one pixel per lane: the neighbours' offsets, the Philox words
 // and the search candidates, the bound and the removal of repeats, into a list per pixel in shared memory.  The
-// patch costs run with one tap per lane, the warp walking its 32 pixels' lists in turn; list B is built once
-// list A is evaluated for all 32 pixels.
+// patch costs run with one tap per lane, the warp walking its pixels' lists in turn; list B is built once
+// list A is evaluated for all of them.
 template <int R, int ST>
-__global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Batch bt, int it, int phase,
+__global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Batch bt, int it, int phase, int rows,
                                                       uint32_t k0, uint32_t k1) {
     using TL = Tile0L<R>;
     using Tex = typename TexelOf<ST>::type;
@@ -1055,50 +1085,63 @@ __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Ba
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int W = pv.W, H = pv.H, Wp = pv.Wp;
     const int hw = (W + 1) >> 1;
-    const int ntx = (hw + TL::TXC - 1) / TL::TXC, nty = (H + TL::TY - 1) / TL::TY;
+    const int ntx = (hw + TL::TXC - 1) / TL::TXC, nty = (H + rows - 1) / rows;
     if ((int)blockIdx.x >= ntx * nty) return;  // block-uniform: the grid covers the largest pair of the batch
     const int tyi = blockIdx.x / ntx, txi = blockIdx.x - tyi * ntx;
-    const int x0 = TL::TX * txi, y0 = TL::TY * tyi;
+    const int x0 = TL::TX * txi, y0 = rows * tyi;
     {
         // the tile's source region, from the padded copy (entries past its edge are clamped and unused)
         const Tex* sp = reinterpret_cast<const Tex*>(pv.imgp[dir]);
         const int Hp = H + 2 * kPad;
-        for (int e = threadIdx.x; e < TL::TH * TL::TW; e += blockDim.x) {
+        for (int e = threadIdx.x; e < (rows + 2 * R) * TL::TW; e += blockDim.x) {
             const int ly = e / TL::TW, lx = e - ly * TL::TW;
             const int gx = min(x0 - R + lx + kPad, Wp - 1), gy = min(y0 - R + ly + kPad, Hp - 1);
             stile[e] = sp[gy * Wp + gx];
         }
     }
+    TapOffsets<R> to;
+#pragma unroll
+    for (int j = 0; j < Patch<R>::NT; ++j) {
+        const int t = lane + 32 * j, tt = t < Patch<R>::T ? t : 0;
+        const int dy = tt / Patch<R>::D - R, dx = tt % Patch<R>::D - R;
+        to.tile[j] = (dy + R) * TL::TW + dx + R;
+        to.at[j] = (unsigned)(dy * Wp + dx) * (unsigned)sizeof(Tex);
+    }
     __syncthreads();
     const void* tgtp = pv.imgp[1 - dir];
     uint32_t(*list)[32] = slist[wid];
     int2* __restrict__ nnf = pv.nnf[dir];
+    uint8_t* __restrict__ moved = pv.resid[dir];
     const float4* __restrict__ boxt = pv.box[1 - dir];
-    // the lane's pixel
-    const int yq = y0 + 2 * wid + (lane >> 4);
-    const int xq = 2 * (TL::TXC * txi + (lane & 15)) + ((yq + phase) & 1);
-    const bool mine = yq < H && xq < W;
+    // the lane's pixel: the wid * npix + lane-th of the tile, 16 a row
+    const int npix = 4 * rows;
+    const int yq = y0 + ((wid * npix + lane) >> 4);
+    const int xq = 2 * (TL::TXC * txi + ((wid * npix + lane) & 15)) + ((yq + phase) & 1);
+    const bool mine = lane < npix && yq < H && xq < W;
     const int iq = mine ? yq * W + xq : 0;
     int2 best = make_int2(0, 0);
-    float bc = 0.f;
+    uint32_t before = 0;
+    float bc = 0.f;  // times 2^23
     if (mine) {
         best = nnf[iq];
-        bc = pv.cost[dir][iq];
+        before = pack_off(best);
+        bc = pv.cost[dir][iq] * 8388608.f;
     }
     // interior pixels: the patch-sum bound applies
     const bool prune = mine && xq >= R && yq >= R && xq < W - R && yq < H - R;
+    const unsigned inside = __ballot_sync(FULL, prune);
     const float4 b1 = prune ? pv.box[dir][iq] : make_float4(0.f, 0.f, 0.f, 0.f);
-    unsigned npr = 0, nev = 0, ntap = 0;
+    unsigned npr = 0, nev = 0;
     // list A, one pixel per lane: the four neighbours' offsets whose target is in the frame, neither the
     // incumbent nor a repeat, and not excluded by the bound
     int n = 0;
     if (mine) {
-        const float thr = box_threshold(bc);
+        const float thr = box_threshold(bc * 1.1920928955078125e-07f);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int nx = xq + (k == 0 ? -1 : (k == 1 ? 1 : 0));
             const int ny = yq + (k == 2 ? -1 : (k == 3 ? 1 : 0));
-            if (nx < 0 || nx >= W || ny < 0 || ny >= H) continue;
+            if (nx < 0 || nx >= W || ny < 0 || ny >= H || (it > 0 && !moved[ny * W + nx])) continue;
             const int2 c = nnf[ny * W + nx];
             const int tx = xq + c.x, ty = yq + c.y;
             if (tx < 0 || tx >= W || ty < 0 || ty >= H || (c.x == best.x && c.y == best.y)) continue;
@@ -1109,80 +1152,71 @@ __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Ba
             list_push(list, n, c, lane);
         }
     }
-    __syncwarp();
-    // list A, one tap per lane, pixel by pixel
-    for (int p = 0; p < 32; ++p) {
-        const int np_ = __shfl_sync(FULL, n, p);
-        if (np_ == 0) continue;  // warp-uniform
-        const int yp = y0 + 2 * wid + (p >> 4);
-        const int xp = 2 * (TL::TXC * txi + (p & 15)) + ((yp + phase) & 1);
-        LanePatch<R> lp;
-        load_patch_tile<R, ST, TL::TW>(lp, stile, x0, y0, W, H, xp, yp, lane, Wp);
-        int2 b = make_int2(__shfl_sync(FULL, best.x, p), __shfl_sync(FULL, best.y, p));
-        float c = __shfl_sync(FULL, bc, p);
-        eval_listed<R, ST>(lp, tgtp, Wp, list, p, np_, b, c, nev, ntap);
-        if (lane == p) {
-            best = b;
-            bc = c;
+    for (int part = 0;; ++part) {
+        __syncwarp();
+        // the list's costs, one tap per lane, pixel by pixel
+        nev += n;
+        for (unsigned todo = __ballot_sync(FULL, n > 0); todo; todo &= todo - 1) {
+            const int p = __ffs(todo) - 1, np_ = __shfl_sync(FULL, n, p);
+            const int yp = y0 + ((wid * npix + p) >> 4);
+            const int xp = 2 * (TL::TXC * txi + ((wid * npix + p) & 15)) + ((yp + phase) & 1);
+            SquarePatch<R> sp;
+            load_square<R, ST, TL::TW>(sp, to, stile, x0, y0, W, H, xp, yp, (inside >> p) & 1u, lane, Wp);
+            int2 b = make_int2(__shfl_sync(FULL, best.x, p), __shfl_sync(FULL, best.y, p));
+            float c = __shfl_sync(FULL, bc, p);
+            eval_listed<R, ST>(sp, tgtp, Wp, list, p, np_, lane, b, c);
+            if (lane == p) {
+                best = b;
+                bc = c;
+            }
         }
-    }
-    __syncwarp();
-    // list B, one pixel per lane: random search around v0, the best offset after list A (Philox words two radii
-    // per call, as in k_pm_sweep)
-    n = 0;
-    if (mine) {
-        const int2 v0 = best;
-        const int R0 = max(W, H);
-        int nrad = 0;
-        while ((R0 >> nrad) >= 1) ++nrad;
-        const uint32_t tag = stream_tag(RNG_SEARCH, dir, 0, 0);
-        const float thr = box_threshold(bc);
-        for (int call = 0; 2 * call < nrad; ++call) {
-            const uint4 rw = philox((uint32_t)iq, ((uint32_t)it << 8) | (uint32_t)call, tag, pv.pair_id, k0, k1);
+        if (part) break;
+        __syncwarp();
+        // list B, one pixel per lane: random search around v0, the best offset after list A (Philox words two radii
+        // per call, as in k_pm_sweep)
+        n = 0;
+        if (mine) {
+            const int2 v0 = best;
+            const int R0 = max(W, H);
+            int nrad = 0;
+            while ((R0 >> nrad) >= 1) ++nrad;
+            const uint32_t tag = stream_tag(RNG_SEARCH, dir, 0, 0);
+            const float thr = box_threshold(bc * 1.1920928955078125e-07f);
+            for (int call = 0; 2 * call < nrad; ++call) {
+                const uint4 rw = philox((uint32_t)iq, ((uint32_t)it << 8) | (uint32_t)call, tag, pv.pair_id, k0, k1);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int k = 2 * call + h;
-                if (k >= nrad) break;
-                const uint32_t wx = h ? rw.z : rw.x, wy = h ? rw.w : rw.y;
-                const int Rk = R0 >> k;
-                const int ox = (int)bounded_u32(wx, (uint32_t)(2 * Rk + 1)) - Rk;
-                const int oy = (int)bounded_u32(wy, (uint32_t)(2 * Rk + 1)) - Rk;
-                const int tx = min(max(xq + v0.x + ox, 0), W - 1), ty = min(max(yq + v0.y + oy, 0), H - 1);
-                const int2 c = make_int2(tx - xq, ty - yq);
-                if (c.x == v0.x && c.y == v0.y) continue;
-                if (prune && box_lb(b1, boxt[iq + c.y * W + c.x]) >= thr) {
-                    ++npr;
-                    continue;
+                for (int h = 0; h < 2; ++h) {
+                    const int k = 2 * call + h;
+                    if (k >= nrad) break;
+                    const uint32_t wx = h ? rw.z : rw.x, wy = h ? rw.w : rw.y;
+                    const int Rk = R0 >> k;
+                    const int ox = (int)bounded_u32(wx, (uint32_t)(2 * Rk + 1)) - Rk;
+                    const int oy = (int)bounded_u32(wy, (uint32_t)(2 * Rk + 1)) - Rk;
+                    const int tx = min(max(xq + v0.x + ox, 0), W - 1), ty = min(max(yq + v0.y + oy, 0), H - 1);
+                    const int2 c = make_int2(tx - xq, ty - yq);
+                    if (c.x == v0.x && c.y == v0.y) continue;
+                    if (prune && box_lb(b1, boxt[iq + c.y * W + c.x]) >= thr) {
+                        ++npr;
+                        continue;
+                    }
+                    list_push(list, n, c, lane);
                 }
-                list_push(list, n, c, lane);
             }
         }
     }
-    __syncwarp();
-    for (int p = 0; p < 32; ++p) {
-        const int np_ = __shfl_sync(FULL, n, p);
-        if (np_ == 0) continue;
-        const int yp = y0 + 2 * wid + (p >> 4);
-        const int xp = 2 * (TL::TXC * txi + (p & 15)) + ((yp + phase) & 1);
-        LanePatch<R> lp;
-        load_patch_tile<R, ST, TL::TW>(lp, stile, x0, y0, W, H, xp, yp, lane, Wp);
-        int2 b = make_int2(__shfl_sync(FULL, best.x, p), __shfl_sync(FULL, best.y, p));
-        float c = __shfl_sync(FULL, bc, p);
-        eval_listed<R, ST>(lp, tgtp, Wp, list, p, np_, b, c, nev, ntap);
-        if (lane == p) {
-            best = b;
-            bc = c;
+    if (mine) {
+        const bool m = pack_off(best) != before;
+        moved[iq] = m;
+        if (m) {
+            nnf[iq] = best;
+            pv.cost[dir][iq] = bc * 1.1920928955078125e-07f;
         }
     }
-    if (mine) {
-        nnf[iq] = best;
-        pv.cost[dir][iq] = bc;
-    }
     if (pv.evals) {
-        const unsigned npw = __reduce_add_sync(FULL, npr);
+        const unsigned npw = __reduce_add_sync(FULL, npr), nevw = __reduce_add_sync(FULL, nev);
         if (lane == 0) {
-            atomicAdd(&pv.evals[GPM_COUNT_SWEEP0], (unsigned long long)nev);
-            atomicAdd(&pv.evals[GPM_COUNT_SWEEP0_TAPS], (unsigned long long)ntap);
+            atomicAdd(&pv.evals[GPM_COUNT_SWEEP0], (unsigned long long)nevw);
+            atomicAdd(&pv.evals[GPM_COUNT_SWEEP0_TAPS], (unsigned long long)nevw * Patch<R>::T);
             if (npw) atomicAdd(&pv.evals[GPM_COUNT_SWEEP0_PRUNED], (unsigned long long)npw);
         }
     }
@@ -1204,6 +1238,7 @@ __global__ void k_build_lists(const __grid_constant__ Batch bt) {
         int col = 0;
         if (i < n) {
             ok = !pv.frozen[dir][i];
+            if (!ok) pv.resid[dir][i] = 0;  // a frozen pixel never moves in the sweeps
             const int y = i / W, x = i - y * W;
             col = (x + y) & 1;
         }
@@ -1236,7 +1271,7 @@ static void launch_pm_r(const PmLaunch& L, cudaStream_t st) {
             if (L.level == 0 && L.census)
                 k_pm_sweep<R, 0, false, true><<<grid, block, 0, st>>>(L.bt, 0, L.it, L.phase, L.k0, L.k1);
             else if (L.level == 0)
-                k_pm_sweep0<R, ST><<<dim3(L.tiles0, 2, L.np), dim3(32 * Tile0L<R>::WARPS), 0, st>>>(L.bt, L.it, L.phase,
+                k_pm_sweep0<R, ST><<<dim3(L.tiles0, 2, L.np), dim3(32 * Tile0L<R>::WARPS), 0, st>>>(L.bt, L.it, L.phase, L.rows0,
                                                                                                   L.k0, L.k1);
             else
                 k_pm_sweep<R, ST, true, false><<<grid, block, 0, st>>>(L.bt, L.level, L.it, L.phase, L.k0, L.k1);
