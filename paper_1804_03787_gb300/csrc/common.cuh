@@ -496,7 +496,8 @@ struct PairView {
     uint32_t pair_id;
     const void* img[2];   // ingested I1, I2 (RGBX in storage type)
     const void* imgp[2];  // the same, (W + 2 kPad) x (H + 2 kPad) with replicated borders (level-0 PatchMatch)
-    float4* box[2];       // per pixel, the RGB sums over its square patch of clamped taps (level-0 lower bound)
+    float4* box[2];       // per pixel, the RGB sums over its square patch of clamped taps (level-0 lower bound); after
+                          // the level-0 sweeps, FP16 sums of 3 x 3 minima and maxima (plane levels' bound)
     int Wp;               // row length of imgp
     int2* nnf[2];
     float* cost[2];

@@ -618,6 +618,13 @@ gpm_status gpm_match(gpm_ctx* c, const gpm_pair* pairs, int32_t n_pairs, int32_t
             build_lists(c, 0, n_pairs, D.max_n);  // every pixel (nothing frozen) for the recost
         }
         pm_sweeps(c, D, 0);
+        if (c->P.num_scales > 0) {  // for the plane levels' sweeps, in the level-0 sweep's box buffers
+            pbeg(c, GPM_PROF_INGEST, batches(n_pairs));
+            each_batch(c, 0, n_pairs, [&](const Batch& b, int nb) {
+                launch_interval_sums(b, nb, D.max_w, D.max_h, c->P.patch_radius, c->P.storage, c->stream);
+            });
+            pend(c);
+        }
         for (int i = 0; i < n_pairs; ++i) c->slots[i].stage = 0;
     } else {
         for (int i = 0; i < n_pairs; ++i)

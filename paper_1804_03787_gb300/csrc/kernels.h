@@ -62,6 +62,8 @@ void launch_ingest(const float* f1, const float* f2, int W, int H, int64_t strid
 void launch_pad_frames(const Batch& bt, int np, int storage, int grid_blocks, cudaStream_t st);
 // Patch sums of both ingested frames (pv.box), after launch_pad_frames: the level-0 sweep's lower bound.
 void launch_box_sums(const Batch& bt, int np, int max_w, int max_h, int radius, int storage, cudaStream_t st);
+// Interval sums of both ingested frames (into pv.box, after the level-0 sweeps): the plane sweeps' lower bound.
+void launch_interval_sums(const Batch& bt, int np, int max_w, int max_h, int radius, int storage, cudaStream_t st);
 // The unfrozen pixels of each colour (the restricted sweeps' lists), counts cleared first.
 void launch_build_lists(const Batch& bt, int np, int grid_blocks, cudaStream_t st);
 // dst[i] = src[i] / (3 (2 radius + 1)^2), or / 24 (2 radius + 1)^2 for census costs: the NNF cost buffer holds
