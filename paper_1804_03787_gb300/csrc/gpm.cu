@@ -31,7 +31,6 @@ struct Slot {
     LevelGeom geoms[GPM_MAX_SCALES];
     int total_cells = 0, m = 0;
     double* partial = nullptr;
-    double* gain = nullptr;
     bool census_costs = false;  // the NNF costs are census Hamming sums (level 0 with the census data term)
     int* eq_hist = nullptr;    // 2 x 256 V-histogram counts (HSV equalisation)
     float* eq_lut = nullptr;   // 2 x 256 equalised V per bin
@@ -206,7 +205,6 @@ size_t layout_slot(const gpm_params& P, int max_n, int max_np, int max_models, i
     pv.flag = (int*)take(sizeof(int));
     pv.gq = (int*)take(n * sizeof(int));
     double* partial = (double*)take(sizeof(double) * 2 * kPartialBlocks);
-    double* gain = (double*)take(sizeof(double));
     int* eq_hist = (int*)take(2 * 256 * sizeof(int));
     float* eq_lut = (float*)take(2 * 256 * sizeof(float));
     unsigned long long* evals = (unsigned long long*)take(GPM_COUNTERS * sizeof(unsigned long long));
@@ -214,7 +212,6 @@ size_t layout_slot(const gpm_params& P, int max_n, int max_np, int max_models, i
         s->d_evals = evals;
         s->pv = pv;
         s->partial = partial;
-        s->gain = gain;
         s->eq_hist = eq_hist;
         s->eq_lut = eq_lut;
     }
@@ -573,7 +570,6 @@ gpm_status gpm_match(gpm_ctx* c, const gpm_pair* pairs, int32_t n_pairs, int32_t
                 j.H = p.height;
                 j.stride = p.row_stride;
                 j.partial = s.partial;
-                j.gain = s.gain;
                 j.o1 = const_cast<void*>(s.pv.img[0]);
                 j.o2 = const_cast<void*>(s.pv.img[1]);
                 j.hist = c->P.equalize ? s.eq_hist : nullptr;
@@ -588,7 +584,7 @@ gpm_status gpm_match(gpm_ctx* c, const gpm_pair* pairs, int32_t n_pairs, int32_t
                 mn = std::max(mn, s.n);
                 mh = std::max(mh, s.H);
             }
-            pbeg(c, GPM_PROF_INGEST, (c->P.equalize ? 6 : 3) + (c->P.census ? 2 : 0) + (c->P.interp ? 1 : 0));
+            pbeg(c, GPM_PROF_INGEST, (c->P.equalize ? 5 : 2) + (c->P.census ? 2 : 0) + (c->P.interp ? 1 : 0));
             launch_ingest_jobs(J, nj, mn, mh, c->P.gain_normalize, c->P.storage, c->stream);
             pend(c);
         }

@@ -24,7 +24,7 @@ void launch_pm(const PmLaunch& L, cudaStream_t st);
 // to take for a launch over `pairs` such frames on nsm SMs.
 int sweep0_tiles(int W, int H, int rows);
 int sweep0_rows(int W, int H, int pairs, int nsm);
-// Blocks of the FP64 frame sums behind the gain (a fixed grid, so a fixed summation order): partial holds
+// Blocks of the frame sums behind the gain (a fixed grid, so a fixed summation order): partial holds
 // 2 * kIngestPartialBlocks doubles.
 constexpr int kIngestPartialBlocks = 128;
 // One pair's ingest: its frames as given and the buffers the ingest fills.
@@ -35,7 +35,6 @@ struct IngestJob {
     int W, H;
     int64_t stride;
     double* partial;  // 2 * kIngestPartialBlocks doubles
-    double* gain;     // one double
     void* o1;         // ingested frames (RGBX in the storage type)
     void* o2;
     int* hist;        // HSV equalisation (Sec. 4.2): 2 x 256 counts and tables, or nullptr
@@ -56,8 +55,7 @@ void launch_ingest_jobs(const IngestJobs& J, int nj, int max_n, int max_h, int g
                         cudaStream_t st);
 // One pair: eq_hist / eq_lut (2 x 256 each, device) non-null: HSV histogram equalisation of both frames first.
 void launch_ingest(const float* f1, const float* f2, int W, int H, int64_t stride, int gain_enable, int storage,
-                   double* partial, int nblk, double* gain, void* o1, void* o2, int* eq_hist, float* eq_lut,
-                   cudaStream_t st);
+                   double* partial, void* o1, void* o2, int* eq_hist, float* eq_lut, cudaStream_t st);
 // Padded copies of both ingested frames (imgp), borders replicating the edges.
 void launch_pad_frames(const Batch& bt, int np, int storage, int grid_blocks, cudaStream_t st);
 // Patch sums of both ingested frames (pv.box), after launch_pad_frames: the level-0 sweep's lower bound.

@@ -59,11 +59,18 @@ __global__ void k_vhist(const __grid_constant__ IngestJobs J) {
     __syncthreads();
     const void* f = blockIdx.y ? j.f2 : j.f1;
     const int n = W * H;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int y = i / W, x = i - y * W;
-        const int64_t e = (int64_t)y * stride + 3 * x;
-        const float r = in_elem(f, j.dtype, e), g = in_elem(f, j.dtype, e + 1), b = in_elem(f, j.dtype, e + 2);
-        atomicAdd(&h[v_bin(fmaxf(r, fmaxf(g, b)))], 1);
+    const int step = gridDim.x * blockDim.x;
+    for (int i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {  // four pixels' loads in flight
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = min(i0 + q * step, n - 1), y = i / W, x = i - y * W;
+            const int64_t e = (int64_t)y * stride + 3 * x;
+            v[q] = fmaxf(in_elem(f, j.dtype, e), fmaxf(in_elem(f, j.dtype, e + 1), in_elem(f, j.dtype, e + 2)));
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (i0 + q * step < n) atomicAdd(&h[v_bin(v[q])], 1);
     }
     __syncthreads();
     for (int k = threadIdx.x; k < 256; k += blockDim.x)
@@ -78,18 +85,20 @@ __global__ void k_vlut(const __grid_constant__ IngestJobs J) {
     const int n = j.W * j.H;
     float* lut = j.lut;
     __shared__ int c[256];
-    __shared__ int cmin;
+    __shared__ int cmin, first[8];
     const int t = threadIdx.x;
     const int* hf = hist + blockIdx.x * 256;
     c[t] = hf[t];
-    if (t == 0) {
-        cmin = -1;
-        for (int b = 0; b < 256; ++b)
-            if (hf[b] > 0) {
-                cmin = hf[b];
-                break;
-            }
+    if (t == 0) cmin = -1;
+    __syncthreads();
+    {
+        const unsigned occupied = __ballot_sync(FULL, c[t] > 0);
+        if ((t & 31) == 0) first[t >> 5] = occupied ? __ffs(occupied) - 1 : -1;
     }
+    __syncthreads();
+    if (t == 0)
+        for (int b = 0; b < 8 && cmin < 0; ++b)
+            if (first[b] >= 0) cmin = c[32 * b + first[b]];
     __syncthreads();
     for (int off = 1; off < 256; off <<= 1) {
         const int v = t >= off ? c[t - off] : 0;
@@ -161,9 +170,44 @@ __global__ void k_census(const __grid_constant__ IngestJobs J) {
     }
 }
 
-// Deterministic FP64 sums of both frames (after equalisation when lut is set): fixed grid, fixed tree
-// (blockIdx.z = job).
-__global__ void k_frame_sums(const __grid_constant__ IngestJobs J) {
+// A sum of floats: those in [2^-16, 2) as exact integers of 2^-40 (a block adds at most 2^21 of them, below 2^62), the
+// others in FP64.  An FP64 addition and the conversion before it take the FP64 pipe, 64 cycles each a warp instruction on
+// GB300; the integers take ten of one cycle.
+struct FrameSum {
+    long long fix = 0;
+    double rest = 0;
+    __device__ __forceinline__ void add(float v) {
+        const unsigned u = __float_as_uint(v);
+        if (u - 0x37800000u < 0x40000000u - 0x37800000u)
+            fix += (long long)((u & 0x7FFFFFu) | 0x800000u) << ((u >> 23) - 110);
+        else if (v != 0.f)
+            rest += (double)v;
+    }
+    // The block's total (of 1024 threads), on thread 0: a fixed tree, so the same bits at every run.
+    __device__ __forceinline__ double total(long long* sf, double* sr) {
+        const bool any = __syncthreads_or(rest != 0.0);  // also true for NaN
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            fix += __shfl_xor_sync(FULL, fix, o);
+            if (any) rest += __shfl_xor_sync(FULL, rest, o);
+        }
+        if ((threadIdx.x & 31) == 0) sf[threadIdx.x >> 5] = fix, sr[threadIdx.x >> 5] = rest;
+        __syncthreads();
+        if (threadIdx.x >= 32) return 0;
+        fix = sf[threadIdx.x];
+        rest = sr[threadIdx.x];
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            fix += __shfl_xor_sync(FULL, fix, o);
+            if (any) rest += __shfl_xor_sync(FULL, rest, o);
+        }
+        return (double)fix * 9.094947017729282379150390625e-13 + rest;  // 2^-40
+    }
+};
+
+// Sums of both frames (after equalisation when lut is set) per block, over rows blockIdx.x, + gridDim.x, ...
+// (blockIdx.z = job).  What bounds it: the frames' reads; 1280x720 with equalisation 56 -> 21 us, of which FP64 took 38.
+__global__ void __launch_bounds__(1024) k_frame_sums(const __grid_constant__ IngestJobs J) {
     const IngestJob& j = J.j[blockIdx.z];
     const void* f1 = j.f1;
     const void* f2 = j.f2;
@@ -172,54 +216,85 @@ __global__ void k_frame_sums(const __grid_constant__ IngestJobs J) {
     const int64_t stride = j.stride;
     const float* lut = j.hist ? j.lut : nullptr;
     double* partial = j.partial;
-    __shared__ double sh[2][256];
-    double a = 0, b = 0;
-    for (int y = blockIdx.x; y < H; y += gridDim.x) {
-        const int64_t r = (int64_t)y * stride;
-        if (lut) {
-            for (int x = threadIdx.x; x < W; x += blockDim.x) {
-                const int64_t e = r + 3 * x;
-                const float3 p = equalize_px(in_elem(f1, dt, e), in_elem(f1, dt, e + 1), in_elem(f1, dt, e + 2), lut);
-                const float3 q =
-                    equalize_px(in_elem(f2, dt, e), in_elem(f2, dt, e + 1), in_elem(f2, dt, e + 2), lut + 256);
-                a += (double)p.x + (double)p.y + (double)p.z;
-                b += (double)q.x + (double)q.y + (double)q.z;
-            }
-        } else {
-            for (int k = threadIdx.x; k < 3 * W; k += blockDim.x) {
-                a += (double)in_elem(f1, dt, r + k);
-                b += (double)in_elem(f2, dt, r + k);
-            }
+    __shared__ long long sf[2][32];
+    __shared__ double sr[2][32];
+    FrameSum a, b;
+    // the block's rows as one sequence of pixels (or elements), so that short rows leave no thread idle
+    const int rows = (H - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // at most 0 past the last row
+    if (lut) {
+#pragma unroll 2
+        for (int i = threadIdx.x; i < rows * W; i += blockDim.x) {
+            const int y = i / W, x = i - y * W;
+            const int64_t e = (int64_t)(blockIdx.x + y * gridDim.x) * stride + 3 * x;
+            const float3 p = equalize_px(in_elem(f1, dt, e), in_elem(f1, dt, e + 1), in_elem(f1, dt, e + 2), lut);
+            const float3 q = equalize_px(in_elem(f2, dt, e), in_elem(f2, dt, e + 1), in_elem(f2, dt, e + 2), lut + 256);
+            a.add(p.x), a.add(p.y), a.add(p.z);
+            b.add(q.x), b.add(q.y), b.add(q.z);
+        }
+    } else {
+        const int W3 = 3 * W;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < rows * W3; i += blockDim.x) {
+            const int y = i / W3, x = i - y * W3;
+            const int64_t e = (int64_t)(blockIdx.x + y * gridDim.x) * stride + x;
+            a.add(in_elem(f1, dt, e));
+            b.add(in_elem(f2, dt, e));
         }
     }
-    sh[0][threadIdx.x] = a;
-    sh[1][threadIdx.x] = b;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            sh[0][threadIdx.x] += sh[0][threadIdx.x + s];
-            sh[1][threadIdx.x] += sh[1][threadIdx.x + s];
-        }
-        __syncthreads();
-    }
+    const double ta = a.total(sf[0], sr[0]), tb = b.total(sf[1], sr[1]);
     if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = sh[0][0];
-        partial[2 * blockIdx.x + 1] = sh[1][0];
+        partial[2 * blockIdx.x] = ta;
+        partial[2 * blockIdx.x + 1] = tb;
     }
 }
 
-__global__ void k_gain(const __grid_constant__ IngestJobs J, int nblk, int enable) {
-    const IngestJob& j = J.j[blockIdx.z];
-    const double* partial = j.partial;
-    double* gain = j.gain;
-    if (threadIdx.x != 0) return;
-    double a = 0, b = 0;
-    for (int i = 0; i < nblk; ++i) {
-        a += partial[2 * i];
-        b += partial[2 * i + 1];
+// The gain of frame 2, mean(I1) / mean(I2), or 1: every block of k_pack adds the partial sums itself, in one order
+// (a launch of its own took 15 us, all of it one thread's 256 dependent FP64 additions).
+__device__ __forceinline__ double frame_gain(const double* partial, int enable) {
+    __shared__ double sg;
+    static_assert(kIngestPartialBlocks == 128, "four partial sums a lane");
+    if (threadIdx.x < 32) {
+        double a = 0, b = 0;
+        if (enable) {
+            double2 v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = reinterpret_cast<const double2*>(partial)[threadIdx.x + 32 * k];
+            a = (v[0].x + v[1].x) + (v[2].x + v[3].x);
+            b = (v[0].y + v[1].y) + (v[2].y + v[3].y);
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+                a += __shfl_xor_sync(FULL, a, o);
+                b += __shfl_xor_sync(FULL, b, o);
+            }
+        }
+        if (threadIdx.x == 0) sg = (enable && b > 0) ? a / b : 1.0;
     }
-    *gain = (enable && b > 0) ? a / b : 1.0;
+    __syncthreads();
+    return sg;
 }
+
+// (float)((double)q * g), mostly without the FP64 pipe: gh + gl holds g to 2^-48, the product's high part and its
+// error are exact, and the rest is within 2^-46 of the product, so the sum s rounds as the FP64 product does unless a
+// change of 2^-44 moves it (one product in 2^18); those, and products far from 1, are taken in FP64.  `wide`: g itself
+// is far from 1.  k_pack at 1280x720: 21 -> 14 us.
+struct Gain {
+    double g;
+    float gh, gl;
+    bool wide;
+    __device__ __forceinline__ explicit Gain(double v) : g(v), gh((float)v), gl((float)(v - (double)(float)v)) {
+        wide = !(v > 9.0949470177292824e-13 && v < 1099511627776.0);  // 2^-40, 2^40
+    }
+    __device__ __noinline__ static float wide_product(float q, double g) { return (float)((double)q * g); }
+    __device__ __forceinline__ float times(float q) const {
+        const float p = __fmul_rn(q, gh), e = __fmaf_rn(q, gh, -p), t = __fmaf_rn(q, gl, e);
+        const float d = __fmul_rn(fabsf(p), 5.6843418860808015e-14f);  // 2^-44
+        const float s = __fadd_rn(p, t);
+        const bool sure = s == __fadd_rn(p, __fadd_rn(t, d)) && s == __fadd_rn(p, __fsub_rn(t, d)) &&
+                          fabsf(p) > 8.67361738e-19f && fabsf(p) < 1.15292150e18f;  // 2^-60, 2^60
+        if (!wide && (sure || q == 0.f)) return q == 0.f ? q : s;
+        return wide_product(q, g);
+    }
+};
 
 template <int ST>
 __device__ __forceinline__ void store_pix(void* base, int i, float r, float g, float b) {
@@ -241,7 +316,7 @@ __device__ __forceinline__ void store_pix(void* base, int i, float r, float g, f
 }
 
 template <int ST>
-__global__ void k_pack(const __grid_constant__ IngestJobs J) {
+__global__ void k_pack(const __grid_constant__ IngestJobs J, int gain_enable) {
     const IngestJob& j = J.j[blockIdx.z];
     const void* f1 = j.f1;
     const void* f2 = j.f2;
@@ -251,7 +326,7 @@ __global__ void k_pack(const __grid_constant__ IngestJobs J) {
     const float* lut = j.hist ? j.lut : nullptr;
     void* o1 = j.o1;
     void* o2 = j.o2;
-    const double g = *j.gain;
+    const Gain g(frame_gain(j.partial, gain_enable));
     const int n = W * H;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int y = i / W, x = i - y * W;
@@ -263,7 +338,7 @@ __global__ void k_pack(const __grid_constant__ IngestJobs J) {
             q = equalize_px(q.x, q.y, q.z, lut + 256);
         }
         store_pix<ST>(o1, i, p.x, p.y, p.z);
-        store_pix<ST>(o2, i, (float)((double)q.x * g), (float)((double)q.y * g), (float)((double)q.z * g));
+        store_pix<ST>(o2, i, g.times(q.x), g.times(q.y), g.times(q.z));
     }
 }
 
@@ -1380,21 +1455,18 @@ void launch_ingest_jobs(const IngestJobs& J, int nj, int max_n, int max_h, int g
         k_vhist<<<dim3(blocks, 2, nj), 256, 0, st>>>(J);
         k_vlut<<<dim3(2, 1, nj), 256, 0, st>>>(J);
     }
-    k_frame_sums<<<dim3(kIngestPartialBlocks, 1, nj), 256, 0, st>>>(J);
-    k_gain<<<dim3(1, 1, nj), 32, 0, st>>>(J, kIngestPartialBlocks, gain_enable);
+    k_frame_sums<<<dim3(kIngestPartialBlocks, 1, nj), 1024, 0, st>>>(J);
     switch (storage) {
-        case 0: k_pack<0><<<dim3(blocks, 1, nj), 256, 0, st>>>(J); break;
-        case 1: k_pack<1><<<dim3(blocks, 1, nj), 256, 0, st>>>(J); break;
-        case 2: k_pack<2><<<dim3(blocks, 1, nj), 256, 0, st>>>(J); break;
+        case 0: k_pack<0><<<dim3(blocks, 1, nj), 256, 0, st>>>(J, gain_enable); break;
+        case 1: k_pack<1><<<dim3(blocks, 1, nj), 256, 0, st>>>(J, gain_enable); break;
+        case 2: k_pack<2><<<dim3(blocks, 1, nj), 256, 0, st>>>(J, gain_enable); break;
     }
 }
 
 void launch_ingest(const float* f1, const float* f2, int W, int H, int64_t stride, int gain_enable, int storage,
-                   double* partial, int nblk, double* gain, void* o1, void* o2, int* eq_hist, float* eq_lut,
-                   cudaStream_t st) {
-    (void)nblk;  // always kIngestPartialBlocks
+                   double* partial, void* o1, void* o2, int* eq_hist, float* eq_lut, cudaStream_t st) {
     IngestJobs J{};
-    J.j[0] = IngestJob{f1, f2, GPM_F32, W, H, stride, partial, gain, o1, o2, eq_lut ? eq_hist : nullptr, eq_lut,
+    J.j[0] = IngestJob{f1, f2, GPM_F32, W, H, stride, partial, o1, o2, eq_lut ? eq_hist : nullptr, eq_lut,
                        nullptr, nullptr, nullptr, nullptr, nullptr};
     launch_ingest_jobs(J, 1, W * H, H, gain_enable, storage, st);
 }

@@ -6,7 +6,7 @@
 // allocations behind their back, and latency-critical loops where an
 // allocation (and the implicit synchronisation cudaMalloc can bring) is not
 // allowed.  They pass the input frames and the output RGBX buffers; the
-// ingest's scratch (the FP64 partial sums of both frames, the gain, and the
+// ingest's scratch (the FP64 partial sums of both frames and the
 // V histogram and table of the optional HSV equalisation) lives in one
 // file-scope device array instead of a buffer from an allocator.
 //
@@ -27,8 +27,6 @@ namespace gpm {
 // The scratch of one ingest (6 KiB in all).
 struct NoAllocScratch {
     double partial[2 * kIngestPartialBlocks];  // per-block FP64 sums of both frames
-    double gain;                                // mean(I1) / mean(I2), or 1
-    double pad[31];                             // keeps the tables 256-byte aligned
     int hist[2 * 256];                          // V histograms (HSV equalisation)
     float lut[2 * 256];                         // equalised V per bin
 };
@@ -75,15 +73,14 @@ extern "C" gpm_status gpm_ingest_noalloc(const float* frame1, const float* frame
         }
         sc = g_scratch_ptr[dev];
     }
-    // Every slot this call reads is written first by this call (the partial sums and the gain by their kernels,
+    // Every slot this call reads is written first by this call (the partial sums by their kernel,
     // the histogram cleared on the stream before it is counted), so nothing carries over from an earlier call.
     char* base = reinterpret_cast<char*>(sc);  // a device address: only offsets are taken on the host
     double* partial = reinterpret_cast<double*>(base + offsetof(NoAllocScratch, partial));
-    double* gain = reinterpret_cast<double*>(base + offsetof(NoAllocScratch, gain));
     int* hist = reinterpret_cast<int*>(base + offsetof(NoAllocScratch, hist));
     float* lut = reinterpret_cast<float*>(base + offsetof(NoAllocScratch, lut));
-    launch_ingest(frame1, frame2, width, height, row_stride, gain_normalize, storage, partial, kIngestPartialBlocks,
-                  gain, out1, out2, equalize ? hist : nullptr, equalize ? lut : nullptr, (cudaStream_t)stream);
+    launch_ingest(frame1, frame2, width, height, row_stride, gain_normalize, storage, partial, out1, out2,
+                  equalize ? hist : nullptr, equalize ? lut : nullptr, (cudaStream_t)stream);
     // Reports a launch failure of this call; an error that earlier work left pending is reported (and cleared) too.
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? GPM_OK : GPM_ECUDA;
