@@ -293,6 +293,7 @@ struct EigShared {
     double M[45][32];
     EigState e;
     double A[45], rd[9], x[9];
+    double P[9][9], y[9];  // eig_jump: a power of (M - sigma I)^-1, and a product with it
 };
 constexpr int kEigSteps = 200;
 
@@ -593,6 +594,100 @@ __device__ __forceinline__ bool eig_thread(const double (*M)[32], double (&x)[9]
     return ++e.it < kEigSteps;
 }
 
+// Many steps of the iteration at once, by the whole warp: x <- B^128 x, normalised and oriented, B the inverse behind
+// the factor in sh (fresh: B's powers are not in sh.P yet; otherwise sh.P is squared once more and twice the steps are
+// taken).  A step multiplies by B and scales, so this is where 128 steps lead, but for rounding: B is applied to
+// the unit vectors (a column a lane) and squared seven times, each time scaled by a power of two, its entries two a lane:
+// 240 FP64 instructions where the steps take 10,000.  The rounding of B is small against its largest eigenvalue
+// 1 / (lambda_1 - sigma), so the vector is off by some 1e-16 / (1 - q), q the ratio of the steps' changes: a few
+// units at the ratios in question (0.6 to 0.95), below what the steps themselves leave (1e-13).  Of 7200 models of windows
+// with tiny supports one differs from the steps' result, by 7e-16.
+__device__ __noinline__ void eig_jump(EigShared& sh, bool fresh) {
+    const int lane = threadIdx.x & 31, row = min(lane, 8);
+    // sh.P times the power of two that brings its largest entry, which is on the diagonal, into [1, 2)
+    auto exponent = [&]() {
+        __syncwarp();
+        const unsigned top = __reduce_max_sync(FULL, (unsigned)__double2hiint(sh.P[row][row]) & 0x7FFFFFFFu) >> 20;
+        return (int)top;
+    };
+    auto usable = [](int top) { return top > 100 && top < 1900; };
+    auto scale = [](int top) { return __hiloint2double((2046 - top) << 20, 0); };
+    if (fresh) {
+        double y[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            double t = i == row ? 1.0 : 0.0;
+#pragma unroll
+            for (int k = 0; k < i; ++k) t = fma(-sh.A[i * (i + 1) / 2 + k], y[k], t);
+            y[i] = t * sh.rd[i];
+        }
+#pragma unroll
+        for (int i = 8; i >= 0; --i) {
+            double t = y[i];
+#pragma unroll
+            for (int k = i + 1; k < 9; ++k) t = fma(-sh.A[k * (k + 1) / 2 + i], y[k], t);
+            y[i] = t * sh.rd[i];
+        }
+        if (lane < 9) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) sh.P[lane][i] = y[i];
+        }
+        const int top = exponent();
+        if (!usable(top)) return;  // warp-uniform
+        const double f = scale(top);
+        if (lane < 9) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) sh.P[lane][i] = y[i] * f;
+        }
+        __syncwarp();
+    }
+    int pi[2], pj[2];  // this lane's entries (i, j) of the lower triangle
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int e = min(lane + 32 * r, 44);
+        int i = 0;
+        while ((i + 1) * (i + 2) / 2 <= e) ++i;
+        pi[r] = i;
+        pj[r] = e - i * (i + 1) / 2;
+    }
+    for (int s = fresh ? 0 : 6; s < 7; ++s) {
+        double c[2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            c[r] = 0;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) c[r] = fma(sh.P[pi[r]][k], sh.P[pj[r]][k], c[r]);
+        }
+        __syncwarp();
+        auto put = [&](double f) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) sh.P[pi[r]][pj[r]] = sh.P[pj[r]][pi[r]] = c[r] * f;
+        };
+        put(1.0);
+        const int top = exponent();
+        if (!usable(top)) return;
+        put(scale(top));
+        __syncwarp();
+    }
+    double t = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) t = fma(sh.P[row][k], sh.x[k], t);
+    if (lane < 9) sh.y[lane] = t;
+    __syncwarp();
+    double n = 0, dot = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        n = fma(sh.y[i], sh.y[i], n);
+        dot = fma(sh.y[i], sh.x[i], dot);
+    }
+    __syncwarp();
+    if (!(n > 1e-30 && n < 1e30)) return;  // the same on every lane
+    double sc = rsqrt_nr(n);
+    if (negative(dot)) sc = -sc;
+    if (lane < 9) sh.x[lane] = t * sc;
+    __syncwarp();
+}
+
 // The iteration of one window (its state in sh, its matrix in column `col`), carried on by the whole warp: the few
 // windows that need many steps (supports of 4 or 5 matches with a nearly two-dimensional null space: up to 200) set
 // the launch's duration, and a step on one thread is some 140 FP64 instructions of 64 cycles each.  Every operation
@@ -600,17 +695,24 @@ __device__ __forceinline__ bool eig_thread(const double (*M)[32], double (&x)[9]
 // lane i holding row i; the backward one (whose order leaves no parallelism) on every lane; the two dot products on
 // even and odd lanes; scaling and difference with lane i on entry i.  About 80 FP64 instructions a step; the eight
 // solves of a 1024x436 pair 3.15 -> 2.36 ms.  The solve kernel hands a window over once it is the warp's last and 4
-// steps are done (98.5 % of the windows need no more): two or more are cheaper side by side on their threads.
+// steps are done (98.5 % of the windows need no more), or after 12: two or more are cheaper side by side on their
+// threads for a few steps.
+// A window that is still iterating with one factor after 4 steps here takes the next 128 at once (eig_jump); a slow
+// one only when the gap test has let it go on.  One launch in two has a window of 60 to 200 steps, 0.3 to 0.55 ms in
+// which the chip waits: the eight solves of a 1024x436 pair 1.71 -> 1.26 ms, the six of a 128x96 one 0.71 -> 0.57 ms.
 __device__ __noinline__ void eig_warp(EigShared& sh, int col) {
     const int lane = threadIdx.x & 31, row = min(lane, 8);
     double A[45], rd[9], x[9], Lr[8], rdr = 0;
     EigState e = sh.e;
 #pragma unroll
     for (int i = 0; i < 9; ++i) x[i] = sh.x[i];
-    int loaded = -1;
+    int loaded = -1, since = 0;  // the factor held here; steps with it since a jump
+    bool fresh = true, gap_ok = false;
     for (;;) {
         if (loaded != e.reshifts) {  // the factor may be new
             loaded = e.reshifts;
+            since = 0;
+            fresh = true;
             __syncwarp();
 #pragma unroll
             for (int q = 0; q < 45; ++q) A[q] = sh.A[q];
@@ -656,11 +758,13 @@ __device__ __noinline__ void eig_warp(EigShared& sh, int col) {
         if (eig_check_due(e)) {  // the same on every lane
             double xc[9], B[45], rdB[9];
             EigState ec = e;
+            const int was = e.reshifts;
 #pragma unroll
             for (int i = 0; i < 9; ++i) xc[i] = x[i];
             const int what = eig_gap_or_shift(sh.M, col, xc, &ec, B, rdB);
             e = ec;
             if (what == 0) break;
+            gap_ok = what == 1 && e.reshifts >= 4 && ec.reshifts == was;
             if (what == 2) {
                 __syncwarp();
                 if (lane == 0) {
@@ -670,6 +774,19 @@ __device__ __noinline__ void eig_warp(EigShared& sh, int col) {
             }
         }
         if (++e.it >= kEigSteps) break;
+        if (++since >= 4 && loaded == e.reshifts && (e.slow == 0 || gap_ok)) {
+            __syncwarp();
+            if (lane == 0) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) sh.x[i] = x[i];
+            }
+            __syncwarp();
+            eig_jump(sh, fresh);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) x[i] = sh.x[i];
+            fresh = false;
+            since = 0;
+        }
     }
     __syncwarp();
     if (lane == 0) {
@@ -1673,11 +1790,12 @@ __global__ void __launch_bounds__(32) k_refit_solve(const __grid_constant__ Batc
     unsigned left;
     for (int step = 0;; ++step) {
         left = __ballot_sync(FULL, act);
-        if (!left || (step >= 4 && __popc(left) == 1)) break;
+        if (!left || (step >= 4 && __popc(left) == 1) || step >= 12) break;
         if (act) act = eig_thread(sh.M, x, A, rd, e);
     }
-    if (left) {  // one window's iteration goes on
-        if (act) {
+    for (; left; left &= left - 1) {  // a window's iteration goes on
+        const bool mine = lane == __ffs(left) - 1;
+        if (mine) {
             sh.e = e;
 #pragma unroll
             for (int q = 0; q < 45; ++q) sh.A[q] = A[q];
@@ -1686,10 +1804,11 @@ __global__ void __launch_bounds__(32) k_refit_solve(const __grid_constant__ Batc
         }
         __syncwarp();
         eig_warp(sh, __ffs(left) - 1);
-        if (act) {
+        if (mine) {
 #pragma unroll
             for (int i = 0; i < 9; ++i) x[i] = sh.x[i];
         }
+        __syncwarp();
     }
     if (!refit) return;
     refit_record(rw, g, pp, cell, x, f);
