@@ -511,7 +511,7 @@ struct PairView {
     int* list[2];         // unfrozen pixel indices, colour 0 then colour 1
     int* list_count;      // [2 dirs][2 colours]
     int* flag;            // device consistency flag: set (non-zero) by a check that failed, read by gpm_sync
-    unsigned long long* m2o_key[2];
+    unsigned long long* m2o_key[2];  // many-to-one keys; census: grey keys; level-0 sweeps: region sums (RegionSums)
     RefitWork* rw[2];     // [cells of the largest level]
     uint32_t* code[2];    // census codes of each frame (census data term)
     int* gq;              // floor(1024 (R + G + B)) of frame 1 as given (edge-aware fill)

@@ -819,6 +819,39 @@ __device__ __forceinline__ float box_threshold(float bc) {
     return fmaf(bc, 1.52587890625e-05f, bc) + 3.814697265625e-06f;
 }
 
+// A second, tighter bound for the random candidates that pass the first, at r = 4 with 16-byte texels: the patch is nine
+// regions of 3 x 3 texels, and the raw cost is at least the sum over them of sum_ch |region sum of a - region sum of b|,
+// the region sums from k_box_sums (in the many-to-one keys' buffer, idle at level 0).  Half of those candidates go;
+// a test costs a lane 100 instructions and 9 gathers of 8 bytes, an evaluation the warp as many and 81 gathers of 16.
+// 1024x436: the 16 sweeps 5.20 -> 4.73 ms.  Where it does not pay: 8-byte texels (half the gathers' cost: 1920x1080 FP16
+// 17.7 -> 17.8 ms), r = 3 (49 texels, four 3 x 3 corners and the cross between them: 511x383 1.17 -> 1.19 ms), and
+// propagated candidates (mostly good ones: with them tested 4.87 ms).
+// A sum is held as 16-bit multiples of 2^-11 per channel (.x = r | g << 16, .y = b; at most 9 * 2), off by at most
+// 2^-12 and eight FP32 roundings, 2.54e-4 in all; bit 31 of .y marks a texel out of the domain of in_domain, for which
+// nothing is dropped.  The margin: 54 such values, 0.0138 = 28.2 units.
+template <int R, int ST>
+constexpr bool kRegionBound = R == 4 && ST == 0;
+struct RegionSums {
+    uint2 a[9];  // the source patch's
+    __device__ __forceinline__ static int at(int k, int W) { return (k / 3 - 1) * 3 * W + (k % 3 - 1) * 3; }
+    __device__ __forceinline__ void load(const uint2* s1, int W) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) a[k] = __ldg(s1 + at(k, W));
+    }
+    // Whether a candidate cannot cost less than thr (box_threshold's); s2: the sums at its target pixel.
+    __device__ __forceinline__ bool excludes(const uint2* s2, int W, float thr) const {
+        unsigned flags = 0, lb = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const uint2 b = __ldg(s2 + at(k, W));
+            flags |= a[k].y | b.y;
+            lb = __dp2a_lo(__vmaxu2(a[k].x, b.x) - __vminu2(a[k].x, b.x), 0x0101u, lb);
+            lb = __dp2a_lo(__vmaxu2(a[k].y, b.y) - __vminu2(a[k].y, b.y), 0x0001u, lb);
+        }
+        return !(flags >> 31) && (float)lb - 29.f >= thr * 2048.f;
+    }
+};
+
 // ---------------------------------------------------------------- interval lower bound (levels >= 1)
 // A warped tap samples between pixels, so the patch sums above do not apply; but a bilinear sample less than one pixel
 // from a place lies between the least and the greatest texel of the 3 x 3 around it.  k_interval_sums replaces
@@ -1252,6 +1285,8 @@ __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Ba
     const bool prune = mine && xq >= R && yq >= R && xq < W - R && yq < H - R;
     const unsigned inside = __ballot_sync(FULL, prune);
     const float4 b1 = prune ? pv.box[dir][iq] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint2* __restrict__ region1 = reinterpret_cast<const uint2*>(pv.m2o_key[dir]) + iq;
+    const uint2* __restrict__ region2 = reinterpret_cast<const uint2*>(pv.m2o_key[1 - dir]) + iq;
     unsigned npr = 0, nev = 0;
     // list A, one pixel per lane: the four neighbours' offsets whose target is in the frame, neither the
     // incumbent nor a repeat, and not excluded by the bound
@@ -1274,6 +1309,25 @@ __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Ba
         }
     }
     for (int part = 0;; ++part) {
+        if constexpr (kRegionBound<R, ST>) {
+            // list B by the regions' bound, one pixel per lane (targets whose patch stays in the frame, as the regions must)
+            if (part && prune && n > 0) {
+                RegionSums regions;
+                regions.load(region1, W);
+                const float thr = box_threshold(bc * 1.1920928955078125e-07f);
+                int kept = 0;
+                for (int k = 0; k < n; ++k) {
+                    const uint32_t key = list[k][lane];
+                    const int2 c = unpack_off(key);
+                    if ((unsigned)(xq + c.x - R) < (unsigned)(W - 2 * R) && (unsigned)(yq + c.y - R) < (unsigned)(H - 2 * R) &&
+                        regions.excludes(region2 + c.y * W + c.x, W, thr))
+                        ++npr;
+                    else
+                        list[kept++][lane] = key;
+                }
+                n = kept;
+            }
+        }
         __syncwarp();
         // the list's costs, one tap per lane, pixel by pixel
         nev += n;
@@ -1535,6 +1589,18 @@ __global__ void __launch_bounds__(256) k_box_sums(const __grid_constant__ Batch 
             a.z += v.z;
         }
         pv.box[dir][y * W + x] = make_float4(a.x, a.y, a.z, 0.f);
+        if constexpr (kRegionBound<R, ST>) {  // the 3 x 3 sums
+            float3 t = make_float3(0.f, 0.f, 0.f);
+            bool ok = true;
+#pragma unroll
+            for (int d = 0; d < 9; ++d) {
+                const float3 v = tex[ly + R - 1 + d / 3][lx + R - 1 + d % 3];
+                ok = ok && in_domain(v.x, v.y, v.z);
+                t = make_float3(t.x + v.x, t.y + v.y, t.z + v.z);
+            }
+            const unsigned r = __float2uint_rn(t.x * 2048.f), g = __float2uint_rn(t.y * 2048.f), b = __float2uint_rn(t.z * 2048.f);
+            reinterpret_cast<uint2*>(pv.m2o_key[dir])[y * W + x] = ok ? make_uint2(r | g << 16, b) : make_uint2(0u, 0x80000000u);
+        }
     }
 }
 template <int ST>

@@ -15,3 +15,12 @@ def test_restricted_sweeps_equal_oracle(W, H, r, cells):
     import torch
     gpm.load()
     parity.test_restricted_patchmatch_level1_lockstep(torch, W, H, r, cells)
+
+
+@pytest.mark.parametrize("W,H", [(61, 43), (40, 97), (129, 21), (24, 17)])
+def test_level0_sweeps_with_region_bound_equal_oracle(W, H):
+    """Radius 4 with FP32 texels, where list B is tested by the 3 x 3 regions' sums too: ragged tiles, and frames with
+    few or no pixels whose patch stays inside."""
+    import torch
+    gpm.load()
+    parity.test_level0_patchmatch_matches_oracle_up_to_near_ties(torch, W, H, 4, (8,))
