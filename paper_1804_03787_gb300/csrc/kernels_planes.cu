@@ -1765,6 +1765,7 @@ __device__ __forceinline__ void refit_record(RefitWork* rw, const LevelGeom& g, 
 // integer ones, the smallest eigenvector of A^T A started from the winner,
 // denormalisation, and the geometry checks of the winner and of the refit.
 __global__ void __launch_bounds__(32) k_refit_solve(const __grid_constant__ Batch bt, int level, PlaneParams pp) {
+    begin_long_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     __shared__ EigShared sh;
@@ -1909,6 +1910,7 @@ constexpr int kRansacWarps = 4;
 template <int CAP>
 __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     k_ransac_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
+    begin_long_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     __shared__ __align__(16) float planes[kRansacWarps][4 * CAP];
@@ -1931,6 +1933,7 @@ __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
+    begin_long_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     __shared__ float4 match[8][256];
@@ -1945,6 +1948,7 @@ __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constan
 __host__ __device__ constexpr int block_cap(int s) { return (s * s + 127) / 128 * 128; }
 __global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__ Batch bt, int level, int stage,
                                                          PlaneParams pp) {
+    begin_long_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int cell = blockIdx.x, dir = blockIdx.y;
@@ -1969,6 +1973,7 @@ __global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
+    begin_long_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     if ((int)blockIdx.x >= g.ncells()) return;  // past this pair's windows (block-uniform)
@@ -1988,6 +1993,7 @@ __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_consta
 // smallest L = delta (first window on ties), with flow H p - p.
 template <int ST>
 __global__ void k_assign(const __grid_constant__ Batch bt, int level, int stage, int which, int write_resid, PlaneParams pp) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int dir = blockIdx.y;
@@ -2040,6 +2046,7 @@ __global__ void k_assign(const __grid_constant__ Batch bt, int level, int stage,
 
 // ---------------------------------------------------------------- occlusion cues (Sec. 3.4)
 __global__ void k_cue_zero(const __grid_constant__ Batch bt, int level, int stage) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int dir = blockIdx.y;
@@ -2054,6 +2061,7 @@ __global__ void k_cue_zero(const __grid_constant__ Batch bt, int level, int stag
 // this level and stage with flow f is symmetric iff q = round(p + f) holds an
 // assigned pixel of the other direction with flow g, |f + g| < t_fb.
 __global__ void k_cue_counts(const __grid_constant__ Batch bt, int level, int stage, int which, PlaneParams pp) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int dir = blockIdx.y;
@@ -2082,6 +2090,7 @@ __global__ void k_cue_counts(const __grid_constant__ Batch bt, int level, int st
 
 // Discard planes failing the symmetry cue (eta) or the RANSAC/colour overlap cue (kappa).
 __global__ void k_cue_invalidate(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int dir = blockIdx.y;
@@ -2108,12 +2117,14 @@ __global__ void k_cue_invalidate(const __grid_constant__ Batch bt, int level, in
 // Many-to-one: per target q = round(p + f), the lowest (L, index) keeps it;
 // a loser whose flow differs from the winner's by t_fb or more is occluded.
 __global__ void k_m2o_init(const __grid_constant__ Batch bt) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pv.n; i += gridDim.x * blockDim.x)
         pv.m2o_key[dir][i] = ~0ull;
 }
 __global__ void k_m2o_claim(const __grid_constant__ Batch bt) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const int W = pv.W, n = pv.n;
@@ -2129,6 +2140,7 @@ __global__ void k_m2o_claim(const __grid_constant__ Batch bt) {
     }
 }
 __global__ void k_m2o_resolve(const __grid_constant__ Batch bt, PlaneParams pp) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const int W = pv.W, n = pv.n;
@@ -2154,6 +2166,7 @@ __global__ void k_m2o_resolve(const __grid_constant__ Batch bt, PlaneParams pp) 
 
 // Sec. 3.3 merge with coarse priority, then the NNF update of Sec. 3.3.1.
 __global__ void k_merge_update(const __grid_constant__ Batch bt, PlaneParams pp) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const int n = pv.n;
@@ -2177,6 +2190,7 @@ __global__ void k_merge_update(const __grid_constant__ Batch bt, PlaneParams pp)
 // One Jacobi iteration: labels from acc into tent (flip = 0) or from tent into acc (flip = 1).
 template <int ST>
 __global__ void k_fill(const __grid_constant__ Batch bt, int flip, PlaneParams pp) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const int W = pv.W, H = pv.H, n = pv.n;
@@ -2245,6 +2259,7 @@ __global__ void k_fill(const __grid_constant__ Batch bt, int flip, PlaneParams p
 __device__ __forceinline__ long long* seed_dist(const PairView& pv) { return reinterpret_cast<long long*>(pv.m2o_key[0]); }
 __device__ __forceinline__ int* seed_of(const PairView& pv) { return pv.list[0]; }
 __global__ void k_seed_init(const __grid_constant__ Batch bt) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int* am = pv.acc[0].m;
     const int n = pv.n;
@@ -2272,6 +2287,7 @@ __device__ __forceinline__ long long seed_step(int q, int before) { return 256 +
 // Rows, a warp each: left to right, then right to left, 32 pixels at a time (their steps' prefix sums, then the
 // offers' prefix minima, by shuffles; the last pixel's offer goes on to the next 32).
 __global__ void __launch_bounds__(128) k_seed_rows(const __grid_constant__ Batch bt) {
+    begin_long_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int W = pv.W, y = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (y >= pv.H) return;
@@ -2323,6 +2339,7 @@ __global__ void __launch_bounds__(128) k_seed_rows(const __grid_constant__ Batch
 // lane a column: it walks its section for the steps' sum and the offer at its end, adds up the sections before it, and walks
 // it again with that offer.
 __global__ void __launch_bounds__(1024) k_seed_columns(const __grid_constant__ Batch bt) {
+    begin_long_kernel();
     constexpr int U = 8;  // rows loaded together
     const PairView& pv = bt.view(blockIdx.z);
     const int W = pv.W, H = pv.H, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -2390,6 +2407,7 @@ __global__ void __launch_bounds__(1024) k_seed_columns(const __grid_constant__ B
 // after warping by the final flow >= occ_thresh.
 template <int ST>
 __global__ void k_final(const __grid_constant__ Batch bt, PlaneParams pp, int interp, const __grid_constant__ FinalOut out) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = 0;
     const int* seed = interp ? seed_of(pv) : nullptr;
@@ -2448,6 +2466,7 @@ __global__ void k_final(const __grid_constant__ Batch bt, PlaneParams pp, int in
 // ---------------------------------------------------------------- state import / export helpers
 // Evaluation forms of imported absolute homographies.
 __global__ void k_import_models(const __grid_constant__ Batch bt, int nlev, int m) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom* geoms = bt.geo[blockIdx.z];
     const int dir = blockIdx.y;
@@ -2470,6 +2489,7 @@ __global__ void k_import_models(const __grid_constant__ Batch bt, int nlev, int 
 
 // labels <-> (model, L, flow) with flow = v + r in double
 __global__ void k_labels_export(Labels l, int n, int* om, float* oL, double* of) {
+    begin_kernel();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         om[i] = l.m[i];
         oL[i] = l.L[i];
@@ -2479,6 +2499,7 @@ __global__ void k_labels_export(Labels l, int n, int* om, float* oL, double* of)
 }
 __global__ void k_labels_import(Labels l, int n, int m, const int* im, const float* iL, const double* iF,
                                 int* flag) {
+    begin_kernel();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         int id = im[i];
         const double fx = iF[2 * i], fy = iF[2 * i + 1];
@@ -2511,11 +2532,11 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
     if (s <= 16) {
         const dim3 fgrid((nc + kRansacWarps - 1) / kRansacWarps, 2, np), grid((nc + 7) / 8, 2, np);
         if (s <= 8)
-            k_ransac_warp<64><<<fgrid, 32 * kRansacWarps, 0, st>>>(bt, level, stage, pp);
+            launch_kernel(k_ransac_warp<64>, fgrid, 32 * kRansacWarps, 0, st, bt, level, stage, pp);
         else
-            k_ransac_warp<256><<<fgrid, 32 * kRansacWarps, 0, st>>>(bt, level, stage, pp);
-        k_refit_solve<<<dim3((2 * nc + 31) / 32, 1, np), 32, 0, st>>>(bt, level, pp);
-        k_ransac_finish_warp<ST><<<grid, 256, 0, st>>>(bt, level, stage, pp);
+            launch_kernel(k_ransac_warp<256>, fgrid, 32 * kRansacWarps, 0, st, bt, level, stage, pp);
+        launch_kernel(k_refit_solve, dim3((2 * nc + 31) / 32, 1, np), 32, 0, st, bt, level, pp);
+        launch_kernel(k_ransac_finish_warp<ST>, grid, 256, 0, st, bt, level, stage, pp);
         return;
     }
     const size_t smem = (size_t)s * s * sizeof(float4), fit_smem = (size_t)block_cap(s) * sizeof(float4);
@@ -2526,9 +2547,9 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
         cudaFuncSetAttribute(k_ransac_finish_block<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
         attr_set = true;
     }
-    k_ransac_block<<<dim3(nc, 2, np), 256, fit_smem, st>>>(bt, level, stage, pp);
-    k_refit_solve<<<dim3((2 * nc + 31) / 32, 1, np), 32, 0, st>>>(bt, level, pp);
-    k_ransac_finish_block<ST><<<dim3(nc, 2, np), 256, smem, st>>>(bt, level, stage, pp);
+    launch_kernel(k_ransac_block, dim3(nc, 2, np), 256, fit_smem, st, bt, level, stage, pp);
+    launch_kernel(k_refit_solve, dim3((2 * nc + 31) / 32, 1, np), 32, 0, st, bt, level, pp);
+    launch_kernel(k_ransac_finish_block<ST>, dim3(nc, 2, np), 256, smem, st, bt, level, stage, pp);
 }
 void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int stage, const PlaneParams& pp,
                    cudaStream_t st) {
@@ -2543,28 +2564,28 @@ void launch_assign(const Batch& bt, int np, int level, int stage, int which, int
                    int grid_blocks, cudaStream_t st) {
     const dim3 grid(grid_blocks, 2, np);
     switch (pp.storage) {
-        case 0: k_assign<0><<<grid, 256, 0, st>>>(bt, level, stage, which, write_resid, pp); break;
-        case 1: k_assign<1><<<grid, 256, 0, st>>>(bt, level, stage, which, write_resid, pp); break;
-        case 2: k_assign<2><<<grid, 256, 0, st>>>(bt, level, stage, which, write_resid, pp); break;
+        case 0: launch_kernel(k_assign<0>, grid, 256, 0, st, bt, level, stage, which, write_resid, pp); break;
+        case 1: launch_kernel(k_assign<1>, grid, 256, 0, st, bt, level, stage, which, write_resid, pp); break;
+        case 2: launch_kernel(k_assign<2>, grid, 256, 0, st, bt, level, stage, which, write_resid, pp); break;
     }
 }
 
 void launch_cues(const Batch& bt, int np, int level, int max_cells, int stage, int which, const PlaneParams& pp,
                  int grid_blocks, cudaStream_t st) {
     const int cb = (max_cells + 255) / 256;
-    k_cue_zero<<<dim3(cb, 2, np), 256, 0, st>>>(bt, level, stage);
-    k_cue_counts<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt, level, stage, which, pp);
-    k_cue_invalidate<<<dim3(cb, 2, np), 256, 0, st>>>(bt, level, stage, pp);
+    launch_kernel(k_cue_zero, dim3(cb, 2, np), 256, 0, st, bt, level, stage);
+    launch_kernel(k_cue_counts, dim3(grid_blocks, 2, np), 256, 0, st, bt, level, stage, which, pp);
+    launch_kernel(k_cue_invalidate, dim3(cb, 2, np), 256, 0, st, bt, level, stage, pp);
 }
 
 void launch_many_to_one(const Batch& bt, int np, const PlaneParams& pp, int grid_blocks, cudaStream_t st) {
-    k_m2o_init<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt);
-    k_m2o_claim<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt);
-    k_m2o_resolve<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt, pp);
+    launch_kernel(k_m2o_init, dim3(grid_blocks, 2, np), 256, 0, st, bt);
+    launch_kernel(k_m2o_claim, dim3(grid_blocks, 2, np), 256, 0, st, bt);
+    launch_kernel(k_m2o_resolve, dim3(grid_blocks, 2, np), 256, 0, st, bt, pp);
 }
 
 void launch_merge_update(const Batch& bt, int np, const PlaneParams& pp, int grid_blocks, cudaStream_t st) {
-    k_merge_update<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt, pp);
+    launch_kernel(k_merge_update, dim3(grid_blocks, 2, np), 256, 0, st, bt, pp);
 }
 
 // Label sets of a pair: 0 acc, 1 tent, 2 st1, 3 lvl.
@@ -2572,6 +2593,7 @@ __device__ __forceinline__ Labels label_set(const PairView& pv, int set, int dir
     return set == 0 ? pv.acc[dir] : (set == 1 ? pv.tent[dir] : (set == 2 ? pv.st1[dir] : pv.lvl[dir]));
 }
 __global__ void k_copy_labels(const __grid_constant__ Batch bt, int from, int to) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const Labels a = label_set(pv, from, dir), b = label_set(pv, to, dir);
@@ -2583,7 +2605,7 @@ __global__ void k_copy_labels(const __grid_constant__ Batch bt, int from, int to
     }
 }
 void launch_copy_labels(const Batch& bt, int np, int from, int to, int grid_blocks, cudaStream_t st) {
-    k_copy_labels<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt, from, to);
+    launch_kernel(k_copy_labels, dim3(grid_blocks, 2, np), 256, 0, st, bt, from, to);
 }
 
 void launch_fill(const Batch& bt, int np, const PlaneParams& pp, int iters, int grid_blocks, cudaStream_t st) {
@@ -2591,19 +2613,19 @@ void launch_fill(const Batch& bt, int np, const PlaneParams& pp, int iters, int 
     const dim3 grid(grid_blocks, 2, np);
     for (int it = 0; it < iters; ++it) {
         switch (pp.storage) {
-            case 0: k_fill<0><<<grid, 256, 0, st>>>(bt, it & 1, pp); break;
-            case 1: k_fill<1><<<grid, 256, 0, st>>>(bt, it & 1, pp); break;
-            case 2: k_fill<2><<<grid, 256, 0, st>>>(bt, it & 1, pp); break;
+            case 0: launch_kernel(k_fill<0>, grid, 256, 0, st, bt, it & 1, pp); break;
+            case 1: launch_kernel(k_fill<1>, grid, 256, 0, st, bt, it & 1, pp); break;
+            case 2: launch_kernel(k_fill<2>, grid, 256, 0, st, bt, it & 1, pp); break;
         }
     }
     if (iters & 1) launch_copy_labels(bt, np, 1, 0, grid_blocks, st);  // the result sits in tent
 }
 
 void launch_fill_seeds(const Batch& bt, int np, int max_w, int max_h, int rounds, int grid_blocks, cudaStream_t st) {
-    k_seed_init<<<dim3(grid_blocks, 1, np), 256, 0, st>>>(bt);
+    launch_kernel(k_seed_init, dim3(grid_blocks, 1, np), 256, 0, st, bt);
     for (int r = 0; r < rounds; ++r) {
-        k_seed_rows<<<dim3((max_h + 3) / 4, 1, np), 128, 0, st>>>(bt);
-        k_seed_columns<<<dim3((max_w + 31) / 32, 1, np), 1024, 0, st>>>(bt);
+        launch_kernel(k_seed_rows, dim3((max_h + 3) / 4, 1, np), 128, 0, st, bt);
+        launch_kernel(k_seed_columns, dim3((max_w + 31) / 32, 1, np), 1024, 0, st, bt);
     }
 }
 
@@ -2611,14 +2633,15 @@ void launch_final(const Batch& bt, int np, const PlaneParams& pp, int interp, co
                   cudaStream_t st) {
     const dim3 grid(grid_blocks, 1, np);
     switch (pp.storage) {
-        case 0: k_final<0><<<grid, 256, 0, st>>>(bt, pp, interp, out); break;
-        case 1: k_final<1><<<grid, 256, 0, st>>>(bt, pp, interp, out); break;
-        case 2: k_final<2><<<grid, 256, 0, st>>>(bt, pp, interp, out); break;
+        case 0: launch_kernel(k_final<0>, grid, 256, 0, st, bt, pp, interp, out); break;
+        case 1: launch_kernel(k_final<1>, grid, 256, 0, st, bt, pp, interp, out); break;
+        case 2: launch_kernel(k_final<2>, grid, 256, 0, st, bt, pp, interp, out); break;
     }
 }
 
 // Clears the models of every window of every level (model ids below m_models).
 __global__ void k_reset_models(const __grid_constant__ Batch bt) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < pv.m_models; id += gridDim.x * blockDim.x) {
@@ -2631,10 +2654,11 @@ __global__ void k_reset_models(const __grid_constant__ Batch bt) {
 }
 void launch_reset_models(const Batch& bt, int np, int max_models, cudaStream_t st) {
     if (max_models <= 0) return;  // no plane levels: no model table (an empty grid is not a launch)
-    k_reset_models<<<dim3((max_models + 255) / 256, 2, np), 256, 0, st>>>(bt);
+    launch_kernel(k_reset_models, dim3((max_models + 255) / 256, 2, np), 256, 0, st, bt);
 }
 
 __global__ void k_reset_labels(const __grid_constant__ Batch bt, float eps) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pv.n; i += gridDim.x * blockDim.x) {
@@ -2647,21 +2671,23 @@ __global__ void k_reset_labels(const __grid_constant__ Batch bt, float eps) {
     }
 }
 __global__ void k_frozen_from_labels(const __grid_constant__ Batch bt) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pv.n; i += gridDim.x * blockDim.x)
         pv.frozen[dir][i] = pv.acc[dir].m[i] >= 0;
 }
 void launch_frozen_from_labels(const Batch& bt, int np, int grid_blocks, cudaStream_t st) {
-    k_frozen_from_labels<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt);
+    launch_kernel(k_frozen_from_labels, dim3(grid_blocks, 2, np), 256, 0, st, bt);
 }
 
 void launch_reset_labels(const Batch& bt, int np, float eps, int grid_blocks, cudaStream_t st) {
-    k_reset_labels<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt, eps);
+    launch_kernel(k_reset_labels, dim3(grid_blocks, 2, np), 256, 0, st, bt, eps);
 }
 
 template <int ST>
 __global__ void k_frames_export(const __grid_constant__ Batch bt, float* dst) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pv.n; i += gridDim.x * blockDim.x) {
@@ -2672,23 +2698,23 @@ __global__ void k_frames_export(const __grid_constant__ Batch bt, float* dst) {
 void launch_frames_export(const Batch& bt, int n, int storage, float* dst, cudaStream_t st) {
     const dim3 grid((n + 255) / 256, 2);
     switch (storage) {
-        case 0: k_frames_export<0><<<grid, 256, 0, st>>>(bt, dst); break;
-        case 1: k_frames_export<1><<<grid, 256, 0, st>>>(bt, dst); break;
-        case 2: k_frames_export<2><<<grid, 256, 0, st>>>(bt, dst); break;
+        case 0: launch_kernel(k_frames_export<0>, grid, 256, 0, st, bt, dst); break;
+        case 1: launch_kernel(k_frames_export<1>, grid, 256, 0, st, bt, dst); break;
+        case 2: launch_kernel(k_frames_export<2>, grid, 256, 0, st, bt, dst); break;
     }
 }
 
 void launch_import_models(const Batch& bt, int nlev, int m, cudaStream_t st) {
     if (m <= 0) return;  // no model table
-    k_import_models<<<dim3((m + 255) / 256, 2), 256, 0, st>>>(bt, nlev, m);
+    launch_kernel(k_import_models, dim3((m + 255) / 256, 2), 256, 0, st, bt, nlev, m);
 }
 
 void launch_labels_export(const Labels& l, int n, int* om, float* oL, double* of, cudaStream_t st) {
-    k_labels_export<<<(n + 255) / 256, 256, 0, st>>>(l, n, om, oL, of);
+    launch_kernel(k_labels_export, (n + 255) / 256, 256, 0, st, l, n, om, oL, of);
 }
 void launch_labels_import(const Labels& l, int n, int m, const int* im, const float* iL, const double* iF, int* flag,
                           cudaStream_t st) {
-    k_labels_import<<<(n + 255) / 256, 256, 0, st>>>(l, n, m, im, iL, iF, flag);
+    launch_kernel(k_labels_import, (n + 255) / 256, 256, 0, st, l, n, m, im, iL, iF, flag);
 }
 
 }  // namespace gpm

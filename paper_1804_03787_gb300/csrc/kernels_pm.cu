@@ -42,6 +42,7 @@ __device__ __forceinline__ int v_bin(float v) {
 
 // Clears the V histograms of the jobs that equalise (blockIdx.z = job).
 __global__ void k_vhist_zero(const __grid_constant__ IngestJobs J) {
+    begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     if (j.hist)
         for (int k = threadIdx.x; k < 2 * 256; k += blockDim.x) j.hist[k] = 0;
@@ -49,6 +50,7 @@ __global__ void k_vhist_zero(const __grid_constant__ IngestJobs J) {
 
 // V histogram of each frame (blockIdx.y = frame, blockIdx.z = job); hist holds 2 x 256 zeroed counts.
 __global__ void k_vhist(const __grid_constant__ IngestJobs J) {
+    begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     if (!j.hist) return;  // block-uniform
     const int W = j.W, H = j.H;
@@ -79,6 +81,7 @@ __global__ void k_vhist(const __grid_constant__ IngestJobs J) {
 
 // Equalised V per bin (blockIdx.x = frame, blockIdx.z = job, 256 threads): an inclusive scan of the counts.
 __global__ void k_vlut(const __grid_constant__ IngestJobs J) {
+    begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     if (!j.hist) return;  // block-uniform
     const int* hist = j.hist;
@@ -128,6 +131,7 @@ __device__ __forceinline__ float3 equalize_px(float r, float g, float b, const f
 // turns -0 into +0.  The 24 comparisons per pixel then run on the integer
 // pipe with exactly the outcomes of comparing the doubles.
 __global__ void k_grey_keys(const __grid_constant__ IngestJobs J) {
+    begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     if (!j.k1) return;  // block-uniform
     const int W = j.W, n = j.W * j.H;
@@ -147,6 +151,7 @@ __global__ void k_grey_keys(const __grid_constant__ IngestJobs J) {
 // 5x5 census code per pixel: bit k (raster order without the centre, neighbours clamped into the frame) set iff
 // the neighbour's grey is below the centre's.
 __global__ void k_census(const __grid_constant__ IngestJobs J) {
+    begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     if (!j.k1) return;  // block-uniform
     const int W = j.W, H = j.H, n = j.W * j.H;
@@ -208,6 +213,7 @@ struct FrameSum {
 // Sums of both frames (after equalisation when lut is set) per block, over rows blockIdx.x, + gridDim.x, ...
 // (blockIdx.z = job).  What bounds it: the frames' reads; 1280x720 with equalisation 56 -> 21 us, of which FP64 took 38.
 __global__ void __launch_bounds__(1024) k_frame_sums(const __grid_constant__ IngestJobs J) {
+    begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     const void* f1 = j.f1;
     const void* f2 = j.f2;
@@ -317,6 +323,7 @@ __device__ __forceinline__ void store_pix(void* base, int i, float r, float g, f
 
 template <int ST>
 __global__ void k_pack(const __grid_constant__ IngestJobs J, int gain_enable) {
+    begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     const void* f1 = j.f1;
     const void* f2 = j.f2;
@@ -700,6 +707,7 @@ __device__ __forceinline__ void patch_sum_pair_in(const LanePatch<R>& l1, const 
 
 template <int R, int ST, bool CENSUS>
 __global__ void __launch_bounds__(256) k_pm_init(const __grid_constant__ Batch bt, uint32_t k0, uint32_t k1) {
+    begin_long_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const int lane = threadIdx.x & 31;
@@ -759,6 +767,7 @@ __global__ void __launch_bounds__(256) k_pm_init(const __grid_constant__ Batch b
 // ---------------------------------------------------------------- recost (level >= 1)
 template <int R, int ST>
 __global__ void __launch_bounds__(256) k_pm_recost(const __grid_constant__ Batch bt, int level) {
+    begin_long_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int dir = blockIdx.y;
@@ -917,6 +926,7 @@ __device__ __forceinline__ bool patch_sums(const LanePatch<R>& lp, int lane, flo
 template <int R, int ST, bool PLANES, bool CENSUS>
 __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Batch bt, int level, int it, int phase, uint32_t k0,
                                                   uint32_t k1) {
+    begin_long_kernel();
     static_assert(!(PLANES && CENSUS), "the census data term is for square patches");
     static_assert(PLANES || CENSUS, "level 0 with colour patches runs k_pm_sweep0");
     __shared__ PairView spv;
@@ -1230,6 +1240,7 @@ __device__ __forceinline__ void eval_listed(const SquarePatch<R>& sp, const void
 template <int R, int ST>
 __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Batch bt, int it, int phase, int rows,
                                                       uint32_t k0, uint32_t k1) {
+    begin_long_kernel();
     using TL = Tile0L<R>;
     using Tex = typename TexelOf<ST>::type;
     __shared__ Tex stile[TL::TH * TL::TW];
@@ -1400,9 +1411,11 @@ __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Ba
 // Unfrozen pixels of each colour, for the restricted sweeps (order is free:
 // pixels of one colour are independent within a half-iteration).
 __global__ void k_lists_zero(const __grid_constant__ Batch bt) {
+    begin_kernel();
     if (threadIdx.x < 4) bt.view(blockIdx.z).list_count[threadIdx.x] = 0;
 }
 __global__ void k_build_lists(const __grid_constant__ Batch bt) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const int n = pv.n, W = pv.W;
@@ -1435,21 +1448,21 @@ static void launch_pm_r(const PmLaunch& L, cudaStream_t st) {
     switch (L.op) {
         case PmLaunch::INIT:  // census codes do not depend on the texel storage: one instance serves all
             if (L.census)
-                k_pm_init<R, 0, true><<<grid, block, 0, st>>>(L.bt, L.k0, L.k1);
+                launch_kernel(k_pm_init<R, 0, true>, grid, block, 0, st, L.bt, L.k0, L.k1);
             else
-                k_pm_init<R, ST, false><<<grid, block, 0, st>>>(L.bt, L.k0, L.k1);
+                launch_kernel(k_pm_init<R, ST, false>, grid, block, 0, st, L.bt, L.k0, L.k1);
             break;
         case PmLaunch::RECOST:
-            k_pm_recost<R, ST><<<grid, block, 0, st>>>(L.bt, L.level);
+            launch_kernel(k_pm_recost<R, ST>, grid, block, 0, st, L.bt, L.level);
             break;
         case PmLaunch::SWEEP:
             if (L.level == 0 && L.census)
-                k_pm_sweep<R, 0, false, true><<<grid, block, 0, st>>>(L.bt, 0, L.it, L.phase, L.k0, L.k1);
+                launch_kernel(k_pm_sweep<R, 0, false, true>, grid, block, 0, st, L.bt, 0, L.it, L.phase, L.k0, L.k1);
             else if (L.level == 0)
-                k_pm_sweep0<R, ST><<<dim3(L.tiles0, 2, L.np), dim3(32 * Tile0L<R>::WARPS), 0, st>>>(L.bt, L.it, L.phase, L.rows0,
+                launch_kernel(k_pm_sweep0<R, ST>, dim3(L.tiles0, 2, L.np), dim3(32 * Tile0L<R>::WARPS), 0, st, L.bt, L.it, L.phase, L.rows0,
                                                                                                   L.k0, L.k1);
             else
-                k_pm_sweep<R, ST, true, false><<<grid, block, 0, st>>>(L.bt, L.level, L.it, L.phase, L.k0, L.k1);
+                launch_kernel(k_pm_sweep<R, ST, true, false>, grid, block, 0, st, L.bt, L.level, L.it, L.phase, L.k0, L.k1);
             break;
     }
 }
@@ -1475,6 +1488,7 @@ void launch_pm(const PmLaunch& L, cudaStream_t st) {
 
 // Greys of frame 1 as given, for the edge-aware fill (the jobs that ask for them).
 __global__ void k_grey_q(const __grid_constant__ IngestJobs J) {
+    begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     if (!j.gq) return;
     const int W = j.W, n = j.W * j.H;
@@ -1500,20 +1514,20 @@ void launch_ingest_jobs(const IngestJobs& J, int nj, int max_n, int max_h, int g
         grey |= J.j[k].gq != nullptr;
     }
     if (census) {
-        k_grey_keys<<<dim3(blocks, 2, nj), 256, 0, st>>>(J);
-        k_census<<<dim3(blocks, 2, nj), 256, 0, st>>>(J);
+        launch_kernel(k_grey_keys, dim3(blocks, 2, nj), 256, 0, st, J);
+        launch_kernel(k_census, dim3(blocks, 2, nj), 256, 0, st, J);
     }
-    if (grey) k_grey_q<<<dim3(blocks, 1, nj), 256, 0, st>>>(J);
+    if (grey) launch_kernel(k_grey_q, dim3(blocks, 1, nj), 256, 0, st, J);
     if (eq) {
-        k_vhist_zero<<<dim3(1, 1, nj), 256, 0, st>>>(J);
-        k_vhist<<<dim3(blocks, 2, nj), 256, 0, st>>>(J);
-        k_vlut<<<dim3(2, 1, nj), 256, 0, st>>>(J);
+        launch_kernel(k_vhist_zero, dim3(1, 1, nj), 256, 0, st, J);
+        launch_kernel(k_vhist, dim3(blocks, 2, nj), 256, 0, st, J);
+        launch_kernel(k_vlut, dim3(2, 1, nj), 256, 0, st, J);
     }
-    k_frame_sums<<<dim3(kIngestPartialBlocks, 1, nj), 1024, 0, st>>>(J);
+    launch_kernel(k_frame_sums, dim3(kIngestPartialBlocks, 1, nj), 1024, 0, st, J);
     switch (storage) {
-        case 0: k_pack<0><<<dim3(blocks, 1, nj), 256, 0, st>>>(J, gain_enable); break;
-        case 1: k_pack<1><<<dim3(blocks, 1, nj), 256, 0, st>>>(J, gain_enable); break;
-        case 2: k_pack<2><<<dim3(blocks, 1, nj), 256, 0, st>>>(J, gain_enable); break;
+        case 0: launch_kernel(k_pack<0>, dim3(blocks, 1, nj), 256, 0, st, J, gain_enable); break;
+        case 1: launch_kernel(k_pack<1>, dim3(blocks, 1, nj), 256, 0, st, J, gain_enable); break;
+        case 2: launch_kernel(k_pack<2>, dim3(blocks, 1, nj), 256, 0, st, J, gain_enable); break;
     }
 }
 
@@ -1530,6 +1544,7 @@ void launch_ingest(const float* f1, const float* f2, int W, int H, int64_t strid
 // clamped coordinates (T: one texel, 16 or 8 bytes).
 template <typename T>
 __global__ void k_pad_frames(const __grid_constant__ Batch bt) {
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const T* src = reinterpret_cast<const T*>(pv.img[dir]);
@@ -1549,6 +1564,7 @@ __global__ void k_pad_frames(const __grid_constant__ Batch bt) {
 // (at most 16 FP32 roundings per sum, which the sweep's test allows for).
 template <int R, int ST>
 __global__ void __launch_bounds__(256) k_box_sums(const __grid_constant__ Batch bt) {
+    begin_kernel();
     constexpr int BX = 32, BY = 8, TWB = BX + 2 * R, THB = BY + 2 * R;
     __shared__ float3 tex[THB][TWB];
     __shared__ float3 hs[THB][BX];
@@ -1606,10 +1622,10 @@ __global__ void __launch_bounds__(256) k_box_sums(const __grid_constant__ Batch 
 template <int ST>
 static void launch_box_st(const Batch& bt, dim3 grid, int radius, cudaStream_t st) {
     switch (radius) {
-        case 1: k_box_sums<1, ST><<<grid, 256, 0, st>>>(bt); break;
-        case 2: k_box_sums<2, ST><<<grid, 256, 0, st>>>(bt); break;
-        case 3: k_box_sums<3, ST><<<grid, 256, 0, st>>>(bt); break;
-        case 4: k_box_sums<4, ST><<<grid, 256, 0, st>>>(bt); break;
+        case 1: launch_kernel(k_box_sums<1, ST>, grid, 256, 0, st, bt); break;
+        case 2: launch_kernel(k_box_sums<2, ST>, grid, 256, 0, st, bt); break;
+        case 3: launch_kernel(k_box_sums<3, ST>, grid, 256, 0, st, bt); break;
+        case 4: launch_kernel(k_box_sums<4, ST>, grid, 256, 0, st, bt); break;
     }
 }
 void launch_box_sums(const Batch& bt, int np, int max_w, int max_h, int radius, int storage, cudaStream_t st) {
@@ -1628,6 +1644,7 @@ void launch_box_sums(const Batch& bt, int np, int max_w, int max_h, int radius, 
 // 1024x436, both frames: 0.04 ms, for 60 % of the plane sweeps' evaluations.
 template <int R, int ST>
 __global__ void __launch_bounds__(256) k_interval_sums(const __grid_constant__ Batch bt) {
+    begin_kernel();
     constexpr int BX = 32, BY = 8, MW = BX + 2 * R, MH = BY + 2 * R, TWI = MW + 2, THI = MH + 2;
     __shared__ float3 tex[THI][TWI];
     __shared__ float3 mn[MH][MW], mx[MH][MW];
@@ -1709,10 +1726,10 @@ __global__ void __launch_bounds__(256) k_interval_sums(const __grid_constant__ B
 template <int ST>
 static void launch_interval_st(const Batch& bt, dim3 grid, int radius, cudaStream_t st) {
     switch (radius) {
-        case 1: k_interval_sums<1, ST><<<grid, 256, 0, st>>>(bt); break;
-        case 2: k_interval_sums<2, ST><<<grid, 256, 0, st>>>(bt); break;
-        case 3: k_interval_sums<3, ST><<<grid, 256, 0, st>>>(bt); break;
-        case 4: k_interval_sums<4, ST><<<grid, 256, 0, st>>>(bt); break;
+        case 1: launch_kernel(k_interval_sums<1, ST>, grid, 256, 0, st, bt); break;
+        case 2: launch_kernel(k_interval_sums<2, ST>, grid, 256, 0, st, bt); break;
+        case 3: launch_kernel(k_interval_sums<3, ST>, grid, 256, 0, st, bt); break;
+        case 4: launch_kernel(k_interval_sums<4, ST>, grid, 256, 0, st, bt); break;
     }
 }
 void launch_interval_sums(const Batch& bt, int np, int max_w, int max_h, int radius, int storage, cudaStream_t st) {
@@ -1726,24 +1743,25 @@ void launch_interval_sums(const Batch& bt, int np, int max_w, int max_h, int rad
 
 void launch_pad_frames(const Batch& bt, int np, int storage, int grid_blocks, cudaStream_t st) {
     if (storage == 0)
-        k_pad_frames<uint4><<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt);
+        launch_kernel(k_pad_frames<uint4>, dim3(grid_blocks, 2, np), 256, 0, st, bt);
     else
-        k_pad_frames<uint2><<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt);
+        launch_kernel(k_pad_frames<uint2>, dim3(grid_blocks, 2, np), 256, 0, st, bt);
 }
 
 void launch_build_lists(const Batch& bt, int np, int grid_blocks, cudaStream_t st) {
-    k_lists_zero<<<dim3(1, 1, np), 32, 0, st>>>(bt);
-    k_build_lists<<<dim3(grid_blocks, 2, np), 256, 0, st>>>(bt);
+    launch_kernel(k_lists_zero, dim3(1, 1, np), 32, 0, st, bt);
+    launch_kernel(k_build_lists, dim3(grid_blocks, 2, np), 256, 0, st, bt);
 }
 
 // Exported patch costs: the raw sums divided by 3T (the same division, so the same bits, as a mean taken
 // at evaluation time).
 __global__ void k_cost_export(const float* src, float* dst, int n, float scale) {
+    begin_kernel();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i] / scale;
 }
 void launch_cost_export(const float* src, float* dst, int n, int radius, int census, cudaStream_t st) {
     const int d = 2 * radius + 1;
-    k_cost_export<<<(n + 255) / 256, 256, 0, st>>>(src, dst, n, (float)((census ? 24 : 3) * d * d));
+    launch_kernel(k_cost_export, (n + 255) / 256, 256, 0, st, src, dst, n, (float)((census ? 24 : 3) * d * d));
 }
 
 
