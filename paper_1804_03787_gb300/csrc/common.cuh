@@ -10,16 +10,11 @@
 
 namespace gpm {
 
-// First statement of every kernel started by launch_kernel, before any global access and on every thread: lets the next
-// kernel's blocks take their places, then waits until the kernels before this one are complete and their writes visible.
-__device__ __forceinline__ void begin_kernel() {
-    cudaTriggerProgrammaticLaunchCompletion();
-    cudaGridDependencySynchronize();
-}
-// The same for the kernels that do the main work: the next one's blocks take their places only when all of these are
-// done.  Earlier they take slots and bandwidth from the last of these and, while the refit solve ends on a few warps, from
-// the other streams (letting them: 253x187 4.53 ms instead of 4.24, the batch on two streams 37.6 instead of 37.2).
-__device__ __forceinline__ void begin_long_kernel() { cudaGridDependencySynchronize(); }
+// First statement of every kernel started by launch_kernel, before any global access and on every thread: waits until the
+// kernels before this one are complete and their writes visible.  No kernel lets the next one's blocks in before it ends:
+// they take slots and bandwidth from its last blocks and from other streams (let in early by every kernel 253x187 took
+// 4.53 ms, by the short ones alone 4.24, by none 4.08).
+__device__ __forceinline__ void begin_kernel() { cudaGridDependencySynchronize(); }
 
 constexpr int kMaxCell = 96;  // largest window side (its matches fill 144 KiB of shared memory in RANSAC)
 // Border of the padded frame copies read by the level-0 PatchMatch: the

@@ -1765,7 +1765,7 @@ __device__ __forceinline__ void refit_record(RefitWork* rw, const LevelGeom& g, 
 // integer ones, the smallest eigenvector of A^T A started from the winner,
 // denormalisation, and the geometry checks of the winner and of the refit.
 __global__ void __launch_bounds__(32) k_refit_solve(const __grid_constant__ Batch bt, int level, PlaneParams pp) {
-    begin_long_kernel();
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     __shared__ EigShared sh;
@@ -1910,7 +1910,7 @@ constexpr int kRansacWarps = 4;
 template <int CAP>
 __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     k_ransac_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
-    begin_long_kernel();
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     __shared__ __align__(16) float planes[kRansacWarps][4 * CAP];
@@ -1933,7 +1933,7 @@ __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
-    begin_long_kernel();
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     __shared__ float4 match[8][256];
@@ -1948,7 +1948,7 @@ __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constan
 __host__ __device__ constexpr int block_cap(int s) { return (s * s + 127) / 128 * 128; }
 __global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__ Batch bt, int level, int stage,
                                                          PlaneParams pp) {
-    begin_long_kernel();
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int cell = blockIdx.x, dir = blockIdx.y;
@@ -1973,7 +1973,7 @@ __global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
-    begin_long_kernel();
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     if ((int)blockIdx.x >= g.ncells()) return;  // past this pair's windows (block-uniform)
@@ -2287,7 +2287,7 @@ __device__ __forceinline__ long long seed_step(int q, int before) { return 256 +
 // Rows, a warp each: left to right, then right to left, 32 pixels at a time (their steps' prefix sums, then the
 // offers' prefix minima, by shuffles; the last pixel's offer goes on to the next 32).
 __global__ void __launch_bounds__(128) k_seed_rows(const __grid_constant__ Batch bt) {
-    begin_long_kernel();
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int W = pv.W, y = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (y >= pv.H) return;
@@ -2339,7 +2339,7 @@ __global__ void __launch_bounds__(128) k_seed_rows(const __grid_constant__ Batch
 // lane a column: it walks its section for the steps' sum and the offer at its end, adds up the sections before it, and walks
 // it again with that offer.
 __global__ void __launch_bounds__(1024) k_seed_columns(const __grid_constant__ Batch bt) {
-    begin_long_kernel();
+    begin_kernel();
     constexpr int U = 8;  // rows loaded together
     const PairView& pv = bt.view(blockIdx.z);
     const int W = pv.W, H = pv.H, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

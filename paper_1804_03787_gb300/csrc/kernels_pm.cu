@@ -707,7 +707,7 @@ __device__ __forceinline__ void patch_sum_pair_in(const LanePatch<R>& l1, const 
 
 template <int R, int ST, bool CENSUS>
 __global__ void __launch_bounds__(256) k_pm_init(const __grid_constant__ Batch bt, uint32_t k0, uint32_t k1) {
-    begin_long_kernel();
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const int dir = blockIdx.y;
     const int lane = threadIdx.x & 31;
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(256) k_pm_init(const __grid_constant__ Batch b
 // ---------------------------------------------------------------- recost (level >= 1)
 template <int R, int ST>
 __global__ void __launch_bounds__(256) k_pm_recost(const __grid_constant__ Batch bt, int level) {
-    begin_long_kernel();
+    begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int dir = blockIdx.y;
@@ -926,7 +926,7 @@ __device__ __forceinline__ bool patch_sums(const LanePatch<R>& lp, int lane, flo
 template <int R, int ST, bool PLANES, bool CENSUS>
 __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Batch bt, int level, int it, int phase, uint32_t k0,
                                                   uint32_t k1) {
-    begin_long_kernel();
+    begin_kernel();
     static_assert(!(PLANES && CENSUS), "the census data term is for square patches");
     static_assert(PLANES || CENSUS, "level 0 with colour patches runs k_pm_sweep0");
     __shared__ PairView spv;
@@ -1240,7 +1240,7 @@ __device__ __forceinline__ void eval_listed(const SquarePatch<R>& sp, const void
 template <int R, int ST>
 __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Batch bt, int it, int phase, int rows,
                                                       uint32_t k0, uint32_t k1) {
-    begin_long_kernel();
+    begin_kernel();
     using TL = Tile0L<R>;
     using Tex = typename TexelOf<ST>::type;
     __shared__ Tex stile[TL::TH * TL::TW];
