@@ -305,10 +305,10 @@ gpm_status set_dims(gpm_ctx* c, Slot& s, int W, int H) {
     return cuda_check(c, "set_dims");
 }
 
-// Restricted-sweep lists of pairs [first, first + np).
-void build_lists(gpm_ctx* c, int first, int np, int max_n) {
-    pbeg(c, GPM_PROF_LISTS, 2 * batches(np));
-    each_batch(c, first, np, [&](const Batch& b, int nb) { launch_build_lists(b, nb, grid_for(c, max_n), c->stream); });
+// Restricted-sweep lists of pairs [first, first + np); cleared: launch_merge_update has cleared their counts.
+void build_lists(gpm_ctx* c, int first, int np, int max_n, bool cleared = false) {
+    pbeg(c, GPM_PROF_LISTS, (cleared ? 1 : 2) * batches(np));
+    each_batch(c, first, np, [&](const Batch& b, int nb) { launch_build_lists(b, nb, cleared, grid_for(c, max_n), c->stream); });
     pend(c);
 }
 
@@ -362,40 +362,34 @@ void fit_level(gpm_ctx* c, const Dims& D, int level) {
     pbeg(c, GPM_PROF_RANSAC, 3 * nb);
     each([&](const Batch& b, int n) { launch_ransac(b, n, level, s, mc, 1, pp, st); });
     pend(c);
-    pbeg(c, GPM_PROF_ASSIGN, nb);
-    each([&](const Batch& b, int n) { launch_assign(b, n, level, 1, 0, 0, pp, gb, st); });
-    pend(c);
-    pbeg(c, GPM_PROF_CUES, 3 * nb);
-    each([&](const Batch& b, int n) { launch_cues(b, n, level, mc, 1, 0, pp, gb, st); });
-    pend(c);
-    pbeg(c, GPM_PROF_ASSIGN, nb);
-    each([&](const Batch& b, int n) { launch_assign(b, n, level, 1, 1, 1, pp, gb, st); });
-    pend(c);
+    auto assign = [&](int stage, int again) {
+        pbeg(c, GPM_PROF_ASSIGN, nb);
+        each([&](const Batch& b, int n) { launch_assign(b, n, level, stage, again, pp, gb, st); });
+        pend(c);
+    };
+    auto cues = [&](int stage, int which) {
+        pbeg(c, GPM_PROF_CUES, 2 * nb);
+        each([&](const Batch& b, int n) { launch_cues(b, n, level, mc, stage, which, pp, gb, st); });
+        pend(c);
+    };
+    assign(1, 0);
+    cues(1, 0);
+    assign(1, 1);
     // second stage on the residual pixels
     pbeg(c, GPM_PROF_RANSAC, 3 * nb);
     each([&](const Batch& b, int n) { launch_ransac(b, n, level, s, mc, 2, pp, st); });
     pend(c);
-    for (int pass = 0; pass < 2; ++pass) {  // assignment, cues, then the assignment after the cues
-        pbeg(c, GPM_PROF_ASSIGN, 2 * nb);
-        each([&](const Batch& b, int n) {
-            launch_copy_labels(b, n, 2, 3, gb, st);
-            launch_assign(b, n, level, 2, 2, 0, pp, gb, st);
-        });
-        pend(c);
-        if (pass == 0) {
-            pbeg(c, GPM_PROF_CUES, 3 * nb);
-            each([&](const Batch& b, int n) { launch_cues(b, n, level, mc, 2, 2, pp, gb, st); });
-            pend(c);
-        }
-    }
+    assign(2, 0);
+    cues(2, 2);
+    assign(2, 1);
     // many-to-one, merge, NNF update, lists for the restricted sweeps
-    pbeg(c, GPM_PROF_MANY_TO_ONE, 3 * nb);
+    pbeg(c, GPM_PROF_MANY_TO_ONE, 2 * nb);
     each([&](const Batch& b, int n) { launch_many_to_one(b, n, pp, gb, st); });
     pend(c);
     pbeg(c, GPM_PROF_MERGE, nb);
     each([&](const Batch& b, int n) { launch_merge_update(b, n, pp, gb, st); });
     pend(c);
-    build_lists(c, 0, np, D.max_n);
+    build_lists(c, 0, np, D.max_n, true);
 }
 
 }  // namespace

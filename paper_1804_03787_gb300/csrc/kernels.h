@@ -82,8 +82,8 @@ void launch_pad_frames(const Batch& bt, int np, int storage, int grid_blocks, cu
 void launch_box_sums(const Batch& bt, int np, int max_w, int max_h, int radius, int storage, cudaStream_t st);
 // Interval sums of both ingested frames (into pv.box, after the level-0 sweeps): the plane sweeps' lower bound.
 void launch_interval_sums(const Batch& bt, int np, int max_w, int max_h, int radius, int storage, cudaStream_t st);
-// The unfrozen pixels of each colour (the restricted sweeps' lists), counts cleared first.
-void launch_build_lists(const Batch& bt, int np, int grid_blocks, cudaStream_t st);
+// The unfrozen pixels of each colour (the restricted sweeps' lists), counts cleared first unless the merge has done so.
+void launch_build_lists(const Batch& bt, int np, bool cleared, int grid_blocks, cudaStream_t st);
 // dst[i] = src[i] / (3 (2 radius + 1)^2), or / 24 (2 radius + 1)^2 for census costs: the NNF cost buffer holds
 // raw tap sums, the export means.
 void launch_cost_export(const float* src, float* dst, int n, int radius, int census, cudaStream_t st);
@@ -99,9 +99,11 @@ struct PlaneParams {
 // RANSAC per window for both directions (blockIdx.y = direction); s: the level's window side.
 void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int stage, const PlaneParams& pp,
                    cudaStream_t st);
-// Assignment by eq. 3-4 into `which` (0 tent, 1 st1, 2 lvl); stage 1 or 2; masked by resid for stage 2.
-void launch_assign(const Batch& bt, int np, int level, int stage, int which, int write_resid, const PlaneParams& pp,
-                   int grid_blocks, cudaStream_t st);
+// Assignment by eq. 3-4: stage 1 into tent, or again (after the cues) into st1 and resid; stage 2 into lvl (pixels of resid,
+// the others from st1), or again there, clearing the many-to-one keys.
+void launch_assign(const Batch& bt, int np, int level, int stage, int again, const PlaneParams& pp, int grid_blocks,
+                   cudaStream_t st);
+// Cue counts (cleared by launch_ransac) and the planes that fail them.
 void launch_cues(const Batch& bt, int np, int level, int max_cells, int stage, int which, const PlaneParams& pp,
                  int grid_blocks, cudaStream_t st);
 void launch_many_to_one(const Batch& bt, int np, const PlaneParams& pp, int grid_blocks, cudaStream_t st);

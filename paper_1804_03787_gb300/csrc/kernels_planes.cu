@@ -1991,23 +1991,62 @@ __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_consta
 // absolute RGB difference between I_src(p) and the bilinear I_tgt(H p); the
 // pixel is an inlier iff delta < eps, and takes the inlier plane with the
 // smallest L = delta (first window on ties), with flow H p - p.
-template <int ST>
-__global__ void k_assign(const __grid_constant__ Batch bt, int level, int stage, int which, int write_resid, PlaneParams pp) {
+//
+// A level assigns four times: the first stage's planes into tent, again into st1 once the cues have discarded some, then the
+// residual stage's on the pixels without one into lvl (the others copied from st1), and again there.  The second
+// assignment of a stage differs from its first only where a window that covers the pixel lost its plane in between,
+// so it is computed there and taken over elsewhere (the winner alone does not tell: without a discarded plane a
+// near tie between two others may fall the other way).
+// What bounds it: the gathers of up to nine windows' models and four texels each.  1024x436, sixteen launches: 0.46 -> 0.38 ms.
+enum AssignMode { ASSIGN_TENT, ASSIGN_ST1, ASSIGN_LVL, ASSIGN_LVL_AGAIN };
+template <int ST, int MODE>
+__global__ void k_assign(const __grid_constant__ Batch bt, int level, PlaneParams pp) {
     begin_kernel();
+    constexpr int stage = MODE <= ASSIGN_ST1 ? 1 : 2;
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int dir = blockIdx.y;
     const int W = pv.W, H = pv.H, n = pv.n;
-    Labels out = which == 0 ? pv.tent[dir] : (which == 1 ? pv.st1[dir] : pv.lvl[dir]);
+    const Labels out = MODE == ASSIGN_TENT ? pv.tent[dir] : (MODE == ASSIGN_ST1 ? pv.st1[dir] : pv.lvl[dir]);
     const void* src = pv.img[dir];
     const void* tgt = pv.img[1 - dir];
     const Mef* mef = pv.mef[dir];
-    const uint8_t* resid = pv.resid[dir];
+    const int* mi = pv.mi[dir];
+    uint8_t* resid = pv.resid[dir];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        if (stage == 2 && !resid[i]) continue;
+        if (MODE == ASSIGN_LVL_AGAIN) pv.m2o_key[dir][i] = ~0ull;  // for the many-to-one test that follows
+        if (MODE == ASSIGN_LVL && !resid[i]) {
+            const Labels in = pv.st1[dir];
+            out.m[i] = in.m[i];
+            out.L[i] = in.L[i];
+            out.v[i] = in.v[i];
+            out.r[i] = in.r[i];
+            continue;
+        }
+        if (MODE == ASSIGN_LVL_AGAIN && !resid[i]) continue;
         const int y = i / W, x = i - y * W;
         int ix3[3], iy3[3];
         const int nxw = covering(g.gx, g.s, g.h, x, ix3), nyw = covering(g.gy, g.s, g.h, y, iy3);
+        if (MODE == ASSIGN_ST1 || MODE == ASSIGN_LVL_AGAIN) {
+            bool lost = false;
+            for (int a = 0; a < nyw; ++a)
+                for (int b = 0; b < nxw; ++b) {
+                    const int id = (g.base + iy3[a] * g.gx.count + ix3[b]) * 2 + (stage - 1);
+                    lost = lost || (mi[(size_t)id * kMI + MI_FLAGS] & (F_BAD_FB | F_BAD_KAPPA)) != 0;
+                }
+            if (!lost) {
+                if (MODE == ASSIGN_ST1) {
+                    const Labels in = pv.tent[dir];
+                    const int m = in.m[i];
+                    out.m[i] = m;
+                    out.L[i] = in.L[i];
+                    out.v[i] = in.v[i];
+                    out.r[i] = in.r[i];
+                    resid[i] = m < 0;
+                }
+                continue;
+            }
+        }
         int bm = -1, bkx = 0, bky = 0;
         float bL = FLT_MAX, bfx = 0.f, bfy = 0.f;
         for (int a = 0; a < nyw; ++a)
@@ -2040,23 +2079,11 @@ __global__ void k_assign(const __grid_constant__ Batch bt, int level, int stage,
         out.L[i] = bm >= 0 ? bL : pp.eps;
         out.v[i] = make_int2(vx, vy);
         out.r[i] = make_float2(rx, ry);
-        if (write_resid) pv.resid[dir][i] = bm < 0;
+        if (MODE == ASSIGN_ST1) resid[i] = bm < 0;
     }
 }
 
 // ---------------------------------------------------------------- occlusion cues (Sec. 3.4)
-__global__ void k_cue_zero(const __grid_constant__ Batch bt, int level, int stage) {
-    begin_kernel();
-    const PairView& pv = bt.view(blockIdx.z);
-    const LevelGeom g = bt.geom(blockIdx.z, level);
-    const int dir = blockIdx.y;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < g.ncells(); c += gridDim.x * blockDim.x) {
-        int* f = pv.mi[dir] + (size_t)((g.base + c) * 2 + stage - 1) * kMI;
-        f[MI_NASSIGN] = 0;
-        f[MI_NSYM] = 0;
-    }
-}
-
 // Forward-backward plane projection symmetry: a pixel assigned to a plane of
 // this level and stage with flow f is symmetric iff q = round(p + f) holds an
 // assigned pixel of the other direction with flow g, |f + g| < t_fb.
@@ -2068,23 +2095,35 @@ __global__ void k_cue_counts(const __grid_constant__ Batch bt, int level, int st
     const int W = pv.W, H = pv.H, n = pv.n;
     const Labels lab = which == 0 ? pv.tent[dir] : pv.lvl[dir];
     const Labels oth = which == 0 ? pv.tent[1 - dir] : pv.lvl[1 - dir];
-    const int lo = g.base * 2, hi = (g.base + g.ncells()) * 2;
+    const int lo = g.base * 2, hi = (g.base + g.ncells()) * 2, lane = threadIdx.x & 31;
     int* mi = pv.mi[dir];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int m = lab.m[i];
-        if (m < lo || m >= hi || (m & 1) != stage - 1) continue;
-        atomicAdd(&mi[(size_t)m * kMI + MI_NASSIGN], 1);
+    // a warp's pixels of one plane count together (its neighbours mostly share it, and their additions one address:
+    // the level's first 32 us, much of it that; the cues of 1024x436, eight launches fewer, 0.16 -> 0.11 ms)
+    for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
+        const int i = i0 + lane;
+        const int m = i < n ? lab.m[i] : -1;
+        const bool counts = m >= lo && m < hi && (m & 1) == stage - 1;
+        const unsigned some = __ballot_sync(0xffffffffu, counts);
+        if (!counts) continue;
+        bool symmetric = false;
         const int y = i / W, x = i - y * W;
         const int2 v = lab.v[i];
         const int qx = x + v.x, qy = y + v.y;
-        if (qx < 0 || qx >= W || qy < 0 || qy >= H) continue;
-        const int j = qy * W + qx;
-        if (oth.m[j] < 0) continue;
-        const int2 w = oth.v[j];
-        const float2 r = lab.r[i], s = oth.r[j];
-        const float ex = (float)(v.x + w.x) + (r.x + s.x);
-        const float ey = (float)(v.y + w.y) + (r.y + s.y);
-        if (ex * ex + ey * ey < pp.fb2) atomicAdd(&mi[(size_t)m * kMI + MI_NSYM], 1);
+        if (qx >= 0 && qx < W && qy >= 0 && qy < H) {
+            const int j = qy * W + qx;
+            if (oth.m[j] >= 0) {
+                const int2 w = oth.v[j];
+                const float2 r = lab.r[i], s = oth.r[j];
+                const float ex = (float)(v.x + w.x) + (r.x + s.x);
+                const float ey = (float)(v.y + w.y) + (r.y + s.y);
+                symmetric = ex * ex + ey * ey < pp.fb2;
+            }
+        }
+        const unsigned same = __match_any_sync(some, m), sym = __ballot_sync(some, symmetric) & same;
+        if (lane == __ffs(same) - 1) {
+            atomicAdd(&mi[(size_t)m * kMI + MI_NASSIGN], __popc(same));
+            if (sym) atomicAdd(&mi[(size_t)m * kMI + MI_NSYM], __popc(sym));
+        }
     }
 }
 
@@ -2115,14 +2154,7 @@ __global__ void k_cue_invalidate(const __grid_constant__ Batch bt, int level, in
 }
 
 // Many-to-one: per target q = round(p + f), the lowest (L, index) keeps it;
-// a loser whose flow differs from the winner's by t_fb or more is occluded.
-__global__ void k_m2o_init(const __grid_constant__ Batch bt) {
-    begin_kernel();
-    const PairView& pv = bt.view(blockIdx.z);
-    const int dir = blockIdx.y;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pv.n; i += gridDim.x * blockDim.x)
-        pv.m2o_key[dir][i] = ~0ull;
-}
+// a loser whose flow differs from the winner's by t_fb or more is occluded.  (The level's last assignment clears the keys.)
 __global__ void k_m2o_claim(const __grid_constant__ Batch bt) {
     begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
@@ -2171,6 +2203,7 @@ __global__ void k_merge_update(const __grid_constant__ Batch bt, PlaneParams pp)
     const int dir = blockIdx.y;
     const int n = pv.n;
     const Labels lab = pv.lvl[dir], acc = pv.acc[dir];
+    if (blockIdx.x == 0 && threadIdx.x < 2) pv.list_count[dir * 2 + threadIdx.x] = 0;  // for the lists that follow
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int m = lab.m[i];
         int am = acc.m[i];
@@ -2560,26 +2593,35 @@ void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int
     }
 }
 
-void launch_assign(const Batch& bt, int np, int level, int stage, int which, int write_resid, const PlaneParams& pp,
-                   int grid_blocks, cudaStream_t st) {
+template <int ST>
+static void launch_assign_st(const Batch& bt, dim3 grid, int level, int stage, int again, const PlaneParams& pp, cudaStream_t st) {
+    if (stage == 1 && !again)
+        launch_kernel(k_assign<ST, ASSIGN_TENT>, grid, 256, 0, st, bt, level, pp);
+    else if (stage == 1)
+        launch_kernel(k_assign<ST, ASSIGN_ST1>, grid, 256, 0, st, bt, level, pp);
+    else if (!again)
+        launch_kernel(k_assign<ST, ASSIGN_LVL>, grid, 256, 0, st, bt, level, pp);
+    else
+        launch_kernel(k_assign<ST, ASSIGN_LVL_AGAIN>, grid, 256, 0, st, bt, level, pp);
+}
+void launch_assign(const Batch& bt, int np, int level, int stage, int again, const PlaneParams& pp, int grid_blocks,
+                   cudaStream_t st) {
     const dim3 grid(grid_blocks, 2, np);
     switch (pp.storage) {
-        case 0: launch_kernel(k_assign<0>, grid, 256, 0, st, bt, level, stage, which, write_resid, pp); break;
-        case 1: launch_kernel(k_assign<1>, grid, 256, 0, st, bt, level, stage, which, write_resid, pp); break;
-        case 2: launch_kernel(k_assign<2>, grid, 256, 0, st, bt, level, stage, which, write_resid, pp); break;
+        case 0: launch_assign_st<0>(bt, grid, level, stage, again, pp, st); break;
+        case 1: launch_assign_st<1>(bt, grid, level, stage, again, pp, st); break;
+        case 2: launch_assign_st<2>(bt, grid, level, stage, again, pp, st); break;
     }
 }
 
 void launch_cues(const Batch& bt, int np, int level, int max_cells, int stage, int which, const PlaneParams& pp,
                  int grid_blocks, cudaStream_t st) {
     const int cb = (max_cells + 255) / 256;
-    launch_kernel(k_cue_zero, dim3(cb, 2, np), 256, 0, st, bt, level, stage);
     launch_kernel(k_cue_counts, dim3(grid_blocks, 2, np), 256, 0, st, bt, level, stage, which, pp);
     launch_kernel(k_cue_invalidate, dim3(cb, 2, np), 256, 0, st, bt, level, stage, pp);
 }
 
 void launch_many_to_one(const Batch& bt, int np, const PlaneParams& pp, int grid_blocks, cudaStream_t st) {
-    launch_kernel(k_m2o_init, dim3(grid_blocks, 2, np), 256, 0, st, bt);
     launch_kernel(k_m2o_claim, dim3(grid_blocks, 2, np), 256, 0, st, bt);
     launch_kernel(k_m2o_resolve, dim3(grid_blocks, 2, np), 256, 0, st, bt, pp);
 }

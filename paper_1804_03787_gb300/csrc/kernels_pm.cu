@@ -1748,8 +1748,8 @@ void launch_pad_frames(const Batch& bt, int np, int storage, int grid_blocks, cu
         launch_kernel(k_pad_frames<uint2>, dim3(grid_blocks, 2, np), 256, 0, st, bt);
 }
 
-void launch_build_lists(const Batch& bt, int np, int grid_blocks, cudaStream_t st) {
-    launch_kernel(k_lists_zero, dim3(1, 1, np), 32, 0, st, bt);
+void launch_build_lists(const Batch& bt, int np, bool cleared, int grid_blocks, cudaStream_t st) {
+    if (!cleared) launch_kernel(k_lists_zero, dim3(1, 1, np), 32, 0, st, bt);
     launch_kernel(k_build_lists, dim3(grid_blocks, 2, np), 256, 0, st, bt);
 }
 
