@@ -2097,8 +2097,8 @@ __global__ void k_cue_counts(const __grid_constant__ Batch bt, int level, int st
     const Labels oth = which == 0 ? pv.tent[1 - dir] : pv.lvl[1 - dir];
     const int lo = g.base * 2, hi = (g.base + g.ncells()) * 2, lane = threadIdx.x & 31;
     int* mi = pv.mi[dir];
-    // a warp's pixels of one plane count together (its neighbours mostly share it, and their additions one address:
-    // the level's first 32 us, much of it that; the cues of 1024x436, eight launches fewer, 0.16 -> 0.11 ms)
+    // a warp's pixels of one plane count together: neighbours mostly share theirs, and one by one their additions queue at
+    // its counters (1024x436: the cues' sixteen launches 0.16 ms with one addition a pixel and eight more launches, 0.11 now)
     for (int i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
         const int i = i0 + lane;
         const int m = i < n ? lab.m[i] : -1;
