@@ -578,7 +578,7 @@ gpm_status gpm_match(gpm_ctx* c, const gpm_pair* pairs, int32_t n_pairs, int32_t
                 mn = std::max(mn, s.n);
                 mh = std::max(mh, s.H);
             }
-            pbeg(c, GPM_PROF_INGEST, (c->P.equalize ? 5 : 2) + (c->P.census ? 2 : 0) + (c->P.interp ? 1 : 0));
+            pbeg(c, GPM_PROF_INGEST, (c->P.equalize ? 4 : 2) + (c->P.census ? 2 : 0) + (c->P.interp ? 1 : 0));
             launch_ingest_jobs(J, nj, mn, mh, c->P.gain_normalize, c->P.storage, c->stream);
             pend(c);
         }

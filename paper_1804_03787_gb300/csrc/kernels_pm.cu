@@ -40,6 +40,24 @@ __device__ __forceinline__ int v_bin(float v) {
     return (int)fminf(x, 255.f);
 }
 
+// Up to four pixels of a row from element e (a multiple of 12 from the row's start), as 12 floats; `wide`: FP32 rows on
+// 16-byte boundaries, so that four whole pixels are three loads.  Elements past `cnt` pixels are 0.
+__device__ __forceinline__ bool wide_rows(const void* f, int dtype, int64_t stride) {
+    return dtype == GPM_F32 && (stride & 3) == 0 && (reinterpret_cast<uintptr_t>(f) & 15) == 0;
+}
+__device__ __forceinline__ void load_px4(const void* f, int dtype, int64_t e, int cnt, bool wide, float (&v)[12]) {
+    if (wide && cnt == 4) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(f) + e) + k);
+            v[4 * k] = a.x, v[4 * k + 1] = a.y, v[4 * k + 2] = a.z, v[4 * k + 3] = a.w;
+        }
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v[k] = k < 3 * cnt ? in_elem(f, dtype, e + k) : 0.f;
+}
+
 // Clears the V histograms of the jobs that equalise (blockIdx.z = job).
 __global__ void k_vhist_zero(const __grid_constant__ IngestJobs J) {
     begin_kernel();
@@ -49,68 +67,58 @@ __global__ void k_vhist_zero(const __grid_constant__ IngestJobs J) {
 }
 
 // V histogram of each frame (blockIdx.y = frame, blockIdx.z = job); hist holds 2 x 256 zeroed counts.
-__global__ void k_vhist(const __grid_constant__ IngestJobs J) {
+__global__ void __launch_bounds__(512) k_vhist(const __grid_constant__ IngestJobs J) {
     begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
     if (!j.hist) return;  // block-uniform
     const int W = j.W, H = j.H;
-    const int64_t stride = j.stride;
-    int* hist = j.hist;
     __shared__ int h[256];
     for (int k = threadIdx.x; k < 256; k += blockDim.x) h[k] = 0;
     __syncthreads();
     const void* f = blockIdx.y ? j.f2 : j.f1;
-    const int n = W * H;
-    const int step = gridDim.x * blockDim.x;
-    for (int i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += 4 * step) {  // four pixels' loads in flight
-        float v[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int i = min(i0 + q * step, n - 1), y = i / W, x = i - y * W;
-            const int64_t e = (int64_t)y * stride + 3 * x;
-            v[q] = fmaxf(in_elem(f, j.dtype, e), fmaxf(in_elem(f, j.dtype, e + 1), in_elem(f, j.dtype, e + 2)));
-        }
+    const bool wide = wide_rows(f, j.dtype, j.stride);
+    const int Q = (W + 3) >> 2, n = Q * H;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int y = i / Q, x = 4 * (i - y * Q), cnt = min(4, W - x);
+        float v[12];
+        load_px4(f, j.dtype, (int64_t)y * j.stride + 3 * x, cnt, wide, v);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (i0 + q * step < n) atomicAdd(&h[v_bin(v[q])], 1);
+            if (q < cnt) atomicAdd(&h[v_bin(fmaxf(v[3 * q], fmaxf(v[3 * q + 1], v[3 * q + 2])))], 1);
     }
     __syncthreads();
     for (int k = threadIdx.x; k < 256; k += blockDim.x)
-        if (h[k]) atomicAdd(&hist[blockIdx.y * 256 + k], h[k]);
+        if (h[k]) atomicAdd(&j.hist[blockIdx.y * 256 + k], h[k]);
 }
 
-// Equalised V per bin (blockIdx.x = frame, blockIdx.z = job, 256 threads): an inclusive scan of the counts.
-__global__ void k_vlut(const __grid_constant__ IngestJobs J) {
-    begin_kernel();
-    const IngestJob& j = J.j[blockIdx.z];
-    if (!j.hist) return;  // block-uniform
-    const int* hist = j.hist;
-    const int n = j.W * j.H;
-    float* lut = j.lut;
-    __shared__ int c[256];
-    __shared__ int cmin, first[8];
-    const int t = threadIdx.x;
-    const int* hf = hist + blockIdx.x * 256;
-    c[t] = hf[t];
-    if (t == 0) cmin = -1;
-    __syncthreads();
-    {
-        const unsigned occupied = __ballot_sync(FULL, c[t] > 0);
-        if ((t & 31) == 0) first[t >> 5] = occupied ? __ffs(occupied) - 1 : -1;
+// Equalised V per bin of both frames, into lut (shared memory), from their counts: an inclusive scan, a frame by 256
+// threads each.  Every thread of the block must call it (at least 512); it ends with a barrier.
+__device__ __forceinline__ void equalized_v(const int* hist, int n, float* lut) {
+    __shared__ int total[16], lowest[16];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int own = 0, sum = 0;
+    if (t < 512) {  // warp-uniform
+        own = sum = hist[t];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(FULL, sum, o);
+            if (lane >= o) sum += v;
+        }
+        const unsigned occupied = __ballot_sync(FULL, own > 0);
+        const int low = __shfl_sync(FULL, own, occupied ? __ffs(occupied) - 1 : 0);  // 0 if none
+        if (lane == 31) total[warp] = sum, lowest[warp] = low;
     }
     __syncthreads();
-    if (t == 0)
-        for (int b = 0; b < 8 && cmin < 0; ++b)
-            if (first[b] >= 0) cmin = c[32 * b + first[b]];
-    __syncthreads();
-    for (int off = 1; off < 256; off <<= 1) {
-        const int v = t >= off ? c[t - off] : 0;
-        __syncthreads();
-        c[t] += v;
-        __syncthreads();
+    if (t < 512) {
+        int cmin = 0;  // the count of the lowest occupied bin
+        for (int b = (warp & 8) + 7; b >= (warp & 8); --b) {
+            if (b < warp) sum += total[b];
+            if (lowest[b] > 0) cmin = lowest[b];
+        }
+        // counts below 2^24 are exact floats, so this is the correctly rounded quotient
+        lut[t] = cmin == 0 || cmin == n ? -1.f : (float)(sum - cmin) / (float)(n - cmin);
     }
-    // counts below 2^24 are exact floats, so this is the correctly rounded quotient
-    lut[blockIdx.x * 256 + t] = (cmin < 0 || cmin == n) ? -1.f : (float)(c[t] - cmin) / (float)(n - cmin);
+    __syncthreads();
 }
 
 __device__ __forceinline__ float3 equalize_px(float r, float g, float b, const float* lut) {
@@ -175,6 +183,25 @@ __global__ void k_census(const __grid_constant__ IngestJobs J) {
     }
 }
 
+template <int ST>
+__device__ __forceinline__ void store_pix(void* base, int i, float r, float g, float b) {
+    if constexpr (ST == 0) {
+        reinterpret_cast<float4*>(base)[i] = make_float4(r, g, b, 0.f);
+    } else if constexpr (ST == 1) {
+        __half2 lo = __floats2half2_rn(r, g), hi = __floats2half2_rn(b, 0.f);
+        uint2 u;
+        u.x = *reinterpret_cast<uint32_t*>(&lo);
+        u.y = *reinterpret_cast<uint32_t*>(&hi);
+        reinterpret_cast<uint2*>(base)[i] = u;
+    } else {
+        __nv_bfloat162 lo = __floats2bfloat162_rn(r, g), hi = __floats2bfloat162_rn(b, 0.f);
+        uint2 u;
+        u.x = *reinterpret_cast<uint32_t*>(&lo);
+        u.y = *reinterpret_cast<uint32_t*>(&hi);
+        reinterpret_cast<uint2*>(base)[i] = u;
+    }
+}
+
 // A sum of floats: those in [2^-16, 2) as exact integers of 2^-40 (a block adds at most 2^21 of them, below 2^62), the
 // others in FP64.  An FP64 addition and the conversion before it take the FP64 pipe, 64 cycles each a warp instruction on
 // GB300; the integers take ten of one cycle.
@@ -210,47 +237,48 @@ struct FrameSum {
     }
 };
 
-// Sums of both frames (after equalisation when lut is set) per block, over rows blockIdx.x, + gridDim.x, ...
-// (blockIdx.z = job).  What bounds it: the frames' reads; 1280x720 with equalisation 56 -> 21 us, of which FP64 took 38.
+// Sums of both frames (equalised where the job asks for it) per block, over rows blockIdx.x, + gridDim.x, ...
+// (blockIdx.z = job), and frame 1 stored, which needs no gain.  What bounds it: the FP32 and integer pipes (a pixel pair with
+// equalisation takes 150 instructions).  1280x720 with equalisation: sums and table 60 us with FP64 additions, 25 with
+// integers and the table in a launch of its own, 17 now with frame 1's half of k_pack besides.
+template <int ST>
 __global__ void __launch_bounds__(1024) k_frame_sums(const __grid_constant__ IngestJobs J) {
     begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
-    const void* f1 = j.f1;
-    const void* f2 = j.f2;
-    const int dt = j.dtype;
     const int W = j.W, H = j.H;
-    const int64_t stride = j.stride;
-    const float* lut = j.hist ? j.lut : nullptr;
-    double* partial = j.partial;
     __shared__ long long sf[2][32];
     __shared__ double sr[2][32];
-    FrameSum a, b;
-    // the block's rows as one sequence of pixels (or elements), so that short rows leave no thread idle
-    const int rows = (H - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // at most 0 past the last row
-    if (lut) {
-#pragma unroll 2
-        for (int i = threadIdx.x; i < rows * W; i += blockDim.x) {
-            const int y = i / W, x = i - y * W;
-            const int64_t e = (int64_t)(blockIdx.x + y * gridDim.x) * stride + 3 * x;
-            const float3 p = equalize_px(in_elem(f1, dt, e), in_elem(f1, dt, e + 1), in_elem(f1, dt, e + 2), lut);
-            const float3 q = equalize_px(in_elem(f2, dt, e), in_elem(f2, dt, e + 1), in_elem(f2, dt, e + 2), lut + 256);
-            a.add(p.x), a.add(p.y), a.add(p.z);
-            b.add(q.x), b.add(q.y), b.add(q.z);
-        }
-    } else {
-        const int W3 = 3 * W;
-#pragma unroll 4
-        for (int i = threadIdx.x; i < rows * W3; i += blockDim.x) {
-            const int y = i / W3, x = i - y * W3;
-            const int64_t e = (int64_t)(blockIdx.x + y * gridDim.x) * stride + x;
-            a.add(in_elem(f1, dt, e));
-            b.add(in_elem(f2, dt, e));
-        }
+    __shared__ float lut[512];
+    if (j.hist) {  // block-uniform
+        equalized_v(j.hist, W * H, lut);
+        if (blockIdx.x == 0 && threadIdx.x < 512) j.lut[threadIdx.x] = lut[threadIdx.x];
     }
-    const double ta = a.total(sf[0], sr[0]), tb = b.total(sf[1], sr[1]);
+    FrameSum sum[2];
+    // the block's rows as one sequence of four-pixel groups, so that short rows leave no thread idle
+    const int rows = (H - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // at most 0 past the last row
+    const int Q = (W + 3) >> 2;
+    const bool wide = wide_rows(j.f1, j.dtype, j.stride) && wide_rows(j.f2, j.dtype, j.stride);
+    for (int i = threadIdx.x; i < rows * Q; i += blockDim.x) {
+        const int r = i / Q, x = 4 * (i - r * Q), y = blockIdx.x + r * gridDim.x, cnt = min(4, W - x);
+        const int64_t e = (int64_t)y * j.stride + 3 * x;
+        float v[2][12];
+        load_px4(j.f1, j.dtype, e, cnt, wide, v[0]);
+        load_px4(j.f2, j.dtype, e, cnt, wide, v[1]);
+#pragma unroll
+        for (int f = 0; f < 2; ++f)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (q >= cnt) break;
+                float3 p = make_float3(v[f][3 * q], v[f][3 * q + 1], v[f][3 * q + 2]);
+                if (j.hist) p = equalize_px(p.x, p.y, p.z, lut + 256 * f);
+                sum[f].add(p.x), sum[f].add(p.y), sum[f].add(p.z);
+                if (f == 0) store_pix<ST>(j.o1, y * W + x + q, p.x, p.y, p.z);
+            }
+    }
+    const double ta = sum[0].total(sf[0], sr[0]), tb = sum[1].total(sf[1], sr[1]);
     if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = ta;
-        partial[2 * blockIdx.x + 1] = tb;
+        j.partial[2 * blockIdx.x] = ta;
+        j.partial[2 * blockIdx.x + 1] = tb;
     }
 }
 
@@ -302,50 +330,21 @@ struct Gain {
     }
 };
 
-template <int ST>
-__device__ __forceinline__ void store_pix(void* base, int i, float r, float g, float b) {
-    if constexpr (ST == 0) {
-        reinterpret_cast<float4*>(base)[i] = make_float4(r, g, b, 0.f);
-    } else if constexpr (ST == 1) {
-        __half2 lo = __floats2half2_rn(r, g), hi = __floats2half2_rn(b, 0.f);
-        uint2 u;
-        u.x = *reinterpret_cast<uint32_t*>(&lo);
-        u.y = *reinterpret_cast<uint32_t*>(&hi);
-        reinterpret_cast<uint2*>(base)[i] = u;
-    } else {
-        __nv_bfloat162 lo = __floats2bfloat162_rn(r, g), hi = __floats2bfloat162_rn(b, 0.f);
-        uint2 u;
-        u.x = *reinterpret_cast<uint32_t*>(&lo);
-        u.y = *reinterpret_cast<uint32_t*>(&hi);
-        reinterpret_cast<uint2*>(base)[i] = u;
-    }
-}
-
+// Frame 2 stored, equalised where the job asks for it and times the gain (blockIdx.z = job).
 template <int ST>
 __global__ void k_pack(const __grid_constant__ IngestJobs J, int gain_enable) {
     begin_kernel();
     const IngestJob& j = J.j[blockIdx.z];
-    const void* f1 = j.f1;
-    const void* f2 = j.f2;
-    const int dt = j.dtype;
     const int W = j.W, H = j.H;
-    const int64_t stride = j.stride;
-    const float* lut = j.hist ? j.lut : nullptr;
-    void* o1 = j.o1;
-    void* o2 = j.o2;
+    const float* lut = j.hist ? j.lut + 256 : nullptr;
     const Gain g(frame_gain(j.partial, gain_enable));
     const int n = W * H;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int y = i / W, x = i - y * W;
-        const int64_t e = (int64_t)y * stride + 3 * x;
-        float3 p = make_float3(in_elem(f1, dt, e), in_elem(f1, dt, e + 1), in_elem(f1, dt, e + 2));
-        float3 q = make_float3(in_elem(f2, dt, e), in_elem(f2, dt, e + 1), in_elem(f2, dt, e + 2));
-        if (lut) {
-            p = equalize_px(p.x, p.y, p.z, lut);
-            q = equalize_px(q.x, q.y, q.z, lut + 256);
-        }
-        store_pix<ST>(o1, i, p.x, p.y, p.z);
-        store_pix<ST>(o2, i, g.times(q.x), g.times(q.y), g.times(q.z));
+        const int64_t e = (int64_t)y * j.stride + 3 * x;
+        float3 q = make_float3(in_elem(j.f2, j.dtype, e), in_elem(j.f2, j.dtype, e + 1), in_elem(j.f2, j.dtype, e + 2));
+        if (lut) q = equalize_px(q.x, q.y, q.z, lut);
+        store_pix<ST>(j.o2, i, g.times(q.x), g.times(q.y), g.times(q.z));
     }
 }
 
@@ -1476,14 +1475,22 @@ void launch_ingest_jobs(const IngestJobs& J, int nj, int max_n, int max_h, int g
     if (grey) launch_kernel(k_grey_q, dim3(blocks, 1, nj), 256, 0, st, J);
     if (eq) {
         launch_kernel(k_vhist_zero, dim3(1, 1, nj), 256, 0, st, J);
-        launch_kernel(k_vhist, dim3(blocks, 2, nj), 256, 0, st, J);
-        launch_kernel(k_vlut, dim3(2, 1, nj), 256, 0, st, J);
+        launch_kernel(k_vhist, dim3(152, 2, nj), 512, 0, st, J);
     }
-    launch_kernel(k_frame_sums, dim3(kIngestPartialBlocks, 1, nj), 1024, 0, st, J);
+    const dim3 sums(kIngestPartialBlocks, 1, nj), pack(blocks, 1, nj);
     switch (storage) {
-        case 0: launch_kernel(k_pack<0>, dim3(blocks, 1, nj), 256, 0, st, J, gain_enable); break;
-        case 1: launch_kernel(k_pack<1>, dim3(blocks, 1, nj), 256, 0, st, J, gain_enable); break;
-        case 2: launch_kernel(k_pack<2>, dim3(blocks, 1, nj), 256, 0, st, J, gain_enable); break;
+        case 0:
+            launch_kernel(k_frame_sums<0>, sums, 1024, 0, st, J);
+            launch_kernel(k_pack<0>, pack, 256, 0, st, J, gain_enable);
+            break;
+        case 1:
+            launch_kernel(k_frame_sums<1>, sums, 1024, 0, st, J);
+            launch_kernel(k_pack<1>, pack, 256, 0, st, J, gain_enable);
+            break;
+        case 2:
+            launch_kernel(k_frame_sums<2>, sums, 1024, 0, st, J);
+            launch_kernel(k_pack<2>, pack, 256, 0, st, J, gain_enable);
+            break;
     }
 }
 
