@@ -911,6 +911,9 @@ __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Bat
     // Plane levels: the compacted pixel list, grid-strided.
     const int wid = threadIdx.x >> 5;
     const int ntx = (hw + 7) >> 3, ntiles = ntx * ((H + 7) >> 3);
+    int w = blockIdx.x * (blockDim.x >> 5) + wid;
+    int next = PLANES && w < total ? list[w] : 0;  // the warp's next listed pixel, loaded a visit ahead (128x96 pair
+                                                       // 1.59 -> 1.53 ms, 80/40 px levels of 1024x436 10.04 -> 9.74)
     for (int rnd = 0;; ++rnd) {
         int x, y, i;
         if (!PLANES) {
@@ -924,9 +927,10 @@ __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Bat
             if (x >= W) continue;
             i = y * W + x;
         } else {
-            const int w = blockIdx.x * (blockDim.x >> 5) + wid + rnd * nw;
             if (w >= total) break;
-            i = list[w];
+            i = next;
+            w += nw;
+            if (w < total) next = list[w];
             y = i / W;
             x = i - y * W;
         }
