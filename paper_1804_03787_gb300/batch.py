@@ -3,7 +3,7 @@
 The pairs go to one or more gpm contexts, one CUDA stream each, balanced by
 pixel count.  Inside a context the pair index is on the device: every stage
 is one launch per eight of the context's pairs (blockIdx.z = pair), so a
-context of eight pairs makes the same ~190 launches as one of a single pair.  Each stream's whole pipeline (every scale, both directions,
+context of eight pairs makes the same ~170 launches as one of a single pair.  Each stream's whole pipeline (every scale, both directions,
 flow and occlusion) is captured once into a CUDA graph and replayed as a
 single launch per step.  The number of streams and the PatchMatch launch
 shape (blocks per SM) are picked by a small autotuner that times replays of

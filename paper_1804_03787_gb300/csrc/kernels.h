@@ -11,7 +11,7 @@ namespace gpm {
 // Launches a kernel that begins with begin_kernel() as a programmatic dependent of the one before it
 // on the stream: it is set up while that one runs and its blocks start as that one's end, so that a launch does not cost
 // the stream its latency.  (After a copy, an event of another stream or a foreign kernel a launch waits as ever.)
-// A pass is 130 to 200 launches in sequence, most of a few microseconds: 128x96 1.91 -> 1.62 ms, 253x187 4.55 -> 4.08,
+// A pass is 100 to 200 launches in sequence, most of a few microseconds: 128x96 1.91 -> 1.62 ms, 253x187 4.55 -> 4.08,
 // 1024x436 17.0 -> 16.6, 1920x1080 51.1 -> 50.6, a batch of four sizes on two streams 37.3 -> 37.1 ms.
 template <class... P, class... A>
 inline void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t shared, cudaStream_t st, A&&... args) {

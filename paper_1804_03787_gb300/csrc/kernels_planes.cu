@@ -1515,7 +1515,7 @@ __device__ __forceinline__ unsigned long long search_warp(const Window& w, const
     return best;
 }
 
-// Larger windows, one block of 256 threads each: 256 hypotheses a round, solved one per thread into shared memory.
+// Larger windows, one block of 256 or 512 threads each: 256 hypotheses a round, solved one per thread into shared memory.
 // The warps first test every hypothesis on an eighth of the matches (chunks of 128, spread over the window); the
 // one with the most is counted from below on all of them, by the whole block, which gives the bound the others have
 // to reach from the start; then the warps take the hypotheses that still can, one at a time, chunk by chunk.
@@ -1529,7 +1529,8 @@ struct BlockSearch {
     unsigned long long best;        // a lower bound of the best key; the winner's at the end
     int next, n_ok, n_loose;
 };
-__device__ __forceinline__ unsigned long long search_block(const BlockGroup<256>& grp, const Window& w,
+template <int NT>
+__device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>& grp, const Window& w,
                                                            const PlaneParams& pp, int cell, uint32_t tag,
                                                            uint32_t pair_id, BlockSearch& bs, RansacStats& st) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, N = w.N;
@@ -1556,13 +1557,14 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<256>
         int status = HYP_DEAD;
         {
             FastHyp h;
-            if (k < pp.num_hyp) status = fast_hypothesis(w, cell, k, tag, pair_id, pp.k0, pp.k1, t, h);
+            if (tid < kHypRound && k < pp.num_hyp)
+                status = fast_hypothesis(w, cell, k, tag, pair_id, pp.k0, pp.k1, t, h);
             if (status == HYP_OK) bs.form[tid] = h;
         }
-        bs.cnt[tid] = status == HYP_OK ? 0 : -1;
+        if (tid < kHypRound) bs.cnt[tid] = status == HYP_OK ? 0 : -1;
         if (tid == 0) bs.next = bs.n_ok = bs.n_loose = 0;
         __syncthreads();
-        for (int e = warp; e < kHypRound; e += 8) {
+        for (int e = warp; e < kHypRound; e += NT / 32) {
             if (bs.cnt[e] < 0) continue;  // warp-uniform
             const PairHyp ph = pair_hyp(bs.form[e]);
             int c = 0, ch = 0;
@@ -1578,19 +1580,19 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<256>
         __syncthreads();
         const int rest = 128 * (nch - nfirst);
         {
-            const int mine = bs.cnt[tid];
+            const int mine = tid < kHypRound ? bs.cnt[tid] : -1;
             const unsigned long long lead = grp.max(mine >= 0 ? hyp_key(mine, k) : 0ull);
             if (lead && hyp_key(min(key_score(lead) + rest, N), key_index(lead)) >= *vbest) {  // block-uniform
                 const FastHyp h = bs.form[key_index(lead) - b];
                 int lo = 0;
-                for (int j = tid; j < N; j += 256) {
+                for (int j = tid; j < N; j += NT) {
                     bool sure, maybe;
                     test_match(w, h, tl, t, j, sure, maybe);
                     lo += sure;
                 }
                 lo = grp.sum(lo);
                 if (tid == 0) bs.best = max(bs.best, hyp_key(lo, key_index(lead)));
-                st.tests += lane == 0 ? N / 8 : 0;
+                st.tests += lane == 0 ? N / (NT / 32) : 0;
                 __syncthreads();
             }
             const bool go = mine >= 0 && hyp_key(min(mine + rest, N), k) >= *vbest;
@@ -1944,22 +1946,28 @@ __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constan
     ransac_finish<WarpGroup, ST>(grp, pv, g, stage, pp, blockIdx.y, cell, match[warp]);
 }
 
-// Larger windows: one 256-thread block per window (matches in dynamic shared memory: four planes of block_cap(s)).
+// Larger windows: one block per window (matches in dynamic shared memory: four planes of block_cap(s)).
 __host__ __device__ constexpr int block_cap(int s) { return (s * s + 127) / 128 * 128; }
-__global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__ Batch bt, int level, int stage,
-                                                         PlaneParams pp) {
+// 512 threads a window instead of 256: where the matches leave an SM room for two blocks only (s > 60: 3 blocks' 16 s^2 +
+// 14 KB are above its 228 KB), and where all windows are resident at once, so that the launch lasts as one window (three
+// 256-thread blocks on each of 152 SMs).  First stage: 64 px windows of 1024x436 0.81 -> 0.72 ms, of 512x384 0.49 -> 0.37,
+// of 253x187 0.30 -> 0.24; 80 px of 1024x436 1.05 -> 0.82; 330 32 px windows 0.12 -> 0.12, their second stage 0.10 -> 0.08.
+// Elsewhere 256 is faster: 3300 32 px windows 0.51 against 0.56 ms, 2000 40 px ones 0.52 against 0.54.
+static bool ransac_wide(int s, int windows) { return s > 60 || windows <= 3 * 152; }
+template <int NT>
+__global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
     begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
     const LevelGeom g = bt.geom(blockIdx.z, level);
     const int cell = blockIdx.x, dir = blockIdx.y;
     if (cell >= g.ncells()) return;  // past this pair's windows (block-uniform)
     extern __shared__ __align__(16) float planes_dyn[];
-    __shared__ double red_d[8];
-    __shared__ int red_i[8];
-    __shared__ unsigned long long red_u[8];
+    __shared__ double red_d[NT / 32];
+    __shared__ int red_i[NT / 32];
+    __shared__ unsigned long long red_u[NT / 32];
     __shared__ __align__(16) BlockSearch bs;
     __shared__ double whl[16];  // also two sums per warp
-    const BlockGroup<256> grp{red_d, red_i, red_u};
+    const BlockGroup<NT> grp{red_d, red_i, red_u};
     const int id = (g.base + cell) * 2 + (stage - 1);
     RefitWork* rw = pv.rw[dir] + cell;
     Window w;
@@ -1969,7 +1977,18 @@ __global__ void __launch_bounds__(256, 3) k_ransac_block(const __grid_constant__
     const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
     RansacStats st;
     const unsigned long long best = search_block(grp, w, pp, cell, tag, pv.pair_id, bs, st);
-    finish_fit(grp, pv, w, pp, dir, cell, id, tag, best, st, whl, reinterpret_cast<long long*>(bs.form), rw);
+    // the winner's sums by 256 threads, whatever the block: their FP64 ones are in one order (barriers wait for the
+    // threads that are left)
+    if (NT > 256 && threadIdx.x >= 256) {
+        if (pv.evals && (threadIdx.x & 31) == 0) {
+            atomicAdd(&pv.evals[GPM_COUNT_RANSAC], (unsigned long long)st.tests);
+            atomicAdd(&pv.evals[GPM_COUNT_RANSAC_FP64], (unsigned long long)st.fp64);
+            atomicAdd(&pv.evals[GPM_COUNT_RANSAC_LOOSE], (unsigned long long)st.loose);
+        }
+        return;
+    }
+    finish_fit(BlockGroup<256>{red_d, red_i, red_u}, pv, w, pp, dir, cell, id, tag, best, st, whl,
+               reinterpret_cast<long long*>(bs.form), rw);
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
@@ -2576,11 +2595,15 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
     static bool attr_set = false;
     if (!attr_set) {
         const int mx = kMaxCell * kMaxCell * (int)sizeof(float4);  // the largest window's matches
-        cudaFuncSetAttribute(k_ransac_block, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        cudaFuncSetAttribute(k_ransac_block<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        cudaFuncSetAttribute(k_ransac_block<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
         cudaFuncSetAttribute(k_ransac_finish_block<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
         attr_set = true;
     }
-    launch_kernel(k_ransac_block, dim3(nc, 2, np), 256, fit_smem, st, bt, level, stage, pp);
+    if (ransac_wide(s, 2 * nc * np))
+        launch_kernel(k_ransac_block<512>, dim3(nc, 2, np), 512, fit_smem, st, bt, level, stage, pp);
+    else
+        launch_kernel(k_ransac_block<256>, dim3(nc, 2, np), 256, fit_smem, st, bt, level, stage, pp);
     launch_kernel(k_refit_solve, dim3((2 * nc + 31) / 32, 1, np), 32, 0, st, bt, level, pp);
     launch_kernel(k_ransac_finish_block<ST>, dim3(nc, 2, np), 256, smem, st, bt, level, stage, pp);
 }
