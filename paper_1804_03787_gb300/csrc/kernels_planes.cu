@@ -1529,6 +1529,11 @@ struct BlockSearch {
     unsigned long long best;        // a lower bound of the best key; the winner's at the end
     int next, n_ok, n_loose;
 };
+// A key in shared memory that other warps may raise meanwhile, the same value on every lane: what it decides holds
+// collectives of the whole warp, and the lanes' own loads may fall on either side of a change.  A stale bound only drops less.
+__device__ __forceinline__ unsigned long long shared_key(const volatile unsigned long long* key) {
+    return __shfl_sync(FULL, (threadIdx.x & 31) == 0 ? *key : 0ull, 0);
+}
 template <int NT>
 __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>& grp, const Window& w,
                                                            const PlaneParams& pp, int cell, uint32_t tag,
@@ -1609,14 +1614,15 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>&
             const bool loose = at >= n_ok;
             const int e = bs.todo[loose ? kHypRound - 1 - (at - n_ok) : at];
             int score = -1;
+            unsigned long long floor = shared_key(vbest);
             if (loose) {
                 ++st.loose;
-                if (hyp_key(N, b + e) >= *vbest)
-                    score = exact_support(w, cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, *vbest, st);
+                if (hyp_key(N, b + e) >= floor)
+                    score = exact_support(w, cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, floor, st);
             } else {
                 const PairHyp ph = pair_hyp(bs.form[e]);
                 int have = bs.cnt[e], left = rest, ch = (int)((long long)nfirst * step % nch);
-                bool alive = hyp_key(min(have + left, N), b + e) >= *vbest;
+                bool alive = hyp_key(min(have + left, N), b + e) >= floor;
                 while (alive && left > 0) {
                     int c = 0;
                     count_quad(w, ph, tt, 128 * ch + 4 * lane, c);
@@ -1625,10 +1631,11 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>&
                     left -= 128;
                     have += (int)__reduce_add_sync(FULL, (unsigned)c);
                     st.tests += 128;
-                    alive = hyp_key(min(have + left, N), b + e) >= *vbest;
+                    floor = shared_key(vbest);
+                    alive = hyp_key(min(have + left, N), b + e) >= floor;
                 }
                 if (alive)
-                    score = contender_support(w, &bs.form[e], cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, *vbest, st);
+                    score = contender_support(w, &bs.form[e], cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, floor, st);
             }
             if (score >= 0 && lane == 0) atomicMax(&bs.best, hyp_key(score, b + e));
             __syncwarp();
