@@ -369,21 +369,21 @@ struct LanePatch {
     uint32_t code[Patch<R>::NT];  // census data term: source codes of the lane's taps
     int tx[Patch<R>::NT], ty[Patch<R>::NT], tidx[Patch<R>::NT];
     float fx[Patch<R>::NT], fy[Patch<R>::NT];
-    // offsets c with oxlo <= c.x <= oxlo + oxspan and oylo <= c.y <= oylo + oyspan keep every texel of
-    // the patch inside the frame (the unclamped, one-add indexing path)
-    int oxlo, oxspan, oylo, oyspan;
+    // offsets c with oxlo <= c.x < oxlo + oxnum and oylo <= c.y < oylo + oynum keep every texel of the patch
+    // inside the frame (the unclamped, one-add indexing path)
+    int oxlo, oxnum, oylo, oynum;
     bool warped;
 };
 
 // The patch touches texels [xlo, xhi] x [ylo, yhi] at offset 0; offsets keep them inside the frame iff
-// -xlo <= c.x <= W-1-xhi (likewise y).  An empty range gets a start no offset reaches.
+// -xlo <= c.x <= W-1-xhi (likewise y).  A patch wider than the frame has no such offset (an incumbent may be any
+// imported value, so a start that no offset reaches would not do).
 template <int R>
 __device__ __forceinline__ void set_interior_box(LanePatch<R>& lp, int xlo, int xhi, int ylo, int yhi, int W, int H) {
-    const int sx = (W - 1 - xhi) + xlo, sy = (H - 1 - yhi) + ylo;
-    lp.oxlo = sx >= 0 ? -xlo : (1 << 30);
-    lp.oxspan = max(sx, 0);
-    lp.oylo = sy >= 0 ? -ylo : (1 << 30);
-    lp.oyspan = max(sy, 0);
+    lp.oxlo = -xlo;
+    lp.oxnum = max((W - xhi) + xlo, 0);
+    lp.oylo = -ylo;
+    lp.oynum = max((H - yhi) + ylo, 0);
 }
 
 // CENSUS: src holds the frame's census codes (uint32 per pixel) instead of texels.
@@ -483,7 +483,7 @@ __device__ __forceinline__ float3 tap_sample(const LanePatch<R>& lp, const void*
 
 template <int R>
 __device__ __forceinline__ bool interior_of(const LanePatch<R>& lp, int2 c) {
-    return (unsigned)(c.x - lp.oxlo) <= (unsigned)lp.oxspan && (unsigned)(c.y - lp.oylo) <= (unsigned)lp.oyspan;
+    return (unsigned)(c.x - lp.oxlo) < (unsigned)lp.oxnum && (unsigned)(c.y - lp.oylo) < (unsigned)lp.oynum;
 }
 
 // Raw patch cost of offset (vx, vy): the sum over taps and channels of
@@ -743,7 +743,11 @@ __global__ void __launch_bounds__(256) k_pm_recost(const __grid_constant__ Batch
             const int i = list[w];
             const int y = i / W, x = i - y * W;
             LanePatch<R> lp;
-            const int2 v = pv.nnf[dir][i];
+            // an imported offset may be any integer: past 2^30 on either side every tap is off the frame on that side,
+            // and sums of coordinates stay in range
+            int2 v = pv.nnf[dir][i];
+            v.x = min(max(v.x, -(1 << 30)), 1 << 30);
+            v.y = min(max(v.y, -(1 << 30)), 1 << 30);
             float c;
             // the padded copy serves square patches whose target pixel is in the frame (an imported offset
             // need not be)

@@ -1,0 +1,48 @@
+"""Imported offsets that leave the frame, as a matcher marks pixels it found no match for."""
+import numpy as np
+import pytest
+
+from paper_1804_03787_gb300 import gpm
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("zoom", [1.0, 1.9])
+@pytest.mark.parametrize("mark", [(1 << 30, 1 << 30), (1 << 30, 0), (-(1 << 31), 1 << 30), (5, -9)])
+def test_recost_of_far_offsets_on_a_frame_narrower_than_the_patch(mark, zoom):
+    """A plane of scale 1.9 spreads the taps of a 9 x 9 patch wider than an 8 x 8 frame: no offset keeps them inside, and
+    every one of these offsets puts every sample (tap displacements stay below 8 px) beyond the frame on each axis that is
+    far, where it reads the border texels."""
+    import torch
+    W = H = 8
+    gp = gpm.default_params(patch_radius=4, cells=(8,), pm_iters=0, num_hyp=32, gain_normalize=0)
+    rng = np.random.default_rng(8)
+    f1, f2 = (rng.random((H, W, 3)).astype(np.float32) for _ in range(2))
+    ctx = gpm.Context(gp, W, H)
+    ctx.match([(torch.from_numpy(f1).cuda(), torch.from_numpy(f2).cuda())])
+    n, m = W * H, ctx.export(gpm.MODELS).shape[1]
+    c = 3.5 - 3.5 * zoom
+    mh = np.tile(np.array([zoom, 0, c, 0, zoom, c, 0, 0, 1.0]), (2, m, 1))
+    mi = ctx.export(gpm.MODEL_INFO).copy()
+    mi[:, :, 0] = 1
+    nnf = np.tile(np.array(mark, np.int32), (2, n, 1))
+    for what, data in ((gpm.NNF, nnf), (gpm.MODELS, mh), (gpm.MODEL_INFO, mi),
+                       (gpm.LABELS, (np.full((2, n), -1, np.int32), np.full((2, n), 0.06, np.float32), np.zeros((2, n, 2))))):
+        ctx.import_state(what, data, 1, after_fit=True)
+    ctx.match(None, 1)
+    got = ctx.export(gpm.COST)
+    ctx.close()
+    d = np.arange(-4, 5)
+    p = np.arange(8)
+    tap = np.clip(p[:, None] + d, 0, 7)                                  # [pixel][tap] on one axis
+    at = [np.clip(p[:, None] + v + zoom * (tap - p[:, None]), 0, 7) for v in map(float, mark)]
+    lo = [np.minimum(np.floor(a).astype(int), 6) for a in at]
+    for k, (a, b) in enumerate(((f1, f2), (f2, f1))):
+        a, b = a.astype(np.float64), b.astype(np.float64)
+        rows = b[lo[1]] * (1 - (at[1] - lo[1]))[..., None, None] + b[lo[1] + 1] * (at[1] - lo[1])[..., None, None]
+        wx = (at[0] - lo[0])[:, None, None, :, None]
+        s = rows[:, :, lo[0]].transpose(2, 0, 1, 3, 4) * (1 - wx) + rows[:, :, lo[0] + 1].transpose(2, 0, 1, 3, 4) * wx
+        src = a[tap[:, :, None, None], tap[None, None]].transpose(2, 0, 1, 3, 4)  # [x][y][ty][tx][channel]
+        want = np.abs(src - s).mean((2, 3, 4)).T.reshape(-1)
+        # tap positions to 1e-6 px, blends and sums to some 1e-6: far below the differences of wrong texels (0.1)
+        assert np.abs(np.asarray(got[k]).reshape(-1) - want).max() < 1e-5
