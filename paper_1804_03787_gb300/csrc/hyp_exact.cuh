@@ -3,8 +3,7 @@
 // GB300 runs FP64 at a small fraction of its FP32 rate, and a 4-point
 // homography in FP64 was the bottleneck of the per-window fit.  Here the
 // projective-basis solution H ~ B adj(A) is formed exactly in 128-bit
-// integers -- frames up to 32767 px a side keep every entry below 2^89 -- and
-// the FP32 evaluation form is derived from exact integer numerators with one
+// integers (minimal_h_exact states their bounds) and the FP32 evaluation form is derived from exact integer numerators with one
 // rounding each; the translation, which needs ~1e-7 px absolute accuracy on
 // flows of hundreds of pixels, is split into hi + lo with an exact integer
 // remainder.
@@ -38,18 +37,20 @@ __host__ __device__ __forceinline__ float u32_to_float(uint32_t v) {
 #endif
 }
 
-// Float near a 128-bit integer below 2^96 in magnitude (ours stay below 2^92):
-// the 32-bit limbs combined by fused multiply-adds, within about 1 ulp -- every
-// caller tolerates that (the translation is corrected by an exact remainder).
+// Float near a 128-bit integer: the 32-bit limbs combined by fused multiply-adds, within about 1 ulp -- every
+// caller tolerates that (the translation is corrected by an exact remainder).  Samples inside a frame stay below
+// 2^92; with imported offsets far out of it mixed in, entries reach 2^111.
 __host__ __device__ __forceinline__ float i128_to_float(i128 x) {
     const bool neg = x < 0;
     const u128 u = neg ? (u128)0 - (u128)x : (u128)x;  // magnitude: no cancellation between limbs
-    const uint32_t l0 = (uint32_t)u, l1 = (uint32_t)(u >> 32), l2 = (uint32_t)(u >> 64);
+    const uint32_t l0 = (uint32_t)u, l1 = (uint32_t)(u >> 32), l2 = (uint32_t)(u >> 64), l3 = (uint32_t)(u >> 96);
 #ifdef __CUDA_ARCH__
-    const float f = __fmaf_rn(u32_to_float(l2), 18446744073709551616.f,
-                              __fmaf_rn(u32_to_float(l1), 4294967296.f, u32_to_float(l0)));
+    float f = __fmaf_rn(u32_to_float(l2), 18446744073709551616.f,
+                        __fmaf_rn(u32_to_float(l1), 4294967296.f, u32_to_float(l0)));
+    if (l3) f = __fmaf_rn(u32_to_float(l3), 79228162514264337593543950336.f, f);
 #else
-    const float f = (float)l2 * 18446744073709551616.f + (float)l1 * 4294967296.f + (float)l0;
+    float f = (float)l2 * 18446744073709551616.f + (float)l1 * 4294967296.f + (float)l0;
+    if (l3) f += (float)l3 * 79228162514264337593543950336.f;
 #endif
     return neg ? -f : f;
 }
@@ -115,16 +116,16 @@ __host__ __device__ inline void split_ratio(i128 num, i128 den, float rden, floa
     hi = i128_to_float(num) * rden;
     lo = 0.f;
     const float a = hi < 0 ? -hi : hi;
-    if (!(a >= 9.5367431640625e-07f && a < 1048576.f)) return;  // 2^-20 <= |hi| < 2^20, else hi alone
+    if (!(a >= 9.5367431640625e-07f)) return;  // below 2^-20: hi alone
     int e;
 #ifdef __CUDA_ARCH__
     const float mant = frexpf(hi, &e);
 #else
     const float mant = __builtin_frexpf(hi, &e);
 #endif
-    const int m = (int)(mant * 16777216.f);  // hi = m * 2^(e - 24), exactly
-    const int sh = 24 - e;                   // in [4, 44]
-    const i128 R = num * ((i128)1 << sh) - (i128)m * den;
+    const int sh = e < 24 ? 24 - e : 0;  // at most 44
+    const i128 M = (i128)(int)(mant * 16777216.f) * ((i128)1 << (e < 24 ? 0 : e - 24));  // hi = M 2^-sh, exactly
+    const i128 R = num * ((i128)1 << sh) - M * den;
 #ifdef __CUDA_ARCH__
     lo = __fmul_rn(i128_to_float(R) * rden, __int_as_float((127 - sh) << 23));
 #else
