@@ -1248,13 +1248,12 @@ __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Ba
     const bool mine = lane < npix && yq < H && xq < W;
     const int iq = mine ? yq * W + xq : 0;
     int2 best = make_int2(0, 0);
-    uint32_t before = 0;
     float bc = 0.f;  // times 2^23
     if (mine) {
         best = nnf[iq];
-        before = pack_off(best);
         bc = pv.cost[dir][iq] * 8388608.f;
     }
+    const float before = bc;
     // interior pixels: the patch-sum bound applies
     const bool prune = mine && xq >= R && yq >= R && xq < W - R && yq < H - R;
     const unsigned inside = __ballot_sync(FULL, prune);
@@ -1354,7 +1353,8 @@ __global__ void __launch_bounds__(128, 6) k_pm_sweep0(const __grid_constant__ Ba
         }
     }
     if (mine) {
-        const bool m = pack_off(best) != before;
+        // a candidate is only taken at a lower cost; the offsets packed would not tell, as an imported one may be any integer
+        const bool m = bc < before;
         moved[iq] = m;
         if (m) {
             nnf[iq] = best;

@@ -46,3 +46,43 @@ def test_recost_of_far_offsets_on_a_frame_narrower_than_the_patch(mark, zoom):
         want = np.abs(src - s).mean((2, 3, 4)).T.reshape(-1)
         # tap positions to 1e-6 px, blends and sums to some 1e-6: far below the differences of wrong texels (0.1)
         assert np.abs(np.asarray(got[k]).reshape(-1) - want).max() < 1e-5
+
+
+@pytest.mark.parametrize("mark,motion", [((1 << 20, 1 << 20), 0), ((65536 + 3, 0), 3)])
+def test_level0_sweeps_replace_far_incumbents(mark, motion):
+    """Half the pixels start from a marker equal to the motion modulo 2^16, among neighbours that hold the motion: a pixel that
+    takes it over must store it."""
+    import torch
+
+    import oracle as O
+
+    from _parity import TIE, dilate, oracle_frames, oracle_params
+    W, H = 61, 43
+    gp = gpm.default_params(patch_radius=2, cells=(), pm_iters=2, num_hyp=64, pm_init=0, gain_normalize=0)
+    P = oracle_params(gp, W, H)
+    rng = np.random.default_rng(5)
+    f1 = rng.random((H, W, 3)).astype(np.float32)
+    f2 = (np.roll(f1, motion, 1) * 0.99 + 0.01 * rng.random((H, W, 3))).astype(np.float32)
+    truth = np.stack([np.tile((m, 0), (W * H, 1)) for m in (motion, -motion)])
+    far = np.stack([np.tile(mark, (W * H, 1)), np.tile((mark[0] - 2 * motion, mark[1]), (W * H, 1))])
+    nnf = np.where(rng.random((2, W * H, 1)) < 0.5, far, truth).astype(np.int32)
+    ctx = gpm.Context(gp, W, H)
+    pair = (torch.from_numpy(f1).cuda(), torch.from_numpy(f2).cuda())
+    ctx.match([pair])
+    ctx.import_state(gpm.NNF, nnf, level=0)
+    ctx.match([pair])
+    got = ctx.export(gpm.NNF)
+    ctx.close()
+    frames, _ = oracle_frames(P, f1, f2)
+    for d in range(2):
+        vx, vy = (np.ascontiguousarray(nnf[d][:, c]) for c in range(2))
+        c = np.zeros(W * H)
+        O.pm_recost(P, *frames[d], 0, None, None, None, vx, vy, c)
+        cone = np.zeros((H, W), bool)
+        for k in range(2 * P.pm_iters):
+            amb = np.full(W * H, np.inf)
+            O.pm_sweep(P, *frames[d], d, 0, k >> 1, k & 1, None, None, None, vx, vy, c, amb)
+            cone |= dilate((amb < TIE).reshape(H, W), 2 * P.pm_iters - 1 - k)
+        sure = ~cone.reshape(-1)
+        assert sure.mean() > 0.5
+        assert (got[d][:, 0] == vx)[sure].all() and (got[d][:, 1] == vy)[sure].all()
