@@ -390,17 +390,20 @@ __device__ __forceinline__ bool mef_inlier_pt(const Mef& m, float ux, float uy, 
 
 // Exact-arithmetic stand-in for the residual test: H in window-local
 // coordinates as doubles (any positive scale, oriented so that the
-// denominator is positive at the window centre), the test in FP64 without a
-// division: den = h6 ux + h7 uy + h8 > 0 and |h_xy . (u, 1) - (u + v) den|^2
+// denominator is positive at the window centre), the test of a match u -> q in FP64
+// without a division: den = h6 x + h7 y + h8 > 0 and |h_xy . (u, 1) - q den|^2
 // < t2 den^2.  Its rounding is some 1e-15 of the terms, far inside the
 // 1e-5 near-tie band of the comparison.
-__device__ __forceinline__ bool hyp_inlier_fp64(const double* Hl, float ux, float uy, float vx, float vy, double t2) {
-    const double x = ux, y = uy, qx = (double)ux + (double)vx, qy = (double)uy + (double)vy;
+__device__ __forceinline__ bool hyp_inlier_fp64(const double* Hl, double x, double y, double qx, double qy, double t2) {
     const double w = Hl[6] * x + Hl[7] * y + Hl[8];
     if (!(w > 0.0)) return false;
     const double nx = Hl[0] * x + Hl[1] * y + Hl[2] - qx * w;
     const double ny = Hl[3] * x + Hl[4] * y + Hl[5] - qy * w;
     return nx * nx + ny * ny < t2 * w * w;
+}
+// The same for a match (u, u + v) held as floats.
+__device__ __forceinline__ bool hyp_inlier_fp64(const double* Hl, float ux, float uy, float vx, float vy, double t2) {
+    return hyp_inlier_fp64(Hl, (double)ux, (double)uy, (double)ux + (double)vx, (double)uy + (double)vy, t2);
 }
 
 // Local homography (double, rows, maps u -> local target) to the evaluation
@@ -482,14 +485,15 @@ struct Labels {
 // solve, finish) and reused by every level and stage.
 struct __align__(16) RefitWork {
     long long mom[24];      // exact DLT moments of the winner's inliers about (cx, cy, cu, cv)
-    int sample[16];         // the winner's sample, window-local: source x[4], y[4], target x[4], y[4]
+    int sample[8];          // the winner's sample, window-local: source x[4], y[4]
+    long long target[8];    // and target x[4], y[4]
     Mef mef0, mef1;         // evaluation forms (origin 0) of the winner and of the refit, with test bounds
     double hl_w[9], hl_r[9];  // the winner and the refit in window-local coordinates, denominator positive at the
                               // window centre (FP64 tests)
     double ds, dt;          // sums of nin times the inliers' distances to the source / target centroids
     double ha_w[9], ha_r[9];  // absolute homographies of the winner and of the refit
     int cx, cy, cu, cv;     // integer centres of the moments
-    int status;             // 2: refit pending (set by the fit), else the window is final
+    int status;             // 1: fit pending (far matches); 2: refit pending (set by the fit); else the window is final
     int nin;                // winner's inliers
     int refit_ok, geo_w, geo_r;
     float vmax;             // largest |offset| component among the window's matches (test bounds)

@@ -35,6 +35,10 @@ struct Slot {
     int* eq_hist = nullptr;    // 2 x 256 V-histogram counts (HSV equalisation)
     float* eq_lut = nullptr;   // 2 x 256 equalised V per bin
     unsigned long long* d_evals = nullptr;
+    // Whether the field may hold any integers: imported, and not yet replaced by a random initial one.  Launches that are
+    // captured run later and often, so what they leave is known only inside the same capture (capture_id).
+    bool any_offsets = false, any_in_graph = false;
+    unsigned long long init_capture = 0;
 };
 
 }  // namespace
@@ -305,6 +309,30 @@ gpm_status set_dims(gpm_ctx* c, Slot& s, int W, int H) {
     return cuda_check(c, "set_dims");
 }
 
+// The capture under way on the context's stream; 0: none.
+unsigned long long capture_id(gpm_ctx* c) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(c->stream, &st, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return ~0ull;
+    }
+    return st == cudaStreamCaptureStatusNone ? 0 : id;
+}
+
+// Whether a window of the pairs [0, np) may hold matches that are far from each other (kNearOffsets): fields that match
+// inside a frame this narrow do not.
+bool any_offsets(gpm_ctx* c, int np) {
+    const unsigned long long id = capture_id(c);
+    bool any = !c->P.pm_init;
+    for (int i = 0; i < np; ++i) {
+        const Slot& s = c->slots[i];
+        any = any || s.any_in_graph || (id ? s.init_capture != id : s.any_offsets) ||
+              2 * std::max(s.W, s.H) + kMaxCell > kNearOffsets;
+    }
+    return any;
+}
+
 // Restricted-sweep lists of pairs [first, first + np); cleared: launch_merge_update has cleared their counts.
 void build_lists(gpm_ctx* c, int first, int np, int max_n, bool cleared = false) {
     pbeg(c, GPM_PROF_LISTS, (cleared ? 1 : 2) * batches(np));
@@ -359,8 +387,9 @@ void fit_level(gpm_ctx* c, const Dims& D, int level) {
     cudaStream_t st = c->stream;
     auto each = [&](auto&& f) { each_batch(c, 0, np, f); };
     // first stage: fit, tentative assignment, cues on both directions, final assignment
-    pbeg(c, GPM_PROF_RANSAC, 3 * nb);
-    each([&](const Batch& b, int n) { launch_ransac(b, n, level, s, mc, 1, pp, st); });
+    const bool any = any_offsets(c, np);
+    pbeg(c, GPM_PROF_RANSAC, (3 + any) * nb);
+    each([&](const Batch& b, int n) { launch_ransac(b, n, level, s, mc, 1, any, pp, st); });
     pend(c);
     auto assign = [&](int stage, int again) {
         pbeg(c, GPM_PROF_ASSIGN, nb);
@@ -376,8 +405,8 @@ void fit_level(gpm_ctx* c, const Dims& D, int level) {
     cues(1, 0);
     assign(1, 1);
     // second stage on the residual pixels
-    pbeg(c, GPM_PROF_RANSAC, 3 * nb);
-    each([&](const Batch& b, int n) { launch_ransac(b, n, level, s, mc, 2, pp, st); });
+    pbeg(c, GPM_PROF_RANSAC, (3 + any) * nb);
+    each([&](const Batch& b, int n) { launch_ransac(b, n, level, s, mc, 2, any, pp, st); });
     pend(c);
     assign(2, 0);
     cues(2, 2);
@@ -604,6 +633,11 @@ gpm_status gpm_match(gpm_ctx* c, const gpm_pair* pairs, int32_t n_pairs, int32_t
             pbeg(c, GPM_PROF_PM_INIT, batches(n_pairs));
             launch_pm_all(c, L, n_pairs);
             pend(c);
+            const unsigned long long id = capture_id(c);
+            for (int i = 0; i < n_pairs; ++i) {
+                c->slots[i].init_capture = id;
+                if (!id) c->slots[i].any_offsets = false;
+            }
         } else {
             build_lists(c, 0, n_pairs, D.max_n);  // every pixel (nothing frozen) for the recost
         }
@@ -796,6 +830,9 @@ gpm_status gpm_import(gpm_ctx* c, int32_t pair, int32_t what, const void* src, i
         case GPM_NNF:
             for (int k = 0; k < 2; ++k)
                 cudaMemcpyAsync(s.pv.nnf[k], d + k * n * sizeof(int2), n * sizeof(int2), cudaMemcpyDeviceToDevice, st);
+            s.any_offsets = true;
+            s.any_in_graph = s.any_in_graph || capture_id(c) != 0;
+            s.init_capture = 0;
             break;
         case GPM_MODELS:
             for (int k = 0; k < 2; ++k)

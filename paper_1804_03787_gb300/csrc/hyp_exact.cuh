@@ -62,20 +62,21 @@ __host__ __device__ __forceinline__ float i128_to_float(i128 x) {
 // weights the cross products mu_k, sum_k mu_k (q_k - q3) = 0, and
 //   H = T(q3) H' T(-p3),   H' = sum_k w_k (q_k - q3, 1) adj(P')_k,   w_k = mu_k l_i l_j,
 // the same integers as the products with the untranslated points, in 18 wide
-// products instead of 45, most of them on short factors.  Bounds for windows
-// up to 96 px (|l| < 2^14.2) and target differences below 2^23 (frames below
-// 2^15 a side; imported offsets may leave the frame): |mu| < 2^47,
-// |w| < 2^75.4, |H| < 2^110.
-__host__ __device__ inline void minimal_h_exact(const int* px, const int* py, const int* qx, const int* qy,
-                                                i128* H) {
+// products instead of 45, most of them on short factors.  For windows up to
+// 96 px (|l| < 2^13.2), m the largest |mu| and q the largest target component
+// or difference: |w| < 2^26.4 m, the last row < 2^42.2 m, the others < 2^43 m q.
+// Targets within 2^22 (frames are below 2^15 a side): m < 2^47, |H| < 2^113;
+// others (imported offsets may be any integer) only if sample_in_range.
+template <class T>
+__host__ __device__ inline void minimal_h_exact(const int* px, const int* py, const T* qx, const T* qy, i128* H) {
     int dx[3], dy[3];
     int64_t X[3], Y[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         dx[k] = px[k] - px[3];
         dy[k] = py[k] - py[3];
-        X[k] = qx[k] - qx[3];
-        Y[k] = qy[k] - qy[3];
+        X[k] = (int64_t)qx[k] - qx[3];
+        Y[k] = (int64_t)qy[k] - qy[3];
     }
     int l[3];
     int64_t mu[3];
@@ -108,6 +109,28 @@ __host__ __device__ inline void minimal_h_exact(const int* px, const int* py, co
     H[3] = h[1][0] + h[2][0] * qy[3];
     H[4] = h[1][1] + h[2][1] * qy[3];
     H[5] = H[8] * qy[3] - h[1][0] * px[3] - h[1][1] * py[3];
+}
+
+// Whether minimal_h_exact and make_mef_exact hold a sample with these targets (below 2^33), moved by up to `shift`: the
+// largest |mu| below 2^57 (split_ratio multiplies twice the last row by 2^24) and its product with the largest target
+// below 2^82.  True of any targets within 2^22, and of targets about two places however far from each other.
+__host__ __device__ inline bool sample_in_range(const int64_t* qx, const int64_t* qy, int64_t shift) {
+    i128 m = 0, q = 0;
+    auto raise = [](i128& a, i128 v) {
+        v = v < 0 ? -v : v;
+        a = v > a ? v : a;
+    };
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int i = (k + 1) % 3, j = (k + 2) % 3;
+        const int64_t xi = qx[i] - qx[3], yi = qy[i] - qy[3], xj = qx[j] - qx[3], yj = qy[j] - qy[3];
+        raise(m, (i128)xi * yj - (i128)xj * yi);
+        raise(q, xi);
+        raise(q, yi);
+    }
+    raise(q, qx[3]);
+    raise(q, qy[3]);
+    return m < (i128)1 << 57 && m * (q + shift) < (i128)1 << 82;
 }
 
 // num / den (den > 0) as hi + lo floats: hi the rounded quotient, lo the

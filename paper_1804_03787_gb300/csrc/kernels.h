@@ -96,9 +96,11 @@ struct PlaneParams {
 
 // Every launch below covers np <= kBatch pairs (blockIdx.z) whose views and level geometries are in bt; grid
 // sizes come from the largest pair (max_cells: the most windows a pair has at the level).
-// RANSAC per window for both directions (blockIdx.y = direction); s: the level's window side.
-void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int stage, const PlaneParams& pp,
-                   cudaStream_t st);
+// RANSAC per window for both directions (blockIdx.y = direction); s: the level's window side.  any_offsets: the field may
+// hold offsets further than kNearOffsets apart, whose windows take a launch of their own (5 us where there are none).
+constexpr int kNearOffsets = 16383;
+void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int stage, bool any_offsets,
+                   const PlaneParams& pp, cudaStream_t st);
 // Assignment by eq. 3-4: stage 1 into tent, or again (after the cues) into st1 and resid; stage 2 into lvl (pixels of resid,
 // the others from st1), or again there, clearing the many-to-one keys.
 void launch_assign(const Batch& bt, int np, int level, int stage, int again, const PlaneParams& pp, int grid_blocks,

@@ -839,31 +839,60 @@ __device__ __forceinline__ void window_origin(const LevelGeom& g, int cell, int&
     oy = y0 + g.s / 2;
 }
 
-// The window's matches in raster order, in shared memory, as planes of floats holding exact integers (so a lane
-// loads four consecutive matches with one 16-byte load per plane): the pixel u in window coordinates, and its
-// target u + v relative to the window's reference offset v0.  Entries past N, up to the next multiple of `pad`,
-// are no match's inlier.
-struct Window {
-    float *x, *y, *qx, *qy;
-    int N;
-    float v0x, v0y;
-    float U;     // half the window side: bounds |u|
-    float vq;    // largest component of |u + v - v0|
-    float vmax;  // largest component of |v|
-    __device__ __forceinline__ float4 match(int j) const {
-        const float a = x[j], b = y[j];
-        return make_float4(a, b, (qx[j] + v0x) - a, (qy[j] + v0y) - b);
-    }
-};
 // A target no hypothesis reaches within the inlier radius (its square stays finite for any accepted hypothesis).
 constexpr float kFarTarget = 1e15f;
 // Up to this |u + v - v0|, differences of targets stay below 2^15 and their cross products fit 32 bits.
-constexpr float kFastReach = 16383.f;
+constexpr int kNearReach = kNearOffsets;
+
+// A target this far from v0 is out of reach: only a sample whose four targets are all far has it as an inlier.  Any other
+// hypothesis gets there only along its vanishing line, where a solve in FP64 is off by some q^2 2^-53 / (window side), a
+// pixel from about 2^28 on; a marker that a sample happens to hold then bends the line to itself, and counts for nothing.
+constexpr long long kFarthest = 1ll << 26;
+__device__ __forceinline__ bool out_of_reach(longlong2 q) { return max(llabs(q.x), llabs(q.y)) >= kFarthest; }
+// What the far matches of a window need (shared memory, one per window): how many, and how many of them are in reach, the
+// offsets in memory and the reference offset.
+struct WindowFar {
+    const int2* nnf;
+    int W, ox, oy, v0x, v0y, n, n_reach;
+};
+// A far match's target relative to v0 (components below 2^33), from its pixel.  Out of line (rare).
+__device__ __noinline__ longlong2 far_target(const WindowFar* far, float x, float y) {
+    const int ux = exact_int(x), uy = exact_int(y);
+    const int2 v = far->nnf[(far->oy + uy) * far->W + far->ox + ux];
+    return make_longlong2((long long)v.x - far->v0x + ux, (long long)v.y - far->v0y + uy);
+}
+// The window's matches in raster order, in shared memory, as planes of floats holding exact integers (so a lane
+// loads four consecutive matches with one 16-byte load per plane): the pixel u in window coordinates, and its
+// target u + v relative to the window's reference offset v0.  An imported offset may be any integer: a match whose
+// target is beyond kNearReach of v0 is far, its target in the planes is kFarTarget (no hypothesis counts it), and
+// far_target reads its offset again.  A window with far matches is left to the FAR instances of the kernels and functions
+// below, so that the others keep their registers and code (with both in one kernel 512x384 planes took 3.86 ms, with a
+// launch each 3.64; without any far matches to serve 3.54).
+// Entries past N, up to the next multiple of `pad`, are no match's inlier.
+struct Window {
+    float *x, *y, *qx, *qy;
+    const WindowFar* far;
+    int N;
+    float U;     // half the window side: bounds |u|
+    float vq;    // largest component of |u + v - v0| among the near matches
+    float vmax;  // largest component of |v|
+    __device__ __forceinline__ bool is_far(int j) const { return qx[j] == kFarTarget; }
+    // a near match, its offset relative to v0
+    __device__ __forceinline__ float4 match(int j) const {
+        const float a = x[j], b = y[j];
+        return make_float4(a, b, qx[j] - a, qy[j] - b);
+    }
+    __device__ __forceinline__ longlong2 far_target(int j) const { return gpm::far_target(far, x[j], y[j]); }
+    // any match's target relative to v0
+    __device__ __forceinline__ longlong2 target(int j) const {
+        return is_far(j) ? far_target(j) : make_longlong2(exact_int(qx[j]), exact_int(qy[j]));
+    }
+};
 
 // Gathers the window's matches (stage 1: every pixel; stage 2: the residual ones) into planes of `cap` floats.
 template <class G>
 __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, const LevelGeom& g, int stage, int dir,
-                                              int cell, float* planes, int cap, int pad, Window& w) {
+                                              int cell, float* planes, int cap, int pad, WindowFar* far, Window& w) {
     const int tid = grp.rank(), s = g.s, W = pv.W;
     int x0, y0, ox, oy;
     window_origin<G>(g, cell, x0, y0, ox, oy);
@@ -873,6 +902,7 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
     w.y = planes + cap;
     w.qx = planes + 2 * cap;
     w.qy = planes + 3 * cap;
+    w.far = far;
     int N = 0;
     for (int base = 0; base < s * s; base += G::size) {
         const int j = base + tid;
@@ -885,11 +915,10 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
         }
         if (take) {
             const int2 v = nnf[i];
-            const int ux = x0 + xl - ox, uy = y0 + yl - oy;
-            w.x[at] = (float)ux;
-            w.y[at] = (float)uy;
-            w.qx[at] = (float)(ux + v.x);
-            w.qy[at] = (float)(uy + v.y);
+            w.x[at] = (float)(x0 + xl - ox);
+            w.y[at] = (float)(y0 + yl - oy);
+            w.qx[at] = __int_as_float(v.x);  // integers until the reference is known
+            w.qy[at] = __int_as_float(v.y);
         }
         N += total;
     }
@@ -897,38 +926,54 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
     w.U = 0.5f * (float)s;
     grp.sync();
     // reference offset: the component-wise median of eight matches spread over the list (any value is correct;
-    // one near the window's main motion keeps the rounding bounds of its hypotheses small)
-    float mx = 0.f, my = 0.f;
+    // one near the window's main motion keeps the rounding bounds of its hypotheses small and few matches far)
+    int mx = 0, my = 0;
     if (N > 0) {
         const int lane = tid & 31, j = ((2 * (lane & 7) + 1) * N) >> 4;
-        mx = w.qx[j] - w.x[j];
-        my = w.qy[j] - w.y[j];
+        mx = __float_as_int(w.qx[j]);
+        my = __float_as_int(w.qy[j]);
     }
     int rx = 0, ry = 0;
 #pragma unroll
     for (int l = 0; l < 8; ++l) {
-        const float a = __shfl_sync(FULL, mx, l), b = __shfl_sync(FULL, my, l);
+        const int a = __shfl_sync(FULL, mx, l), b = __shfl_sync(FULL, my, l);
         const bool before = l < (int)(threadIdx.x & 7);
         rx += a < mx || (a == mx && before);
         ry += b < my || (b == my && before);
     }
-    w.v0x = __shfl_sync(FULL, mx, __ffs(__ballot_sync(FULL, rx == 3)) - 1);
-    w.v0y = __shfl_sync(FULL, my, __ffs(__ballot_sync(FULL, ry == 3)) - 1);
+    const int v0x = __shfl_sync(FULL, mx, __ffs(__ballot_sync(FULL, rx == 3)) - 1);
+    const int v0y = __shfl_sync(FULL, my, __ffs(__ballot_sync(FULL, ry == 3)) - 1);
+    if (tid == 0) *far = WindowFar{nnf, W, ox, oy, v0x, v0y, 0, 0};
     grp.sync();
-    float vm = 0.f, vq = 0.f;
+    unsigned vm = 0, vq = 0;
+    int n_far = 0;  // and those in reach, times 2^16
     for (int j = tid; j < N; j += G::size) {
-        const float ax = w.qx[j], ay = w.qy[j], bx = ax - w.v0x, by = ay - w.v0y;
-        vm = fmaxf(vm, fmaxf(fabsf(ax - w.x[j]), fabsf(ay - w.y[j])));
-        vq = fmaxf(vq, fmaxf(fabsf(bx), fabsf(by)));
-        w.qx[j] = bx;
-        w.qy[j] = by;
+        const int vx = __float_as_int(w.qx[j]), vy = __float_as_int(w.qy[j]);
+        const int dx = (int)((unsigned)vx - (unsigned)v0x), dy = (int)((unsigned)vy - (unsigned)v0y);
+        const int bx = (int)((unsigned)dx + (unsigned)exact_int(w.x[j])), by = (int)((unsigned)dy + (unsigned)exact_int(w.y[j]));
+        vm = max(vm, max((unsigned)abs(vx), (unsigned)abs(vy)));
+        // in range, and the subtractions did not wrap
+        const bool near = max((unsigned)(bx + kNearReach), (unsigned)(by + kNearReach)) <= 2u * kNearReach &&
+                          (((vx ^ v0x) & (vx ^ dx)) | ((vy ^ v0y) & (vy ^ dy))) >= 0;
+        if (near)
+            vq = max(vq, (unsigned)max(abs(bx), abs(by)));
+        else  // rounded: at the limit it may count as in reach without being so
+            n_far += fmaxf(fabsf((float)vx - (float)v0x), fabsf((float)vy - (float)v0y)) > 1.01f * (float)kFarthest ? 1 : 0x10001;
+        w.qx[j] = near ? (float)bx : kFarTarget;
+        w.qy[j] = near ? (float)by : kFarTarget;
     }
     for (int j = N + tid; j < (N + pad - 1) / pad * pad; j += G::size) {
         w.x[j] = w.y[j] = 0.f;
         w.qx[j] = w.qy[j] = kFarTarget;
     }
-    w.vmax = (float)grp.max((unsigned)vm);  // non-negative integers
-    w.vq = (float)grp.max((unsigned)vq);
+    w.vmax = (float)grp.max(vm);
+    unsigned reach = grp.max(n_far ? 1u << 14 : vq);  // vq is below 2^14
+    if (reach >> 14) {  // uniform over the window
+        n_far = grp.sum(n_far);
+        if (tid == 0) far->n = n_far & 0xFFFF, far->n_reach = n_far >> 16;
+        reach = grp.max(vq);
+    }
+    w.vq = (float)reach;
     grp.sync();
 }
 
@@ -943,8 +988,8 @@ __device__ __forceinline__ void draw_indices(int N, int cell, int k, uint32_t ta
     idx[3] = (int)bounded_u32(r.w, (uint32_t)N);
 }
 
-// Hypothesis k of a window, exact (128-bit integers, hyp_exact.cuh), in window coordinates; false if the sample is
-// degenerate (three source or three target points collinear).
+// Hypothesis k of a window, exact (128-bit integers, hyp_exact.cuh), from window coordinates to targets relative to v0;
+// false if the sample is degenerate (three source or three target points collinear).
 __device__ __forceinline__ bool draw_exact(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id,
                                            uint32_t k0, uint32_t k1, i128* Hk) {
     int idx[4], px[4], py[4], qx[4], qy[4];
@@ -953,8 +998,8 @@ __device__ __forceinline__ bool draw_exact(const Window& w, int cell, int k, uin
     for (int j = 0; j < 4; ++j) {
         px[j] = exact_int(w.x[idx[j]]);
         py[j] = exact_int(w.y[idx[j]]);
-        qx[j] = exact_int(w.qx[idx[j]] + w.v0x);
-        qy[j] = exact_int(w.qy[idx[j]] + w.v0y);
+        qx[j] = exact_int(w.qx[idx[j]]);
+        qy[j] = exact_int(w.qy[idx[j]]);
     }
     bool degen = false;
     const int T3[4][3] = {{0, 1, 2}, {0, 1, 3}, {0, 2, 3}, {1, 2, 3}};
@@ -969,10 +1014,44 @@ __device__ __forceinline__ bool draw_exact(const Window& w, int cell, int k, uin
     return true;
 }
 
+// Hypothesis k of a window with far matches, whose targets are read from their own integers, as its FP64 and its evaluation
+// form; false also if the targets are too far apart for the products (sample_in_range) or the denominator is 0 at the
+// centre.  all_far: whether all of the sample's targets are.  Out of line.
+__device__ __noinline__ bool solve_far(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id, uint32_t k0,
+                                       uint32_t k1, double* Hl, Mef& m, bool& all_far) {
+    int idx[4], px[4], py[4];
+    int64_t qx[4], qy[4];
+    draw_indices(w.N, cell, k, tag, pair_id, k0, k1, idx);
+    all_far = true;
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+        px[j] = exact_int(w.x[idx[j]]);
+        py[j] = exact_int(w.y[idx[j]]);
+        all_far = all_far && w.is_far(idx[j]);
+        const longlong2 q = w.target(idx[j]);
+        qx[j] = q.x;
+        qy[j] = q.y;
+    }
+    bool degen = false;
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+        const int a = t == 3 ? 1 : 0, b = t < 2 ? 1 : 2, c = t == 0 ? 2 : 3;
+        degen |= collinear3(px[a], py[a], px[b], py[b], px[c], py[c]);
+        degen |= (i128)(qx[b] - qx[a]) * (qy[c] - qy[a]) == (i128)(qy[b] - qy[a]) * (qx[c] - qx[a]);
+    }
+    if (degen || !sample_in_range(qx, qy, max(llabs((long long)w.far->v0x), llabs((long long)w.far->v0y)))) return false;
+    i128 Hk[9];
+    minimal_h_exact(px, py, qx, qy, Hk);
+    if (!make_mef_exact(Hk, m)) return false;
+    exact_local_fp64(Hk, Hl);
+    return true;
+}
+
 // A hypothesis in FP32, for scoring: den(u) = c0 + g0 ux + g1 uy (positive at the window centre), the target
 // relative to v0 times den, X(u) = xc + x0 ux + x1 uy and Y(u) likewise, and kap, a bound of everything rounding
 // can do to the inlier test: with n = (X - qx den, Y - qy den), an inlier has |n| < t den, so it passes
-// |n| <= t den + kap as computed, and a match that passes |n| < t den - kap as computed is an inlier.
+// |n| <= t den + kap as computed, and a match that passes |n| < t den - kap as computed is an inlier.  kap is for the
+// near matches; far_allowance and far_maybe derive the far ones' from it.
 struct FastHyp {
     float g0, g1, c0, kap, x0, x1, xc, pad0, y0, y1, yc, pad1;
 };
@@ -992,11 +1071,12 @@ __device__ __forceinline__ float t_below(float t2) { return sqrtf(t2) * (1.f - 9
 // 32 (SQ + |q3|_1 (1 + S)), n in addition |q|_1 28 (1 + S).  A match that can pass has
 // |q|_1 <= (|X| + |Y|) / den + 2 t, which the window's extremes of the form bound where den stays positive; else
 // the window's largest |q| does.  (34 and 30 below leave the second order room.)
+template <bool FAR>
 __device__ __forceinline__ int fast_hypothesis(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id,
                                                uint32_t k0, uint32_t k1, float t, FastHyp& h) {
-    if (!(w.vq <= kFastReach)) return HYP_LOOSE;  // uniform over the window
     int idx[4];
     draw_indices(w.N, cell, k, tag, pair_id, k0, k1, idx);
+    if (FAR && (w.is_far(idx[0]) || w.is_far(idx[1]) || w.is_far(idx[2]) || w.is_far(idx[3]))) return HYP_LOOSE;
     const float p3x = w.x[idx[3]], p3y = w.y[idx[3]], q3x = w.qx[idx[3]], q3y = w.qy[idx[3]];
     float dx[3], dy[3], X[3], Y[3], l[3];
     int Xi[3], Yi[3], mu[3];
@@ -1109,6 +1189,26 @@ __device__ __forceinline__ void test_match(const Window& w, const FastHyp& h, fl
     sure = b > 0.f && n2 < b * b;
 }
 
+// How many far matches a scored hypothesis may have as inliers: those in reach, unless its targets in the window stay near
+// (the bound on them in fast_hypothesis, with kap / t for ed, which is below it).
+__device__ __forceinline__ int far_allowance(const Window& w, const FastHyp& h, float t) {
+    const float dmin = h.c0 - (fabsf(h.g0) + fabsf(h.g1)) * w.U - 2.f * h.kap / t;
+    const float XY = fabsf(h.xc) + fabsf(h.yc) + (fabsf(h.x0) + fabsf(h.x1) + fabsf(h.y0) + fabsf(h.y1)) * w.U;
+    return dmin > 0.f && 1.05f * XY + t + 2.2f * t * dmin < 0.999f * (float)kNearReach * dmin ? 0 : w.far->n_reach;
+}
+// Whether a far match can be an inlier of a scored hypothesis.  Its bound: with one = 1 + U S, kap is at least
+// 34 u (|q3|_1 one + SQ U) + 30 u t one, so for a target q, rounded to floats itself,
+// 40 u ((|q3|_1 + |q|_1) one + SQ U) + 30 u t one is at most kap (1.2 + 1.34 |q|_1 / t).
+__device__ __forceinline__ bool far_maybe(const Window& w, const FastHyp& h, float t, int j) {
+    const longlong2 q = w.far_target(j);
+    const float ux = w.x[j], uy = w.y[j], qx = (float)q.x, qy = (float)q.y;
+    const float den = fmaf(h.g1, uy, fmaf(h.g0, ux, h.c0));
+    const float nx = fmaf(-qx, den, fmaf(h.x1, uy, fmaf(h.x0, ux, h.xc)));
+    const float ny = fmaf(-qy, den, fmaf(h.y1, uy, fmaf(h.y0, ux, h.yc)));
+    const float a = fmaf(t, den, h.kap * (1.21f + 1.35f * (fabsf(qx) + fabsf(qy)) / t));
+    return !out_of_reach(q) && a > 0.f && fmaf(nx, nx, ny * ny) < a * a;
+}
+
 // The order of two hypotheses: more inliers, then the lower index.  Zero is below every hypothesis.
 __device__ __forceinline__ unsigned long long hyp_key(int score, int k) {
     return ((unsigned long long)(unsigned)(score + 1) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)k);
@@ -1128,6 +1228,13 @@ __device__ __forceinline__ bool exact_inlier(const Mef& m, const double* Hl, con
     return hyp_inlier_fp64(Hl, mt.x, mt.y, mt.z, mt.w, (double)t2);
 }
 
+// The test of any match by a hypothesis in FP64 (all_far: of its sample), a far one from its own integers.
+__device__ __forceinline__ bool inlier_fp64(const Window& w, const double* Hl, bool all_far, int j, float t2) {
+    const longlong2 q = w.target(j);
+    return (all_far || !out_of_reach(q)) &&
+           hyp_inlier_fp64(Hl, (double)w.x[j], (double)w.y[j], (double)q.x, (double)q.y, (double)t2);
+}
+
 // What a warp counts of its work (profiling counters).
 struct RansacStats {
     int tests = 0, fp64 = 0, loose = 0;
@@ -1135,23 +1242,33 @@ struct RansacStats {
 
 // The exact support of hypothesis k, by one warp: -1 if its sample is degenerate, or as soon as it cannot reach
 // `floor` (a key).  Out of line: for the few hypotheses that contend with uncertain tests, and the loose ones.
+template <bool FAR>
 __device__ __noinline__ int exact_support(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id,
                                           uint32_t k0, uint32_t k1, float t2, unsigned long long floor,
                                           RansacStats& st) {
     const int lane = threadIdx.x & 31;
     double Hl[9];
     Mef m;
-    {
+    bool all_far = false;
+    if constexpr (FAR) {
+        if (!solve_far(w, cell, k, tag, pair_id, k0, k1, Hl, m, all_far)) return -1;
+    } else {
         i128 Hk[9];
         if (!draw_exact(w, cell, k, tag, pair_id, k0, k1, Hk) || !make_mef_exact(Hk, m)) return -1;
         exact_local_fp64(Hk, Hl);
     }
-    mef_set_bounds(m, w.U, w.vmax, t2);
+    mef_set_bounds(m, w.U, w.vq + w.U, t2);
     int score = 0, f = 0;
     for (int c = 0; c < w.N; c += 128) {
 #pragma unroll 1
         for (int j = c + lane; j < c + 128 + lane; j += 32) {
-            const bool in = j < w.N && exact_inlier(m, Hl, w.match(j), t2, f);
+            bool in = false;
+            if (FAR && j < w.N && w.is_far(j)) {
+                in = inlier_fp64(w, Hl, all_far, j, t2);
+                ++f;
+            } else if (j < w.N) {
+                in = exact_inlier(m, Hl, w.match(j), t2, f);
+            }
             score += __popc(__ballot_sync(FULL, in));
         }
         st.tests += min(128, w.N - c);
@@ -1163,6 +1280,7 @@ __device__ __noinline__ int exact_support(const Window& w, int cell, int k, uint
 
 // The support of scored hypothesis k (its form in `form`, shared memory), by one warp: the FP32 count if no test is
 // uncertain, else exact; -1 if it cannot reach `floor`.  Out of line (contenders only).
+template <bool FAR>
 __device__ __noinline__ int contender_support(const Window& w, const FastHyp* form, int cell, int k, uint32_t tag,
                                               uint32_t pair_id, uint32_t k0, uint32_t k1, float t2,
                                               unsigned long long floor, RansacStats& st) {
@@ -1170,8 +1288,11 @@ __device__ __noinline__ int contender_support(const Window& w, const FastHyp* fo
     const float tl = t_below(t2), th = t_above(t2);
     int lo = 0, hi = 0;
     for (int j = threadIdx.x & 31; j < w.N; j += 32) {
-        bool sure, maybe;
-        test_match(w, h, tl, th, j, sure, maybe);
+        bool sure = false, maybe;
+        if (FAR && w.is_far(j))
+            maybe = far_maybe(w, h, th, j);
+        else
+            test_match(w, h, tl, th, j, sure, maybe);
         lo += sure;
         hi += maybe;
     }
@@ -1179,7 +1300,7 @@ __device__ __noinline__ int contender_support(const Window& w, const FastHyp* fo
     hi = (int)__reduce_add_sync(FULL, (unsigned)hi);
     st.tests += w.N;
     if (hyp_key(hi, k) < floor) return -1;
-    return hi == lo ? lo : exact_support(w, cell, k, tag, pair_id, k0, k1, t2, floor, st);
+    return hi == lo ? lo : exact_support<FAR>(w, cell, k, tag, pair_id, k0, k1, t2, floor, st);
 }
 
 // The window's matches in raster order into `match`; returns their number.
@@ -1308,6 +1429,7 @@ __device__ __forceinline__ void group_dists(const BlockGroup<NT>&, double s, dou
     }
 }
 
+constexpr int kFarPending = 1;  // RefitWork::status of a window with far matches that is yet to be fitted
 // The window's model record, cleared before its fit.
 __device__ __forceinline__ void clear_model(const PairView& pv, int dir, int id, int N, RefitWork* rw) {
     int* mi = pv.mi[dir] + (size_t)id * kMI;
@@ -1330,11 +1452,63 @@ __device__ __noinline__ void winner_fp64(const Window& w, int cell, int k, uint3
         for (int q = 0; q < 9; ++q) whl[q] = Hl[q];
 }
 
+// finish_fit's first part in a window with far matches: the winner's inliers among this thread's matches, all decided in
+// FP64, its sample into rw, and, if there are far inliers, the inliers' targets in the planes about another reference, the
+// offset of the winner's first match, now in v0: far inliers are near it.  beyond: one is beyond kRefitReach of it all the
+// same, which leaves the window without a refit (inliers so far apart are no plane of any scale in use, and their sums
+// would not fit: within it an inlier is at most 3/4 of their span from their mean, and squares stay below 2^30).
+template <class G>
+__device__ __forceinline__ unsigned long long far_winner(const G& grp, const Window& w, int cell, int k, uint32_t tag,
+                                                      uint32_t pair_id, uint32_t k0, uint32_t k1, float t2, RefitWork* rw,
+                                                      int2& v0, bool& beyond) {
+    constexpr int kRefitReach = 20000;
+    const int tid = grp.rank();
+    double Hl[9];
+    Mef m;
+    bool all_far;
+    solve_far(w, cell, k, tag, pair_id, k0, k1, Hl, m, all_far);
+    unsigned long long inm = 0;
+    bool far = false;
+    for (int j = tid, c = 0; j < w.N; j += G::size, ++c)
+        if (inlier_fp64(w, Hl, all_far, j, t2)) {
+            inm |= 1ull << c;
+            far = far || w.is_far(j);
+        }
+    int idx[4];
+    draw_indices(w.N, cell, k, tag, pair_id, k0, k1, idx);
+    if (tid < 4) {
+        const int j = tid == 0 ? idx[0] : (tid == 1 ? idx[1] : (tid == 2 ? idx[2] : idx[3]));
+        const longlong2 q = w.target(j);
+        rw->sample[tid] = exact_int(w.x[j]);
+        rw->sample[4 + tid] = exact_int(w.y[j]);
+        rw->target[tid] = v0.x + q.x;
+        rw->target[4 + tid] = v0.y + q.y;
+    }
+    beyond = false;
+    if (!grp.any(far)) return inm;
+    longlong2 shift = w.target(idx[0]);
+    shift.x -= exact_int(w.x[idx[0]]);
+    shift.y -= exact_int(w.y[idx[0]]);
+    grp.sync();  // the targets are read
+    for (unsigned long long b = inm; b; b &= b - 1) {
+        const int j = tid + (__ffsll((long long)b) - 1) * G::size;
+        longlong2 q = w.target(j);
+        q.x -= shift.x;
+        q.y -= shift.y;
+        beyond = beyond || max(llabs(q.x), llabs(q.y)) > kRefitReach;
+        w.qx[j] = beyond ? 0.f : (float)(int)q.x;
+        w.qy[j] = beyond ? 0.f : (float)(int)q.y;
+    }
+    v0 = make_int2((int)(v0.x + shift.x), (int)(v0.y + shift.y));
+    beyond = grp.any(beyond);
+    return inm;
+}
+
 // What follows the search: the refit's inputs on the winner's inliers (Hartley centroids as exact integer sums,
 // distances, and the DLT moments as exact integers about the rounded centroids) and the winner's sample, from which
 // the solve (a thread per window) forms the exact homography.  best: the winner's key, 0 if there is none; whl: 9
 // doubles of shared memory; scratch: 24 values per warp of a block.
-template <class G>
+template <bool FAR, class G>
 __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, const Window& w, const PlaneParams& pp,
                                            int dir, int cell, int id, uint32_t tag, unsigned long long best,
                                            const RansacStats& st, double* whl, long long* scratch, RefitWork* rw) {
@@ -1362,27 +1536,43 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
     // the winner's inliers among this thread's matches (bit c: match tid + c G::size; N <= 64 G::size for every
     // group: 256 matches per warp window, 96 x 96 per block window), uncertain ones decided in FP64
     static_assert(kMaxCell * kMaxCell <= 64 * 256 && 16 * 16 <= 64 * 32, "inlier mask too small");
-    unsigned long long inm = 0, um = 0;
-    {
-        FastHyp h;
-        const float tl = t_below(pp.t2), th = t_above(pp.t2);
-        const bool scored = fast_hypothesis(w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, th, h) == HYP_OK;
-        for (int j = tid, c = 0; j < N; j += G::size, ++c) {
-            bool sure = false, maybe = true;
-            if (scored) test_match(w, h, tl, th, j, sure, maybe);
-            if (sure)
-                inm |= 1ull << c;
-            else if (maybe)
-                um |= 1ull << c;
+    unsigned long long inm = 0;
+    int2 v0 = make_int2(w.far->v0x, w.far->v0y);
+    bool beyond = false;
+    if constexpr (FAR) {
+        inm = far_winner(grp, w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, pp.t2, rw, v0, beyond);
+    } else {
+        unsigned long long um = 0;
+        {
+            FastHyp h;
+            const float tl = t_below(pp.t2), th = t_above(pp.t2);
+            const bool scored = fast_hypothesis<false>(w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, th, h) == HYP_OK;
+            for (int j = tid, c = 0; j < N; j += G::size, ++c) {
+                bool sure = false, maybe = true;
+                if (scored) test_match(w, h, tl, th, j, sure, maybe);
+                if (sure)
+                    inm |= 1ull << c;
+                else if (maybe)
+                    um |= 1ull << c;
+            }
         }
-    }
-    if (grp.any(um != 0)) {
-        if (tid < 32) winner_fp64(w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, whl);
-        grp.sync();
-        for (; um; um &= um - 1) {
-            const int c = __ffsll((long long)um) - 1;
-            const float4 mt = w.match(tid + c * G::size);
-            if (hyp_inlier_fp64(whl, mt.x, mt.y, mt.z, mt.w, (double)pp.t2)) inm |= 1ull << c;
+        if (grp.any(um != 0)) {
+            if (tid < 32) winner_fp64(w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, whl);
+            grp.sync();
+            for (; um; um &= um - 1) {
+                const int c = __ffsll((long long)um) - 1;
+                const float4 mt = w.match(tid + c * G::size);
+                if (hyp_inlier_fp64(whl, mt.x, mt.y, mt.z, mt.w, (double)pp.t2)) inm |= 1ull << c;
+            }
+        }
+        if (tid < 4) {
+            int idx[4];
+            draw_indices(N, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, idx);
+            const int j = tid == 0 ? idx[0] : (tid == 1 ? idx[1] : (tid == 2 ? idx[2] : idx[3]));
+            rw->sample[tid] = exact_int(w.x[j]);
+            rw->sample[4 + tid] = exact_int(w.y[j]);
+            rw->target[tid] = (long long)v0.x + exact_int(w.qx[j]);
+            rw->target[4 + tid] = (long long)v0.y + exact_int(w.qy[j]);
         }
     }
     int sx = 0, sy = 0, tx = 0, ty = 0;  // target sums about v0
@@ -1393,17 +1583,18 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
         tx += exact_int(w.qx[j]);
         ty += exact_int(w.qy[j]);
     }
-    const int v0x = exact_int(w.v0x), v0y = exact_int(w.v0y);
     sx = grp.sum(sx);
     sy = grp.sum(sy);
-    tx = grp.sum(tx) + nw * v0x;
-    ty = grp.sum(ty) + nw * v0y;
+    tx = grp.sum(tx);
+    ty = grp.sum(ty);
     const float fn = (float)nw;
     const int cx = __float2int_rn(__fdiv_rn((float)sx, fn)), cy = __float2int_rn(__fdiv_rn((float)sy, fn));
-    const int cu = __float2int_rn(__fdiv_rn((float)tx, fn)), cv = __float2int_rn(__fdiv_rn((float)ty, fn));
+    const int cu = __float2int_rn(__fdiv_rn((float)((long long)nw * v0.x + tx), fn));
+    const int cv = __float2int_rn(__fdiv_rn((float)((long long)nw * v0.y + ty), fn));
+    const int du = (int)((long long)v0.x - cu), dv = (int)((long long)v0.y - cv);  // small: cu is v0 and a mean about it
     // Hartley scales: distances to the exact centroids, as n |p - mean| = |n p - sum| from exact integers
     // (the least-squares refit of a noisy support moves with its normalisation, so the scale must carry no
-    // more than float rounding); n |coordinate| < 2^31 for frames up to 32767 px and windows up to 96 px
+    // more than float rounding); windows up to 96 px: n |coordinate about v0| < 2^31
     double ds = 0.0, dt = 0.0;
     long long R[24];
 #pragma unroll
@@ -1411,10 +1602,10 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
     for (; inm; inm &= inm - 1) {
         const int j = tid + (__ffsll((long long)inm) - 1) * G::size;
         const int ax = exact_int(w.x[j]), ay = exact_int(w.y[j]);
-        const int bx = exact_int(w.qx[j]) + v0x, by = exact_int(w.qy[j]) + v0y;
+        const int bx = exact_int(w.qx[j]), by = exact_int(w.qy[j]);
         add_dist(ds, nw * ax - sx, nw * ay - sy);
         add_dist(dt, nw * bx - tx, nw * by - ty);
-        const int X = ax - cx, Y = ay - cy, U = bx - cu, V = by - cv;
+        const int X = ax - cx, Y = ay - cy, U = bx + du, V = by + dv;
         const int zz[6] = {X * X, X * Y, X, Y * Y, Y, 1};
         const int w3 = U * U + V * V;
 #pragma unroll
@@ -1425,17 +1616,9 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
             R[18 + q] += (long long)w3 * zz[q];
         }
     }
+    if (beyond) ds = dt = 0.0;  // no extent: no refit
     group_dists(grp, ds, dt, reinterpret_cast<double*>(whl), rw);
     group_moments(grp, R, scratch, rw->mom);
-    if (tid < 4) {
-        int idx[4];
-        draw_indices(N, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, idx);
-        const int j = tid == 0 ? idx[0] : (tid == 1 ? idx[1] : (tid == 2 ? idx[2] : idx[3]));
-        rw->sample[tid] = exact_int(w.x[j]);
-        rw->sample[4 + tid] = exact_int(w.y[j]);
-        rw->sample[8 + tid] = exact_int(w.qx[j]) + v0x;
-        rw->sample[12 + tid] = exact_int(w.qy[j]) + v0y;
-    }
     if (tid == 0) {
         rw->cx = cx;
         rw->cy = cy;
@@ -1462,6 +1645,7 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
 // What bounds it: instruction fetch, then the FP32 pipe in the tests (12 operations a match).  1024x436, stage 1:
 // the 16 px windows 1.44 -> 0.41 ms, the 8 px windows 1.73 -> 0.53 ms, against scoring exact 128-bit hypotheses
 // (0.64 and 1.12 ms of these gains while the winner was still solved here, in 180 KB of code, not 97).
+template <bool FAR>
 __device__ __forceinline__ unsigned long long search_warp(const Window& w, const PlaneParams& pp, int cell,
                                                           uint32_t tag, uint32_t pair_id, FastHyp* slot,
                                                           RansacStats& st) {
@@ -1474,10 +1658,11 @@ __device__ __forceinline__ unsigned long long search_warp(const Window& w, const
         const int k = b + lane;
         FastHyp h;
         const int status =
-            k < pp.num_hyp ? fast_hypothesis(w, cell, k, tag, pair_id, pp.k0, pp.k1, t, h) : (int)HYP_DEAD;
+            k < pp.num_hyp ? fast_hypothesis<FAR>(w, cell, k, tag, pair_id, pp.k0, pp.k1, t, h) : (int)HYP_DEAD;
         st.loose += __popc(__ballot_sync(FULL, status == HYP_LOOSE));
         unsigned alive = __ballot_sync(FULL, status == HYP_OK);
         int cnt = 0, left = 4 * nq;  // maybe tests passed; matches not yet tested
+        if (FAR && status == HYP_OK) cnt = far_allowance(w, h, t);  // taken as passed
         if (alive) {
             const PairHyp ph = pair_hyp(h);
             for (int pass = 0; pass < 4; ++pass) {
@@ -1504,8 +1689,8 @@ __device__ __forceinline__ unsigned long long search_warp(const Window& w, const
             if (lane == l) *slot = h;
             __syncwarp();
             const int score =
-                ok ? contender_support(w, slot, cell, b + l, tag, pair_id, pp.k0, pp.k1, pp.t2, best, st)
-                   : exact_support(w, cell, b + l, tag, pair_id, pp.k0, pp.k1, pp.t2, best, st);
+                ok ? contender_support<FAR>(w, slot, cell, b + l, tag, pair_id, pp.k0, pp.k1, pp.t2, best, st)
+                   : exact_support<FAR>(w, cell, b + l, tag, pair_id, pp.k0, pp.k1, pp.t2, best, st);
             __syncwarp();
             if (score >= 0) best = max(best, hyp_key(score, b + l));
             alive &= ~(1u << l);
@@ -1534,7 +1719,7 @@ struct BlockSearch {
 __device__ __forceinline__ unsigned long long shared_key(const volatile unsigned long long* key) {
     return __shfl_sync(FULL, (threadIdx.x & 31) == 0 ? *key : 0ull, 0);
 }
-template <int NT>
+template <bool FAR, int NT>
 __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>& grp, const Window& w,
                                                            const PlaneParams& pp, int cell, uint32_t tag,
                                                            uint32_t pair_id, BlockSearch& bs, RansacStats& st) {
@@ -1563,7 +1748,7 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>&
         {
             FastHyp h;
             if (tid < kHypRound && k < pp.num_hyp)
-                status = fast_hypothesis(w, cell, k, tag, pair_id, pp.k0, pp.k1, t, h);
+                status = fast_hypothesis<FAR>(w, cell, k, tag, pair_id, pp.k0, pp.k1, t, h);
             if (status == HYP_OK) bs.form[tid] = h;
         }
         if (tid < kHypRound) bs.cnt[tid] = status == HYP_OK ? 0 : -1;
@@ -1579,6 +1764,7 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>&
                 if (ch >= nch) ch -= nch;
             }
             c = (int)__reduce_add_sync(FULL, (unsigned)c);
+            if (FAR) c += far_allowance(w, bs.form[e], t);  // taken as passed
             if (lane == 0) bs.cnt[e] = (short)c;
             st.tests += 128 * nfirst;
         }
@@ -1618,7 +1804,7 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>&
             if (loose) {
                 ++st.loose;
                 if (hyp_key(N, b + e) >= floor)
-                    score = exact_support(w, cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, floor, st);
+                    score = exact_support<FAR>(w, cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, floor, st);
             } else {
                 const PairHyp ph = pair_hyp(bs.form[e]);
                 int have = bs.cnt[e], left = rest, ch = (int)((long long)nfirst * step % nch);
@@ -1635,7 +1821,7 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>&
                     alive = hyp_key(min(have + left, N), b + e) >= floor;
                 }
                 if (alive)
-                    score = contender_support(w, &bs.form[e], cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, floor, st);
+                    score = contender_support<FAR>(w, &bs.form[e], cell, b + e, tag, pair_id, pp.k0, pp.k1, pp.t2, floor, st);
             }
             if (score >= 0 && lane == 0) atomicMax(&bs.best, hyp_key(score, b + e));
             __syncwarp();
@@ -1660,7 +1846,7 @@ __device__ __forceinline__ bool refit_system(RefitWork* rw, const LevelGeom& g, 
     double Hw[9];
     {
         i128 hx[9];
-        minimal_h_exact(rw->sample, rw->sample + 4, rw->sample + 8, rw->sample + 12, hx);
+        minimal_h_exact(rw->sample, rw->sample + 4, rw->target, rw->target + 4, hx);
         Mef m0;
         make_mef_exact(hx, m0);
         mef_set_bounds(m0, 0.5f * (float)g.s, rw->vmax, pp.t2);
@@ -1916,7 +2102,8 @@ __device__ void ransac_finish(const G& grp, const PairView& pv, const LevelGeom&
 // (A) Windows up to 16 x 16: one warp per window, kRansacWarps windows per block.  CAP: the most matches a window
 // has (64 for sides up to 8, else 256).
 constexpr int kRansacWarps = 4;
-template <int CAP>
+// FAR: the windows that the other instance has left (kFarPending), otherwise the rest.
+template <int CAP, bool FAR>
 __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     k_ransac_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
     begin_kernel();
@@ -1924,6 +2111,7 @@ __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     const LevelGeom g = bt.geom(blockIdx.z, level);
     __shared__ __align__(16) float planes[kRansacWarps][4 * CAP];
     __shared__ FastHyp slot[kRansacWarps];
+    __shared__ WindowFar far[kRansacWarps];
     __shared__ double whl[kRansacWarps][9];
     const int warp = threadIdx.x >> 5, dir = blockIdx.y;
     const int cell = blockIdx.x * kRansacWarps + warp;
@@ -1931,14 +2119,19 @@ __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     const WarpGroup grp;
     const int id = (g.base + cell) * 2 + (stage - 1);
     RefitWork* rw = pv.rw[dir] + cell;
+    if (FAR && rw->status != kFarPending) return;
     Window w;
-    gather_window(grp, pv, g, stage, dir, cell, planes[warp], CAP, 4, w);
+    gather_window(grp, pv, g, stage, dir, cell, planes[warp], CAP, 4, &far[warp], w);
     if (grp.rank() == 0) clear_model(pv, dir, id, w.N, rw);
     if (w.N < pp.min_inliers || w.N < 4) return;
+    if (!FAR && w.far->n) {
+        if (grp.rank() == 0) rw->status = kFarPending;
+        return;
+    }
     const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
     RansacStats st;
-    const unsigned long long best = search_warp(w, pp, cell, tag, pv.pair_id, &slot[warp], st);
-    finish_fit(grp, pv, w, pp, dir, cell, id, tag, best, st, whl[warp], nullptr, rw);
+    const unsigned long long best = search_warp<FAR>(w, pp, cell, tag, pv.pair_id, &slot[warp], st);
+    finish_fit<FAR>(grp, pv, w, pp, dir, cell, id, tag, best, st, whl[warp], nullptr, rw);
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
@@ -1961,7 +2154,7 @@ __host__ __device__ constexpr int block_cap(int s) { return (s * s + 127) / 128 
 // of 253x187 0.30 -> 0.24; 80 px of 1024x436 1.05 -> 0.82; 330 32 px windows 0.12 -> 0.12, their second stage 0.10 -> 0.08.
 // Elsewhere 256 is faster: 3300 32 px windows 0.51 against 0.56 ms, 2000 40 px ones 0.52 against 0.54.
 static bool ransac_wide(int s, int windows) { return s > 60 || windows <= 3 * 152; }
-template <int NT>
+template <int NT, bool FAR>
 __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
     begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
@@ -1974,16 +2167,22 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __g
     __shared__ unsigned long long red_u[NT / 32];
     __shared__ __align__(16) BlockSearch bs;
     __shared__ double whl[16];  // also two sums per warp
+    __shared__ WindowFar far;
     const BlockGroup<NT> grp{red_d, red_i, red_u};
     const int id = (g.base + cell) * 2 + (stage - 1);
     RefitWork* rw = pv.rw[dir] + cell;
+    if (FAR && rw->status != kFarPending) return;  // block-uniform: cleared behind the barriers of gather_window
     Window w;
-    gather_window(grp, pv, g, stage, dir, cell, planes_dyn, block_cap(g.s), 128, w);
+    gather_window(grp, pv, g, stage, dir, cell, planes_dyn, block_cap(g.s), 128, &far, w);
     if (threadIdx.x == 0) clear_model(pv, dir, id, w.N, rw);
     if (w.N < pp.min_inliers || w.N < 4) return;
+    if (!FAR && w.far->n) {
+        if (threadIdx.x == 0) rw->status = kFarPending;
+        return;
+    }
     const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
     RansacStats st;
-    const unsigned long long best = search_block(grp, w, pp, cell, tag, pv.pair_id, bs, st);
+    const unsigned long long best = search_block<FAR>(grp, w, pp, cell, tag, pv.pair_id, bs, st);
     // the winner's sums by 256 threads, whatever the block: their FP64 ones are in one order (barriers wait for the
     // threads that are left)
     if (NT > 256 && threadIdx.x >= 256) {
@@ -1994,8 +2193,8 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __g
         }
         return;
     }
-    finish_fit(BlockGroup<256>{red_d, red_i, red_u}, pv, w, pp, dir, cell, id, tag, best, st, whl,
-               reinterpret_cast<long long*>(bs.form), rw);
+    finish_fit<FAR>(BlockGroup<256>{red_d, red_i, red_u}, pv, w, pp, dir, cell, id, tag, best, st, whl,
+                    reinterpret_cast<long long*>(bs.form), rw);
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
@@ -2589,16 +2788,16 @@ __global__ void k_labels_import(Labels l, int n, int m, const int* im, const flo
 // Every launch covers np pairs (blockIdx.z); grids are sized for the largest pair, and each block past its own
 // pair's pixels or windows does nothing.
 template <int ST>
-static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_cells, int stage,
+static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_cells, int stage, bool any_offsets,
                              const PlaneParams& pp, cudaStream_t st) {
     const int nc = max_cells;
+    const dim3 solve((2 * nc + 31) / 32, 1, np);
     if (s <= 16) {
         const dim3 fgrid((nc + kRansacWarps - 1) / kRansacWarps, 2, np), grid((nc + 7) / 8, 2, np);
-        if (s <= 8)
-            launch_kernel(k_ransac_warp<64>, fgrid, 32 * kRansacWarps, 0, st, bt, level, stage, pp);
-        else
-            launch_kernel(k_ransac_warp<256>, fgrid, 32 * kRansacWarps, 0, st, bt, level, stage, pp);
-        launch_kernel(k_refit_solve, dim3((2 * nc + 31) / 32, 1, np), 32, 0, st, bt, level, pp);
+        auto fit = [&](auto kernel) { launch_kernel(kernel, fgrid, 32 * kRansacWarps, 0, st, bt, level, stage, pp); };
+        fit(s <= 8 ? k_ransac_warp<64, false> : k_ransac_warp<256, false>);
+        if (any_offsets) fit(s <= 8 ? k_ransac_warp<64, true> : k_ransac_warp<256, true>);
+        launch_kernel(k_refit_solve, solve, 32, 0, st, bt, level, pp);
         launch_kernel(k_ransac_finish_warp<ST>, grid, 256, 0, st, bt, level, stage, pp);
         return;
     }
@@ -2606,24 +2805,24 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
     static bool attr_set = false;
     if (!attr_set) {
         const int mx = kMaxCell * kMaxCell * (int)sizeof(float4);  // the largest window's matches
-        cudaFuncSetAttribute(k_ransac_block<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_ransac_block<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        cudaFuncSetAttribute(k_ransac_finish_block<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+        for (auto* k : {k_ransac_block<256, false>, k_ransac_block<512, false>, k_ransac_block<256, true>,
+                        k_ransac_block<512, true>, k_ransac_finish_block<ST>})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
         attr_set = true;
     }
-    if (ransac_wide(s, 2 * nc * np))
-        launch_kernel(k_ransac_block<512>, dim3(nc, 2, np), 512, fit_smem, st, bt, level, stage, pp);
-    else
-        launch_kernel(k_ransac_block<256>, dim3(nc, 2, np), 256, fit_smem, st, bt, level, stage, pp);
-    launch_kernel(k_refit_solve, dim3((2 * nc + 31) / 32, 1, np), 32, 0, st, bt, level, pp);
+    const bool wide = ransac_wide(s, 2 * nc * np);
+    auto fit = [&](auto kernel) { launch_kernel(kernel, dim3(nc, 2, np), wide ? 512 : 256, fit_smem, st, bt, level, stage, pp); };
+    fit(wide ? k_ransac_block<512, false> : k_ransac_block<256, false>);
+    if (any_offsets) fit(wide ? k_ransac_block<512, true> : k_ransac_block<256, true>);
+    launch_kernel(k_refit_solve, solve, 32, 0, st, bt, level, pp);
     launch_kernel(k_ransac_finish_block<ST>, dim3(nc, 2, np), 256, smem, st, bt, level, stage, pp);
 }
-void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int stage, const PlaneParams& pp,
-                   cudaStream_t st) {
+void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int stage, bool any_offsets,
+                   const PlaneParams& pp, cudaStream_t st) {
     switch (pp.storage) {
-        case 0: launch_ransac_st<0>(bt, np, level, s, max_cells, stage, pp, st); break;
-        case 1: launch_ransac_st<1>(bt, np, level, s, max_cells, stage, pp, st); break;
-        case 2: launch_ransac_st<2>(bt, np, level, s, max_cells, stage, pp, st); break;
+        case 0: launch_ransac_st<0>(bt, np, level, s, max_cells, stage, any_offsets, pp, st); break;
+        case 1: launch_ransac_st<1>(bt, np, level, s, max_cells, stage, any_offsets, pp, st); break;
+        case 2: launch_ransac_st<2>(bt, np, level, s, max_cells, stage, any_offsets, pp, st); break;
     }
 }
 

@@ -86,3 +86,49 @@ def test_level0_sweeps_replace_far_incumbents(mark, motion):
         sure = ~cone.reshape(-1)
         assert sure.mean() > 0.5
         assert (got[d][:, 0] == vx)[sure].all() and (got[d][:, 1] == vy)[sure].all()
+
+
+def _marked(W, H, seed, mark, share):
+    """Two motions (left and right part) with a sixth of the offsets random, and a share of the pixels marked."""
+    rng = np.random.default_rng(seed)
+    y, x = np.mgrid[0:H, 0:W].astype(np.float64)
+    t = np.where((x < 0.6 * W)[..., None], np.stack([1.01 * x + 0.02 * y + 3, 0.99 * y - 0.015 * x - 2], -1),
+                 np.stack([x - 11 + 0.05 * y, y * 1.04 + 6], -1)) + rng.normal(0, 0.4, (H, W, 2))
+    t = np.where((rng.random((H, W)) < 1 / 6)[..., None], rng.random((H, W, 2)) * (W, H), t)
+    v = np.rint(t - np.stack([x, y], -1)).astype(np.int64)
+    v[rng.random((H, W)) < share] = mark
+    return np.ascontiguousarray(v.reshape(-1, 2).astype(np.int32))
+
+
+# windows of 8 and 16 px (a warp each), 18 px with 512 threads a window, and 18 px with 256 (more than 456 windows)
+@pytest.mark.parametrize("W,H,s,hyp", [(37, 29, 8, 96), (53, 41, 16, 128), (41, 30, 18, 96), (200, 160, 18, 257)])
+@pytest.mark.parametrize("share", [0.1, 0.55, 0.75])
+@pytest.mark.parametrize("mark", [1 << 20, -(1 << 20), 1 << 23, -(1 << 23), 1 << 30, -(1 << 30), -(1 << 31)])
+def test_planes_of_marked_fields_equal_oracle(mark, share, W, H, s, hyp):
+    """Markers are matches like any other: outliers of a window's motion, or its plane where they prevail."""
+    import torch
+
+    import oracle as O
+
+    from _parity import oracle_params, ransac_equal
+    gp = gpm.default_params(patch_radius=2, cells=(s,), pm_iters=0, num_hyp=hyp)
+    P = oracle_params(gp, W, H)
+    f = np.random.default_rng(s).random((H, W, 3)).astype(np.float32) * 0.2 + 0.4
+    nnf = np.stack([_marked(W, H, 10 * s + d, mark, share) for d in range(2)])
+    ctx = gpm.Context(gp, W, H)
+    fr = torch.from_numpy(f).cuda()
+    ctx.match([(fr, fr.clone())])
+    ctx.import_state(gpm.NNF, nnf, level=0)
+    ctx.fit_planes(1)
+    gmh, gmi = ctx.export(gpm.MODELS), ctx.export(gpm.MODEL_INFO)
+    ctx.close()
+    frame = np.asarray(f, np.float64)
+    first = np.arange(int(O.cell_base(P)[1])) * 2
+    for d in range(2):
+        mh, mi = O.empty_models(P)
+        vx, vy = (np.ascontiguousarray(nnf[d][:, c]) for c in range(2))
+        O.fit_level(P, frame, frame, d, 1, 1, vx, vy, None, mh, mi)
+        sure = first[(mi[first, O.MI_FLAGS] & O.F_AMBIG) == 0]
+        assert len(sure) > len(first) // 4
+        bad = sure[~ransac_equal(gmh[d], gmi[d], mh, mi, sure)]
+        assert len(bad) == 0, f"dir {d}: windows {bad // 2} differ"
