@@ -844,13 +844,22 @@ constexpr float kFarTarget = 1e15f;
 // Up to this |u + v - v0|, differences of targets stay below 2^15 and their cross products fit 32 bits.
 constexpr int kNearReach = kNearOffsets;
 
-// A target this far from v0 is out of reach: only a sample whose four targets are all far has it as an inlier.  Any other
-// hypothesis gets there only along its vanishing line, where a solve in FP64 is off by some q^2 2^-53 / (window side), a
-// pixel from about 2^28 on; a marker that a sample happens to hold then bends the line to itself, and counts for nothing.
+// A target this far from the sample's median target (sample_centre) is out of the hypothesis's reach, and no inlier.  It
+// gets there only along its vanishing line, where a solve in FP64 is off by some q^2 2^-53 / (window side), a pixel from
+// about 2^28 on: a marker that a sample happens to hold bends the line to itself, and counts for nothing.
 constexpr long long kFarthest = 1ll << 26;
-__device__ __forceinline__ bool out_of_reach(longlong2 q) { return max(llabs(q.x), llabs(q.y)) >= kFarthest; }
-// What the far matches of a window need (shared memory, one per window): how many, and how many of them are in reach, the
-// offsets in memory and the reference offset.
+__device__ __forceinline__ bool out_of_reach(longlong2 q, longlong2 centre) {
+    return max(llabs(q.x - centre.x), llabs(q.y - centre.y)) >= kFarthest;
+}
+// The second smallest of a sample's targets, by components: among three or four that are together.
+__device__ __forceinline__ longlong2 sample_centre(longlong2 a, longlong2 b, longlong2 c, longlong2 d) {
+    auto second = [](long long a, long long b, long long c, long long d) {
+        return min(max(min(a, b), min(c, d)), min(max(a, b), max(c, d)));
+    };
+    return make_longlong2(second(a.x, b.x, c.x, d.x), second(a.y, b.y, c.y, d.y));
+}
+// What the far matches of a window need (shared memory, one per window): how many, and how many of them are in reach of
+// near samples (a few more at the limit), the offsets in memory and the reference offset.
 struct WindowFar {
     const int2* nnf;
     int W, ox, oy, v0x, v0y, n, n_reach;
@@ -889,8 +898,26 @@ struct Window {
     }
 };
 
-// Gathers the window's matches (stage 1: every pixel; stage 2: the residual ones) into planes of `cap` floats.
+// For a window with far matches: the reference is moved to one of the eight matches (offset mx, my of the lane) if more are
+// near that one (planes still in integers).  Samples that mix places are bounded by how many matches are far: with at most
+// half of them, most are dropped by the bound.
 template <class G>
+__device__ __forceinline__ void choose_reference(const G& grp, const Window& w, int mx, int my, int& v0x, int& v0y) {
+    auto near = [&](int x, int y) {
+        int n = 0;
+        for (int j = grp.rank(); j < w.N; j += G::size)
+            n += max(llabs((long long)__float_as_int(w.qx[j]) - x), llabs((long long)__float_as_int(w.qy[j]) - y)) < kNearReach / 2;
+        return grp.sum(n);
+    };
+    int most = near(v0x, v0y);
+    for (int l = 0; l < 8 && 2 * most < w.N; ++l) {  // uniform over the window
+        const int x = __shfl_sync(FULL, mx, l), y = __shfl_sync(FULL, my, l), n = near(x, y);
+        if (n > most) most = n, v0x = x, v0y = y;
+    }
+}
+
+// Gathers the window's matches (stage 1: every pixel; stage 2: the residual ones) into planes of `cap` floats.
+template <bool FAR, class G>
 __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, const LevelGeom& g, int stage, int dir,
                                               int cell, float* planes, int cap, int pad, WindowFar* far, Window& w) {
     const int tid = grp.rank(), s = g.s, W = pv.W;
@@ -941,8 +968,9 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
         rx += a < mx || (a == mx && before);
         ry += b < my || (b == my && before);
     }
-    const int v0x = __shfl_sync(FULL, mx, __ffs(__ballot_sync(FULL, rx == 3)) - 1);
-    const int v0y = __shfl_sync(FULL, my, __ffs(__ballot_sync(FULL, ry == 3)) - 1);
+    int v0x = __shfl_sync(FULL, mx, __ffs(__ballot_sync(FULL, rx == 3)) - 1);
+    int v0y = __shfl_sync(FULL, my, __ffs(__ballot_sync(FULL, ry == 3)) - 1);
+    if constexpr (FAR) choose_reference(grp, w, mx, my, v0x, v0y);
     if (tid == 0) *far = WindowFar{nnf, W, ox, oy, v0x, v0y, 0, 0};
     grp.sync();
     unsigned vm = 0, vq = 0;
@@ -958,7 +986,7 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
         if (near)
             vq = max(vq, (unsigned)max(abs(bx), abs(by)));
         else  // rounded: at the limit it may count as in reach without being so
-            n_far += fmaxf(fabsf((float)vx - (float)v0x), fabsf((float)vy - (float)v0y)) > 1.01f * (float)kFarthest ? 1 : 0x10001;
+            n_far += fmaxf(fabsf((float)vx - (float)v0x), fabsf((float)vy - (float)v0y)) > 1.02f * (float)kFarthest ? 1 : 0x10001;
         w.qx[j] = near ? (float)bx : kFarTarget;
         w.qy[j] = near ? (float)by : kFarTarget;
     }
@@ -1016,22 +1044,22 @@ __device__ __forceinline__ bool draw_exact(const Window& w, int cell, int k, uin
 
 // Hypothesis k of a window with far matches, whose targets are read from their own integers, as its FP64 and its evaluation
 // form; false also if the targets are too far apart for the products (sample_in_range) or the denominator is 0 at the
-// centre.  all_far: whether all of the sample's targets are.  Out of line.
+// centre.  middle: sample_centre.  Out of line.
 __device__ __noinline__ bool solve_far(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id, uint32_t k0,
-                                       uint32_t k1, double* Hl, Mef& m, bool& all_far) {
+                                       uint32_t k1, double* Hl, Mef& m, longlong2& middle) {
     int idx[4], px[4], py[4];
     int64_t qx[4], qy[4];
     draw_indices(w.N, cell, k, tag, pair_id, k0, k1, idx);
-    all_far = true;
 #pragma unroll 1
     for (int j = 0; j < 4; ++j) {
         px[j] = exact_int(w.x[idx[j]]);
         py[j] = exact_int(w.y[idx[j]]);
-        all_far = all_far && w.is_far(idx[j]);
         const longlong2 q = w.target(idx[j]);
         qx[j] = q.x;
         qy[j] = q.y;
     }
+    auto q = [&](int j) { return make_longlong2(qx[j], qy[j]); };
+    middle = sample_centre(q(0), q(1), q(2), q(3));
     bool degen = false;
 #pragma unroll 1
     for (int t = 0; t < 4; ++t) {
@@ -1051,61 +1079,38 @@ __device__ __noinline__ bool solve_far(const Window& w, int cell, int k, uint32_
 // relative to v0 times den, X(u) = xc + x0 ux + x1 uy and Y(u) likewise, and kap, a bound of everything rounding
 // can do to the inlier test: with n = (X - qx den, Y - qy den), an inlier has |n| < t den, so it passes
 // |n| <= t den + kap as computed, and a match that passes |n| < t den - kap as computed is an inlier.  kap is for the
-// near matches; far_allowance and far_maybe derive the far ones' from it.
+// near matches.  For a far one (FAR only) it is 1.2 kap + far_kap |q|_1; away: the sample's centre is far.
 struct FastHyp {
-    float g0, g1, c0, kap, x0, x1, xc, pad0, y0, y1, yc, pad1;
+    float g0, g1, c0, kap, x0, x1, xc, far_kap, y0, y1, yc;
+    int away;
 };
 enum { HYP_DEAD = 0, HYP_OK = 1, HYP_LOOSE = 2 };  // degenerate; scored in FP32; the FP32 form says too little
 // t widened by 2^-20: covers the relative roundings of both sides of the comparison (at most 6 units of 2^-24).
 __device__ __forceinline__ float t_above(float t2) { return sqrtf(t2) * (1.f + 9.5367431640625e-07f); }
 __device__ __forceinline__ float t_below(float t2) { return sqrtf(t2) * (1.f - 9.5367431640625e-07f); }
 
-// Draws hypothesis k and solves it in FP32.  Relative to the fourth pair, with the cross products l_k, mu_k of
-// hyp_exact.cuh (exact: floats below 2^24 and 32-bit integers) and rho_k = mu_k / (M l_k), M = sum mu, the form's
+// A hypothesis solved in FP32.  Relative to the fourth pair (p3, q3), with the cross products l_k, mu_k of
+// hyp_exact.cuh (exact: floats below 2^24 and integers) and rho_k = mu_k / (M l_k), M = sum mu, the form's
 // coefficients are sums over k of rho_k (dy_i - dy_j), rho_k (dx_j - dx_i) and their products with the target
-// differences, normalised to 1 at p3.  The degeneracy test is exact: the eight triangle areas are the l_k, the mu_k
-// and their sums.
+// differences, normalised to 1 at p3.
 // Rounding, in units of u = 2^-24, first order: mu, M, M l one each, the division 4 (2 ulp): rho 7; a product with
 // an exact integer 8, the sums 11 (g) and 12 (h00..h11).  With e_k = |rho_k| (|dy_i - dy_j| + |dx_j - dx_i|),
 // S = U sum e_k and SQ = U sum e_k (|X_k| + |Y_k|): den carries at most 28 (1 + S), X and Y together at most
 // 32 (SQ + |q3|_1 (1 + S)), n in addition |q|_1 28 (1 + S).  A match that can pass has
 // |q|_1 <= (|X| + |Y|) / den + 2 t, which the window's extremes of the form bound where den stays positive; else
 // the window's largest |q| does.  (34 and 30 below leave the second order room.)
-template <bool FAR>
-__device__ __forceinline__ int fast_hypothesis(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id,
-                                               uint32_t k0, uint32_t k1, float t, FastHyp& h) {
-    int idx[4];
-    draw_indices(w.N, cell, k, tag, pair_id, k0, k1, idx);
-    if (FAR && (w.is_far(idx[0]) || w.is_far(idx[1]) || w.is_far(idx[2]) || w.is_far(idx[3]))) return HYP_LOOSE;
-    const float p3x = w.x[idx[3]], p3y = w.y[idx[3]], q3x = w.qx[idx[3]], q3y = w.qy[idx[3]];
-    float dx[3], dy[3], X[3], Y[3], l[3];
-    int Xi[3], Yi[3], mu[3];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        dx[j] = w.x[idx[j]] - p3x;
-        dy[j] = w.y[idx[j]] - p3y;
-        X[j] = w.qx[idx[j]] - q3x;
-        Y[j] = w.qy[idx[j]] - q3y;
-        Xi[j] = exact_int(X[j]);
-        Yi[j] = exact_int(Y[j]);
-    }
-    bool degen = false;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const int a = (j + 1) % 3, b = (j + 2) % 3;
-        l[j] = dx[a] * dy[b] - dx[b] * dy[a];
-        mu[j] = Xi[a] * Yi[b] - Xi[b] * Yi[a];
-        degen |= l[j] == 0.f || mu[j] == 0;
-    }
-    const int M = (int)((unsigned)mu[0] + (unsigned)mu[1] + (unsigned)mu[2]);
-    if (degen || l[0] + l[1] + l[2] == 0.f || M == 0) return HYP_DEAD;
-    const float Mf = (float)M;
+// FAR_SAMPLE: mu and M are within 2 units and the target differences are rounded themselves, which makes 15 of the 12
+// above: the bounds are taken half as large again.
+template <bool FAR, bool FAR_SAMPLE>
+__device__ __forceinline__ int solve_form(const Window& w, float p3x, float p3y, float q3x, float q3y, const float (&dx)[3],
+                                          const float (&dy)[3], const float (&X)[3], const float (&Y)[3],
+                                          const float (&l)[3], const float (&mu)[3], float M, float t, FastHyp& h) {
     float S = 0.f, SQ = 0.f, h00 = 0.f, h01 = 0.f, h10 = 0.f, h11 = 0.f;
     h.g0 = h.g1 = 0.f;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         const int a = (j + 1) % 3, b = (j + 2) % 3;
-        const float rho = __fdividef((float)mu[j], Mf * l[j]);
+        const float rho = __fdividef(mu[j], M * l[j]);
         const float al = rho * (dy[a] - dy[b]), be = rho * (dx[b] - dx[a]);
         const float e = fabsf(al) + fabsf(be);
         S += e;
@@ -1124,7 +1129,7 @@ __device__ __forceinline__ int fast_hypothesis(const Window& w, int cell, int k,
     h.y0 = fmaf(q3y, h.g0, h10);
     h.y1 = fmaf(q3y, h.g1, h11);
     h.yc = fmaf(-h11, p3y, fmaf(-h10, p3x, q3y * h.c0));
-    const float u = 5.9604644775390625e-08f, U = w.U;
+    const float u = (FAR_SAMPLE ? 1.5f : 1.f) * 5.9604644775390625e-08f, U = w.U;
     const float one = fmaf(U, S, 1.f), ed = 30.f * u * one;
     const float dc = h.c0 - 0.5f * (h.g0 + h.g1);
     if (!(fabsf(dc) > 2.f * ed)) return HYP_LOOSE;  // its orientation needs the exact form
@@ -1140,7 +1145,92 @@ __device__ __forceinline__ int fast_hypothesis(const Window& w, int cell, int k,
         Q = fminf(Q, __fdividef(1.05f * XY + t, dmin) + 2.2f * t);
     }
     h.kap = 1.0001f * fmaf(34.f * u, fmaf(fabsf(q3x) + fabsf(q3y) + Q, one, SQ * U), t * ed);
-    return h.kap < 1e6f ? HYP_OK : HYP_LOOSE;  // a wide bound still excludes most; NaN: loose
+    if (FAR) h.far_kap = 40.f * u * one;  // the target rounded itself; the rest of kap grows from 34 to 40 u
+    // a wide bound still excludes most (far targets are up to 2^18 times as far); NaN: loose
+    return h.kap < (FAR_SAMPLE ? 1e14f : 1e6f) ? HYP_OK : HYP_LOOSE;
+}
+
+// A sample with far targets, solved relative to a near one, so that q3 is small and the far targets' differences come with
+// a small rho_k of their own: the bound is not much wider than for near samples.  With targets out of reach of each other
+// it is solved relative to the one next to the centre, since three of them together make every rho_k large otherwise.
+// 512x384 planes (3.67 ms without markers) with 15 and 50 % at 2^20: 42 -> 9.3 and 287 -> 76 ms; at 2^30, 50 %: 68.
+__device__ __forceinline__ int far_hypothesis(const Window& w, const int (&idx)[4], float t, FastHyp& h) {
+    longlong2 q[4];
+    bool apart = false, any_near = false;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        q[j] = w.target(idx[j]);
+        apart = apart || out_of_reach(q[j], make_longlong2(0, 0));
+        any_near = any_near || !w.is_far(idx[j]);
+    }
+    const longlong2 c = sample_centre(q[0], q[1], q[2], q[3]);
+    h.away = max(llabs(c.x), llabs(c.y)) > kNearReach;
+    const longlong2 at = apart || !any_near ? c : make_longlong2(0, 0);
+    int r = 0, i3 = idx[0];
+    longlong2 q3 = q[0];
+#pragma unroll
+    for (int j = 1; j < 4; ++j)
+        if (llabs(q[j].x - at.x) + llabs(q[j].y - at.y) < llabs(q3.x - at.x) + llabs(q3.y - at.y)) r = j, i3 = idx[j], q3 = q[j];
+    const float p3x = w.x[i3], p3y = w.y[i3];
+    float dx[3], dy[3], X[3], Y[3], l[3], mu[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int i = j == r ? idx[3] : idx[j];
+        if (j == r) q[j] = q[3];
+        dx[j] = w.x[i] - p3x;
+        dy[j] = w.y[i] - p3y;
+        X[j] = (float)(q[j].x - q3.x);
+        Y[j] = (float)(q[j].y - q3.y);
+    }
+    i128 M = 0;
+    bool degen = false;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int a = (j + 1) % 3, b = (j + 2) % 3;
+        const i128 m = (i128)(q[a].x - q3.x) * (q[b].y - q3.y) - (i128)(q[b].x - q3.x) * (q[a].y - q3.y);
+        l[j] = dx[a] * dy[b] - dx[b] * dy[a];
+        M += m;
+        mu[j] = i128_to_float(m);
+        degen |= l[j] == 0.f || m == 0;
+    }
+    if (degen || l[0] + l[1] + l[2] == 0.f || M == 0) return HYP_DEAD;
+    return solve_form<true, true>(w, p3x, p3y, (float)q3.x, (float)q3.y, dx, dy, X, Y, l, mu, i128_to_float(M), t, h);
+}
+
+// Draws hypothesis k and solves it in FP32.  The degeneracy test is exact: the eight triangle areas are the l_k, the mu_k
+// and their sums.
+template <bool FAR>
+__device__ __forceinline__ int fast_hypothesis(const Window& w, int cell, int k, uint32_t tag, uint32_t pair_id,
+                                               uint32_t k0, uint32_t k1, float t, FastHyp& h) {
+    int idx[4];
+    draw_indices(w.N, cell, k, tag, pair_id, k0, k1, idx);
+    if (FAR && (w.is_far(idx[0]) || w.is_far(idx[1]) || w.is_far(idx[2]) || w.is_far(idx[3])))
+        return far_hypothesis(w, idx, t, h);
+    if (FAR) h.away = 0;
+    const float p3x = w.x[idx[3]], p3y = w.y[idx[3]], q3x = w.qx[idx[3]], q3y = w.qy[idx[3]];
+    float dx[3], dy[3], X[3], Y[3], l[3], mu[3];
+    int Xi[3], Yi[3], M = 0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        dx[j] = w.x[idx[j]] - p3x;
+        dy[j] = w.y[idx[j]] - p3y;
+        X[j] = w.qx[idx[j]] - q3x;
+        Y[j] = w.qy[idx[j]] - q3y;
+        Xi[j] = exact_int(X[j]);
+        Yi[j] = exact_int(Y[j]);
+    }
+    bool degen = false;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int a = (j + 1) % 3, b = (j + 2) % 3;
+        l[j] = dx[a] * dy[b] - dx[b] * dy[a];
+        const int m = Xi[a] * Yi[b] - Xi[b] * Yi[a];
+        M = (int)((unsigned)M + (unsigned)m);
+        mu[j] = (float)m;
+        degen |= l[j] == 0.f || m == 0;
+    }
+    if (degen || l[0] + l[1] + l[2] == 0.f || M == 0) return HYP_DEAD;
+    return solve_form<FAR, false>(w, p3x, p3y, q3x, q3y, dx, dy, X, Y, l, mu, (float)M, t, h);
 }
 
 // The form of a hypothesis with every coefficient in both halves of a pair, for tests of two matches per
@@ -1190,23 +1280,23 @@ __device__ __forceinline__ void test_match(const Window& w, const FastHyp& h, fl
 }
 
 // How many far matches a scored hypothesis may have as inliers: those in reach, unless its targets in the window stay near
-// (the bound on them in fast_hypothesis, with kap / t for ed, which is below it).
+// (the bound on them in solve_form, with kap / t for ed, which is below it).
 __device__ __forceinline__ int far_allowance(const Window& w, const FastHyp& h, float t) {
+    if (h.away) return w.far->n;
     const float dmin = h.c0 - (fabsf(h.g0) + fabsf(h.g1)) * w.U - 2.f * h.kap / t;
     const float XY = fabsf(h.xc) + fabsf(h.yc) + (fabsf(h.x0) + fabsf(h.x1) + fabsf(h.y0) + fabsf(h.y1)) * w.U;
     return dmin > 0.f && 1.05f * XY + t + 2.2f * t * dmin < 0.999f * (float)kNearReach * dmin ? 0 : w.far->n_reach;
 }
-// Whether a far match can be an inlier of a scored hypothesis.  Its bound: with one = 1 + U S, kap is at least
-// 34 u (|q3|_1 one + SQ U) + 30 u t one, so for a target q, rounded to floats itself,
-// 40 u ((|q3|_1 + |q|_1) one + SQ U) + 30 u t one is at most kap (1.2 + 1.34 |q|_1 / t).
+// Whether a far match can be an inlier of a scored hypothesis.
 __device__ __forceinline__ bool far_maybe(const Window& w, const FastHyp& h, float t, int j) {
     const longlong2 q = w.far_target(j);
     const float ux = w.x[j], uy = w.y[j], qx = (float)q.x, qy = (float)q.y;
     const float den = fmaf(h.g1, uy, fmaf(h.g0, ux, h.c0));
     const float nx = fmaf(-qx, den, fmaf(h.x1, uy, fmaf(h.x0, ux, h.xc)));
     const float ny = fmaf(-qy, den, fmaf(h.y1, uy, fmaf(h.y0, ux, h.yc)));
-    const float a = fmaf(t, den, h.kap * (1.21f + 1.35f * (fabsf(qx) + fabsf(qy)) / t));
-    return !out_of_reach(q) && a > 0.f && fmaf(nx, nx, ny * ny) < a * a;
+    const float a = fmaf(t, den, 1.001f * fmaf(h.far_kap, fabsf(qx) + fabsf(qy), 1.2f * h.kap));
+    const bool reach = h.away || fmaxf(fabsf(qx), fabsf(qy)) < 1.01f * (float)kFarthest;
+    return reach && a > 0.f && fmaf(nx, nx, ny * ny) < a * a;
 }
 
 // The order of two hypotheses: more inliers, then the lower index.  Zero is below every hypothesis.
@@ -1228,10 +1318,10 @@ __device__ __forceinline__ bool exact_inlier(const Mef& m, const double* Hl, con
     return hyp_inlier_fp64(Hl, mt.x, mt.y, mt.z, mt.w, (double)t2);
 }
 
-// The test of any match by a hypothesis in FP64 (all_far: of its sample), a far one from its own integers.
-__device__ __forceinline__ bool inlier_fp64(const Window& w, const double* Hl, bool all_far, int j, float t2) {
+// The test of any match by a hypothesis in FP64 (middle: its sample's centre), a far one from its own integers.
+__device__ __forceinline__ bool inlier_fp64(const Window& w, const double* Hl, longlong2 middle, int j, float t2) {
     const longlong2 q = w.target(j);
-    return (all_far || !out_of_reach(q)) &&
+    return !out_of_reach(q, middle) &&
            hyp_inlier_fp64(Hl, (double)w.x[j], (double)w.y[j], (double)q.x, (double)q.y, (double)t2);
 }
 
@@ -1249,9 +1339,9 @@ __device__ __noinline__ int exact_support(const Window& w, int cell, int k, uint
     const int lane = threadIdx.x & 31;
     double Hl[9];
     Mef m;
-    bool all_far = false;
+    longlong2 middle = make_longlong2(0, 0);
     if constexpr (FAR) {
-        if (!solve_far(w, cell, k, tag, pair_id, k0, k1, Hl, m, all_far)) return -1;
+        if (!solve_far(w, cell, k, tag, pair_id, k0, k1, Hl, m, middle)) return -1;
     } else {
         i128 Hk[9];
         if (!draw_exact(w, cell, k, tag, pair_id, k0, k1, Hk) || !make_mef_exact(Hk, m)) return -1;
@@ -1264,9 +1354,9 @@ __device__ __noinline__ int exact_support(const Window& w, int cell, int k, uint
         for (int j = c + lane; j < c + 128 + lane; j += 32) {
             bool in = false;
             if (FAR && j < w.N && w.is_far(j)) {
-                in = inlier_fp64(w, Hl, all_far, j, t2);
+                in = inlier_fp64(w, Hl, middle, j, t2);
                 ++f;
-            } else if (j < w.N) {
+            } else if (j < w.N && !(FAR && out_of_reach(w.target(j), middle))) {
                 in = exact_inlier(m, Hl, w.match(j), t2, f);
             }
             score += __popc(__ballot_sync(FULL, in));
@@ -1293,7 +1383,7 @@ __device__ __noinline__ int contender_support(const Window& w, const FastHyp* fo
             maybe = far_maybe(w, h, th, j);
         else
             test_match(w, h, tl, th, j, sure, maybe);
-        lo += sure;
+        lo += sure && !(FAR && h.away);  // it may be out of reach
         hi += maybe;
     }
     lo = (int)__reduce_add_sync(FULL, (unsigned)lo);
@@ -1465,12 +1555,12 @@ __device__ __forceinline__ unsigned long long far_winner(const G& grp, const Win
     const int tid = grp.rank();
     double Hl[9];
     Mef m;
-    bool all_far;
-    solve_far(w, cell, k, tag, pair_id, k0, k1, Hl, m, all_far);
+    longlong2 middle;
+    solve_far(w, cell, k, tag, pair_id, k0, k1, Hl, m, middle);
     unsigned long long inm = 0;
     bool far = false;
     for (int j = tid, c = 0; j < w.N; j += G::size, ++c)
-        if (inlier_fp64(w, Hl, all_far, j, t2)) {
+        if (inlier_fp64(w, Hl, middle, j, t2)) {
             inm |= 1ull << c;
             far = far || w.is_far(j);
         }
@@ -1779,7 +1869,7 @@ __device__ __forceinline__ unsigned long long search_block(const BlockGroup<NT>&
                 for (int j = tid; j < N; j += NT) {
                     bool sure, maybe;
                     test_match(w, h, tl, t, j, sure, maybe);
-                    lo += sure;
+                    lo += sure && !(FAR && h.away);
                 }
                 lo = grp.sum(lo);
                 if (tid == 0) bs.best = max(bs.best, hyp_key(lo, key_index(lead)));
@@ -2121,7 +2211,7 @@ __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     RefitWork* rw = pv.rw[dir] + cell;
     if (FAR && rw->status != kFarPending) return;
     Window w;
-    gather_window(grp, pv, g, stage, dir, cell, planes[warp], CAP, 4, &far[warp], w);
+    gather_window<FAR>(grp, pv, g, stage, dir, cell, planes[warp], CAP, 4, &far[warp], w);
     if (grp.rank() == 0) clear_model(pv, dir, id, w.N, rw);
     if (w.N < pp.min_inliers || w.N < 4) return;
     if (!FAR && w.far->n) {
@@ -2173,7 +2263,7 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __g
     RefitWork* rw = pv.rw[dir] + cell;
     if (FAR && rw->status != kFarPending) return;  // block-uniform: cleared behind the barriers of gather_window
     Window w;
-    gather_window(grp, pv, g, stage, dir, cell, planes_dyn, block_cap(g.s), 128, &far, w);
+    gather_window<FAR>(grp, pv, g, stage, dir, cell, planes_dyn, block_cap(g.s), 128, &far, w);
     if (threadIdx.x == 0) clear_model(pv, dir, id, w.N, rw);
     if (w.N < pp.min_inliers || w.N < 4) return;
     if (!FAR && w.far->n) {

@@ -132,3 +132,40 @@ def test_planes_of_marked_fields_equal_oracle(mark, share, W, H, s, hyp):
         assert len(sure) > len(first) // 4
         bad = sure[~ransac_equal(gmh[d], gmi[d], mh, mi, sure)]
         assert len(bad) == 0, f"dir {d}: windows {bad // 2} differ"
+
+
+def test_far_windows_are_fitted_by_graphs_captured_before_an_import():
+    """A fit captured before the field is imported serves far windows all the same; whole runs, which replace the field, take
+    the launches of before once more afterwards."""
+    import torch
+    W, H, s = 53, 41, 16
+    gp = gpm.default_params(patch_radius=2, cells=(s,), pm_iters=0, num_hyp=64)
+    f = torch.from_numpy(np.random.default_rng(3).random((H, W, 3)).astype(np.float32)).cuda()
+    nnf = np.stack([_marked(W, H, 7 + d, 1 << 20, 0.2) for d in range(2)])
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(st):
+        ctx = gpm.Context(gp, W, H, stream=st)
+        counts = []
+        for _ in range(2):
+            n = ctx.launch_count()
+            ctx.run([(f, f)])
+            counts.append(ctx.launch_count() - n)
+            ctx.match([(f, f)])
+            ctx.import_state(gpm.NNF, nnf, level=0)
+            ctx.fit_planes(1)
+            want = ctx.export(gpm.MODEL_INFO), ctx.export(gpm.MODELS)
+        assert counts[0] == counts[1]
+        ctx.close()
+        ctx = gpm.Context(gp, W, H, stream=st)
+        ctx.match([(f, f)])
+        ctx.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            ctx.fit_planes(1)
+        ctx.import_state(gpm.NNF, nnf, level=0)
+        g.replay()
+        got = ctx.export(gpm.MODEL_INFO), ctx.export(gpm.MODELS)
+        ctx.close()
+    assert (want[0][:, ::2, 1] > 0).any()  # inliers: the cues drop these planes later
+    assert (got[0] == want[0]).all() and (got[1] == want[1]).all()
