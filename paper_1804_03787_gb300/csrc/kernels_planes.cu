@@ -3,6 +3,8 @@
 // propagation fill and the final flow / occlusion map.
 #include <float.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "hyp_exact.cuh"
 #include "kernels.h"
@@ -2877,6 +2879,22 @@ __global__ void k_labels_import(Labels l, int n, int m, const int* im, const flo
 // ---------------------------------------------------------------- launchers
 // Every launch covers np pairs (blockIdx.z); grids are sized for the largest pair, and each block past its own
 // pair's pixels or windows does nothing.
+// Launches a kernel whose windows' matches are in dynamic shared memory.  Its limit is raised before the first launch on each
+// device, by whichever thread comes first.
+template <auto KERNEL>
+static void launch_windows(dim3 grid, unsigned threads, size_t shared, cudaStream_t st, const Batch& bt, int level, int stage,
+                           const PlaneParams& pp) {
+    static std::atomic<unsigned long long> raised{0};  // bit d: on device d
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (!(raised.load(std::memory_order_acquire) & bit)) {
+        const int largest = kMaxCell * kMaxCell * (int)sizeof(float4);
+        if (cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, largest) == cudaSuccess)
+            raised.fetch_or(bit, std::memory_order_release);
+    }
+    launch_kernel(KERNEL, grid, threads, shared, st, bt, level, stage, pp);
+}
 template <int ST>
 static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_cells, int stage, bool any_offsets,
                              const PlaneParams& pp, cudaStream_t st) {
@@ -2892,20 +2910,16 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
         return;
     }
     const size_t smem = (size_t)s * s * sizeof(float4), fit_smem = (size_t)block_cap(s) * sizeof(float4);
-    static bool attr_set = false;
-    if (!attr_set) {
-        const int mx = kMaxCell * kMaxCell * (int)sizeof(float4);  // the largest window's matches
-        for (auto* k : {k_ransac_block<256, false>, k_ransac_block<512, false>, k_ransac_block<256, true>,
-                        k_ransac_block<512, true>, k_ransac_finish_block<ST>})
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-        attr_set = true;
+    const dim3 grid(nc, 2, np);
+    if (ransac_wide(s, 2 * nc * np)) {
+        launch_windows<k_ransac_block<512, false>>(grid, 512, fit_smem, st, bt, level, stage, pp);
+        if (any_offsets) launch_windows<k_ransac_block<512, true>>(grid, 512, fit_smem, st, bt, level, stage, pp);
+    } else {
+        launch_windows<k_ransac_block<256, false>>(grid, 256, fit_smem, st, bt, level, stage, pp);
+        if (any_offsets) launch_windows<k_ransac_block<256, true>>(grid, 256, fit_smem, st, bt, level, stage, pp);
     }
-    const bool wide = ransac_wide(s, 2 * nc * np);
-    auto fit = [&](auto kernel) { launch_kernel(kernel, dim3(nc, 2, np), wide ? 512 : 256, fit_smem, st, bt, level, stage, pp); };
-    fit(wide ? k_ransac_block<512, false> : k_ransac_block<256, false>);
-    if (any_offsets) fit(wide ? k_ransac_block<512, true> : k_ransac_block<256, true>);
     launch_kernel(k_refit_solve, solve, 32, 0, st, bt, level, pp);
-    launch_kernel(k_ransac_finish_block<ST>, dim3(nc, 2, np), 256, smem, st, bt, level, stage, pp);
+    launch_windows<k_ransac_finish_block<ST>>(grid, 256, smem, st, bt, level, stage, pp);
 }
 void launch_ransac(const Batch& bt, int np, int level, int s, int max_cells, int stage, bool any_offsets,
                    const PlaneParams& pp, cudaStream_t st) {
