@@ -118,36 +118,6 @@ __device__ __forceinline__ float4 ldpix_shared<2>(const void* base, int i) {
     return make_float4(a.x, a.y, b.x, b.y);
 }
 
-// A texel at a shared-memory byte address (a 32-bit shared-window address, as from __cvta_generic_to_shared).
-template <int ST>
-__device__ __forceinline__ float4 ldpix_shared_addr(unsigned addr);
-template <>
-__device__ __forceinline__ float4 ldpix_shared_addr<0>(unsigned addr) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
-    return v;
-}
-template <int ST>
-__device__ __forceinline__ uint2 ld_shared_u2(unsigned addr) {
-    uint2 u;
-    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(u.x), "=r"(u.y) : "r"(addr));
-    return u;
-}
-template <>
-__device__ __forceinline__ float4 ldpix_shared_addr<1>(unsigned addr) {
-    const uint2 u = ld_shared_u2<1>(addr);
-    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
-    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-}
-template <>
-__device__ __forceinline__ float4 ldpix_shared_addr<2>(unsigned addr) {
-    const uint2 u = ld_shared_u2<2>(addr);
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
-    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-}
-
 // Bilinear blend of the four texels around a point with fractions (fx, fy).
 __device__ __forceinline__ float3 blend4(float4 a, float4 b, float4 c, float4 d, float fx, float fy) {
     const float gx = 1.f - fx, gy = 1.f - fy;

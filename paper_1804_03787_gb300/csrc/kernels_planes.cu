@@ -23,11 +23,6 @@ __device__ __forceinline__ bool collinear3(int ax, int ay, int bx, int by, int c
     return (long long)(bx - ax) * (cy - ay) - (long long)(by - ay) * (cx - ax) == 0;
 }
 
-__device__ __forceinline__ void mat3_mul(const double* A, const double* B, double* C) {
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j) C[i * 3 + j] = A[i * 3] * B[j] + A[i * 3 + 1] * B[3 + j] + A[i * 3 + 2] * B[6 + j];
-}
-
 // X = i + f (f in [0,1)) lies in [-kFrameTol, n - 1 + kFrameTol].
 __device__ __forceinline__ bool in_frame_tol(int i, float f, int n) {
     if (i >= 0 && i < n - 1) return true;
@@ -104,11 +99,6 @@ struct WarpGroup {
     static constexpr int size = 32;
     __device__ int rank() const { return threadIdx.x & 31; }
     __device__ void sync() const { __syncwarp(); }
-    __device__ double sum(double v) const {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-        return v;
-    }
     __device__ int sum(int v) const { return (int)__reduce_add_sync(FULL, (unsigned)v); }
     __device__ unsigned max(unsigned v) const { return __reduce_max_sync(FULL, v); }
     __device__ bool any(bool p) const { return __any_sync(FULL, p); }
@@ -123,21 +113,10 @@ struct WarpGroup {
 template <int NT>
 struct BlockGroup {
     static constexpr int size = NT;
-    double* red_d;
     int* red_i;
     unsigned long long* red_u;
     __device__ int rank() const { return threadIdx.x; }
     __device__ void sync() const { __syncthreads(); }
-    __device__ double sum(double v) const {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) red_d[threadIdx.x >> 5] = v;
-        __syncthreads();
-        double t = 0;
-        for (int w = 0; w < NT / 32; ++w) t += red_d[w];  // fixed order: same bits on every thread
-        return t;
-    }
     __device__ int sum(int v) const {
         v = (int)__reduce_add_sync(FULL, (unsigned)v);
         __syncthreads();
@@ -2254,13 +2233,12 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __g
     const int cell = blockIdx.x, dir = blockIdx.y;
     if (cell >= g.ncells()) return;  // past this pair's windows (block-uniform)
     extern __shared__ __align__(16) float planes_dyn[];
-    __shared__ double red_d[NT / 32];
     __shared__ int red_i[NT / 32];
     __shared__ unsigned long long red_u[NT / 32];
     __shared__ __align__(16) BlockSearch bs;
     __shared__ double whl[16];  // also two sums per warp
     __shared__ WindowFar far;
-    const BlockGroup<NT> grp{red_d, red_i, red_u};
+    const BlockGroup<NT> grp{red_i, red_u};
     const int id = (g.base + cell) * 2 + (stage - 1);
     RefitWork* rw = pv.rw[dir] + cell;
     if (FAR && rw->status != kFarPending) return;  // block-uniform: cleared behind the barriers of gather_window
@@ -2285,7 +2263,7 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __g
         }
         return;
     }
-    finish_fit<FAR>(BlockGroup<256>{red_d, red_i, red_u}, pv, w, pp, dir, cell, id, tag, best, st, whl,
+    finish_fit<FAR>(BlockGroup<256>{red_i, red_u}, pv, w, pp, dir, cell, id, tag, best, st, whl,
                     reinterpret_cast<long long*>(bs.form), rw);
 }
 template <int ST>
@@ -2295,10 +2273,9 @@ __global__ void __launch_bounds__(256) k_ransac_finish_block(const __grid_consta
     const LevelGeom g = bt.geom(blockIdx.z, level);
     if ((int)blockIdx.x >= g.ncells()) return;  // past this pair's windows (block-uniform)
     extern __shared__ float4 match_dyn[];
-    __shared__ double red_d[8];
     __shared__ int red_i[8];
     __shared__ unsigned long long red_u[8];
-    BlockGroup<256> grp{red_d, red_i, red_u};
+    BlockGroup<256> grp{red_i, red_u};
     ransac_finish<BlockGroup<256>, ST>(grp, pv, g, stage, pp, blockIdx.y, blockIdx.x, match_dyn);
 }
 

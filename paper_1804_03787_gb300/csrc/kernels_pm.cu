@@ -576,7 +576,7 @@ __device__ __forceinline__ int abandon_threshold(float thr) {
 // function returns false.  Each lane accumulates its taps in the same order
 // as patch_sum and the total is warp_sum_q24's, so a full sum is bitwise the
 // same as patch_sum's.
-template <int R, int ST, bool IN, bool EVERY_CHUNK>
+template <int R, int ST, bool IN>
 __device__ __forceinline__ bool tap_sum_in(const LanePatch<R>& lp, const void* tgt, int W, int H, int2 c, int ithr,
                                         float& sum, int& nch, int lane) {
     const int off = c.y * W + c.x;
@@ -585,7 +585,7 @@ __device__ __forceinline__ bool tap_sum_in(const LanePatch<R>& lp, const void* t
     for (int j = 0; j < Patch<R>::NT; ++j) {
         const int t = lane + 32 * j;
         if (t < Patch<R>::T) s += absdiff3(lp.a[j], tap_sample<R, ST, IN>(lp, tgt, W, H, j, c, off));
-        if (j + 1 < Patch<R>::NT && EVERY_CHUNK) {
+        if (j + 1 < Patch<R>::NT) {
             // floor(min(s * 2^19, 2^23 - 1)): exact scaling, clamp (keeps a lower bound), truncation in the
             // mantissa of 2^23
             const unsigned q =
@@ -600,14 +600,13 @@ __device__ __forceinline__ bool tap_sum_in(const LanePatch<R>& lp, const void* t
     nch = Patch<R>::NT;
     return true;
 }
-// EVERY_CHUNK: test the bound after every chunk but the last (plane levels, where a chunk costs four gathers per
-// tap); otherwise never (level 0, where the patch-sum bound has already removed most losing candidates and a
-// test, with its reduction and the predication it puts on every later gather, cost more than it saved).
-template <int R, int ST, bool EVERY_CHUNK>
+// For the plane levels, where a chunk costs four gathers per tap (level 0 sums in full: the patch-sum bound has
+// already removed most losing candidates there).
+template <int R, int ST>
 __device__ __forceinline__ bool tap_sum(const LanePatch<R>& lp, const void* tgt, int W, int H, int2 c, int ithr,
                                         float& sum, int& nch, int lane) {
-    return interior_of<R>(lp, c) ? tap_sum_in<R, ST, true, EVERY_CHUNK>(lp, tgt, W, H, c, ithr, sum, nch, lane)
-                                 : tap_sum_in<R, ST, false, EVERY_CHUNK>(lp, tgt, W, H, c, ithr, sum, nch, lane);
+    return interior_of<R>(lp, c) ? tap_sum_in<R, ST, true>(lp, tgt, W, H, c, ithr, sum, nch, lane)
+                                 : tap_sum_in<R, ST, false>(lp, tgt, W, H, c, ithr, sum, nch, lane);
 }
 
 // A candidate offset in one word (|c.x|, |c.y| < 2^15 for frames below 2^15 pixels a side).
@@ -1028,7 +1027,7 @@ __global__ void __launch_bounds__(256, 4) k_pm_sweep(const __grid_constant__ Bat
                 } else {
                     float sum;
                     int nch;
-                    const bool done = tap_sum<R, ST, PLANES>(lp, tgt, W, H, c, ithr, sum, nch, lane);
+                    const bool done = tap_sum<R, ST>(lp, tgt, W, H, c, ithr, sum, nch, lane);
                     ntap += min(32 * nch, Patch<R>::T);
                     if (done && sum < bc) {
                         bc = sum;
