@@ -16,6 +16,7 @@ from __future__ import annotations
 import argparse
 import json
 import os
+import re
 import statistics
 import subprocess
 import tempfile
@@ -300,18 +301,32 @@ def measure_fp32_peak(nsm: int, gpu_id: str, launches: int = 24):
                    "(CUDA events), divided by the median SM clock sampled during them"}
 
 
-# DRAM traffic (ncu dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the kernel class, from the
-# captures summarised in profiles/ (null where the kernel changed since, or no capture matches the class).
-TRAFFIC_PER_LAUNCH = {
-    "pm_sweep": (39698432 + 256, "profiles/pm_sweep0_level0_1024x436.md"),
-    "pm_sweep_plane": (17859584 + 1024, "profiles/pm_sweep_plane_level1_1024x436.md"),
-}
-# Issue-slot utilisation of the kernel (ncu smsp__issue_active, one launch of the same workload): the sweeps are
-# bound by gather latency and issue, which the ALU fraction alone does not show.
-ISSUE_PER_LAUNCH = {
-    "pm_sweep": (0.5727, "profiles/pm_sweep0_level0_1024x436.md"),
-    "pm_sweep_plane": (0.6457, "profiles/pm_sweep_plane_level1_1024x436.md"),
-}
+# The captures of one launch of each kernel class (the same workload), summarised in profiles/.
+CAPTURES = {"pm_sweep": "profiles/pm_sweep0_level0_1024x436.md",
+            "pm_sweep_plane": "profiles/pm_sweep_plane_level1_1024x436.md"}
+
+
+def _captured(path, metric):
+    """The value of one metric in a capture's table, with its decimal unit prefix applied; None if it is not there."""
+    try:
+        with open(os.path.join(ROOT, path)) as f:
+            row = re.search(r"\(`" + re.escape(metric) + r"`\) \| ([0-9.,]+) ?(\S*)", f.read())
+    except OSError:
+        return None
+    scale = {"K": 1e3, "M": 1e6, "G": 1e9}.get(row.group(2)[:1], 1.0) if row and "byte" in row.group(2) else 1.0
+    return float(row.group(1).replace(",", "")) * scale if row else None
+
+
+def _traffic(path):
+    both = [_captured(path, f"dram__bytes_{k}.sum") for k in ("read", "write")]
+    return None if None in both else round(sum(both))
+
+
+# DRAM traffic of one launch of the class, and the share of its issue slots in use: the sweeps are bound by gather latency
+# and issue, which the ALU fraction alone does not show.
+TRAFFIC_PER_LAUNCH = {k: (_traffic(p), p) for k, p in CAPTURES.items() if _traffic(p) is not None}
+ISSUE_PER_LAUNCH = {k: (v / 100, p) for k, p in CAPTURES.items()
+                    if (v := _captured(p, "smsp__issue_active.avg.pct_of_peak_sustained_active")) is not None}
 # Algorithmic bytes of a PatchMatch sweep per pixel visit (FP32 storage): the NNF offset and cost read and
 # written (8 + 8 B) and one RGBX texel of each frame (16 + 16 B).
 PM_BYTES_PER_VISIT = 48
@@ -366,11 +381,11 @@ def roofline_block(prof, evals, nsm, clocks, peaks, steps, timed=None, fp32=None
                       "per_launch": {"evaluations": ev, "taps_summed": taps, "taps_per_evaluation": taps / max(ev, 1),
                                      "nominal_taps_per_evaluation": T}})
     elif top == "ransac":
-        # one residual test ||H u - (u + v)||^2 < t^2 in the evaluation form: 14 FP32 operations
-        ops = evals[gpm.COUNT_RANSAC] / n_prof_launches * 14
+        # one bound test ||H u - (u + v)|| < t + bound of a match: 12 FP32 operations
+        ops = evals[gpm.COUNT_RANSAC] / n_prof_launches * 12
         ach = ops / (block["avg_launch_ms"] * 1e-3) / 1e12
         block.update({"bound": "alu", "achieved": ach, "peak": peak_ops, "unit": "TFLOP/s", "frac": ach / peak_ops,
-                      "units": "FP32 lane operations (14 per residual test; hypothesis solves not counted)"})
+                      "units": "FP32 lane operations (12 per residual test; hypothesis solves not counted)"})
     else:
         block.update({"bound": "alu", "achieved": None, "peak": peak_ops, "unit": "TFLOP/s", "frac": None})
     iss = ISSUE_PER_LAUNCH.get(top)
