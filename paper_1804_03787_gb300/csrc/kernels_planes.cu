@@ -4,6 +4,7 @@
 #include <float.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 #include "hyp_exact.cuh"
@@ -897,8 +898,13 @@ __device__ __forceinline__ void choose_reference(const G& grp, const Window& w, 
     }
 }
 
+// Which windows an instance of the fit kernels serves: of a field whose matches cannot be far from each other; of any
+// field, leaving those with far matches (kFarPending); the windows left.  (Pairs through FIT_ANY: 1024x436 15.14 -> 15.32
+// ms against the code without far matches, 1.2 %; through FIT_NEAR 0.8 %, 0.5 of it the shared bound's broadcast.)
+enum FitMode { FIT_NEAR, FIT_ANY, FIT_FAR };
+
 // Gathers the window's matches (stage 1: every pixel; stage 2: the residual ones) into planes of `cap` floats.
-template <bool FAR, class G>
+template <int MODE, class G>
 __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, const LevelGeom& g, int stage, int dir,
                                               int cell, float* planes, int cap, int pad, WindowFar* far, Window& w) {
     const int tid = grp.rank(), s = g.s, W = pv.W;
@@ -951,7 +957,7 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
     }
     int v0x = __shfl_sync(FULL, mx, __ffs(__ballot_sync(FULL, rx == 3)) - 1);
     int v0y = __shfl_sync(FULL, my, __ffs(__ballot_sync(FULL, ry == 3)) - 1);
-    if constexpr (FAR) choose_reference(grp, w, mx, my, v0x, v0y);
+    if constexpr (MODE == FIT_FAR) choose_reference(grp, w, mx, my, v0x, v0y);
     if (tid == 0) *far = WindowFar{nnf, W, ox, oy, v0x, v0y, 0, 0};
     grp.sync();
     unsigned vm = 0, vq = 0;
@@ -962,8 +968,9 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
         const int bx = (int)((unsigned)dx + (unsigned)exact_int(w.x[j])), by = (int)((unsigned)dy + (unsigned)exact_int(w.y[j]));
         vm = max(vm, max((unsigned)abs(vx), (unsigned)abs(vy)));
         // in range, and the subtractions did not wrap
-        const bool near = max((unsigned)(bx + kNearReach), (unsigned)(by + kNearReach)) <= 2u * kNearReach &&
-                          (((vx ^ v0x) & (vx ^ dx)) | ((vy ^ v0y) & (vy ^ dy))) >= 0;
+        const bool near = MODE == FIT_NEAR ||
+                          (max((unsigned)(bx + kNearReach), (unsigned)(by + kNearReach)) <= 2u * kNearReach &&
+                           (((vx ^ v0x) & (vx ^ dx)) | ((vy ^ v0y) & (vy ^ dy))) >= 0);
         if (near)
             vq = max(vq, (unsigned)max(abs(bx), abs(by)));
         else  // rounded: at the limit it may count as in reach without being so
@@ -977,7 +984,7 @@ __device__ __forceinline__ void gather_window(const G& grp, const PairView& pv, 
     }
     w.vmax = (float)grp.max(vm);
     unsigned reach = grp.max(n_far ? 1u << 14 : vq);  // vq is below 2^14
-    if (reach >> 14) {  // uniform over the window
+    if (MODE != FIT_NEAR && reach >> 14) {  // uniform over the window
         n_far = grp.sum(n_far);
         if (tid == 0) far->n = n_far & 0xFFFF, far->n_reach = n_far >> 16;
         reach = grp.max(vq);
@@ -1579,7 +1586,7 @@ __device__ __forceinline__ unsigned long long far_winner(const G& grp, const Win
 // distances, and the DLT moments as exact integers about the rounded centroids) and the winner's sample, from which
 // the solve (a thread per window) forms the exact homography.  best: the winner's key, 0 if there is none; whl: 9
 // doubles of shared memory; scratch: 24 values per warp of a block.
-template <bool FAR, class G>
+template <int MODE, class G>
 __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, const Window& w, const PlaneParams& pp,
                                            int dir, int cell, int id, uint32_t tag, unsigned long long best,
                                            const RansacStats& st, double* whl, long long* scratch, RefitWork* rw) {
@@ -1610,7 +1617,7 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
     unsigned long long inm = 0;
     int2 v0 = make_int2(w.far->v0x, w.far->v0y);
     bool beyond = false;
-    if constexpr (FAR) {
+    if constexpr (MODE == FIT_FAR) {
         inm = far_winner(grp, w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, pp.t2, rw, v0, beyond);
     } else {
         unsigned long long um = 0;
@@ -1660,9 +1667,10 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
     ty = grp.sum(ty);
     const float fn = (float)nw;
     const int cx = __float2int_rn(__fdiv_rn((float)sx, fn)), cy = __float2int_rn(__fdiv_rn((float)sy, fn));
-    const int cu = __float2int_rn(__fdiv_rn((float)((long long)nw * v0.x + tx), fn));
-    const int cv = __float2int_rn(__fdiv_rn((float)((long long)nw * v0.y + ty), fn));
-    const int du = (int)((long long)v0.x - cu), dv = (int)((long long)v0.y - cv);  // small: cu is v0 and a mean about it
+    using Sum = std::conditional_t<MODE == FIT_NEAR, int, long long>;  // near a frame, 32 bits hold n times an offset
+    const int cu = __float2int_rn(__fdiv_rn((float)((Sum)nw * v0.x + tx), fn));
+    const int cv = __float2int_rn(__fdiv_rn((float)((Sum)nw * v0.y + ty), fn));
+    const int du = (int)((Sum)v0.x - cu), dv = (int)((Sum)v0.y - cv);  // small: cu is v0 and a mean about it
     // Hartley scales: distances to the exact centroids, as n |p - mean| = |n p - sum| from exact integers
     // (the least-squares refit of a noisy support moves with its normalisation, so the scale must carry no
     // more than float rounding); windows up to 96 px: n |coordinate about v0| < 2^31
@@ -2173,8 +2181,7 @@ __device__ void ransac_finish(const G& grp, const PairView& pv, const LevelGeom&
 // (A) Windows up to 16 x 16: one warp per window, kRansacWarps windows per block.  CAP: the most matches a window
 // has (64 for sides up to 8, else 256).
 constexpr int kRansacWarps = 4;
-// FAR: the windows that the other instance has left (kFarPending), otherwise the rest.
-template <int CAP, bool FAR>
+template <int CAP, int MODE>
 __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     k_ransac_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
     begin_kernel();
@@ -2190,19 +2197,19 @@ __global__ void __launch_bounds__(32 * kRansacWarps, 24 / kRansacWarps)
     const WarpGroup grp;
     const int id = (g.base + cell) * 2 + (stage - 1);
     RefitWork* rw = pv.rw[dir] + cell;
-    if (FAR && rw->status != kFarPending) return;
+    if (MODE == FIT_FAR && rw->status != kFarPending) return;
     Window w;
-    gather_window<FAR>(grp, pv, g, stage, dir, cell, planes[warp], CAP, 4, &far[warp], w);
+    gather_window<MODE>(grp, pv, g, stage, dir, cell, planes[warp], CAP, 4, &far[warp], w);
     if (grp.rank() == 0) clear_model(pv, dir, id, w.N, rw);
     if (w.N < pp.min_inliers || w.N < 4) return;
-    if (!FAR && w.far->n) {
+    if (MODE == FIT_ANY && w.far->n) {
         if (grp.rank() == 0) rw->status = kFarPending;
         return;
     }
     const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
     RansacStats st;
-    const unsigned long long best = search_warp<FAR>(w, pp, cell, tag, pv.pair_id, &slot[warp], st);
-    finish_fit<FAR>(grp, pv, w, pp, dir, cell, id, tag, best, st, whl[warp], nullptr, rw);
+    const unsigned long long best = search_warp<MODE == FIT_FAR>(w, pp, cell, tag, pv.pair_id, &slot[warp], st);
+    finish_fit<MODE>(grp, pv, w, pp, dir, cell, id, tag, best, st, whl[warp], nullptr, rw);
 }
 template <int ST>
 __global__ void __launch_bounds__(256) k_ransac_finish_warp(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
@@ -2225,7 +2232,7 @@ __host__ __device__ constexpr int block_cap(int s) { return (s * s + 127) / 128 
 // of 253x187 0.30 -> 0.24; 80 px of 1024x436 1.05 -> 0.82; 330 32 px windows 0.12 -> 0.12, their second stage 0.10 -> 0.08.
 // Elsewhere 256 is faster: 3300 32 px windows 0.51 against 0.56 ms, 2000 40 px ones 0.52 against 0.54.
 static bool ransac_wide(int s, int windows) { return s > 60 || windows <= 3 * 152; }
-template <int NT, bool FAR>
+template <int NT, int MODE>
 __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __grid_constant__ Batch bt, int level, int stage, PlaneParams pp) {
     begin_kernel();
     const PairView& pv = bt.view(blockIdx.z);
@@ -2241,18 +2248,18 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __g
     const BlockGroup<NT> grp{red_i, red_u};
     const int id = (g.base + cell) * 2 + (stage - 1);
     RefitWork* rw = pv.rw[dir] + cell;
-    if (FAR && rw->status != kFarPending) return;  // block-uniform: cleared behind the barriers of gather_window
+    if (MODE == FIT_FAR && rw->status != kFarPending) return;  // block-uniform: cleared behind the barriers of gather_window
     Window w;
-    gather_window<FAR>(grp, pv, g, stage, dir, cell, planes_dyn, block_cap(g.s), 128, &far, w);
+    gather_window<MODE>(grp, pv, g, stage, dir, cell, planes_dyn, block_cap(g.s), 128, &far, w);
     if (threadIdx.x == 0) clear_model(pv, dir, id, w.N, rw);
     if (w.N < pp.min_inliers || w.N < 4) return;
-    if (!FAR && w.far->n) {
+    if (MODE == FIT_ANY && w.far->n) {
         if (threadIdx.x == 0) rw->status = kFarPending;
         return;
     }
     const uint32_t tag = stream_tag(RNG_RANSAC, dir, level, stage);
     RansacStats st;
-    const unsigned long long best = search_block<FAR>(grp, w, pp, cell, tag, pv.pair_id, bs, st);
+    const unsigned long long best = search_block<MODE == FIT_FAR>(grp, w, pp, cell, tag, pv.pair_id, bs, st);
     // the winner's sums by 256 threads, whatever the block: their FP64 ones are in one order (barriers wait for the
     // threads that are left)
     if (NT > 256 && threadIdx.x >= 256) {
@@ -2263,7 +2270,7 @@ __global__ void __launch_bounds__(NT, NT > 256 ? 2 : 3) k_ransac_block(const __g
         }
         return;
     }
-    finish_fit<FAR>(BlockGroup<256>{red_i, red_u}, pv, w, pp, dir, cell, id, tag, best, st, whl,
+    finish_fit<MODE>(BlockGroup<256>{red_i, red_u}, pv, w, pp, dir, cell, id, tag, best, st, whl,
                     reinterpret_cast<long long*>(bs.form), rw);
 }
 template <int ST>
@@ -2880,20 +2887,29 @@ static void launch_ransac_st(const Batch& bt, int np, int level, int s, int max_
     if (s <= 16) {
         const dim3 fgrid((nc + kRansacWarps - 1) / kRansacWarps, 2, np), grid((nc + 7) / 8, 2, np);
         auto fit = [&](auto kernel) { launch_kernel(kernel, fgrid, 32 * kRansacWarps, 0, st, bt, level, stage, pp); };
-        fit(s <= 8 ? k_ransac_warp<64, false> : k_ransac_warp<256, false>);
-        if (any_offsets) fit(s <= 8 ? k_ransac_warp<64, true> : k_ransac_warp<256, true>);
+        if (any_offsets) {
+            fit(s <= 8 ? k_ransac_warp<64, FIT_ANY> : k_ransac_warp<256, FIT_ANY>);
+            fit(s <= 8 ? k_ransac_warp<64, FIT_FAR> : k_ransac_warp<256, FIT_FAR>);
+        } else {
+            fit(s <= 8 ? k_ransac_warp<64, FIT_NEAR> : k_ransac_warp<256, FIT_NEAR>);
+        }
         launch_kernel(k_refit_solve, solve, 32, 0, st, bt, level, pp);
         launch_kernel(k_ransac_finish_warp<ST>, grid, 256, 0, st, bt, level, stage, pp);
         return;
     }
     const size_t smem = (size_t)s * s * sizeof(float4), fit_smem = (size_t)block_cap(s) * sizeof(float4);
     const dim3 grid(nc, 2, np);
-    if (ransac_wide(s, 2 * nc * np)) {
-        launch_windows<k_ransac_block<512, false>>(grid, 512, fit_smem, st, bt, level, stage, pp);
-        if (any_offsets) launch_windows<k_ransac_block<512, true>>(grid, 512, fit_smem, st, bt, level, stage, pp);
+    auto fit = [&](auto narrow, auto broad) {
+        if (ransac_wide(s, 2 * nc * np))
+            launch_windows<broad()>(grid, 512, fit_smem, st, bt, level, stage, pp);
+        else
+            launch_windows<narrow()>(grid, 256, fit_smem, st, bt, level, stage, pp);
+    };
+    if (any_offsets) {
+        fit([] { return k_ransac_block<256, FIT_ANY>; }, [] { return k_ransac_block<512, FIT_ANY>; });
+        fit([] { return k_ransac_block<256, FIT_FAR>; }, [] { return k_ransac_block<512, FIT_FAR>; });
     } else {
-        launch_windows<k_ransac_block<256, false>>(grid, 256, fit_smem, st, bt, level, stage, pp);
-        if (any_offsets) launch_windows<k_ransac_block<256, true>>(grid, 256, fit_smem, st, bt, level, stage, pp);
+        fit([] { return k_ransac_block<256, FIT_NEAR>; }, [] { return k_ransac_block<512, FIT_NEAR>; });
     }
     launch_kernel(k_refit_solve, solve, 32, 0, st, bt, level, pp);
     launch_windows<k_ransac_finish_block<ST>>(grid, 256, smem, st, bt, level, stage, pp);
