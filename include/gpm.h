@@ -214,7 +214,12 @@ gpm_status gpm_sync(gpm_ctx* ctx);
    Import accepts GPM_NNF, GPM_MODELS (+ valid bits from GPM_MODEL_INFO when
    imported right after), GPM_LABELS (also sets the frozen pixels: those with
    a plane) and GPM_CUES; it sets the stage order so that the next call may
-   follow the imported state. */
+   follow the imported state.  An imported offset may be any integer, such as
+   a marker of pixels without a match: its cost is that of the border, and it
+   is a match of its window's plane like any other, except that targets 2^26
+   px and more from a hypothesis's own are not its inliers, and that samples
+   whose targets are too far apart in several directions for 128-bit products
+   (beyond some 2^27 px) are dropped. */
 enum {
     GPM_NNF = 0,
     GPM_COST = 1,
@@ -244,19 +249,24 @@ gpm_status gpm_import(gpm_ctx* ctx, int32_t pair, int32_t what, const void* src_
                               3-channel patch cost, possibly abandoned);
      GPM_COUNT_SWEEP_PLANE    the same for the restricted, plane-distorted
                               sweeps of levels >= 1;
-     GPM_COUNT_RANSAC         RANSAC residual tests (scored hypotheses x
-                              window matches);
+     GPM_COUNT_RANSAC         RANSAC residual tests of the search: a
+                              hypothesis is tested until it cannot win, and a
+                              contender's tests are counted again;
      GPM_COUNT_INIT           evaluations of the initial field and recosts;
      GPM_COUNT_SWEEP0_TAPS    taps the level-0 sweep evaluations actually
                               summed (an abandoned evaluation stops early);
      GPM_COUNT_SWEEP_PLANE_TAPS  the same for the plane-level sweeps;
      GPM_COUNT_SWEEP0_PRUNED  level-0 sweep candidates rejected without any
-                              tap by the patch-sum lower bound (not counted
-                              as evaluations);
-     GPM_COUNT_RANSAC_FP64    RANSAC residual tests whose FP32 decision was
-                              within its rounding bound, decided again in FP64;
-     GPM_COUNT_RANSAC_LOOSE   hypotheses whose window-wide rounding bound was
-                              too loose, tested with a bound per match.
+                              tap by a lower bound, of the patch sums or of
+                              its nine regions (not counted as evaluations;
+                              what the plane levels' interval bound rejects is
+                              counted nowhere);
+     GPM_COUNT_RANSAC_FP64    RANSAC residual tests of the search whose FP32
+                              decision was within its rounding bound, or whose
+                              match is far from its window's others, decided
+                              in FP64 (not those of the winner afterwards);
+     GPM_COUNT_RANSAC_LOOSE   hypotheses whose FP32 form says too little,
+                              counted from their exact form at once.
    gpm_profile_read synchronises the stream, returns per kernel class the
    summed device milliseconds and the launch count, and the GPM_COUNTERS
    counts, then clears them.  Host arrays: ms[GPM_PROF_CLASSES],
@@ -324,8 +334,8 @@ gpm_status gpm_fp32_peak_probe(int32_t blocks, int32_t iters, float* sink, void*
    (GPM_F32: 16 bytes each, GPM_F16 / GPM_BF16: 8 bytes); with equalize, each
    frame's HSV value histogram is equalised first (Sec. 4.2); with
    gain_normalize, frame 2 is then scaled by mean(I1) / mean(I2).
-   It allocates nothing: its scratch is one static device array of 6.25 KiB
-   (partial sums, the gain, the histograms and tables), held on every GPU that
+   It allocates nothing: its scratch is one static device array of 6 KiB
+   (partial sums, the histograms and tables), held on every GPU that
    loads the library until the process exits.  Frames up to 32767 x 32767
    and 2^26 pixels (the largest frame a context takes); larger ones, NULL
    pointers, a row stride below 3 * width or a bad storage / equalize value

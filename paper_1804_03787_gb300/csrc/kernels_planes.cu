@@ -1723,7 +1723,8 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
 // those one by one with its lanes over the matches.
 // What bounds it: instruction fetch, then the FP32 pipe in the tests (12 operations a match).  1024x436, stage 1:
 // the 16 px windows 1.44 -> 0.41 ms, the 8 px windows 1.73 -> 0.53 ms, against scoring exact 128-bit hypotheses
-// (0.64 and 1.12 ms of these gains while the winner was still solved here, in 180 KB of code, not 97).
+// (0.64 and 1.12 ms of these gains while the winner was still solved here, in 180 KB of code, not 97; an integer
+// reference offset has since cost 5 %: 8 px 0.67 -> 0.70 ms, a capture each).
 template <bool FAR>
 __device__ __forceinline__ unsigned long long search_warp(const Window& w, const PlaneParams& pp, int cell,
                                                           uint32_t tag, uint32_t pair_id, FastHyp* slot,
@@ -1784,7 +1785,8 @@ __device__ __forceinline__ unsigned long long search_warp(const Window& w, const
 // one with the most is counted from below on all of them, by the whole block, which gives the bound the others have
 // to reach from the start; then the warps take the hypotheses that still can, one at a time, chunk by chunk.
 // What bounds it: the FP32 pipe and the shared loads of the tests.  1024x436, stage 1: the 64 px windows 1.99 ->
-// 0.77 ms, the 32 px windows 1.03 -> 0.47 ms, against scoring in index order from exact 128-bit hypotheses.
+// 0.77 ms, the 32 px windows 1.03 -> 0.47 ms, against scoring in index order from exact 128-bit hypotheses (reading the
+// bound once a warp has since cost 7 %: 64 px 0.73 -> 0.79 ms, a capture each; reading it every fourth chunk gained nothing).
 constexpr int kHypRound = 256;
 struct BlockSearch {
     FastHyp form[kHypRound];

@@ -246,8 +246,8 @@ class Context:
     def profile_read(self):
         """{class: (ms, launches)} and the work counts (a tuple indexed by the COUNT_* constants: level-0 sweep
         evaluations, plane-level sweep evaluations, RANSAC residual tests, init / recost evaluations, taps summed by
-        the level-0 sweeps, taps summed by the plane-level sweeps, level-0 candidates rejected by the patch-sum bound,
-        RANSAC tests decided in FP64, RANSAC hypotheses tested with per-match bounds); clears them."""
+        the level-0 sweeps, taps summed by the plane-level sweeps, level-0 candidates rejected by a lower bound,
+        RANSAC tests decided in FP64, RANSAC hypotheses counted from their exact form at once); clears them."""
         k = len(PROF_CLASSES)
         ms = (C.c_double * k)()
         ln = (C.c_uint64 * k)()
