@@ -313,11 +313,17 @@ gpm_status set_dims(gpm_ctx* c, Slot& s, int W, int H) {
 unsigned long long capture_id(gpm_ctx* c) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     unsigned long long id = 0;
-    if (cudaStreamGetCaptureInfo(c->stream, &st, &id) != cudaSuccess) {
-        cudaGetLastError();
-        return ~0ull;
-    }
+    const cudaError_t e = cudaStreamGetCaptureInfo(c->stream, &st, &id);
+    if (e == cudaErrorStreamCaptureImplicit) cudaGetLastError();  // another stream's capture; other errors stay to be reported
+    if (e != cudaSuccess) return ~0ull;
     return st == cudaStreamCaptureStatusNone ? 0 : id;
+}
+
+// The pair's field holds imported offsets from here on, or will (Slot::any_offsets).
+void imported_offsets(gpm_ctx* c, Slot& s) {
+    s.any_offsets = true;
+    s.any_in_graph = s.any_in_graph || capture_id(c) != 0;
+    s.init_capture = 0;
 }
 
 // Whether a window of the pairs [0, np) may hold matches that are far from each other (kNearOffsets): fields that match
@@ -830,9 +836,7 @@ gpm_status gpm_import(gpm_ctx* c, int32_t pair, int32_t what, const void* src, i
         case GPM_NNF:
             for (int k = 0; k < 2; ++k)
                 cudaMemcpyAsync(s.pv.nnf[k], d + k * n * sizeof(int2), n * sizeof(int2), cudaMemcpyDeviceToDevice, st);
-            s.any_offsets = true;
-            s.any_in_graph = s.any_in_graph || capture_id(c) != 0;
-            s.init_capture = 0;
+            imported_offsets(c, s);
             break;
         case GPM_MODELS:
             for (int k = 0; k < 2; ++k)
@@ -858,6 +862,7 @@ gpm_status gpm_import(gpm_ctx* c, int32_t pair, int32_t what, const void* src, i
                 launch_labels_import(s.pv.acc[k], s.n, s.m, im + k * n, iL + k * n, iF + k * n * 2, s.pv.flag, st);
                 c->launches += 1;
             }
+            imported_offsets(c, s);  // the next merge makes the labels' flows the pixels' offsets
             // frozen pixels and the restricted PatchMatch lists follow the accumulated map
             launch_frozen_from_labels(batch(c, pair, 1), 1, grid_for(c, s.n), st);
             c->launches += 1;

@@ -169,3 +169,37 @@ def test_far_windows_are_fitted_by_graphs_captured_before_an_import():
         ctx.close()
     assert (want[0][:, ::2, 1] > 0).any()  # inliers: the cues drop these planes later
     assert (got[0] == want[0]).all() and (got[1] == want[1]).all()
+
+
+def test_far_flows_of_imported_labels_reach_the_next_level_exactly():
+    """A merge makes the flows of imported labels the pixels' offsets: the fit after it takes them as it takes an imported
+    field with the same offsets."""
+    import torch
+
+    import oracle as O
+
+    from _parity import oracle_params
+    W, H = 53, 41
+    gp = gpm.default_params(patch_radius=2, cells=(16, 8), pm_iters=2, num_hyp=64)
+    rng = np.random.default_rng(9)
+    f = torch.from_numpy(rng.random((H, W, 3)).astype(np.float32)).cuda()
+    far = rng.random((2, W * H)) < 0.3
+    labels = (np.where(far, 0, -1).astype(np.int32), np.zeros((2, W * H), np.float32),
+              np.where(far[..., None], 2.0**29, 0.0) + np.zeros(2))
+    got = []
+    for again in (False, True):
+        ctx = gpm.Context(gp, W, H)
+        ctx.match([(f, f)])
+        ctx.import_state(gpm.LABELS, labels, level=0)
+        ctx.fit_planes(1)
+        ctx.match(None, 1)
+        field = ctx.export(gpm.NNF)
+        assert (field[far] == 1 << 29).all()
+        if again:
+            ctx.import_state(gpm.NNF, field, level=1)
+        ctx.fit_planes(2)
+        got.append((ctx.export(gpm.MODEL_INFO), ctx.export(gpm.MODELS)))
+        ctx.close()
+    level2 = 2 * int(O.cell_base(oracle_params(gp, W, H))[1])
+    assert (got[1][0][:, level2::2, 1] >= 32).any()  # planes of the near matches, half of a window and more
+    assert (got[0][0] == got[1][0]).all() and (got[0][1] == got[1][1]).all()
