@@ -454,7 +454,7 @@ struct Labels {
 // Per-window record of the RANSAC refit, filled in three launches (fit,
 // solve, finish) and reused by every level and stage.
 struct __align__(16) RefitWork {
-    long long mom[24];      // exact DLT moments of the winner's inliers about (cx, cy, cu, cv)
+    long long mom[24];      // exact DLT moments of the winner's inliers about (cx, cy, cu, cv); wide: doubles
     int sample[8];          // the winner's sample, window-local: source x[4], y[4]
     long long target[8];    // and target x[4], y[4]
     Mef mef0, mef1;         // evaluation forms (origin 0) of the winner and of the refit, with test bounds
@@ -463,6 +463,7 @@ struct __align__(16) RefitWork {
     double ds, dt;          // sums of nin times the inliers' distances to the source / target centroids
     double ha_w[9], ha_r[9];  // absolute homographies of the winner and of the refit
     int cx, cy, cu, cv;     // integer centres of the moments
+    int wide;               // the moments are the bits of doubles (inliers too far apart)
     int status;             // 1: fit pending (far matches); 2: refit pending (set by the fit); else the window is final
     int nin;                // winner's inliers
     int refit_ok, geo_w, geo_r;

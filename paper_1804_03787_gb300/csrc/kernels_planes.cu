@@ -101,6 +101,11 @@ struct WarpGroup {
     __device__ int rank() const { return threadIdx.x & 31; }
     __device__ void sync() const { __syncwarp(); }
     __device__ int sum(int v) const { return (int)__reduce_add_sync(FULL, (unsigned)v); }
+    __device__ long long sum(long long v) const {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+        return v;
+    }
     __device__ unsigned max(unsigned v) const { return __reduce_max_sync(FULL, v); }
     __device__ bool any(bool p) const { return __any_sync(FULL, p); }
     // exclusive prefix of `take` over the group and the total
@@ -125,6 +130,15 @@ struct BlockGroup {
         __syncthreads();
         int t = 0;
         for (int w = 0; w < NT / 32; ++w) t += red_i[w];
+        return t;
+    }
+    __device__ long long sum(long long v) const {
+        v = WarpGroup().sum(v);
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) red_u[threadIdx.x >> 5] = (unsigned long long)v;
+        __syncthreads();
+        long long t = 0;
+        for (int w = 0; w < NT / 32; ++w) t += (long long)red_u[w];
         return t;
     }
     __device__ unsigned max(unsigned v) const {
@@ -1532,14 +1546,13 @@ __device__ __noinline__ void winner_fp64(const Window& w, int cell, int k, uint3
 
 // finish_fit's first part in a window with far matches: the winner's inliers among this thread's matches, all decided in
 // FP64, its sample into rw, and, if there are far inliers, the inliers' targets in the planes about another reference, the
-// offset of the winner's first match, now in v0: far inliers are near it.  beyond: one is beyond kRefitReach of it all the
-// same, which leaves the window without a refit (inliers so far apart are no plane of any scale in use, and their sums
-// would not fit: within it an inlier is at most 3/4 of their span from their mean, and squares stay below 2^30).
+// offset of the winner's first match, now in v0: far inliers are near it.  wide: one is not within kPlaneReach of it (within
+// it an inlier is at most 3/4 of their span from their mean, and squares stay below 2^30); then nothing is moved.
 template <class G>
 __device__ __forceinline__ unsigned long long far_winner(const G& grp, const Window& w, int cell, int k, uint32_t tag,
                                                       uint32_t pair_id, uint32_t k0, uint32_t k1, float t2, RefitWork* rw,
-                                                      int2& v0, bool& beyond) {
-    constexpr int kRefitReach = 20000;
+                                                      int2& v0, bool& wide) {
+    constexpr int kPlaneReach = 20000;
     const int tid = grp.rank();
     double Hl[9];
     Mef m;
@@ -1562,24 +1575,90 @@ __device__ __forceinline__ unsigned long long far_winner(const G& grp, const Win
         rw->target[tid] = v0.x + q.x;
         rw->target[4 + tid] = v0.y + q.y;
     }
-    beyond = false;
+    wide = false;
     if (!grp.any(far)) return inm;
     longlong2 shift = w.target(idx[0]);
     shift.x -= exact_int(w.x[idx[0]]);
     shift.y -= exact_int(w.y[idx[0]]);
+    for (unsigned long long b = inm; b; b &= b - 1) {
+        const longlong2 q = w.target(tid + (__ffsll((long long)b) - 1) * G::size);
+        wide = wide || max(llabs(q.x - shift.x), llabs(q.y - shift.y)) > kPlaneReach;
+    }
+    wide = grp.any(wide);
     grp.sync();  // the targets are read
+    if (wide) return inm;
     for (unsigned long long b = inm; b; b &= b - 1) {
         const int j = tid + (__ffsll((long long)b) - 1) * G::size;
-        longlong2 q = w.target(j);
-        q.x -= shift.x;
-        q.y -= shift.y;
-        beyond = beyond || max(llabs(q.x), llabs(q.y)) > kRefitReach;
-        w.qx[j] = beyond ? 0.f : (float)(int)q.x;
-        w.qy[j] = beyond ? 0.f : (float)(int)q.y;
+        const longlong2 q = w.target(j);
+        w.qx[j] = (float)(int)(q.x - shift.x);
+        w.qy[j] = (float)(int)(q.y - shift.y);
     }
     v0 = make_int2((int)(v0.x + shift.x), (int)(v0.y + shift.y));
-    beyond = grp.any(beyond);
     return inm;
+}
+
+// The refit's inputs for inliers whose targets are too far apart for 32 bits (a plane whose vanishing line passes by some of
+// them): the same sums, the moments in 128 bits and stored as doubles (RefitWork::wide).
+template <class G>
+__device__ __noinline__ void wide_sums(const G& grp, const Window& w, unsigned long long inm, int nw, int2 v0, double* whl,
+                                       RefitWork* rw) {
+    const int tid = grp.rank();
+    int sx = 0, sy = 0;
+    long long tx = 0, ty = 0;
+    for (unsigned long long b = inm; b; b &= b - 1) {
+        const int j = tid + (__ffsll((long long)b) - 1) * G::size;
+        const longlong2 q = w.target(j);
+        sx += exact_int(w.x[j]);
+        sy += exact_int(w.y[j]);
+        tx += q.x;
+        ty += q.y;
+    }
+    sx = grp.sum(sx);
+    sy = grp.sum(sy);
+    tx = grp.sum(tx);
+    ty = grp.sum(ty);
+    const double n = nw, lim = 2147483000.0;
+    const int cx = __double2int_rn(sx / n), cy = __double2int_rn(sy / n);
+    const int cu = __double2int_rn(fmin(fmax(tx / n + v0.x, -lim), lim));
+    const int cv = __double2int_rn(fmin(fmax(ty / n + v0.y, -lim), lim));
+    double ds = 0.0, dt = 0.0;
+    for (unsigned long long b = inm; b; b &= b - 1) {
+        const int j = tid + (__ffsll((long long)b) - 1) * G::size;
+        const longlong2 q = w.target(j);
+        const double ax = n * exact_int(w.x[j]) - sx, ay = n * exact_int(w.y[j]) - sy;
+        const double bx = n * (double)q.x - (double)tx, by = n * (double)q.y - (double)ty;
+        ds += sqrt(fma(ax, ax, ay * ay));
+        dt += sqrt(fma(bx, bx, by * by));
+    }
+#pragma unroll 1
+    for (int k = 0; k < 24; ++k) {
+        i128 m = 0;
+        for (unsigned long long b = inm; b; b &= b - 1) {
+            const int j = tid + (__ffsll((long long)b) - 1) * G::size;
+            const longlong2 q = w.target(j);
+            const int X = exact_int(w.x[j]) - cx, Y = exact_int(w.y[j]) - cy;
+            const long long U = q.x + v0.x - cu, V = q.y + v0.y - cv;
+            const int e = k % 6, z = e == 0 ? X * X : (e == 1 ? X * Y : (e == 2 ? X : (e == 3 ? Y * Y : (e == 4 ? Y : 1))));
+            m += (k < 6 ? (i128)1 : (k < 12 ? (i128)U : (k < 18 ? (i128)V : (i128)U * U + (i128)V * V))) * z;
+        }
+        i128 t = 0;  // the group's, by 32-bit limbs
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            const long long limb = l < 3 ? (long long)(uint32_t)(m >> (32 * l)) : (long long)(m >> 96);
+            t += (i128)grp.sum(limb) * ((i128)1 << (32 * l));
+        }
+        const bool neg = t < 0;
+        const u128 a = neg ? (u128)0 - (u128)t : (u128)t;
+        const double d = (double)(unsigned long long)(a >> 64) * 18446744073709551616.0 + (double)(unsigned long long)a;
+        if (tid == 0) rw->mom[k] = __double_as_longlong(neg ? -d : d);
+    }
+    group_dists(grp, ds, dt, whl, rw);
+    if (tid == 0) {
+        rw->cx = cx;
+        rw->cy = cy;
+        rw->cu = cu;
+        rw->cv = cv;
+    }
 }
 
 // What follows the search: the refit's inputs on the winner's inliers (Hartley centroids as exact integer sums,
@@ -1616,9 +1695,9 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
     static_assert(kMaxCell * kMaxCell <= 64 * 256 && 16 * 16 <= 64 * 32, "inlier mask too small");
     unsigned long long inm = 0;
     int2 v0 = make_int2(w.far->v0x, w.far->v0y);
-    bool beyond = false;
+    bool wide = false;
     if constexpr (MODE == FIT_FAR) {
-        inm = far_winner(grp, w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, pp.t2, rw, v0, beyond);
+        inm = far_winner(grp, w, cell, wk, tag, pv.pair_id, pp.k0, pp.k1, pp.t2, rw, v0, wide);
     } else {
         unsigned long long um = 0;
         {
@@ -1653,6 +1732,13 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
             rw->target[4 + tid] = (long long)v0.y + exact_int(w.qy[j]);
         }
     }
+    if (tid == 0) {
+        rw->nin = nw;
+        rw->vmax = w.vmax;
+        rw->wide = wide;
+        rw->status = 2;
+    }
+    if (MODE == FIT_FAR && wide) return wide_sums(grp, w, inm, nw, v0, whl, rw);
     int sx = 0, sy = 0, tx = 0, ty = 0;  // target sums about v0
     for (unsigned long long m = inm; m; m &= m - 1) {
         const int j = tid + (__ffsll((long long)m) - 1) * G::size;
@@ -1695,7 +1781,6 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
             R[18 + q] += (long long)w3 * zz[q];
         }
     }
-    if (beyond) ds = dt = 0.0;  // no extent: no refit
     group_dists(grp, ds, dt, reinterpret_cast<double*>(whl), rw);
     group_moments(grp, R, scratch, rw->mom);
     if (tid == 0) {
@@ -1703,9 +1788,6 @@ __device__ __forceinline__ void finish_fit(const G& grp, const PairView& pv, con
         rw->cy = cy;
         rw->cu = cu;
         rw->cv = cv;
-        rw->nin = nw;
-        rw->vmax = w.vmax;
-        rw->status = 2;
     }
 }
 
@@ -1950,6 +2032,10 @@ __device__ __forceinline__ bool refit_system(RefitWork* rw, const LevelGeom& g, 
     double R[24];
 #pragma unroll
     for (int q = 0; q < 24; ++q) R[q] = (double)rw->mom[q];  // exact: |moment| < 2^53
+    if (rw->wide) {
+#pragma unroll
+        for (int q = 0; q < 24; ++q) R[q] = __longlong_as_double(rw->mom[q]);
+    }
     const double inv_n = 1.0 / (double)rw->nin;
     const double dx = R[2] * inv_n, dy = R[4] * inv_n, du = R[11] * inv_n, dv = R[17] * inv_n;
     const double mx = rw->cx + dx, my = rw->cy + dy, mqx = rw->cu + du, mqy = rw->cv + dv;

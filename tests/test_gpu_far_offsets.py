@@ -203,3 +203,40 @@ def test_far_flows_of_imported_labels_reach_the_next_level_exactly():
     level2 = 2 * int(O.cell_base(oracle_params(gp, W, H))[1])
     assert (got[1][0][:, level2::2, 1] >= 32).any()  # planes of the near matches, half of a window and more
     assert (got[0][0] == got[1][0]).all() and (got[0][1] == got[1][1]).all()
+
+
+@pytest.mark.parametrize("W,H,s,hyp", [(53, 41, 16, 128), (37, 29, 8, 96), (41, 30, 18, 96), (200, 160, 18, 257)])
+@pytest.mark.parametrize("gain", [30.0, 300.0])
+def test_planes_that_reach_far_equal_oracle(gain, W, H, s, hyp):
+    """A projective motion whose vanishing line passes just beyond the right border: inliers of one plane lie 10^4 to 10^6 px
+    apart, too far for 32-bit sums."""
+    import torch
+
+    import oracle as O
+
+    from _parity import oracle_params, ransac_equal
+    gp = gpm.default_params(patch_radius=2, cells=(s,), pm_iters=0, num_hyp=hyp, min_inliers=4)
+    P = oracle_params(gp, W, H)
+    f = np.random.default_rng(s).random((H, W, 3)).astype(np.float32) * 0.2 + 0.4
+    y, x = np.mgrid[0:H, 0:W].astype(np.float64)
+    den = 1 - (x + 0.1 * y) / (W + 0.1 * H)
+    v = np.stack([np.rint(gain * (x - W / 2) / den) - x, np.rint(gain * (y - H / 2) / den) - y], -1).reshape(-1, 2).astype(np.int32)
+    assert np.abs(v).max() > 16383  # beyond what a window holds as near
+    nnf = np.stack([v, v[::-1]])
+    ctx = gpm.Context(gp, W, H)
+    fr = torch.from_numpy(f).cuda()
+    ctx.match([(fr, fr.clone())])
+    ctx.import_state(gpm.NNF, nnf, level=0)
+    ctx.fit_planes(1)
+    gmh, gmi = ctx.export(gpm.MODELS), ctx.export(gpm.MODEL_INFO)
+    ctx.close()
+    frame = np.asarray(f, np.float64)
+    first = np.arange(int(O.cell_base(P)[1])) * 2
+    for d in range(2):
+        mh, mi = O.empty_models(P)
+        vx, vy = (np.ascontiguousarray(nnf[d][:, c]) for c in range(2))
+        O.fit_level(P, frame, frame, d, 1, 1, vx, vy, None, mh, mi)
+        sure = first[(mi[first, O.MI_FLAGS] & O.F_AMBIG) == 0]
+        assert len(sure) > len(first) // 4
+        bad = sure[~ransac_equal(gmh[d], gmi[d], mh, mi, sure)]
+        assert len(bad) == 0, f"dir {d}: windows {bad // 2} differ"
