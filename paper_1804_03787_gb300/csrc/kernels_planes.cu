@@ -2194,17 +2194,24 @@ __device__ void ransac_finish(const G& grp, const PairView& pv, const LevelGeom&
     window_origin<G>(g, cell, x0, y0, ox, oy);
     const int W = pv.W, H = pv.H;
     const float t2 = pp.t2;
+    const int2* nnf = pv.nnf[dir];
+    // a match's test, certified: FP64 where the FP32 form cannot tell, or its offset is no exact float
+    auto inlier = [&](const Mef& m, const double* Hl, const float4& mt) {
+        bool unc;
+        const bool in = cert_inlier(m, mt, t2, unc), far = fmaxf(fabsf(mt.z), fabsf(mt.w)) >= 16777216.f;
+        if (!(unc || far)) return in;
+        int2 v = make_int2(0, 0);
+        if (far) v = nnf[(oy + (int)mt.y) * W + ox + (int)mt.x];
+        return hyp_inlier_fp64(Hl, (double)mt.x, (double)mt.y, (double)mt.x + (far ? (double)v.x : (double)mt.z),
+                               (double)mt.y + (far ? (double)v.y : (double)mt.w), (double)t2);
+    };
     const int wscore = rw->nin;
     const bool have_refit = rw->refit_ok != 0;
     int rcount = 0;
     if (have_refit) {
         const Mef rm = rw->mef1;
         for (int j = tid; j < N; j += G::size) {
-            const float4 mt = match[j];
-            bool unc;
-            bool in = cert_inlier(rm, mt, t2, unc);
-            if (unc) in = hyp_inlier_fp64(rw->hl_r, mt.x, mt.y, mt.z, mt.w, (double)t2);
-            rcount += in;
+            rcount += inlier(rm, rw->hl_r, match[j]);
         }
     }
     rcount = grp.sum(rcount);
@@ -2220,10 +2227,7 @@ __device__ void ransac_finish(const G& grp, const PairView& pv, const LevelGeom&
     int nrc = 0;
     for (int j = tid; j < N; j += G::size) {
         const float4 mt = match[j];
-        bool unc;
-        bool in = cert_inlier(fm, mt, t2, unc);
-        if (unc) in = hyp_inlier_fp64(Hl, mt.x, mt.y, mt.z, mt.w, (double)t2);
-        if (!in) continue;
+        if (!inlier(fm, Hl, mt)) continue;
         const int px = ox + (int)mt.x, py = oy + (int)mt.y;
         int ix, iy, kx, ky;
         float fx, fy;

@@ -240,3 +240,10 @@ def test_planes_that_reach_far_equal_oracle(gain, W, H, s, hyp):
         assert len(sure) > len(first) // 4
         bad = sure[~ransac_equal(gmh[d], gmi[d], mh, mi, sure)]
         assert len(bad) == 0, f"dir {d}: windows {bad // 2} differ"
+
+
+@pytest.mark.parametrize("mark", [(1 << 24) + 3, -(1 << 30) - 12345, (1 << 31) - 129])
+def test_planes_of_markers_that_are_no_floats_equal_oracle(mark):
+    """Far offsets that FP32 rounds by more than the inlier radius: the refit is tested on the matches as they are."""
+    test_planes_of_marked_fields_equal_oracle(mark, 0.75, 53, 41, 16, 128)
+    test_planes_of_marked_fields_equal_oracle(mark, 0.75, 41, 30, 18, 96)
